@@ -1,5 +1,5 @@
 // fdas_api.cu -- the C ABI of libfdas (declared in include/fdas.h): plan life cycle, argument
-// validation, the FP64 template-bank build (step a1) and the launch of the fused kernel.
+// validation and the launch of the fused kernel.
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -42,154 +42,14 @@ namespace {
 
 thread_local int g_last_error = FDAS_OK;
 
-constexpr int kGLPoints = 16;
-__constant__ double c_gl_x[kGLPoints];   // Gauss-Legendre nodes on [-1, 1]
-__constant__ double c_gl_w[kGLPoints];   // and weights
-
-// Gauss-Legendre nodes and weights by Newton iteration on the Legendre polynomial P_n, using
-// the three-term recurrence (n+1) P_{n+1} = (2n+1) x P_n - n P_{n-1} and
-// P_n'(x) = n (x P_n - P_{n-1}) / (x^2 - 1); w_i = 2 / ((1 - x_i^2) P_n'(x_i)^2).
-void gauss_legendre(int n, double* x, double* w) {
-  const double pi = 3.14159265358979323846;
-  for (int i = 0; i < n; ++i) {
-    double z = std::cos(pi * (i + 0.75) / (n + 0.5));
-    double dp = 0.0;
-    for (int it = 0; it < 100; ++it) {
-      double p0 = 1.0, p1 = z;
-      for (int k = 2; k <= n; ++k) {
-        const double p2 = ((2.0 * k - 1.0) * z * p1 - (k - 1.0) * p0) / k;
-        p0 = p1;
-        p1 = p2;
-      }
-      dp = n * (z * p1 - p0) / (z * z - 1.0);
-      const double dz = p1 / dp;
-      z -= dz;
-      if (std::fabs(dz) < 1e-16) break;
-    }
-    x[i] = z;
-    w[i] = 2.0 / ((1.0 - z * z) * dp * dp);
-  }
-}
-
-// The quadrature rule, computed once per process (a function-local static is initialised
-// exactly once even when several host threads build plans at the same time).
-struct GLTable {
-  double x[kGLPoints], w[kGLPoints];
-  GLTable() { gauss_legendre(kGLPoints, x, w); }
-};
-const GLTable& gl_table() {
-  static const GLTable table;
-  return table;
-}
-
-// a1, part 1: raw response H_q(z) = int_0^1 exp(i pi (z u^2 - (z+2q) u)) du by composite
-// 16-point Gauss-Legendre quadrature (panels short enough that the phase turns by at most
-// ~4 rad per panel), then normalisation to unit L2 norm over q = -h..h.  One block per z.
-__global__ void taps_kernel(double2* taps, int zmax, int zstep, int h) {
-  const int zi = blockIdx.x;
-  const double z = (double)(-zmax + zi * zstep);
-  const int ntap = 2 * h + 1;
-  double2* row = taps + (size_t)zi * ntap;
-  double part = 0.0;
-  for (int j = threadIdx.x; j < ntap; j += blockDim.x) {
-    const double q = (double)(j - h);
-    const double b = z + 2.0 * q;
-    const int panels = (int)ceil(3.14159265358979323846 * (fabs(z) + 2.0 * fabs(q) + 1.0) / 4.0) + 1;
-    const double width = 1.0 / panels;
-    double re = 0.0, im = 0.0;
-    for (int k = 0; k < panels; ++k) {
-      const double mid = (k + 0.5) * width;
-      double pr = 0.0, pi = 0.0;
-#pragma unroll
-      for (int g = 0; g < kGLPoints; ++g) {
-        const double u = mid + 0.5 * width * c_gl_x[g];
-        double sn, cs;
-        sincospi(z * u * u - b * u, &sn, &cs);
-        pr += c_gl_w[g] * cs;
-        pi += c_gl_w[g] * sn;
-      }
-      re += pr;
-      im += pi;
-    }
-    re *= 0.5 * width;
-    im *= 0.5 * width;
-    row[j] = make_double2(re, im);
-    part += re * re + im * im;
-  }
-  __shared__ double red[256];
-  red[threadIdx.x] = part;
-  __syncthreads();
-  for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-    if ((int)threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
-    __syncthreads();
-  }
-  const double scale = 1.0 / sqrt(red[0]);
-  for (int j = threadIdx.x; j < ntap; j += blockDim.x) {
-    const double2 v = row[j];
-    row[j] = make_double2(v.x * scale, v.y * scale);
-  }
-}
-
 // Float offset of the real part of element k in the pair-major structure-of-arrays layout
 // (lane k1 = k % n1, k2 = k / n1; pair p = k2/2 of lane k1 is the float4 at p*n1 + k1 holding
 // re(2p), re(2p+1), im(2p), im(2p+1)); the imaginary part is 2 floats further.  n1 = 0 is the
 // interleaved natural order, where the imaginary part is the next float.
-__host__ __device__ __forceinline__ int pair_layout_re(int k, int n1) {
+int pair_layout_re(int k, int n1) {
   if (n1 == 0) return 2 * k;   // natural order (L >= 4096)
   const int k1 = k % n1, k2 = k / n1;
   return ((k2 >> 1) * n1 + k1) * 4 + (k2 & 1);
-}
-
-// a1, part 2: T_z[k] = (1/L) sum_{j=0}^{m} conj(Hn_{j-h}) exp(+i 2pi k j / L) in FP64 (the
-// conjugated template placed at circular index q + h, so that the correlation's valid outputs
-// are the first V of each segment), rounded to complex64 and stored in the kernel layout.
-// grid (L/256, Z), 256 threads; dynamic shared memory L double2 of exp(+i 2pi j / L).
-__global__ void spectra_kernel(const double2* taps, float2* templates, int L, int h, int n1) {
-  extern __shared__ double2 e_tab[];
-  for (int j = threadIdx.x; j < L; j += blockDim.x) {
-    double sn, cs;
-    sincospi(2.0 * (double)j / (double)L, &sn, &cs);
-    e_tab[j] = make_double2(cs, sn);
-  }
-  __syncthreads();
-  const int zi = blockIdx.y;
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= L) return;
-  const int ntap = 2 * h + 1;
-  const double2* row = taps + (size_t)zi * ntap;
-  double re = 0.0, im = 0.0;
-  for (int j = 0; j < ntap; ++j) {
-    const double2 hq = row[j];
-    const double2 e = e_tab[(int)(((long long)k * j) % L)];
-    re += hq.x * e.x + hq.y * e.y;   // Re(conj(h) e)
-    im += hq.x * e.y - hq.y * e.x;   // Im(conj(h) e)
-  }
-  float* dst = reinterpret_cast<float*>(templates + (size_t)zi * L);
-  const int off = pair_layout_re(k, n1);
-  dst[off] = (float)(re / L);
-  dst[off + (n1 ? 2 : 1)] = (float)(im / L);
-}
-
-// Inter-pass twiddles exp(+i 2pi n2 k1 / L), n2 < N2 = L/n1, k1 < n1: lane k1's pair j holds
-// n2 = j and n2 = j + N2/2 (float4 at j*n1 + k1: re, re, im, im).  n1 = 0 (L >= 4096): the
-// natural table exp(-2 pi i t / L).
-__global__ void twist_kernel(float2* tw, int L, int n1) {
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= L) return;
-  if (n1 == 0) {   // L >= 4096: W[t] = exp(-2 pi i t / L) for the Stockham passes
-    double sn, cs;
-    sincospi(2.0 * (double)idx / (double)L, &sn, &cs);
-    tw[idx] = make_float2((float)cs, (float)-sn);
-    return;
-  }
-  const int k1 = idx % n1, n2 = idx / n1;
-  const int h2 = L / n1 / 2;
-  double sn, cs;
-  sincospi(2.0 * (double)(((long long)n2 * k1) % L) / (double)L, &sn, &cs);
-  float* dst = reinterpret_cast<float*>(tw);
-  const int off = ((n2 % h2) * n1 + k1) * 4 + n2 / h2;
-  dst[off] = (float)cs;
-  dst[off + 2] = (float)sn;
 }
 
 // Failure-detection self test: one thread waits, with the given bound, on an mbarrier whose
@@ -685,29 +545,13 @@ int fdas_template_spectrum(fdas_plan* p, int z_idx, float* host_out) {
 }  // extern "C"
 
 // ---------------------------------------------------------------------------------------
-// Helpers for the allocation-free entry point (fdas_static.cu): the same validation, template
-// build kernels and tensor-map encoding as the plan-based calls above, on caller-given memory.
+// Helpers for the allocation-free entry point (fdas_static.cu): the same validation and
+// tensor-map encoding as the plan-based calls above, on caller-given memory.
 // ---------------------------------------------------------------------------------------
 namespace fdas {
 
 int validate_geometry(int64_t n_bins, int zmax, int zstep, int seg_len, int tmpl_len) {
   return validate(n_bins, zmax, zstep, seg_len, tmpl_len);
-}
-
-cudaError_t build_templates_into(double2* taps, float2* templates, float2* twist, int zmax, int zstep, int L,
-                                 int m, cudaStream_t st) {
-  const GLTable& gl = gl_table();
-  cudaError_t e = cudaMemcpyToSymbolAsync(c_gl_x, gl.x, sizeof(gl.x), 0, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaMemcpyToSymbolAsync(c_gl_w, gl.w, sizeof(gl.w), 0, cudaMemcpyHostToDevice, st);
-  if (e != cudaSuccess) return e;
-  const int Z = 2 * (zmax / zstep) + 1, h = m / 2, n1 = conv_group_threads(L);
-  taps_kernel<<<Z, 256, 0, st>>>(taps, zmax, zstep, h);
-  const size_t tab = sizeof(double2) * (size_t)L;
-  e = cudaFuncSetAttribute(spectra_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tab);
-  if (e != cudaSuccess) return e;
-  spectra_kernel<<<dim3((L + 255) / 256, Z), 256, tab, st>>>(taps, templates, L, h, n1);
-  twist_kernel<<<(L + 255) / 256, 256, 0, st>>>(twist, L, n1);
-  return cudaGetLastError();
 }
 
 cudaError_t launch_wait_selftest(int* status, int64_t limit_ns, cudaStream_t st) {

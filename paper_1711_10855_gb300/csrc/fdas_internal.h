@@ -144,6 +144,7 @@ cudaError_t launch_segment_spectra_big(int L, const SegParams& p, int sm_count, 
 namespace fdas {
 // Used by the allocation-free entry point (defined in fdas_api.cu).
 int validate_geometry(int64_t n_bins, int zmax, int zstep, int seg_len, int tmpl_len);
+// Step a1 (defined in fdas_templates.cu): taps, template spectra and twiddle table.
 cudaError_t build_templates_into(double2* taps, float2* templates, float2* twist, int zmax, int zstep, int L,
                                  int m, cudaStream_t st);
 int encode_spectrum_map(CUtensorMap* map, const void* d_spectrum, int64_t n_bins, int L);
