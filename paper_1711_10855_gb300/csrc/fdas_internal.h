@@ -4,6 +4,7 @@
 #include <cstdint>
 
 #include <cuda.h>
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
 namespace fdas {
@@ -150,4 +151,76 @@ cudaError_t build_templates_into(double2* taps, float2* templates, float2* twist
 int encode_spectrum_map(CUtensorMap* map, const void* d_spectrum, int64_t n_bins, int L);
 // One thread waits, for at most limit_ns, on a barrier nothing completes and sets kStatusTimeout.
 cudaError_t launch_wait_selftest(int* status, int64_t limit_ns, cudaStream_t st);
+}  // namespace fdas
+
+// ---------------------------------------------------------------------------------------
+// The z-band network on windows (fdas_train.cu): FP32 forward, backward and Adam.
+// ---------------------------------------------------------------------------------------
+namespace fdas {
+
+constexpr int kNetC = 32;   // channels
+constexpr int kNetK = 9;    // kernel taps
+
+// Flat parameter layout (floats).
+struct NetLayout {
+  int Z, W1, b1, W2, b2, W3, b3, Wl, bl, total;
+  explicit NetLayout(int z) : Z(z) {
+    W1 = 0;
+    b1 = W1 + kNetC * 1 * kNetK;
+    W2 = b1 + kNetC;
+    b2 = W2 + kNetC * kNetC * kNetK;
+    W3 = b2 + kNetC;
+    b3 = W3 + kNetC * kNetC * kNetK;
+    Wl = b3 + kNetC;
+    bl = Wl + Z * kNetC;
+    total = bl + Z;
+  }
+};
+
+// Packed copies of the 32 x 32 x 9 weights, each [32 inputs of the pass][9 taps][32 outputs].
+enum { kPackW2, kPackW3, kPackW2Back, kPackW3Back, kPackW2Half, kPackW3Half, kNetPacks };
+
+struct NetState {
+  NetLayout lay{0};
+  int W = 0, sm_count = 0;
+  float* p = nullptr;          // FP32 master parameters
+  __half* ph = nullptr;        // FP16 copy for inference
+  float* pr = nullptr;         // the FP16 copy's values as FP32
+  float* packs = nullptr;      // kNetPacks packed weight matrices (of p, and of pr: *Half)
+  float* g = nullptr;          // gradients
+  float* m = nullptr;          // Adam moments
+  float* v = nullptr;
+  float* h1 = nullptr;         // activations [B][32] rows of W: W/2 + 160 used,
+  float* h2 = nullptr;         // W/2 + 128 used
+  float* d2 = nullptr;         // gradient of layer 2's pre-activations, as h2
+  float* pool = nullptr;       // per-tile maxima and positions of layer 3
+  int* pool_arg = nullptr;
+  float* pooled = nullptr;     // [B][32]
+  float* seed = nullptr;       // [B][32] gradient of the pooled maxima
+  int* arg = nullptr;          // [B][32]
+  float* logits = nullptr;     // [B][Z]
+  float* dlog = nullptr;       // [B][Z]
+  float* loss = nullptr;       // device scalar
+  float* loss_part = nullptr;  // [B]
+  float* db2_part = nullptr;   // [B][32]
+  float* part1 = nullptr;      // weight-gradient partials of the three layers
+  float* part2 = nullptr;
+  float* part3 = nullptr;
+  float* gl = nullptr;         // head gradients
+};
+
+// Element counts of the buffers whose size is not plain from their shape.
+struct NetSizes {
+  size_t act, pool, part1, part2, part3, gl, packs;
+};
+NetSizes net_sizes(int W, int Z, int max_batch, int sm_count);
+cudaError_t net_prepare();   // function attributes, once per created net
+// The copies (ph, pr, packs) of the parameters p.
+void net_publish(const NetState& s, cudaStream_t st);
+cudaError_t net_predict(const NetState& s, const float* windows, int B, bool half_weights, float* logits,
+                        cudaStream_t st);
+// One step of Adam (`step` counts from 1); gradients in g, the loss in *loss.
+cudaError_t net_train_step(const NetState& s, const float* windows, const float* targets, int B, float lr, int step,
+                           cudaStream_t st);
+
 }  // namespace fdas

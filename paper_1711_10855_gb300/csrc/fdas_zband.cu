@@ -32,35 +32,17 @@
 
 namespace {
 
-constexpr int kC = 32;          // channels
-constexpr int kK = 9;           // kernel taps
+using Layout = fdas::NetLayout;
+constexpr int kC = fdas::kNetC;   // channels
+constexpr int kK = fdas::kNetK;   // kernel taps
 constexpr int kPad = 4;
-constexpr int kTile = 128;      // positions per conv block
+constexpr int kWidthStep = 128;   // window widths are multiples of it
 constexpr int kDil1 = 1, kDil2 = 4, kDil3 = 16;    // layer dilations
 constexpr int kRF = kPad * (kDil1 + kDil2 + kDil3);   // receptive field of a layer-3 position
-
-// Flat parameter layout (floats).
-struct Layout {
-  int W1, b1, W2, b2, W3, b3, Wl, bl, total;
-  explicit Layout(int Z) {
-    W1 = 0;
-    b1 = W1 + kC * 1 * kK;
-    W2 = b1 + kC;
-    b2 = W2 + kC * kC * kK;
-    W3 = b2 + kC;
-    b3 = W3 + kC * kC * kK;
-    Wl = b3 + kC;
-    bl = Wl + Z * kC;
-    total = bl + Z;
-  }
-};
 
 constexpr float kXCap = 64.f;   // input cap: x_r = min(|A_r|^2 ln 2 / median |A|^2, 64)
 constexpr int kSelBlocks = 2048; // grid cap of the median's first pass
 constexpr int kSelBlocks12 = 304; // and of its second and third (2 blocks per SM of a GB300)
-
-__device__ __forceinline__ float to_f(float v) { return v; }
-__device__ __forceinline__ float to_f(__half v) { return __half2float(v); }
 
 // Exact lower median of |A_r|^2 (rank (n-1)/2) by radix selection on the FP32 bit patterns
 // (non-negative floats order as unsigned integers): three passes over the spectrum histogram the
@@ -210,258 +192,6 @@ __global__ void spectrum_windows_kernel(const float2* spec, int64_t n, const flo
   const int64_t r0 = w * hop - Wd / 4;
   const float sc = *scale;
   for (int t = threadIdx.x; t < Wd; t += blockDim.x) x[w * Wd + t] = power_x(spec, n, r0 + t, sc);
-}
-
-// pre[b][o][t] = bias[o] + sum_{i,k} W[o][i][k] * in(b, i, t + (k - 4) D); in = x (CIN = 1) or
-// relu(prev pre-activation).  Block: 128 positions of one window, all 32 output channels;
-// thread (o = tid/8, t = tid%8 + 8j).
-template <int CIN, int D>
-constexpr size_t conv_fwd_smem() {
-  return sizeof(float) * ((size_t)CIN * (kTile + 2 * kPad * D) + (size_t)kC * CIN * kK);
-}
-
-template <int CIN, bool RELU_IN, typename WT, int D>
-__global__ void __launch_bounds__(256) conv_fwd_kernel(const float* in, const WT* W, const WT* bias, float* pre,
-                                                       int Wd) {
-  constexpr int S = kTile + 2 * kPad * D;   // staged positions: the tile and its halo
-  extern __shared__ float dyn[];
-  float (*sIn)[S] = reinterpret_cast<float (*)[S]>(dyn);
-  float* sW = dyn + (size_t)CIN * S;
-  const int b = blockIdx.y, t0 = blockIdx.x * kTile;
-  for (int idx = threadIdx.x; idx < kC * CIN * kK; idx += blockDim.x) sW[idx] = to_f(W[idx]);
-  for (int idx = threadIdx.x; idx < CIN * S; idx += blockDim.x) {
-    const int i = idx / S, tt = idx % S;
-    const int t = t0 + tt - kPad * D;
-    float v = (t >= 0 && t < Wd) ? in[((size_t)b * CIN + i) * Wd + t] : 0.f;
-    if (RELU_IN) v = fmaxf(v, 0.f);
-    sIn[i][tt] = v;
-  }
-  __syncthreads();
-  const int o = threadIdx.x >> 3, tl = threadIdx.x & 7;
-  float acc[kTile / 8];
-  const float bo = to_f(bias[o]);
-#pragma unroll
-  for (int j = 0; j < kTile / 8; ++j) acc[j] = bo;
-  for (int i = 0; i < CIN; ++i) {
-#pragma unroll
-    for (int k = 0; k < kK; ++k) {
-      const float w = sW[(o * CIN + i) * kK + k];
-#pragma unroll
-      for (int j = 0; j < kTile / 8; ++j) acc[j] = fmaf(w, sIn[i][tl + 8 * j + k * D], acc[j]);
-    }
-  }
-#pragma unroll
-  for (int j = 0; j < kTile / 8; ++j) pre[((size_t)b * kC + o) * Wd + t0 + tl + 8 * j] = acc[j];
-}
-
-// Pooling over the central half and the linear head: one block per window.
-template <typename WT>
-__global__ void pool_head_kernel(const float* a3, const WT* Wl, const WT* bl, int Wd, int Z, float* m_out,
-                                 int* arg_out, float* logits) {
-  const int b = blockIdx.x;
-  __shared__ float sm[kC];
-  const int lo = Wd / 4, hi = 3 * Wd / 4;
-  // 8 threads per channel, then combine (first maximum on ties)
-  const int c = threadIdx.x >> 3, l = threadIdx.x & 7;
-  float best = -1.f;
-  int barg = lo;
-  for (int t = lo + l; t < hi; t += 8) {
-    const float v = fmaxf(a3[((size_t)b * kC + c) * Wd + t], 0.f);
-    if (v > best) {
-      best = v;
-      barg = t;
-    }
-  }
-  for (int off = 4; off > 0; off >>= 1) {
-    const float ov = __shfl_down_sync(0xffffffffu, best, off, 8);
-    const int oa = __shfl_down_sync(0xffffffffu, barg, off, 8);
-    if (ov > best || (ov == best && oa < barg)) {
-      best = ov;
-      barg = oa;
-    }
-  }
-  if (l == 0) {
-    sm[c] = best;
-    if (m_out) m_out[b * kC + c] = best;
-    if (arg_out) arg_out[b * kC + c] = barg;
-  }
-  __syncthreads();
-  for (int j = threadIdx.x; j < Z; j += blockDim.x) {
-    float s = to_f(bl[j]);
-#pragma unroll 8
-    for (int cc = 0; cc < kC; ++cc) s = fmaf(to_f(Wl[j * kC + cc]), sm[cc], s);
-    logits[(size_t)b * Z + j] = s;
-  }
-}
-
-// dlog = (sigmoid(l) - target) / (B*Z); loss_part[warp] = that warp's sum of BCE terms / (B*Z),
-// summed afterwards in a fixed order (sum_fixed_kernel), so the loss is the same on every run.
-__global__ void bce_grad_kernel(const float* logits, const float* target, int count, float* dlog, float* loss_part) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  float term = 0.f;
-  if (i < count) {
-    const float l = logits[i], t = target[i];
-    dlog[i] = (1.f / (1.f + expf(-l)) - t) / (float)count;
-    term = fmaxf(l, 0.f) - l * t + log1pf(expf(-fabsf(l)));
-  }
-  for (int off = 16; off > 0; off >>= 1) term += __shfl_down_sync(0xffffffffu, term, off);
-  if ((threadIdx.x & 31) == 0 && i < count) loss_part[i >> 5] = term / (float)count;   // warps with a term
-}
-
-// out = sum of part[0..n) in a fixed order: thread t adds part[t], part[t + 1024], ... in turn,
-// then a fixed-shape tree over the 1024 threads.  One block of 1024 threads.
-__global__ void __launch_bounds__(1024) sum_fixed_kernel(const float* part, int n, float* out) {
-  __shared__ float s[1024];
-  float a = 0.f;
-  for (int j = threadIdx.x; j < n; j += 1024) a += part[j];
-  s[threadIdx.x] = a;
-  __syncthreads();
-  for (int w = 512; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w) s[threadIdx.x] += s[threadIdx.x + w];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) *out = s[0];
-}
-
-// out[j] = sum over blk = 0, 1, ..., nblk-1 (in that order) of part[blk * stride + j], j < n: the
-// fixed-order reduction of per-block weight-gradient partials.
-__global__ void reduce_partials_kernel(const float* part, int nblk, int stride, int n, float* out) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= n) return;
-  float a = 0.f;
-  for (int blk = 0; blk < nblk; ++blk) a += part[(size_t)blk * stride + j];
-  out[j] = a;
-}
-
-// Head backward: dWl[j][c] = sum_b dlog[b][j] m[b][c], dbl[j] = sum_b dlog[b][j].
-__global__ void head_bwd_weights_kernel(const float* dlog, const float* m, int B, int Z, float* dWl, float* dbl) {
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= Z * (kC + 1)) return;
-  const int j = idx / (kC + 1), c = idx % (kC + 1);
-  float s = 0.f;
-  for (int b = 0; b < B; ++b) s += dlog[(size_t)b * Z + j] * (c < kC ? m[b * kC + c] : 1.f);
-  if (c < kC) dWl[j * kC + c] = s;
-  else dbl[j] = s;
-}
-
-// dm[b][c] = sum_j dlog[b][j] Wl[j][c]; then da3 = dm at the pooled position if a3 > 0 there.
-__global__ void head_bwd_data_kernel(const float* dlog, const float* Wl, const int* arg, const float* a3, int Z,
-                                     int Wd, float* da3) {
-  const int b = blockIdx.x, c = threadIdx.x;
-  if (c >= kC) return;
-  float s = 0.f;
-  for (int j = 0; j < Z; ++j) s = fmaf(dlog[(size_t)b * Z + j], Wl[j * kC + c], s);
-  const int t = arg[b * kC + c];
-  const size_t at = ((size_t)b * kC + c) * Wd + t;
-  da3[at] = a3[at] > 0.f ? s : 0.f;
-}
-
-// dIn_pre[b][i][t] = (prev_pre > 0) * sum_{o,k} W[o][i][k] dOut[b][o][t - (k - 4) D].
-template <int D>
-constexpr size_t bwd_data_smem() {
-  return sizeof(float) * ((size_t)kC * (kTile + 2 * kPad * D) + (size_t)kC * kC * kK);
-}
-
-template <int D>
-__global__ void __launch_bounds__(256) conv_bwd_data_kernel(const float* dout, const float* W, const float* prev_pre,
-                                                            float* din, int Wd) {
-  constexpr int S = kTile + 2 * kPad * D;
-  extern __shared__ float dyn[];
-  float (*sD)[S] = reinterpret_cast<float (*)[S]>(dyn);
-  float* sW = dyn + (size_t)kC * S;
-  const int b = blockIdx.y, t0 = blockIdx.x * kTile;
-  for (int idx = threadIdx.x; idx < kC * kC * kK; idx += blockDim.x) sW[idx] = W[idx];
-  for (int idx = threadIdx.x; idx < kC * S; idx += blockDim.x) {
-    const int o = idx / S, tt = idx % S;
-    const int t = t0 + tt - kPad * D;
-    sD[o][tt] = (t >= 0 && t < Wd) ? dout[((size_t)b * kC + o) * Wd + t] : 0.f;
-  }
-  __syncthreads();
-  const int i = threadIdx.x >> 3, tl = threadIdx.x & 7;
-  float acc[kTile / 8];
-#pragma unroll
-  for (int j = 0; j < kTile / 8; ++j) acc[j] = 0.f;
-  for (int o = 0; o < kC; ++o) {
-#pragma unroll
-    for (int k = 0; k < kK; ++k) {
-      const float w = sW[(o * kC + i) * kK + k];
-      // dOut index t - (k - 4) D = (t0 + tl + 8j) - (k - 4) D -> tile offset tl + 8j + (8 - k) D
-#pragma unroll
-      for (int j = 0; j < kTile / 8; ++j) acc[j] = fmaf(w, sD[o][tl + 8 * j + (2 * kPad - k) * D], acc[j]);
-    }
-  }
-#pragma unroll
-  for (int j = 0; j < kTile / 8; ++j) {
-    const size_t at = ((size_t)b * kC + i) * Wd + t0 + tl + 8 * j;
-    din[at] = prev_pre[at] > 0.f ? acc[j] : 0.f;
-  }
-}
-
-// Partials of one block (tile, b): part[blk][(o*CIN + i)*9 + k] = sum_{t in tile} in(b, i, t + (k - 4) D)
-// * dOut[b][o][t] and part[blk][C*CIN*9 + o] = sum_{t in tile} dOut[b][o][t], blk = b*tiles + tile;
-// reduce_partials_kernel then sums them over blocks in a fixed order (no floating-point atomics, so
-// one seed gives one network).  Thread handles (o = tid/8) and i in {tid%8, tid%8 + 8, ...}.
-template <int CIN, int D>
-constexpr size_t bwd_weight_smem() {
-  return sizeof(float) * ((size_t)CIN * (kTile + 2 * kPad * D) + (size_t)kC * kTile);
-}
-
-template <int CIN, bool RELU_IN, int D>
-__global__ void __launch_bounds__(256) conv_bwd_weight_kernel(const float* in, const float* dout, int Wd,
-                                                              float* part) {
-  constexpr int S = kTile + 2 * kPad * D;
-  extern __shared__ float dyn[];
-  float (*sIn)[S] = reinterpret_cast<float (*)[S]>(dyn);
-  float (*sD)[kTile] = reinterpret_cast<float (*)[kTile]>(dyn + (size_t)CIN * S);
-  const int b = blockIdx.y, t0 = blockIdx.x * kTile;
-  for (int idx = threadIdx.x; idx < CIN * S; idx += blockDim.x) {
-    const int i = idx / S, tt = idx % S;
-    const int t = t0 + tt - kPad * D;
-    float v = (t >= 0 && t < Wd) ? in[((size_t)b * CIN + i) * Wd + t] : 0.f;
-    if (RELU_IN) v = fmaxf(v, 0.f);
-    sIn[i][tt] = v;
-  }
-  for (int idx = threadIdx.x; idx < kC * kTile; idx += blockDim.x) {
-    const int o = idx / kTile, tt = idx % kTile;
-    sD[o][tt] = dout[((size_t)b * kC + o) * Wd + t0 + tt];
-  }
-  __syncthreads();
-  const int o = threadIdx.x >> 3, l = threadIdx.x & 7;
-  for (int i = l; i < CIN; i += 8) {
-    float acc[kK];
-#pragma unroll
-    for (int k = 0; k < kK; ++k) acc[k] = 0.f;
-    for (int t = 0; t < kTile; ++t) {
-      const float d = sD[o][t];
-#pragma unroll
-      for (int k = 0; k < kK; ++k) acc[k] = fmaf(sIn[i][t + k * D], d, acc[k]);
-    }
-    float* dst = part + ((size_t)b * gridDim.x + blockIdx.x) * ((size_t)kC * CIN * kK + kC);
-#pragma unroll
-    for (int k = 0; k < kK; ++k) dst[(o * CIN + i) * kK + k] = acc[k];
-  }
-  if (l == 0) {
-    float s = 0.f;
-    for (int t = 0; t < kTile; ++t) s += sD[o][t];
-    part[((size_t)b * gridDim.x + blockIdx.x) * ((size_t)kC * CIN * kK + kC) + (size_t)kC * CIN * kK + o] = s;
-  }
-}
-
-__global__ void adam_kernel(float* p, const float* g, float* m, float* v, int n, float lr, float b1, float b2,
-                            float eps, float c1, float c2) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const float gi = g[i];
-  const float mi = b1 * m[i] + (1.f - b1) * gi;
-  const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-  m[i] = mi;
-  v[i] = vi;
-  p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
-}
-
-__global__ void to_half_kernel(const float* p, __half* h, int n) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) h[i] = __float2half_rn(p[i]);
 }
 
 // Proposal -> correlation work list.  Segment j of group g (G segments of V bins: outputs
@@ -930,24 +660,7 @@ __global__ void __launch_bounds__(256, 1) propose_kernel(const ProposeParams p) 
 
 struct fdas_zband {
   int Wd = 0, Z = 0, max_batch = 0, sm_count = 0;
-  Layout lay{0};
-  float* p = nullptr;        // FP32 master parameters
-  __half* ph = nullptr;      // FP16 copy for inference
-  float* g = nullptr;        // gradients
-  float* m = nullptr;        // Adam moments
-  float* v = nullptr;
-  float* a1 = nullptr;       // pre-activations [B][C][Wd]
-  float* a2 = nullptr;
-  float* a3 = nullptr;
-  float* d1 = nullptr;       // gradient buffers [B][C][Wd]
-  float* d2 = nullptr;
-  float* pooled = nullptr;   // [B][C]
-  int* arg = nullptr;        // [B][C]
-  float* logits = nullptr;   // [B][Z]
-  float* dlog = nullptr;     // [B][Z]
-  float* loss = nullptr;     // device scalar
-  float* loss_part = nullptr; // per-warp loss partials [ceil(B*Z / 32)]
-  float* wpart = nullptr;    // weight-gradient partials [B * Wd/128][C*C*9 + C]
+  fdas::NetState net;
   SelectState* sel = nullptr; // median selection state
   float* scale = nullptr;    // ln 2 / median |A|^2
   int* status = nullptr;     // bit 0: a bounded wait of the inference kernel gave up
@@ -967,9 +680,10 @@ struct fdas_zband {
 
 namespace {
 void free_zband(fdas_zband* z) {
-  void* ptrs[] = {z->p,      z->ph,  z->g,      z->m,    z->v,         z->a1,     z->a2,
-                  z->a3,     z->d1,  z->d2,     z->pooled, z->arg,    z->logits, z->dlog,
-                  z->loss,   z->loss_part, z->wpart, z->sel, z->scale, z->status};
+  const fdas::NetState& s = z->net;
+  void* ptrs[] = {s.p,      s.ph,   s.pr,   s.packs,  s.g,    s.m,         s.v,        s.h1,    s.h2,    s.d2,    s.pool,
+                  s.pool_arg, s.pooled, s.seed, s.arg, s.logits, s.dlog, s.loss, s.loss_part, s.db2_part, s.part1, s.part2,
+                  s.part3,  s.gl,   z->sel, z->scale, z->status};
   for (void* q : ptrs) cudaFree(q);
   if (z->graph_exec) cudaGraphExecDestroy(z->graph_exec);
   if (z->graph) cudaGraphDestroy(z->graph);
@@ -998,32 +712,6 @@ int host_copy(fdas_zband* z, void* dst, const void* src, size_t bytes, cudaMemcp
   return FDAS_OK;
 }
 
-// Layers 1..3, pooling and head on B windows `in` (FP32 activations; FP32 or FP16 weights).
-cudaError_t forward(fdas_zband* z, const float* in, int B, bool half_weights, cudaStream_t st) {
-  const Layout& L = z->lay;
-  const dim3 grid(z->Wd / kTile, B);
-  if (half_weights) {
-    const __half* h = z->ph;
-    conv_fwd_kernel<1, false, __half, kDil1>
-        <<<grid, 256, conv_fwd_smem<1, kDil1>(), st>>>(in, h + L.W1, h + L.b1, z->a1, z->Wd);
-    conv_fwd_kernel<kC, true, __half, kDil2>
-        <<<grid, 256, conv_fwd_smem<kC, kDil2>(), st>>>(z->a1, h + L.W2, h + L.b2, z->a2, z->Wd);
-    conv_fwd_kernel<kC, true, __half, kDil3>
-        <<<grid, 256, conv_fwd_smem<kC, kDil3>(), st>>>(z->a2, h + L.W3, h + L.b3, z->a3, z->Wd);
-    pool_head_kernel<__half><<<B, 256, 0, st>>>(z->a3, h + L.Wl, h + L.bl, z->Wd, z->Z, z->pooled, z->arg, z->logits);
-  } else {
-    const float* p = z->p;
-    conv_fwd_kernel<1, false, float, kDil1>
-        <<<grid, 256, conv_fwd_smem<1, kDil1>(), st>>>(in, p + L.W1, p + L.b1, z->a1, z->Wd);
-    conv_fwd_kernel<kC, true, float, kDil2>
-        <<<grid, 256, conv_fwd_smem<kC, kDil2>(), st>>>(z->a1, p + L.W2, p + L.b2, z->a2, z->Wd);
-    conv_fwd_kernel<kC, true, float, kDil3>
-        <<<grid, 256, conv_fwd_smem<kC, kDil3>(), st>>>(z->a2, p + L.W3, p + L.b3, z->a3, z->Wd);
-    pool_head_kernel<float><<<B, 256, 0, st>>>(z->a3, p + L.Wl, p + L.bl, z->Wd, z->Z, z->pooled, z->arg, z->logits);
-  }
-  return cudaGetLastError();
-}
-
 // scale = ln 2 / median |A|^2 into `scale`: seven launches.
 void launch_power_scale(const float2* spec, int64_t n, SelectState* sel, float* scale, cudaStream_t st) {
   select_init_kernel<<<1, 256, 0, st>>>(sel, n);
@@ -1045,7 +733,7 @@ extern "C" {
 fdas_zband* fdas_zband_create(int window, int n_out, int max_batch) {
   // the window's quarter margins must hold the receptive field (the windowed and whole-sequence
   // forms then agree)
-  if (window < 4 * kRF || window % kTile != 0 || window > (1 << 16) || n_out < 1 || n_out > 65535 ||
+  if (window < 4 * kRF || window % kWidthStep != 0 || window > (1 << 16) || n_out < 1 || n_out > 65535 ||
       max_batch < 1 || max_batch > 65535)
     return nullptr;
   int dev = 0, major = 0, minor = 0, sms = 0;
@@ -1055,21 +743,7 @@ fdas_zband* fdas_zband_create(int window, int n_out, int max_batch) {
     cudaGetLastError();
     return nullptr;
   }
-  constexpr auto kSmemAttr = cudaFuncAttributeMaxDynamicSharedMemorySize;
-  if (cudaFuncSetAttribute(conv_fwd_kernel<kC, true, float, kDil2>, kSmemAttr, (int)conv_fwd_smem<kC, kDil2>()) !=
-          cudaSuccess ||
-      cudaFuncSetAttribute(conv_fwd_kernel<kC, true, float, kDil3>, kSmemAttr, (int)conv_fwd_smem<kC, kDil3>()) !=
-          cudaSuccess ||
-      cudaFuncSetAttribute(conv_fwd_kernel<kC, true, __half, kDil2>, kSmemAttr, (int)conv_fwd_smem<kC, kDil2>()) !=
-          cudaSuccess ||
-      cudaFuncSetAttribute(conv_fwd_kernel<kC, true, __half, kDil3>, kSmemAttr, (int)conv_fwd_smem<kC, kDil3>()) !=
-          cudaSuccess ||
-      cudaFuncSetAttribute(conv_bwd_data_kernel<kDil2>, kSmemAttr, (int)bwd_data_smem<kDil2>()) != cudaSuccess ||
-      cudaFuncSetAttribute(conv_bwd_data_kernel<kDil3>, kSmemAttr, (int)bwd_data_smem<kDil3>()) != cudaSuccess ||
-      cudaFuncSetAttribute(conv_bwd_weight_kernel<kC, true, kDil2>, kSmemAttr, (int)bwd_weight_smem<kC, kDil2>()) !=
-          cudaSuccess ||
-      cudaFuncSetAttribute(conv_bwd_weight_kernel<kC, true, kDil3>, kSmemAttr, (int)bwd_weight_smem<kC, kDil3>()) !=
-          cudaSuccess ||
+  if (fdas::net_prepare() != cudaSuccess ||
       cudaFuncSetAttribute(propose_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, kProposeSmem) !=
           cudaSuccess ||
       cudaFuncSetAttribute(propose_kernel<384>, cudaFuncAttributeMaxDynamicSharedMemorySize, kProposeSmem) !=
@@ -1085,25 +759,34 @@ fdas_zband* fdas_zband_create(int window, int n_out, int max_batch) {
   z->Z = n_out;
   z->max_batch = max_batch;
   z->sm_count = sms;
-  z->lay = Layout(n_out);
-  const size_t P = (size_t)z->lay.total, B = (size_t)max_batch, act = B * kC * (size_t)window;
-  bool ok = cudaMalloc(&z->p, P * 4) == cudaSuccess && cudaMalloc(&z->ph, P * 2) == cudaSuccess &&
-            cudaMalloc(&z->g, P * 4) == cudaSuccess && cudaMalloc(&z->m, P * 4) == cudaSuccess &&
-            cudaMalloc(&z->v, P * 4) == cudaSuccess && cudaMalloc(&z->a1, act * 4) == cudaSuccess &&
-            cudaMalloc(&z->a2, act * 4) == cudaSuccess && cudaMalloc(&z->a3, act * 4) == cudaSuccess &&
-            cudaMalloc(&z->d1, act * 4) == cudaSuccess && cudaMalloc(&z->d2, act * 4) == cudaSuccess &&
-            cudaMalloc(&z->pooled, B * kC * 4) == cudaSuccess && cudaMalloc(&z->arg, B * kC * 4) == cudaSuccess &&
-            cudaMalloc(&z->logits, B * (size_t)n_out * 4) == cudaSuccess &&
-            cudaMalloc(&z->dlog, B * (size_t)n_out * 4) == cudaSuccess && cudaMalloc(&z->loss, 4) == cudaSuccess &&
-            cudaMalloc(&z->loss_part, (B * (size_t)n_out + 31) / 32 * 4) == cudaSuccess &&
-            cudaMalloc(&z->wpart, B * (size_t)(window / kTile) * ((size_t)kC * kC * kK + kC) * 4) == cudaSuccess &&
+  fdas::NetState& s = z->net;
+  s.lay = Layout(n_out);
+  s.W = window;
+  s.sm_count = sms;
+  const size_t P = (size_t)s.lay.total, B = (size_t)max_batch;
+  const fdas::NetSizes n = fdas::net_sizes(window, n_out, max_batch, sms);
+  bool ok = cudaMalloc(&s.p, P * 4) == cudaSuccess && cudaMalloc(&s.ph, P * 2) == cudaSuccess &&
+            cudaMalloc(&s.pr, P * 4) == cudaSuccess && cudaMalloc(&s.packs, n.packs * 4) == cudaSuccess &&
+            cudaMalloc(&s.g, P * 4) == cudaSuccess && cudaMalloc(&s.m, P * 4) == cudaSuccess &&
+            cudaMalloc(&s.v, P * 4) == cudaSuccess && cudaMalloc(&s.h1, n.act * 4) == cudaSuccess &&
+            cudaMalloc(&s.h2, n.act * 4) == cudaSuccess && cudaMalloc(&s.d2, n.act * 4) == cudaSuccess &&
+            cudaMalloc(&s.pool, n.pool * 4) == cudaSuccess && cudaMalloc(&s.pool_arg, n.pool * 4) == cudaSuccess &&
+            cudaMalloc(&s.pooled, B * kC * 4) == cudaSuccess && cudaMalloc(&s.seed, B * kC * 4) == cudaSuccess &&
+            cudaMalloc(&s.arg, B * kC * 4) == cudaSuccess &&
+            cudaMalloc(&s.logits, B * (size_t)n_out * 4) == cudaSuccess &&
+            cudaMalloc(&s.dlog, B * (size_t)n_out * 4) == cudaSuccess && cudaMalloc(&s.loss, 4) == cudaSuccess &&
+            cudaMalloc(&s.loss_part, B * 4) == cudaSuccess && cudaMalloc(&s.db2_part, B * kC * 4) == cudaSuccess &&
+            cudaMalloc(&s.part1, n.part1 * 4) == cudaSuccess && cudaMalloc(&s.part2, n.part2 * 4) == cudaSuccess &&
+            cudaMalloc(&s.part3, n.part3 * 4) == cudaSuccess && cudaMalloc(&s.gl, n.gl * 4) == cudaSuccess &&
             cudaMalloc(&z->sel, sizeof(SelectState)) == cudaSuccess &&
             cudaMalloc(&z->scale, 4) == cudaSuccess && cudaMalloc(&z->status, 4) == cudaSuccess &&
             cudaStreamCreateWithFlags(&z->own, cudaStreamNonBlocking) == cudaSuccess &&
             cudaEventCreateWithFlags(&z->done, cudaEventDisableTiming) == cudaSuccess;
-  if (!ok || cudaMemsetAsync(z->p, 0, P * 4, z->own) != cudaSuccess ||
-      cudaMemsetAsync(z->ph, 0, P * 2, z->own) != cudaSuccess || cudaMemsetAsync(z->m, 0, P * 4, z->own) != cudaSuccess ||
-      cudaMemsetAsync(z->v, 0, P * 4, z->own) != cudaSuccess || cudaMemsetAsync(z->status, 0, 4, z->own) != cudaSuccess ||
+  if (!ok || cudaMemsetAsync(s.p, 0, P * 4, z->own) != cudaSuccess ||
+      cudaMemsetAsync(s.ph, 0, P * 2, z->own) != cudaSuccess || cudaMemsetAsync(s.pr, 0, P * 4, z->own) != cudaSuccess ||
+      cudaMemsetAsync(s.packs, 0, n.packs * 4, z->own) != cudaSuccess ||
+      cudaMemsetAsync(s.m, 0, P * 4, z->own) != cudaSuccess || cudaMemsetAsync(s.v, 0, P * 4, z->own) != cudaSuccess ||
+      cudaMemsetAsync(z->status, 0, 4, z->own) != cudaSuccess ||
       cudaEventRecord(z->done, z->own) != cudaSuccess || cudaStreamSynchronize(z->own) != cudaSuccess) {
     cudaGetLastError();
     free_zband(z);
@@ -1112,15 +795,15 @@ fdas_zband* fdas_zband_create(int window, int n_out, int max_batch) {
   return z;
 }
 
-int fdas_zband_param_count(const fdas_zband* z) { return z ? z->lay.total : FDAS_ERR_INVALID; }
+int fdas_zband_param_count(const fdas_zband* z) { return z ? z->net.lay.total : FDAS_ERR_INVALID; }
 
 int fdas_zband_set_params(fdas_zband* z, const float* host_params) {
   if (!z || !host_params) return FDAS_ERR_INVALID;
-  const int P = z->lay.total;
-  if (host_copy(z, z->p, host_params, (size_t)P * 4, cudaMemcpyHostToDevice) != FDAS_OK) return FDAS_ERR_CUDA;
-  to_half_kernel<<<(P + 255) / 256, 256, 0, z->own>>>(z->p, z->ph, P);
-  cudaMemsetAsync(z->m, 0, (size_t)P * 4, z->own);
-  cudaMemsetAsync(z->v, 0, (size_t)P * 4, z->own);
+  const int P = z->net.lay.total;
+  if (host_copy(z, z->net.p, host_params, (size_t)P * 4, cudaMemcpyHostToDevice) != FDAS_OK) return FDAS_ERR_CUDA;
+  fdas::net_publish(z->net, z->own);
+  cudaMemsetAsync(z->net.m, 0, (size_t)P * 4, z->own);
+  cudaMemsetAsync(z->net.v, 0, (size_t)P * 4, z->own);
   z->step = 0;
   if (note_work(z, z->own, cudaGetLastError()) != FDAS_OK) return FDAS_ERR_CUDA;
   return cudaStreamSynchronize(z->own) == cudaSuccess ? FDAS_OK : FDAS_ERR_CUDA;
@@ -1128,14 +811,14 @@ int fdas_zband_set_params(fdas_zband* z, const float* host_params) {
 
 int fdas_zband_get_params(fdas_zband* z, float* host_params) {
   if (!z || !host_params) return FDAS_ERR_INVALID;
-  return host_copy(z, host_params, z->p, (size_t)z->lay.total * 4, cudaMemcpyDeviceToHost);
+  return host_copy(z, host_params, z->net.p, (size_t)z->net.lay.total * 4, cudaMemcpyDeviceToHost);
 }
 
 int fdas_zband_get_adam(fdas_zband* z, float* host_m, float* host_v, int* host_step) {
   if (!z || !host_m || !host_v || !host_step) return FDAS_ERR_INVALID;
-  const size_t bytes = (size_t)z->lay.total * 4;
-  if (host_copy(z, host_m, z->m, bytes, cudaMemcpyDeviceToHost) != FDAS_OK ||
-      host_copy(z, host_v, z->v, bytes, cudaMemcpyDeviceToHost) != FDAS_OK)
+  const size_t bytes = (size_t)z->net.lay.total * 4;
+  if (host_copy(z, host_m, z->net.m, bytes, cudaMemcpyDeviceToHost) != FDAS_OK ||
+      host_copy(z, host_v, z->net.v, bytes, cudaMemcpyDeviceToHost) != FDAS_OK)
     return FDAS_ERR_CUDA;
   *host_step = z->step;
   return FDAS_OK;
@@ -1143,9 +826,9 @@ int fdas_zband_get_adam(fdas_zband* z, float* host_m, float* host_v, int* host_s
 
 int fdas_zband_set_adam(fdas_zband* z, const float* host_m, const float* host_v, int step) {
   if (!z || !host_m || !host_v || step < 0) return FDAS_ERR_INVALID;
-  const size_t bytes = (size_t)z->lay.total * 4;
-  if (host_copy(z, z->m, host_m, bytes, cudaMemcpyHostToDevice) != FDAS_OK ||
-      host_copy(z, z->v, host_v, bytes, cudaMemcpyHostToDevice) != FDAS_OK)
+  const size_t bytes = (size_t)z->net.lay.total * 4;
+  if (host_copy(z, z->net.m, host_m, bytes, cudaMemcpyHostToDevice) != FDAS_OK ||
+      host_copy(z, z->net.v, host_v, bytes, cudaMemcpyHostToDevice) != FDAS_OK)
     return FDAS_ERR_CUDA;
   z->step = step;
   return FDAS_OK;
@@ -1155,40 +838,12 @@ int fdas_zband_train_step(fdas_zband* z, const float* d_windows, const float* d_
                           float* host_loss, fdas_stream_t stream) {
   if (!z || !d_windows || !d_targets || batch < 1 || batch > z->max_batch || !(lr > 0.f)) return FDAS_ERR_INVALID;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  const Layout& L = z->lay;
-  const int B = batch, Wd = z->Wd, Z = z->Z, P = L.total;
-  if (forward(z, d_windows, B, false, st) != cudaSuccess) return FDAS_ERR_CUDA;
-  bce_grad_kernel<<<(B * Z + 255) / 256, 256, 0, st>>>(z->logits, d_targets, B * Z, z->dlog, z->loss_part);
-  sum_fixed_kernel<<<1, 1024, 0, st>>>(z->loss_part, (B * Z + 31) / 32, z->loss);
-  head_bwd_weights_kernel<<<(Z * (kC + 1) + 255) / 256, 256, 0, st>>>(z->dlog, z->pooled, B, Z, z->g + L.Wl,
-                                                                       z->g + L.bl);
-  const size_t act = (size_t)B * kC * Wd;
-  cudaMemsetAsync(z->d1, 0, act * 4, st);
-  head_bwd_data_kernel<<<B, kC, 0, st>>>(z->dlog, z->p + L.Wl, z->arg, z->a3, Z, Wd, z->d1);   // da3
-  const dim3 grid(Wd / kTile, B);
-  const int nblk = B * (Wd / kTile);
-  // partials of layer `cin` inputs, then their fixed-order sum into the W and b slices (W then b
-  // are adjacent in the parameter layout)
-  auto reduce = [&](int cin, int w_off) {
-    const int n = kC * cin * kK + kC;
-    reduce_partials_kernel<<<(n + 255) / 256, 256, 0, st>>>(z->wpart, nblk, n, n, z->g + w_off);
-  };
-  conv_bwd_weight_kernel<kC, true, kDil3><<<grid, 256, bwd_weight_smem<kC, kDil3>(), st>>>(z->a2, z->d1, Wd, z->wpart);
-  reduce(kC, L.W3);
-  conv_bwd_data_kernel<kDil3><<<grid, 256, bwd_data_smem<kDil3>(), st>>>(z->d1, z->p + L.W3, z->a2, z->d2, Wd);   // da2
-  conv_bwd_weight_kernel<kC, true, kDil2><<<grid, 256, bwd_weight_smem<kC, kDil2>(), st>>>(z->a1, z->d2, Wd, z->wpart);
-  reduce(kC, L.W2);
-  conv_bwd_data_kernel<kDil2><<<grid, 256, bwd_data_smem<kDil2>(), st>>>(z->d2, z->p + L.W2, z->a1, z->d1, Wd);   // da1
-  conv_bwd_weight_kernel<1, false, kDil1><<<grid, 256, bwd_weight_smem<1, kDil1>(), st>>>(d_windows, z->d1, Wd, z->wpart);
-  reduce(1, L.W1);
+  if (fdas::net_train_step(z->net, d_windows, d_targets, batch, lr, z->step + 1, st) != cudaSuccess)
+    return FDAS_ERR_CUDA;
   z->step += 1;
-  const float b1 = 0.9f, b2 = 0.999f;
-  const float c1 = 1.f - powf(b1, (float)z->step), c2 = 1.f - powf(b2, (float)z->step);
-  adam_kernel<<<(P + 255) / 256, 256, 0, st>>>(z->p, z->g, z->m, z->v, P, lr, b1, b2, 1e-8f, c1, c2);
-  to_half_kernel<<<(P + 255) / 256, 256, 0, st>>>(z->p, z->ph, P);
   if (note_work(z, st, cudaGetLastError()) != FDAS_OK) return FDAS_ERR_CUDA;
   if (host_loss) {
-    if (cudaMemcpyAsync(host_loss, z->loss, 4, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+    if (cudaMemcpyAsync(host_loss, z->net.loss, 4, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
         cudaStreamSynchronize(st) != cudaSuccess)
       return FDAS_ERR_CUDA;
   }
@@ -1197,7 +852,7 @@ int fdas_zband_train_step(fdas_zband* z, const float* d_windows, const float* d_
 
 int fdas_zband_gradients(fdas_zband* z, float* host_grads) {
   if (!z || !host_grads) return FDAS_ERR_INVALID;
-  return host_copy(z, host_grads, z->g, (size_t)z->lay.total * 4, cudaMemcpyDeviceToHost);
+  return host_copy(z, host_grads, z->net.g, (size_t)z->net.lay.total * 4, cudaMemcpyDeviceToHost);
 }
 
 int fdas_zband_predict(fdas_zband* z, const float* d_windows, int batch, int half_weights, float* d_logits,
@@ -1206,9 +861,8 @@ int fdas_zband_predict(fdas_zband* z, const float* d_windows, int batch, int hal
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   for (int b0 = 0; b0 < batch; b0 += z->max_batch) {
     const int B = batch - b0 < z->max_batch ? batch - b0 : z->max_batch;
-    if (forward(z, d_windows + (size_t)b0 * z->Wd, B, half_weights != 0, st) != cudaSuccess) return FDAS_ERR_CUDA;
-    if (cudaMemcpyAsync(d_logits + (size_t)b0 * z->Z, z->logits, (size_t)B * z->Z * 4, cudaMemcpyDeviceToDevice,
-                        st) != cudaSuccess)
+    if (fdas::net_predict(z->net, d_windows + (size_t)b0 * z->Wd, B, half_weights != 0, d_logits + (size_t)b0 * z->Z,
+                          st) != cudaSuccess)
       return FDAS_ERR_CUDA;
   }
   return note_work(z, st, cudaGetLastError());
@@ -1224,15 +878,15 @@ static cudaError_t launch_propose(fdas_zband* z, const float* d_spectrum, int64_
   q.spec = reinterpret_cast<const float2*>(d_spectrum);
   q.n = n_bins;
   q.scale = z->scale;
-  q.w = z->ph;
-  q.oW1 = z->lay.W1;
-  q.ob1 = z->lay.b1;
-  q.oW2 = z->lay.W2;
-  q.ob2 = z->lay.b2;
-  q.oW3 = z->lay.W3;
-  q.ob3 = z->lay.b3;
-  q.oWl = z->lay.Wl;
-  q.obl = z->lay.bl;
+  q.w = z->net.ph;
+  q.oW1 = z->net.lay.W1;
+  q.ob1 = z->net.lay.b1;
+  q.oW2 = z->net.lay.W2;
+  q.ob2 = z->net.lay.b2;
+  q.oW3 = z->net.lay.W3;
+  q.ob3 = z->net.lay.b3;
+  q.oWl = z->net.lay.Wl;
+  q.obl = z->net.lay.bl;
   q.Z = z->Z;
   q.hop = hop;
   q.n_blocks = nb;
