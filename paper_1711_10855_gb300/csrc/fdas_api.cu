@@ -44,10 +44,8 @@ thread_local int g_last_error = FDAS_OK;
 
 // Float offset of the real part of element k in the pair-major structure-of-arrays layout
 // (lane k1 = k % n1, k2 = k / n1; pair p = k2/2 of lane k1 is the float4 at p*n1 + k1 holding
-// re(2p), re(2p+1), im(2p), im(2p+1)); the imaginary part is 2 floats further.  n1 = 0 is the
-// interleaved natural order, where the imaginary part is the next float.
+// re(2p), re(2p+1), im(2p), im(2p+1)); the imaginary part is 2 floats further.
 int pair_layout_re(int k, int n1) {
-  if (n1 == 0) return 2 * k;   // natural order (L >= 4096)
   const int k1 = k % n1, k2 = k / n1;
   return ((k2 >> 1) * n1 + k1) * 4 + (k2 & 1);
 }
@@ -91,6 +89,9 @@ EncodeTiledFn get_encode_fn() {
   return fn;
 }
 
+// The other lengths' kernels fetch the spectrum by bulk copies of its in-range part.
+bool needs_spectrum_map(int L) { return L <= 512 || L == 2048; }
+
 // Record the plan's completion event after work enqueued on `st` (skipped while the stream is
 // being captured into a CUDA graph: a captured record is not an event the host can wait on).
 int note_work(fdas_plan* p, cudaStream_t st) {
@@ -107,7 +108,7 @@ int enqueued(fdas_plan* p, cudaStream_t st, cudaError_t launch) {
 // 1-D tensor map over the spectrum: n_bins elements of 8 bytes, box of min(L, 256) elements,
 // zero fill outside [0, n_bins).
 int make_spectrum_map(fdas_plan* p, const void* d_spectrum) {
-  if (p->L >= 4096) return FDAS_OK;   // the L >= 4096 kernels read the spectrum directly
+  if (!needs_spectrum_map(p->L)) return FDAS_OK;
   if (p->map_ptr == d_spectrum) return FDAS_OK;
   EncodeTiledFn enc = get_encode_fn();
   if (!enc) return FDAS_ERR_CUDA;
@@ -536,7 +537,7 @@ int fdas_template_spectrum(fdas_plan* p, int z_idx, float* host_out) {
   for (int k = 0; k < p->L; ++k) {
     const int off = pair_layout_re(k, p->n1);
     host_out[2 * k] = f[off];
-    host_out[2 * k + 1] = f[off + (p->n1 ? 2 : 1)];
+    host_out[2 * k + 1] = f[off + 2];
   }
   std::free(tmp);
   return FDAS_OK;
@@ -560,7 +561,7 @@ cudaError_t launch_wait_selftest(int* status, int64_t limit_ns, cudaStream_t st)
 }
 
 int encode_spectrum_map(CUtensorMap* map, const void* d_spectrum, int64_t n_bins, int L) {
-  if (L >= 4096) return FDAS_OK;   // the L >= 4096 kernels read the spectrum directly
+  if (!needs_spectrum_map(L)) return FDAS_OK;
   EncodeTiledFn enc = get_encode_fn();
   if (!enc) return FDAS_ERR_CUDA;
   cuuint64_t gdim[1] = {(cuuint64_t)n_bins};

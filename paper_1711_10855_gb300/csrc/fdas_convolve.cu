@@ -32,15 +32,13 @@
 #include <cstdio>
 #include <type_traits>
 
-#include "fdas_device.cuh"
+#include "fdas_conv_common.cuh"
 #include "fdas_internal.h"
 
 // The decoupled work-list instantiation leaves the shared-ring loop of the kernel unreachable.
 #pragma nv_diag_suppress 128
 
 namespace fdas {
-
-__host__ __device__ constexpr size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 template <int L_, int N1_, int P_, int XR_, int R_ = 4>
 struct ConvCfg {
@@ -163,56 +161,12 @@ __device__ __forceinline__ void forward_transform(const float2* sx, const float4
   forward_transform_with<Cfg>(sx, [&](cp2 (&v)[Cfg::H2]) { apply_twist2<Cfg, true>(v, stw, k1); }, xb, k1, out);
 }
 
-// Twist with the twiddle pairs held in this lane's TMEM row (4 columns per pair, chunks of 4 pairs).
-template <class Cfg, bool CONJ>
-__device__ __forceinline__ void apply_twist_tmem(cp2 (&v)[Cfg::H2], uint32_t tw_addr) {
-  static_assert(Cfg::H2 % 8 == 0, "twist chunking");
-  static_for<Cfg::H2 / 8>([&](auto cc) {
-    constexpr int c = decltype(cc)::value;
-    float r0[16], r1[16];
-    tmem_ld16(tw_addr + 32 * c, r0);
-    tmem_ld16(tw_addr + 32 * c + 16, r1);
-    tmem_wait_ld();
-    static_for<4>([&](auto qq) {
-      constexpr int q = decltype(qq)::value;
-      const cp2 w0 = cp2{make_float2(r0[4 * q], r0[4 * q + 1]), make_float2(r0[4 * q + 2], r0[4 * q + 3])};
-      const cp2 w1 = cp2{make_float2(r1[4 * q], r1[4 * q + 1]), make_float2(r1[4 * q + 2], r1[4 * q + 3])};
-      v[8 * c + q] = CONJ ? cmul2_conj(v[8 * c + q], w0) : cmul2(v[8 * c + q], w0);
-      v[8 * c + 4 + q] = CONJ ? cmul2_conj(v[8 * c + 4 + q], w1) : cmul2(v[8 * c + 4 + q], w1);
-    });
-  });
-}
-
 // Store X[n] (held by lane t = n mod N1) into the pair-major layout of the inverse transform.
 template <class Cfg>
 __device__ __forceinline__ void store_spectrum_element(float* sx, int t, int k2, float re, float im) {
   const int base = ((k2 >> 1) * Cfg::N1 + t) * 4 + (k2 & 1);
   sx[base] = re;
   sx[base + 2] = im;
-}
-
-// One arrival on a shared-memory consumer counter with acquire-release semantics at CTA scope: the
-// caller's earlier reads of the slot (ordered within the warp by __syncwarp) happen before the
-// arrival, and the last arriver's later refill of the slot happens after every other arrival.
-// Returns the count before this arrival.
-__device__ __forceinline__ unsigned arrive_count(unsigned* counter) {
-  unsigned old;
-  asm volatile("atom.acq_rel.cta.shared::cta.add.u32 %0, [%1], 1;" : "=r"(old) : "r"(smem_u32(counter)) : "memory");
-  return old;
-}
-
-// Bounded wait for a template slot: the common case (already filled) costs one try_wait; the abort
-// flag is read only when the slot is not ready, so one warp's timeout stops the others quickly.
-__device__ __forceinline__ int wait_slot(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
-  if (mbar_try_wait(bar, parity)) return 1;
-  if (*abort_flag) return 0;
-  return mbar_wait(bar, parity) ? 1 : 0;
-}
-
-// Device status word: set kStatusTimeout when a bounded wait gave up.
-__device__ __forceinline__ void report_timeout(int* status, volatile int* abort_flag) {
-  *abort_flag = 1;
-  atomicOr(status, kStatusTimeout);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -1080,7 +1034,16 @@ __global__ void __launch_bounds__(256, 1)
 // ---------------------------------------------------------------------------------------
 // Host dispatch
 // ---------------------------------------------------------------------------------------
-int conv_group_threads(int L) { return L <= 256 ? 8 : (L <= 1024 ? 16 : (L <= 2048 ? 32 : 0)); }
+int conv_group_threads(int L) {
+  switch (L) {
+    case 256: return 8;
+    case 512: return 16;
+    case 1024:
+    case 2048: return 32;
+    case 4096: return 64;
+    default: return 128;
+  }
+}
 
 template <class Cfg>
 static cudaError_t launch_conv_cfg(const CUtensorMap* map, const ConvParams& p, int sm_count, cudaStream_t st) {
@@ -1110,8 +1073,6 @@ static cudaError_t launch_seg_cfg(const CUtensorMap* map, const SegParams& p, cu
 
 using Cfg256 = ConvCfg<256, 8, 1, 1>;
 using Cfg512 = ConvCfg<512, 16, 1, 1>;
-using Cfg1024 = ConvCfg<1024, 16, 2, 1>;
-using Cfg2048 = ConvCfg<2048, 32, 4, 1, 2>;
 
 template <class Cfg, int NV>
 static cudaError_t launch_tmem_nv(const ListParams& p, int sm_count, cudaStream_t st) {
@@ -1278,11 +1239,8 @@ cudaError_t launch_convolve(int L, const CUtensorMap* map, const ConvParams& p, 
   switch (L) {
     case 256: return launch_conv_cfg<Cfg256>(map, p, sm_count, st);
     case 512: return launch_single_desc(512, p, sm_count, st);
-    case 1024: return launch_conv_cfg<Cfg1024>(map, p, sm_count, st);
     case 2048: return launch_single_desc(2048, p, sm_count, st);
-    case 4096:
-    case 8192: return launch_convolve_big(L, p, sm_count, st);
-    default: return cudaErrorInvalidValue;
+    default: return launch_convolve_wide(L, p, sm_count, st);
   }
 }
 
@@ -1290,11 +1248,8 @@ cudaError_t launch_segment_spectra(int L, const CUtensorMap* map, const SegParam
   switch (L) {
     case 256: return launch_seg_cfg<Cfg256>(map, p, st);
     case 512: return launch_seg_cfg<Cfg512>(map, p, st);
-    case 1024: return launch_seg_cfg<Cfg1024>(map, p, st);
     case 2048: return launch_seg_cfg<ConvCfg<2048, 32, 2, 2>>(map, p, st);   // two-round exchange fits
-    case 4096:
-    case 8192: return launch_segment_spectra_big(L, p, sm_count, st);
-    default: return cudaErrorInvalidValue;
+    default: return launch_segment_spectra_wide(L, p, sm_count, st);
   }
 }
 

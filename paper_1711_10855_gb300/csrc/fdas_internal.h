@@ -79,7 +79,7 @@ struct PairParams {
 // Parameters of the forward-transform-only kernel (steps a2 + a3, for tests).
 struct SegParams {
   const float2* twist;
-  const float2* spectrum_in; // n_bins complex64 (read directly by the L >= 4096 kernel)
+  const float2* spectrum_in; // n_bins complex64 (bulk copies of the L = 1024, 4096, 8192 kernel)
   float2* out;              // nseg x L, natural order
   int* status;
   int64_t n_bins;
@@ -89,8 +89,7 @@ struct SegParams {
 
 // Threads per transform group (N1) used for segment length L; the template bank and the
 // twiddle table are stored in the layout of that decomposition (element k = k1 + N1*k2 at
-// ((k2/2)*N1 + k1)*2 + k2%2).  0 for L >= 4096: natural order, and the twiddle table holds
-// exp(-2 pi i t / L), t < L (shared-memory Stockham kernel, fdas_convolve_big.cu).
+// ((k2/2)*N1 + k1)*2 + k2%2).
 int conv_group_threads(int L);
 
 // Segments resident per CTA of the descriptor-driven kernel for segment length L, or 0 if L has
@@ -136,9 +135,9 @@ cudaError_t launch_tc_prepare(const float2* bank, int Z, float2* nat, unsigned* 
 // forward = true: the segment transforms (spectrum -> seg_out); false: the correlation (seg -> plane).
 cudaError_t launch_tc(const TcParams& p, int precision, bool forward, int sm_count, cudaStream_t stream);
 
-// Segment lengths 4096 and 8192 (fdas_convolve_big.cu); no tensor map.
-cudaError_t launch_convolve_big(int L, const ConvParams& p, int sm_count, cudaStream_t stream);
-cudaError_t launch_segment_spectra_big(int L, const SegParams& p, int sm_count, cudaStream_t stream);
+// Segment lengths 1024, 4096 and 8192 (fdas_convolve_wide.cu); no tensor map.
+cudaError_t launch_convolve_wide(int L, const ConvParams& p, int sm_count, cudaStream_t stream);
+cudaError_t launch_segment_spectra_wide(int L, const SegParams& p, int sm_count, cudaStream_t stream);
 
 }  // namespace fdas
 

@@ -103,10 +103,8 @@ __device__ void fft_inplace(double2* buf, int M, int count, const double2* W, in
 
 // Float offset of the real part of element k in the pair-major structure-of-arrays layout
 // (lane k1 = k % n1, k2 = k / n1; pair p = k2/2 of lane k1 is the float4 at p*n1 + k1 holding
-// re(2p), re(2p+1), im(2p), im(2p+1)); the imaginary part is 2 floats further.  n1 = 0 is the
-// interleaved natural order, where the imaginary part is the next float.
-__host__ __device__ __forceinline__ int layout_re(int k, int n1) {
-  if (n1 == 0) return 2 * k;
+// re(2p), re(2p+1), im(2p), im(2p+1)); the imaginary part is 2 floats further.
+__device__ __forceinline__ int layout_re(int k, int n1) {
   const int k1 = k % n1, k2 = k / n1;
   return ((k2 >> 1) * n1 + k1) * 4 + (k2 & 1);
 }
@@ -120,14 +118,8 @@ struct BankShape {
 };
 
 // Inter-pass twiddles exp(+i 2pi n2 k1 / L), n2 < N2 = L/n1, k1 < n1: lane k1's pair j holds
-// n2 = j and n2 = j + N2/2 (float4 at j*n1 + k1: re, re, im, im).  n1 = 0: the natural table
-// exp(-2 pi i t / L).
+// n2 = j and n2 = j + N2/2 (float4 at j*n1 + k1: re, re, im, im).
 __device__ void write_twist(float2* tw, int idx, int L, int n1) {
-  if (n1 == 0) {
-    const double2 w = cispi(-2.0 * (double)idx / (double)L);
-    tw[idx] = make_float2((float)w.x, (float)w.y);
-    return;
-  }
   const int k1 = idx % n1, n2 = idx / n1;
   const int h2 = L / n1 / 2;
   const double2 w = cispi(2.0 * (double)(((long long)n2 * k1) % L) / (double)L);
@@ -243,7 +235,6 @@ __global__ void __launch_bounds__(kThreads) template_bank_kernel(double2* taps, 
   float* tp = reinterpret_cast<float*>(templates + (size_t)(zc + j) * L);
   float* tn = reinterpret_cast<float*>(templates + (size_t)(zc - j) * L);
   const double inv = 1.0 / (double)L;
-  const int im = b.n1 ? 2 : 1;
   for (int k = tid; k < L; k += kThreads) {
     const int t = (int)(((long long)k * h) & (L - 1));            // e^{2 pi i t / L}
     double2 ph = W[(t & (L / 2 - 1)) * (N / L)];
@@ -251,10 +242,10 @@ __global__ void __launch_bounds__(kThreads) template_bank_kernel(double2* taps, 
     const double2 s = buf[k];
     const int off = layout_re(k, b.n1);
     tp[off] = (float)(fma(ph.x, s.x, -ph.y * s.y) * inv);
-    tp[off + im] = (float)(fma(ph.x, s.y, ph.y * s.x) * inv);
+    tp[off + 2] = (float)(fma(ph.x, s.y, ph.y * s.x) * inv);
     if (j) {
       tn[off] = (float)(fma(ph.x, s.x, ph.y * s.y) * inv);
-      tn[off + im] = (float)(fma(-ph.x, s.y, ph.y * s.x) * inv);
+      tn[off + 2] = (float)(fma(-ph.x, s.y, ph.y * s.x) * inv);
     }
   }
 }
