@@ -89,7 +89,8 @@ EncodeTiledFn get_encode_fn() {
   return fn;
 }
 
-// The other lengths' kernels fetch the spectrum by bulk copies of its in-range part.
+// fdas_segment_spectra of the short lengths reads the spectrum through a tensor map; every other kernel
+// fetches its in-range part by bulk copies.
 bool needs_spectrum_map(int L) { return L <= 512 || L == 2048; }
 
 // Record the plan's completion event after work enqueued on `st` (skipped while the stream is
@@ -255,8 +256,6 @@ int fdas_convolve_power(fdas_plan* p, const float* d_spectrum, float* d_plane, f
   if (!p->built) return FDAS_ERR_NOT_BUILT;
   if ((reinterpret_cast<uintptr_t>(d_spectrum) & 15u) || (reinterpret_cast<uintptr_t>(d_plane) & 15u))
     return FDAS_ERR_ALIGN;
-  int rc = make_spectrum_map(p, d_spectrum);
-  if (rc != FDAS_OK) return rc;
   fdas::ConvParams q;
   q.spectrum = reinterpret_cast<const float2*>(d_spectrum);
   q.templates = p->d_templates;
@@ -270,7 +269,7 @@ int fdas_convolve_power(fdas_plan* p, const float* d_spectrum, float* d_plane, f
   q.V = p->V;
   q.h = p->h;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  return enqueued(p, st, fdas::launch_convolve(p->L, &p->map, q, p->sm_count, st));
+  return enqueued(p, st, fdas::launch_convolve(p->L, q, p->sm_count, st));
 }
 
 int fdas_plan_group_segments(const fdas_plan* p) {
@@ -558,20 +557,6 @@ int validate_geometry(int64_t n_bins, int zmax, int zstep, int seg_len, int tmpl
 cudaError_t launch_wait_selftest(int* status, int64_t limit_ns, cudaStream_t st) {
   wait_selftest_kernel<<<1, 1, 0, st>>>(status, (unsigned long long)limit_ns);
   return cudaGetLastError();
-}
-
-int encode_spectrum_map(CUtensorMap* map, const void* d_spectrum, int64_t n_bins, int L) {
-  if (!needs_spectrum_map(L)) return FDAS_OK;
-  EncodeTiledFn enc = get_encode_fn();
-  if (!enc) return FDAS_ERR_CUDA;
-  cuuint64_t gdim[1] = {(cuuint64_t)n_bins};
-  cuuint64_t gstride[1] = {0};
-  cuuint32_t box[1] = {(cuuint32_t)(L < 256 ? L : 256)};
-  cuuint32_t estride[1] = {1};
-  CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 1, const_cast<void*>(d_spectrum), gdim, gstride, box,
-                   estride, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                   CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS ? FDAS_OK : FDAS_ERR_CUDA;
 }
 
 }  // namespace fdas

@@ -106,9 +106,7 @@ cudaError_t launch_per_spectrum(const fdas_batch* b, const float* const* d_spect
     q.Z = d.Z;
     q.V = b->V;
     q.h = b->h;
-    CUtensorMap map;
-    if (fdas::encode_spectrum_map(&map, d_spectra[i], d.n_bins, b->L) != FDAS_OK) return cudaErrorInvalidValue;
-    const cudaError_t e = fdas::launch_convolve(b->L, &map, q, b->sm_count, st);
+    const cudaError_t e = fdas::launch_convolve(b->L, q, b->sm_count, st);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;

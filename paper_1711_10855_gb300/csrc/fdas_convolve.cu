@@ -161,173 +161,6 @@ __device__ __forceinline__ void forward_transform(const float2* sx, const float4
   forward_transform_with<Cfg>(sx, [&](cp2 (&v)[Cfg::H2]) { apply_twist2<Cfg, true>(v, stw, k1); }, xb, k1, out);
 }
 
-// Store X[n] (held by lane t = n mod N1) into the pair-major layout of the inverse transform.
-template <class Cfg>
-__device__ __forceinline__ void store_spectrum_element(float* sx, int t, int k2, float re, float im) {
-  const int base = ((k2 >> 1) * Cfg::N1 + t) * 4 + (k2 & 1);
-  sx[base] = re;
-  sx[base + 2] = im;
-}
-
-// ---------------------------------------------------------------------------------------
-// The fused kernel
-// ---------------------------------------------------------------------------------------
-template <class Cfg>
-__global__ void __launch_bounds__(256, 1)
-    fdas_convolve_kernel(const __grid_constant__ CUtensorMap spec_map, const ConvParams p) {
-  constexpr int L = Cfg::L, N1 = Cfg::N1, R = Cfg::R, P = Cfg::P, G = Cfg::G;
-  extern __shared__ __align__(1024) unsigned char smem[];
-  float2* sX = reinterpret_cast<float2*>(smem + Cfg::OFF_X);
-  float2* sT = reinterpret_cast<float2*>(smem + Cfg::OFF_T);
-  float2* sTw = reinterpret_cast<float2*>(smem + Cfg::OFF_TW);
-  float4* sXb = reinterpret_cast<float4*>(smem + Cfg::OFF_XB);
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + Cfg::OFF_BAR);
-  uint64_t* segbar = full + R;
-  uint64_t* twbar = segbar + 1;
-  int64_t* issued_pos = reinterpret_cast<int64_t*>(twbar + 1);   // [R] last position issued per slot
-  unsigned* cnt = reinterpret_cast<unsigned*>(issued_pos + R);      // [R] consumer arrivals per slot
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(cnt + R);
-
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int gw = lane / N1, k1 = lane % N1;
-  const int par = warp % P;
-  const int seg_slot = (warp / P) * Cfg::F + gw;
-  float2* myX = sX + seg_slot * L;
-  float4* myXb = sXb + warp * Cfg::XWARP + gw * Cfg::XGROUP;
-  const float4* stw4 = reinterpret_cast<const float4*>(sTw);
-
-  const int64_t U = p.units;
-  const int64_t u0 = (int64_t)blockIdx.x * U / gridDim.x;
-  const int64_t u1 = ((int64_t)blockIdx.x + 1) * U / gridDim.x;
-  const int64_t npos = u1 - u0;
-  if (npos <= 0) return;
-
-  if (tid == 0) {
-    for (int r = 0; r < R; ++r) {
-      mbar_init(&full[r], 1);
-      cnt[r] = 0u;
-      issued_pos[r] = -1;
-    }
-    mbar_init(segbar, 1);
-    mbar_init(twbar, 1);
-    *abort_flag = 0;
-    fence_barrier_init();
-  }
-  __syncthreads();
-
-  auto issue_template = [&](int64_t i) {
-    const int slot = (int)(i % R);
-    const int64_t z = (u0 + i) % p.Z;
-    issued_pos[slot] = i;
-    mbar_arrive_expect_tx(&full[slot], L * 8);
-    bulk_g2s(sT + (size_t)slot * L, p.templates + (size_t)z * L, L * 8, &full[slot]);
-  };
-  if (tid == 0) {
-    mbar_arrive_expect_tx(twbar, L * 8);
-    bulk_g2s(sTw, p.twist, L * 8, twbar);
-    const int64_t first = npos < R ? npos : R;
-    for (int64_t i = 0; i < first; ++i) issue_template(i);
-  }
-  // `alive` is CTA-uniform: it only changes through __syncthreads_and.
-  int alive = __syncthreads_and(mbar_wait(twbar, 0) ? 1 : 0);
-  if (!alive && tid == 0) report_timeout(p.status, abort_flag);
-
-  uint32_t seg_phase = 0;
-  bool seg_in_flight = false;
-  const int64_t g_first = u0 / p.Z, g_last = (u1 - 1) / p.Z;
-  for (int64_t grp = g_first; grp <= g_last; ++grp) {
-    const int64_t a = (grp * p.Z > u0 ? grp * p.Z : u0) - u0;
-    const int64_t b = ((grp + 1) * p.Z < u1 ? (grp + 1) * p.Z : u1) - u0;
-    // every warp is done with the previous group's spectra before they are overwritten
-    alive = __syncthreads_and(alive && !*abort_flag);
-    if (!alive) break;
-    if (tid == 0) {
-      mbar_arrive_expect_tx(segbar, G * L * 8);
-      for (int j = 0; j < G; ++j) {
-        const int64_t x0 = (grp * G + j) * (int64_t)p.V - p.h;
-        for (int bx = 0; bx < L / Cfg::BOX; ++bx)
-          tma_load_1d(sX + (size_t)j * L + bx * Cfg::BOX, &spec_map, (int32_t)(x0 + bx * Cfg::BOX), segbar);
-      }
-    }
-    seg_in_flight = true;
-    alive = __syncthreads_and(mbar_wait(segbar, seg_phase) ? 1 : 0);
-    if (!alive) {
-      if (tid == 0) report_timeout(p.status, abort_flag);
-      break;
-    }
-    seg_in_flight = false;
-    seg_phase ^= 1u;
-    if (par == 0) {
-      // a3: forward FFT in place; X[n] goes to the pair-major layout of the inverse transform
-      forward_transform<Cfg>(myX, stw4, myXb, k1, [&](auto rr, auto nn, const cp2& x) {
-        constexpr int r = decltype(rr)::value, n1 = decltype(nn)::value;
-        float* sx = reinterpret_cast<float*>(myX);
-        store_spectrum_element<Cfg>(sx, k1, r + Cfg::C * n1, x.re.x, x.im.x);
-        store_spectrum_element<Cfg>(sx, k1, r + Cfg::CP + Cfg::C * n1, x.re.y, x.im.y);
-      });
-    }
-    __syncthreads();
-
-    const int64_t s = grp * G + seg_slot;
-    const int64_t segbase = s * (int64_t)p.V;
-    const int64_t lim64 = p.n_bins - segbase < (int64_t)p.V ? p.n_bins - segbase : (int64_t)p.V;
-    const int lim = lim64 > 0 ? (int)lim64 : 0;   // outputs n < lim of this segment are stored
-    int64_t i = a + (((par - a) % P) + P) % P;
-    for (; i < b; i += P) {
-      const int slot = (int)(i % R);
-      // warp-uniform bounded wait for the template of position i
-      const int ok = __all_sync(0xffffffffu, wait_slot(&full[slot], (uint32_t)((i / R) & 1), abort_flag));
-      if (!ok) {
-        if (lane == 0) report_timeout(p.status, abort_flag);
-        break;
-      }
-      const int64_t z = (u0 + i) % p.Z;
-      const float2* st = sT + (size_t)slot * L;
-
-      // a4: Y = X * T, loaded as packed pairs in the first pass's bit-reversed order
-      cp2 v[Cfg::H2];
-      static_for<Cfg::H2>([&](auto pp) {
-        constexpr int q = decltype(pp)::value;
-        const cp2 x = cp2_from(reinterpret_cast<const float4*>(myX)[q * N1 + k1]);
-        const cp2 t = cp2_from(reinterpret_cast<const float4*>(st)[q * N1 + k1]);
-        v[bitrev(2 * q, Cfg::LOG_N2)] = cmul2(x, t);
-      });
-      // release the template slot; the last of the W/P consumers refills it R positions ahead
-      __syncwarp();
-      if (lane == 0) {
-        const unsigned old = arrive_count(&cnt[slot]);
-        if ((old + 1u) % (unsigned)(Cfg::W / P) == 0u) {
-          if (i + R < npos) {
-            fence_proxy_async_smem();
-            issue_template(i + R);
-          }
-        }
-      }
-      // a5: inverse FFT
-      fft_split_pairs<Cfg::N2, +1>(v);
-      apply_twist2<Cfg, false>(v, stw4, k1);
-      float* row = p.plane + z * p.n_bins + segbase;
-      exchange_and_pass2<Cfg, +1>(v, myXb, k1, [&](auto rr, auto nn, const cp2& y) {
-        // a6 + a7: keep n < V (and inside the spectrum), store |y|^2
-        constexpr int r = decltype(rr)::value, n1 = decltype(nn)::value;
-        const float2 pw = power2(y);
-        const int n_lo = r * N1 + k1 + Cfg::N2 * n1;
-        const int n_hi = n_lo + Cfg::CP * N1;
-        if (n_lo < lim) __stcs(row + n_lo, pw.x);
-        if (n_hi < lim) __stcs(row + n_hi, pw.y);
-      });
-    }
-  }
-
-  // After a timeout, wait (bounded) for this CTA's copies still in flight before exiting.
-  __syncthreads();
-  if (tid == 0 && (*abort_flag || !alive)) {
-    for (int r = 0; r < R; ++r)
-      if (issued_pos[r] >= 0) (void)mbar_wait(&full[r], (uint32_t)((issued_pos[r] / R) & 1));
-    if (seg_in_flight) (void)mbar_wait(segbar, seg_phase);
-  }
-}
-
 // ---------------------------------------------------------------------------------------
 // Variant with the segment spectra and the twiddle table in tensor memory (one column pair per
 // lane: N2 = 2*N1, i.e. L = 512 and 2048).  Every warp owns its own segment(s); the template of
@@ -336,19 +169,19 @@ __global__ void __launch_bounds__(256, 1)
 // spectrum and the twiddles come from TMEM, a separate store, which relieves the shared-memory
 // bandwidth that otherwise co-limits the kernel with the FP32 pipe.
 // ---------------------------------------------------------------------------------------
-template <int L_, int N1_>
+template <int L_, int N1_, int W_ = 8, int P_ = 1>
 struct TmemCfg {
   static constexpr int L = L_;
   static constexpr int N1 = N1_;
   static constexpr int N2 = L / N1;
   static constexpr int H2 = N2 / 2;
   static constexpr int F = 32 / N1;
-  static constexpr int W = 8;
-  static constexpr int P = 1;
-  static constexpr int G = F * W;          // segments resident per CTA: one group of lanes each
+  static constexpr int W = W_;             // warps per CTA
+  static constexpr int P = P_;             // warps sharing a segment, taking alternate templates
+  static constexpr int G = F * W / P;      // segments resident per CTA: one group of lanes each
   static constexpr int R = 4;
-  static constexpr int C = 2;
-  static constexpr int CP = 1;
+  static constexpr int C = N2 / N1;        // pass-2 columns per lane
+  static constexpr int CP = C / 2;         // and column pairs (exchange rounds)
   static constexpr int XR = 1;
   static constexpr int XCOLS = N1;
   static constexpr int XPITCH = N1 + 1;
@@ -356,7 +189,6 @@ struct TmemCfg {
   static constexpr int XWARP = F * XGROUP;
   static constexpr int LOG_N1 = ilog2(N1);
   static constexpr int LOG_N2 = ilog2(N2);
-  static constexpr int BOX = L < 256 ? L : 256;
   // per-warp shared region: staging of its segments, then its exchange tiles
   static constexpr size_t REGION = align_up(((size_t)F * L * 8 > (size_t)XWARP * 16) ? (size_t)F * L * 8
                                                                                      : (size_t)XWARP * 16, 128);
@@ -364,12 +196,13 @@ struct TmemCfg {
   static constexpr size_t OFF_REG = OFF_T + (size_t)R * L * 8;
   static constexpr size_t OFF_BAR = align_up(OFF_REG + (size_t)W * REGION, 128);
   static constexpr size_t SMEM = OFF_BAR + 256;
-  // TMEM columns of each quadrant: twiddles, then the spectra of its two warps
+  // TMEM columns of each quadrant: twiddles, then the spectra of its segments' warps
   static constexpr uint32_t TMEM_COLS = 512;
   static constexpr uint32_t COL_TW = 0;
   static constexpr uint32_t COL_X = 2 * N2;
-  static_assert(N2 == 2 * N1 && 32 % N1 == 0, "one column pair per lane");
-  static_assert(6 * N2 <= (int)TMEM_COLS, "TMEM columns");
+  static_assert((C == 2 || C == 4) && 32 % N1 == 0, "one or two column pairs per lane");
+  static_assert(W % (4 * P) == 0 && (P == 1 || P == 2), "warps sharing a segment share a TMEM quadrant");
+  static_assert(2 * N2 * (1 + W / P / 4) <= (int)TMEM_COLS, "TMEM columns");
   static_assert(SMEM <= 232448, "shared memory budget");
 };
 
@@ -408,10 +241,11 @@ __device__ __forceinline__ int64_t unit_total(const ListParams& p) { return p.un
 // transform).  The time of a group is then set by its busiest warp, not by the number of listed
 // units: sparse masks cost about their share of (segment, template) pairs.
 template <class Cfg, int NV, bool LIST, bool DEC = false>
-__global__ void __launch_bounds__(256, 1)
+__global__ void __launch_bounds__(32 * Cfg::W, 1)
     fdas_convolve_tmem_kernel(const std::conditional_t<LIST, ListParams, BatchParams> p) {
   static_assert(!DEC || LIST, "decoupled warps serve masked work lists");
-  constexpr int L = Cfg::L, N1 = Cfg::N1, R = Cfg::R, G = Cfg::G, H2 = Cfg::H2, W = Cfg::W;
+  static_assert(!LIST || Cfg::P == 1, "work lists: every warp walks every position");
+  constexpr int L = Cfg::L, N1 = Cfg::N1, R = Cfg::R, G = Cfg::G, H2 = Cfg::H2, W = Cfg::W, P = Cfg::P;
   extern __shared__ __align__(1024) unsigned char smem[];
   float2* sT = reinterpret_cast<float2*>(smem + Cfg::OFF_T);
   unsigned char* sReg = smem + Cfg::OFF_REG;
@@ -421,7 +255,8 @@ __global__ void __launch_bounds__(256, 1)
   unsigned* cnt = reinterpret_cast<unsigned*>(issued_pos + R);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(cnt + R);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(cnt + R + 1);
-  // template-refill cursor (positions are issued in increasing order, one thread at a time)
+  // template-refill cursor, one per position parity with P = 2 (the positions of one parity are issued in
+  // increasing order, one thread at a time)
   struct IssueCursor {
     int64_t u;          // unit of the next position to issue
     int64_t spec_end;   // first unit of the next spectrum
@@ -432,6 +267,9 @@ __global__ void __launch_bounds__(256, 1)
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int gw = lane / N1, k1 = lane % N1;
+  // P = 2: warps w and w + 4 (one TMEM quadrant) hold the same segments and take alternate templates
+  const int par = P == 2 ? (warp >> 2) & 1 : 0;
+  const int wseg = P == 2 ? (warp & 3) + 4 * (warp >> 3) : warp;
   float2* myRegion = reinterpret_cast<float2*>(sReg + (size_t)warp * Cfg::REGION);
   float2* mySeg = myRegion + (size_t)gw * L;
   float4* myXb = reinterpret_cast<float4*>(myRegion) + gw * Cfg::XGROUP;
@@ -473,8 +311,22 @@ __global__ void __launch_bounds__(256, 1)
   tmem_fence_after_sync();
   const uint32_t tmem_row = *tmem_slot + ((uint32_t)(32 * (warp & 3)) << 16);
   const uint32_t tw_addr = tmem_row + Cfg::COL_TW;
-  const uint32_t x_addr = tmem_row + Cfg::COL_X + (uint32_t)(warp >> 2) * (2 * Cfg::N2);
+  const uint32_t x_addr = tmem_row + Cfg::COL_X + (uint32_t)(wseg >> 2) * (2 * Cfg::N2);
 
+  // Move a cursor n units on (P = 2)
+  [[maybe_unused]] auto advance = [&](IssueCursor* c, int n) {
+    c->u += n;
+    c->z += n;
+    while (c->u >= c->spec_end && c->u < U) {   // into a later spectrum
+      const SpecDesc dn = spectrum_desc(p, c->b + 1);
+      c->z = (int)(c->u - c->spec_end);
+      c->b += 1;
+      c->Z = dn.Z;
+      c->z_off = dn.z_off;
+      c->spec_end = c->b + 1 < p.count ? spectrum_desc(p, c->b + 1).unit_base : U;
+    }
+    while (c->z >= c->Z) c->z -= c->Z;
+  };
   // Template of CTA position i (unit u0 + i): bank row z_off_b + (u - unit_base_b) mod Z_b.  The
   // cursor walks units in order, so an issue costs a few shared-memory operations; a descriptor is
   // read from global memory only when the walk enters the next spectrum.
@@ -482,11 +334,16 @@ __global__ void __launch_bounds__(256, 1)
     const int slot = (int)(i % R);
     issued_pos[slot] = i;
     int64_t zrow;
+    IssueCursor* const cp = P == 2 ? cur + (i & 1) : cur;
     if constexpr (LIST) zrow = cur->z_off + unit_at(u0 + i) % cur->Z;
-    else zrow = cur->z_off + cur->z;
+    else zrow = cp->z_off + cp->z;
     mbar_arrive_expect_tx(&full[slot], L * 8);
     bulk_g2s(sT + (size_t)slot * L, p.templates + (size_t)zrow * L, L * 8, &full[slot]);
     if constexpr (LIST) return;   // single spectrum: the cursor's spectrum never changes
+    if constexpr (P == 2) {
+      advance(cp, 2);
+      return;
+    }
     cur->u += 1;
     cur->z = cur->z + 1 == cur->Z ? 0 : cur->z + 1;
     if (cur->u == cur->spec_end && cur->u < U) {
@@ -508,34 +365,22 @@ __global__ void __launch_bounds__(256, 1)
     cur->z_off = d0.z_off;
     cur->z = (int)((u0 - d0.unit_base) % d0.Z);
     cur->spec_end = b0 + 1 < p.count ? spectrum_desc(p, b0 + 1).unit_base : U;
+    if constexpr (P == 2) {
+      cur[1] = cur[0];
+      advance(cur + 1, 1);
+    }
     const int64_t first = npos < R ? npos : R;
     for (int64_t i = 0; i < first; ++i) issue_template(i);
   }
   // twiddle pairs of lane k1 into this quadrant's TMEM rows (one warp per quadrant)
-  if (warp < 4) {
-    const float4* tw4 = reinterpret_cast<const float4*>(p.twist);
-    static_for<H2 / 4>([&](auto cc) {
-      constexpr int c = decltype(cc)::value;
-      float r[16];
-      static_for<4>([&](auto qq) {
-        constexpr int q = decltype(qq)::value;
-        const float4 w = __ldg(tw4 + (4 * c + q) * N1 + k1);
-        r[4 * q] = w.x;
-        r[4 * q + 1] = w.y;
-        r[4 * q + 2] = w.z;
-        r[4 * q + 3] = w.w;
-      });
-      tmem_st16(tw_addr + 16 * c, r);
-    });
-    tmem_wait_st();
-  }
-  // release template slot `slot` of position i; the last of the W consumers refills it R positions
-  // ahead
+  if (warp < 4) twiddles_to_tmem<H2>(p.twist, N1, k1, tw_addr);
+  // release template slot `slot` of position i; the last of the W / P consumers refills it R
+  // positions ahead
   auto release_slot = [&](int64_t i, int slot) {
     __syncwarp();
     if (lane == 0) {
       const unsigned old = arrive_count(&cnt[slot]);
-      if ((old + 1u) % (unsigned)W == 0u) {
+      if ((old + 1u) % (unsigned)(W / P) == 0u) {
         if (i + R < npos) {
           fence_proxy_async_smem();
           issue_template(i + R);
@@ -582,16 +427,17 @@ __global__ void __launch_bounds__(256, 1)
       }
       mbar_arrive_expect_tx(segbar, bytes);
       for (int j = 0; j < G; ++j) {
-        float2* dst = reinterpret_cast<float2*>(sReg + (size_t)(j / Cfg::F) * Cfg::REGION) + (size_t)(j % Cfg::F) * L;
+        const int ws = j / Cfg::F, wj = P == 2 ? (ws & 3) + 8 * (ws >> 2) : ws;   // the segment's first warp
+        float2* dst = reinterpret_cast<float2*>(sReg + (size_t)wj * Cfg::REGION) + (size_t)(j % Cfg::F) * L;
         const int64_t x0 = (grp * G + j) * (int64_t)p.V - p.h;
         const int64_t c0 = x0 > 0 ? x0 : 0;
         const int64_t c1 = x0 + L < d.n_bins ? x0 + L : d.n_bins;
         if (c1 > c0) bulk_g2s(dst + (c0 - x0), d.spec + c0, (uint32_t)((c1 - c0) * 8), segbar);
       }
     }
-    {
+    if (P == 1 || par == 0) {
       // zeros outside [0, n_b) in this lane group's window
-      const int64_t x0 = (grp * G + warp * Cfg::F + gw) * (int64_t)p.V - p.h;
+      const int64_t x0 = (grp * G + wseg * Cfg::F + gw) * (int64_t)p.V - p.h;
       const int64_t lo = x0 < 0 ? (-x0 < L ? -x0 : L) : 0;                           // [0, lo) below 0
       const int64_t hi = d.n_bins - x0 < L ? (d.n_bins - x0 > 0 ? d.n_bins - x0 : 0) : L;  // [hi, L) beyond n
       for (int e = k1; e < L; e += N1)
@@ -607,22 +453,39 @@ __global__ void __launch_bounds__(256, 1)
     seg_phase ^= 1u;
 
     // a3: forward FFT of this lane group's segment; X pairs (k2 = 2p, 2p+1) go to TMEM
-    {
+    if (P == 1 || par == 0) {
       float xr[16];
+      cp2 first[Cfg::CP == 2 ? N1 : 1];   // two column pairs: round 0's, until round 1's complete the pairs
       forward_transform_with<Cfg>(
           mySeg, [&](cp2 (&v)[H2]) { apply_twist_tmem<Cfg, true>(v, tw_addr); }, myXb, k1,
-          [&](auto, auto nn, const cp2& x) {
-            constexpr int n1 = decltype(nn)::value;   // pair p = n1
-            xr[4 * (n1 & 3)] = x.re.x;
-            xr[4 * (n1 & 3) + 1] = x.re.y;
-            xr[4 * (n1 & 3) + 2] = x.im.x;
-            xr[4 * (n1 & 3) + 3] = x.im.y;
-            if constexpr ((n1 & 3) == 3) tmem_st16(x_addr + 4 * (n1 - 3), xr);
+          [&](auto rr, auto nn, const cp2& x) {
+            [[maybe_unused]] constexpr int r = decltype(rr)::value, n1 = decltype(nn)::value;
+            auto put = [&](auto pp, float a, float b, float c, float d) {
+              constexpr int pr = decltype(pp)::value;
+              xr[4 * (pr & 3)] = a;
+              xr[4 * (pr & 3) + 1] = b;
+              xr[4 * (pr & 3) + 2] = c;
+              xr[4 * (pr & 3) + 3] = d;
+              if constexpr ((pr & 3) == 3) tmem_st16(x_addr + 4 * (pr - 3), xr);
+            };
+            if constexpr (Cfg::CP == 1) {   // pair p = n1
+              put(nn, x.re.x, x.re.y, x.im.x, x.im.y);
+            } else if constexpr (r == 0) {  // elements k2 = 4 n1, 4 n1 + 2
+              first[n1] = x;
+            } else {                        // and 4 n1 + 1, 4 n1 + 3
+              put(std::integral_constant<int, 2 * n1>{}, first[n1].re.x, x.re.x, first[n1].im.x, x.im.x);
+              put(std::integral_constant<int, 2 * n1 + 1>{}, first[n1].re.y, x.re.y, first[n1].im.y, x.im.y);
+            }
           });
       tmem_wait_st();
     }
+    if constexpr (P == 2) {   // the other warp of the segment reads the spectrum too
+      tmem_fence_before_sync();
+      __syncthreads();
+      tmem_fence_after_sync();
+    }
 
-    const int64_t s = grp * G + warp * Cfg::F + gw;
+    const int64_t s = grp * G + wseg * Cfg::F + gw;
     const int64_t segbase = s * (int64_t)p.V;
     const int64_t lim64 = d.n_bins - segbase < (int64_t)p.V ? d.n_bins - segbase : (int64_t)p.V;
     const int lim = lim64 > 0 ? (int)lim64 : 0;
@@ -705,7 +568,7 @@ __global__ void __launch_bounds__(256, 1)
       tmem_fence_before_sync();
       continue;
     }
-    for (int64_t i = a; i < bpos; ++i) {
+    for (int64_t i = P == 1 ? a : a + ((par - a) & 1); i < bpos; i += P) {
       const int slot = (int)(i % R);
       const int ok = __all_sync(0xffffffffu, wait_slot(&full[slot], (uint32_t)((i / R) & 1), abort_flag));
       if (!ok) {
@@ -759,13 +622,13 @@ __global__ void __launch_bounds__(256, 1)
       fft_split_pairs<Cfg::N2, +1>(v);
       apply_twist_tmem<Cfg, false>(v, tw_addr);
       float* row = d.plane + z * d.n_bins + segbase;
-      exchange_and_pass2<Cfg, +1>(v, myXb, k1, [&](auto, auto nn, const cp2& y) {
+      exchange_and_pass2<Cfg, +1>(v, myXb, k1, [&](auto rr, auto nn, const cp2& y) {
         // a6 + a7: keep n < V (and inside the spectrum), store |y|^2
-        constexpr int n1 = decltype(nn)::value;
+        constexpr int r = decltype(rr)::value, n1 = decltype(nn)::value;
         if constexpr (n1 < NV) {
           const float2 pw = power2(y);
-          const int n_lo = k1 + Cfg::N2 * n1;
-          const int n_hi = n_lo + N1;
+          const int n_lo = r * N1 + k1 + Cfg::N2 * n1;
+          const int n_hi = n_lo + Cfg::CP * N1;
           if (n_lo < lim_z) __stcs(row + n_lo, pw.x);
           if (n_hi < lim_z) __stcs(row + n_hi, pw.y);
         }
@@ -837,23 +700,7 @@ __global__ void __launch_bounds__(256, 1) fdas_convolve_pairs_kernel(const PairP
   const uint32_t tw_addr = tmem_row + Cfg::COL_TW;
   const uint32_t x_addr = tmem_row + Cfg::COL_X + (uint32_t)(warp >> 2) * (2 * Cfg::N2);
   // twiddle pairs of lane k1 into this quadrant's TMEM rows (one warp per quadrant)
-  if (warp < 4) {
-    const float4* tw4 = reinterpret_cast<const float4*>(p.twist);
-    static_for<H2 / 4>([&](auto cc) {
-      constexpr int c = decltype(cc)::value;
-      float r[16];
-      static_for<4>([&](auto qq) {
-        constexpr int q = decltype(qq)::value;
-        const float4 w = __ldg(tw4 + (4 * c + q) * N1 + k1);
-        r[4 * q] = w.x;
-        r[4 * q + 1] = w.y;
-        r[4 * q + 2] = w.z;
-        r[4 * q + 3] = w.w;
-      });
-      tmem_st16(tw_addr + 16 * c, r);
-    });
-    tmem_wait_st();
-  }
+  if (warp < 4) twiddles_to_tmem<H2>(p.twist, N1, k1, tw_addr);
   tmem_fence_before_sync();
   __syncthreads();
   tmem_fence_after_sync();
@@ -1046,19 +893,6 @@ int conv_group_threads(int L) {
 }
 
 template <class Cfg>
-static cudaError_t launch_conv_cfg(const CUtensorMap* map, const ConvParams& p, int sm_count, cudaStream_t st) {
-  auto kern = fdas_convolve_kernel<Cfg>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::SMEM);
-  if (e != cudaSuccess) return e;
-  ConvParams q = p;
-  const int64_t ngroups = (p.nseg + Cfg::G - 1) / Cfg::G;
-  q.units = ngroups * p.Z;
-  const int64_t grid = q.units < sm_count ? q.units : sm_count;
-  kern<<<(unsigned)grid, 256, Cfg::SMEM, st>>>(*map, q);
-  return cudaGetLastError();
-}
-
-template <class Cfg>
 static cudaError_t launch_seg_cfg(const CUtensorMap* map, const SegParams& p, cudaStream_t st) {
   constexpr int GS = 8 * Cfg::F;
   constexpr size_t smem = align_up(((size_t)GS * Cfg::L + Cfg::L) * 8 + (size_t)8 * Cfg::XWARP * 16, 128) + 64;
@@ -1074,51 +908,57 @@ static cudaError_t launch_seg_cfg(const CUtensorMap* map, const SegParams& p, cu
 using Cfg256 = ConvCfg<256, 8, 1, 1>;
 using Cfg512 = ConvCfg<512, 16, 1, 1>;
 
-template <class Cfg, int NV>
+// Full planes: PlaneCfg.  Work lists: ListCfg (the same segments per CTA; void: none), separate
+// instantiations with their own parameter type, so that the full-plane code stays free of them.
+template <class PlaneCfg, class ListCfg, int NV>
 static cudaError_t launch_tmem_nv(const ListParams& p, int sm_count, cudaStream_t st) {
-  // the work-list variant is a separate instantiation (with its own parameter type): the
-  // full-plane code stays free of it
   const int64_t grid = p.units < sm_count ? p.units : sm_count;
-  if (p.unit_list && p.unit_mask) {
-    auto kern = fdas_convolve_tmem_kernel<Cfg, NV, true, true>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::SMEM);
+  auto launch = [&](auto kern, int warps, size_t smem, const auto& params) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    kern<<<(unsigned)grid, 256, Cfg::SMEM, st>>>(p);
-  } else if (p.unit_list) {
-    auto kern = fdas_convolve_tmem_kernel<Cfg, NV, true>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::SMEM);
-    if (e != cudaSuccess) return e;
-    kern<<<(unsigned)grid, 256, Cfg::SMEM, st>>>(p);
+    kern<<<(unsigned)grid, 32 * warps, smem, st>>>(params);
+    return cudaGetLastError();
+  };
+  if constexpr (std::is_void_v<ListCfg>) {
+    if (p.unit_list) return cudaErrorInvalidValue;
   } else {
-    auto kern = fdas_convolve_tmem_kernel<Cfg, NV, false>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::SMEM);
-    if (e != cudaSuccess) return e;
-    kern<<<(unsigned)grid, 256, Cfg::SMEM, st>>>(static_cast<const BatchParams&>(p));
+    static_assert(PlaneCfg::G == ListCfg::G, "a unit is the same segments in both");
+    if (p.unit_list && p.unit_mask)
+      return launch(fdas_convolve_tmem_kernel<ListCfg, NV, true, true>, ListCfg::W, ListCfg::SMEM, p);
+    if (p.unit_list) return launch(fdas_convolve_tmem_kernel<ListCfg, NV, true>, ListCfg::W, ListCfg::SMEM, p);
   }
-  return cudaGetLastError();
+  return launch(fdas_convolve_tmem_kernel<PlaneCfg, NV, false>, PlaneCfg::W, PlaneCfg::SMEM,
+                static_cast<const BatchParams&>(p));
 }
 
 // Smallest instantiated NV >= ceil(V / N2): N1*3/4, N1*7/8 or N1.
-template <class Cfg>
+template <class PlaneCfg, class ListCfg>
 static cudaError_t launch_tmem_cfg(const ListParams& p, int sm_count, cudaStream_t st) {
-  const int rows = (p.V + Cfg::N2 - 1) / Cfg::N2;
-  if (rows <= Cfg::N1 * 3 / 4) return launch_tmem_nv<Cfg, Cfg::N1 * 3 / 4>(p, sm_count, st);
-  if (rows <= Cfg::N1 * 7 / 8) return launch_tmem_nv<Cfg, Cfg::N1 * 7 / 8>(p, sm_count, st);
-  return launch_tmem_nv<Cfg, Cfg::N1>(p, sm_count, st);
+  constexpr int N1 = PlaneCfg::N1;
+  const int rows = (p.V + PlaneCfg::N2 - 1) / PlaneCfg::N2;
+  if (rows <= N1 * 3 / 4) return launch_tmem_nv<PlaneCfg, ListCfg, N1 * 3 / 4>(p, sm_count, st);
+  if (rows <= N1 * 7 / 8) return launch_tmem_nv<PlaneCfg, ListCfg, N1 * 7 / 8>(p, sm_count, st);
+  return launch_tmem_nv<PlaneCfg, ListCfg, N1>(p, sm_count, st);
 }
+
+using Tmem256 = TmemCfg<256, 8, 16, 2>;
+using Tmem512 = TmemCfg<512, 16, 16, 2>;
+using Tmem512List = TmemCfg<512, 16>;
+using Tmem2048 = TmemCfg<2048, 32>;
 
 int batch_segments_per_cta(int L) {
   switch (L) {
-    case 512: return TmemCfg<512, 16>::G;
-    case 2048: return TmemCfg<2048, 32>::G;
+    case 512: return Tmem512::G;
+    case 2048: return Tmem2048::G;
     default: return 0;
   }
 }
 
 static cudaError_t launch_desc(int L, const ListParams& p, int sm_count, cudaStream_t st) {
   switch (L) {
-    case 512: return launch_tmem_cfg<TmemCfg<512, 16>>(p, sm_count, st);
-    case 2048: return launch_tmem_cfg<TmemCfg<2048, 32>>(p, sm_count, st);
+    case 256: return launch_tmem_cfg<Tmem256, void>(p, sm_count, st);
+    case 512: return launch_tmem_cfg<Tmem512, Tmem512List>(p, sm_count, st);
+    case 2048: return launch_tmem_cfg<Tmem2048, Tmem2048>(p, sm_count, st);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -1131,7 +971,7 @@ cudaError_t launch_batch(int L, const BatchParams& p, int sm_count, cudaStream_t
 
 // Single spectrum: the descriptor-driven kernel with an inline one-entry table where it exists.
 static cudaError_t launch_single_desc(int L, const ConvParams& p, int sm_count, cudaStream_t st) {
-  const int G = batch_segments_per_cta(L);
+  const int G = L == 256 ? Tmem256::G : batch_segments_per_cta(L);
   BatchParams q;
   q.templates = p.templates;
   q.twist = p.twist;
@@ -1235,11 +1075,11 @@ cudaError_t launch_pairs(int L, const PairParams& p, int sm_count, cudaStream_t 
   return launch_pairs_nv<Cfg, Cfg::N1>(p, sm_count, st);
 }
 
-cudaError_t launch_convolve(int L, const CUtensorMap* map, const ConvParams& p, int sm_count, cudaStream_t st) {
+cudaError_t launch_convolve(int L, const ConvParams& p, int sm_count, cudaStream_t st) {
   switch (L) {
-    case 256: return launch_conv_cfg<Cfg256>(map, p, sm_count, st);
-    case 512: return launch_single_desc(512, p, sm_count, st);
-    case 2048: return launch_single_desc(2048, p, sm_count, st);
+    case 256:
+    case 512:
+    case 2048: return launch_single_desc(L, p, sm_count, st);
     default: return launch_convolve_wide(L, p, sm_count, st);
   }
 }

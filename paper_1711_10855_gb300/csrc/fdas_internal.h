@@ -107,8 +107,7 @@ bool pairs_supported(int L);
 cudaError_t launch_pairs(int L, const PairParams& p, int sm_count, cudaStream_t stream);
 
 // Launch helpers (defined in fdas_convolve.cu).  Return a cudaError_t from the launch.
-cudaError_t launch_convolve(int L, const CUtensorMap* spec_map, const ConvParams& p, int sm_count,
-                            cudaStream_t stream);
+cudaError_t launch_convolve(int L, const ConvParams& p, int sm_count, cudaStream_t stream);
 cudaError_t launch_segment_spectra(int L, const CUtensorMap* spec_map, const SegParams& p,
                                    int sm_count, cudaStream_t stream);
 // Tensor-core variant for L = 2048 (fdas_tc.cu): inverse transforms as DFT-matrix contractions.
@@ -147,7 +146,6 @@ int validate_geometry(int64_t n_bins, int zmax, int zstep, int seg_len, int tmpl
 // Step a1 (defined in fdas_templates.cu): taps, template spectra and twiddle table.
 cudaError_t build_templates_into(double2* taps, float2* templates, float2* twist, int zmax, int zstep, int L,
                                  int m, cudaStream_t st);
-int encode_spectrum_map(CUtensorMap* map, const void* d_spectrum, int64_t n_bins, int L);
 // One thread waits, for at most limit_ns, on a barrier nothing completes and sets kStatusTimeout.
 cudaError_t launch_wait_selftest(int* status, int64_t limit_ns, cudaStream_t st);
 }  // namespace fdas

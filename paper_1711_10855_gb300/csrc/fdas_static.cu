@@ -105,9 +105,6 @@ extern "C" int fdas_convolve_power_static(int64_t n_bins, int zmax, int zstep, i
     s.m = m;
   }
 
-  CUtensorMap map;
-  rc = fdas::encode_spectrum_map(&map, d_spectrum, n_bins, L);
-  if (rc != FDAS_OK) return rc;
   fdas::ConvParams q;
   q.spectrum = reinterpret_cast<const float2*>(d_spectrum);
   q.templates = templates;
@@ -120,7 +117,7 @@ extern "C" int fdas_convolve_power_static(int64_t n_bins, int zmax, int zstep, i
   q.Z = Z;
   q.V = V;
   q.h = h;
-  return fdas::launch_convolve(L, &map, q, s.sm_count, st) == cudaSuccess ? FDAS_OK : FDAS_ERR_CUDA;
+  return fdas::launch_convolve(L, q, s.sm_count, st) == cudaSuccess ? FDAS_OK : FDAS_ERR_CUDA;
 }
 
 extern "C" int fdas_static_check(fdas_stream_t stream) {
