@@ -264,7 +264,6 @@ int fdas_convolve_power(fdas_plan* p, const float* d_spectrum, float* d_plane, f
   q.status = p->d_status;
   q.n_bins = p->n_bins;
   q.nseg = p->nseg;
-  q.units = 0;
   q.Z = p->Z;
   q.V = p->V;
   q.h = p->h;
@@ -295,7 +294,6 @@ int fdas_convolve_power_units_masked(fdas_plan* p, const float* d_spectrum, floa
   q.status = p->d_status;
   q.n_bins = p->n_bins;
   q.nseg = p->nseg;
-  q.units = 0;
   q.Z = p->Z;
   q.V = p->V;
   q.h = p->h;
@@ -321,7 +319,6 @@ int fdas_convolve_power_units_device_count(fdas_plan* p, const float* d_spectrum
   q.status = p->d_status;
   q.n_bins = p->n_bins;
   q.nseg = p->nseg;
-  q.units = 0;
   q.Z = p->Z;
   q.V = p->V;
   q.h = p->h;

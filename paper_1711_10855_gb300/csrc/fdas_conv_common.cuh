@@ -52,25 +52,33 @@ __device__ __forceinline__ void report_timeout(int* status, volatile int* abort_
   atomicOr(status, kStatusTimeout);
 }
 
-// Twiddle pairs of lane group position k1 (pair p at p*n1 + k1 of the plan's table) into this lane's
-// TMEM columns from `addr`.
+// Twiddle pairs of transform lane k1 (pair p at p*n1 + k1 of the plan's table) ...
 template <int H2>
-__device__ __forceinline__ void twiddles_to_tmem(const float2* twist, int n1, int k1, uint32_t addr) {
+__device__ __forceinline__ void load_twiddles(float4 (&tw)[H2], const float2* twist, int n1, int k1) {
   const float4* tw4 = reinterpret_cast<const float4*>(twist);
+  static_for<H2>([&](auto jj) { tw[decltype(jj)::value] = __ldg(tw4 + decltype(jj)::value * n1 + k1); });
+}
+// ... into this lane's TMEM columns from `addr`.
+template <int H2>
+__device__ __forceinline__ void twiddles_to_tmem(const float4 (&tw)[H2], uint32_t addr) {
   static_for<H2 / 4>([&](auto cc) {
     constexpr int c = decltype(cc)::value;
     float r[16];
     static_for<4>([&](auto qq) {
       constexpr int q = decltype(qq)::value;
-      const float4 w = __ldg(tw4 + (4 * c + q) * n1 + k1);
-      r[4 * q] = w.x;
-      r[4 * q + 1] = w.y;
-      r[4 * q + 2] = w.z;
-      r[4 * q + 3] = w.w;
+      r[4 * q] = tw[4 * c + q].x;
+      r[4 * q + 1] = tw[4 * c + q].y;
+      r[4 * q + 2] = tw[4 * c + q].z;
+      r[4 * q + 3] = tw[4 * c + q].w;
     });
     tmem_st16(addr + 16 * c, r);
   });
   tmem_wait_st();
+}
+
+// a / b for a >= 0, in 32 bits where a fits.
+__device__ __forceinline__ int64_t quotient(int64_t a, int b) {
+  return (uint64_t)a <= 0xffffffffull ? (int64_t)((uint32_t)a / (uint32_t)b) : a / b;
 }
 
 }  // namespace fdas

@@ -226,6 +226,18 @@ __device__ __forceinline__ SpecDesc spectrum_desc(const BatchParams& p, int b) {
 __device__ __forceinline__ int64_t unit_total(const BatchParams& p) { return p.units; }
 __device__ __forceinline__ int64_t unit_total(const ListParams& p) { return p.unit_count ? *p.unit_count : p.units; }
 
+// First unit of CTA k.  The units are cut into equal ranges; one spectrum's groups count group_cost
+// more units each (what fetching and transforming a group's segments costs), so that a CTA whose
+// range enters a second group gets fewer templates.
+__device__ __forceinline__ int64_t first_unit(const BatchParams& p, unsigned k) {
+  const int64_t v = (int64_t)k * p.span + (k < (unsigned)p.span_extra ? k : (unsigned)p.span_extra);
+  if (p.group_cost == 0) return v;
+  const int per = p.single.Z + p.group_cost;
+  const int64_t g = quotient(v, per);
+  const int64_t r = v - g * per - p.group_cost;
+  return g * p.single.Z + (r > 0 ? r : 0);
+}
+
 // NV: pass-2 output rows n1 < NV can hold valid outputs (NV >= ceil(V / N2)); rows n1 >= NV are
 // dropped at compile time, which also removes the butterfly halves that only feed them.
 //
@@ -285,33 +297,65 @@ __global__ void __launch_bounds__(32 * Cfg::W, 1)
     if constexpr (LIST) return (int64_t)__ldg(p.unit_list + e);
     else return e;
   };
-  const int64_t u0 = (int64_t)blockIdx.x * U / gridDim.x;
-  const int64_t u1 = ((int64_t)blockIdx.x + 1) * U / gridDim.x;
+  int64_t u0, u1;
+  if constexpr (LIST) {
+    u0 = (int64_t)blockIdx.x * U / gridDim.x;
+    u1 = ((int64_t)blockIdx.x + 1) * U / gridDim.x;
+  } else {
+    u0 = first_unit(p, blockIdx.x);
+    u1 = first_unit(p, blockIdx.x + 1);
+  }
   const int64_t npos = u1 - u0;
   if (npos <= 0) return;
 
-  if (tid == 0) {
-    for (int r = 0; r < R; ++r) {
-      mbar_init(&full[r], 1);
-      cnt[r] = 0u;
-      issued_pos[r] = -1;
+  // the segment group holding entry u0
+  int b = find_spectrum(p, unit_at(u0));
+  const SpecDesc d0 = spectrum_desc(p, b);
+  int64_t grp = quotient(unit_at(u0) - d0.unit_base, d0.Z);
+  int64_t z_first = unit_at(u0) - d0.unit_base - grp * d0.Z;
+
+  // a2: bulk copies of the in-range part of every segment of the group, one lane per segment (issued one
+  // after the other by a single thread they took 430 cycles each)
+  static_assert(G <= 32, "one lane per segment");
+  auto fetch_segments = [&](const SpecDesc& d) {   // a whole warp
+    const int64_t x0 = (grp * G + lane) * (int64_t)p.V - p.h;
+    const int64_t c0 = x0 > 0 ? x0 : 0;
+    const int64_t c1 = x0 + L < d.n_bins ? x0 + L : d.n_bins;
+    const uint32_t bytes = lane < G && c1 > c0 ? (uint32_t)((c1 - c0) * 8) : 0u;
+    const uint32_t total = __reduce_add_sync(0xffffffffu, bytes);
+    if (lane == 0) mbar_arrive_expect_tx(segbar, total);
+    __syncwarp();
+    if (bytes) {
+      const int ws = lane / Cfg::F, wj = P == 2 ? (ws & 3) + 8 * (ws >> 2) : ws;   // the segment's first warp
+      float2* dst = reinterpret_cast<float2*>(sReg + (size_t)wj * Cfg::REGION) + (size_t)(lane % Cfg::F) * L;
+      bulk_g2s(dst + (c0 - x0), d.spec + c0, bytes, segbar);
     }
-    mbar_init(segbar, 1);
-    if constexpr (DEC)
-      for (int w = 0; w < W; ++w) mbar_init(&wbar[w], 1);
-    *abort_flag = 0;
-    fence_barrier_init();
-  }
+  };
+
+  // The first group's segments, the first templates, the twiddles and the tensor memory are asked for at
+  // once by different warps.
   if (warp == 0) {
+    if (lane == 0) {
+      mbar_init(segbar, 1);
+      if constexpr (DEC)
+        for (int w = 0; w < W; ++w) mbar_init(&wbar[w], 1);
+      *abort_flag = 0;
+      fence_barrier_init();
+    }
+    __syncwarp();
+    fetch_segments(d0);
+  } else if (warp == 1) {
+    if (lane < R) {
+      mbar_init(&full[lane], 1);
+      cnt[lane] = 0u;
+      issued_pos[lane] = -1;
+      fence_barrier_init();
+    }
+    __syncwarp();
+  } else if (warp == 2) {
     tmem_alloc(tmem_slot, Cfg::TMEM_COLS);
     tmem_relinquish();
   }
-  tmem_fence_before_sync();
-  __syncthreads();
-  tmem_fence_after_sync();
-  const uint32_t tmem_row = *tmem_slot + ((uint32_t)(32 * (warp & 3)) << 16);
-  const uint32_t tw_addr = tmem_row + Cfg::COL_TW;
-  const uint32_t x_addr = tmem_row + Cfg::COL_X + (uint32_t)(wseg >> 2) * (2 * Cfg::N2);
 
   // Move a cursor n units on (P = 2)
   [[maybe_unused]] auto advance = [&](IssueCursor* c, int n) {
@@ -356,15 +400,13 @@ __global__ void __launch_bounds__(32 * Cfg::W, 1)
       cur->spec_end = nb + 1 < p.count ? spectrum_desc(p, nb + 1).unit_base : U;
     }
   };
-  if (tid == 0 && !DEC) {
-    const int b0 = find_spectrum(p, u0);
-    const SpecDesc d0 = spectrum_desc(p, b0);
+  if (tid == 32 && !DEC) {
     cur->u = u0;
-    cur->b = b0;
+    cur->b = b;
     cur->Z = d0.Z;
     cur->z_off = d0.z_off;
-    cur->z = (int)((u0 - d0.unit_base) % d0.Z);
-    cur->spec_end = b0 + 1 < p.count ? spectrum_desc(p, b0 + 1).unit_base : U;
+    cur->z = (int)z_first;
+    cur->spec_end = b + 1 < p.count ? spectrum_desc(p, b + 1).unit_base : U;
     if constexpr (P == 2) {
       cur[1] = cur[0];
       advance(cur + 1, 1);
@@ -372,8 +414,16 @@ __global__ void __launch_bounds__(32 * Cfg::W, 1)
     const int64_t first = npos < R ? npos : R;
     for (int64_t i = 0; i < first; ++i) issue_template(i);
   }
-  // twiddle pairs of lane k1 into this quadrant's TMEM rows (one warp per quadrant)
-  if (warp < 4) twiddles_to_tmem<H2>(p.twist, N1, k1, tw_addr);
+  // twiddle pairs of lane k1, one warp per quadrant (stored once the tensor memory is there)
+  float4 tw[H2];
+  if (warp >= 4 && warp < 8) load_twiddles<H2>(tw, p.twist, N1, k1);
+  tmem_fence_before_sync();
+  __syncthreads();
+  tmem_fence_after_sync();
+  const uint32_t tmem_row = *tmem_slot + ((uint32_t)(32 * (warp & 3)) << 16);
+  const uint32_t tw_addr = tmem_row + Cfg::COL_TW;
+  const uint32_t x_addr = tmem_row + Cfg::COL_X + (uint32_t)(wseg >> 2) * (2 * Cfg::N2);
+  if (warp >= 4 && warp < 8) twiddles_to_tmem<H2>(tw, tw_addr);
   // release template slot `slot` of position i; the last of the W / P consumers refills it R
   // positions ahead
   auto release_slot = [&](int64_t i, int slot) {
@@ -388,6 +438,20 @@ __global__ void __launch_bounds__(32 * Cfg::W, 1)
       }
     }
   };
+  // the group after the one whose positions end at entry e
+  auto next_group = [&](int64_t e) {
+    if (e >= u1) return;
+    if constexpr (LIST) {
+      grp = quotient(unit_at(e), p.single.Z);
+      z_first = unit_at(e) - grp * p.single.Z;
+    } else {
+      z_first = 0;
+      if (++grp == spectrum_desc(p, b).ngroups) {
+        grp = 0;
+        ++b;
+      }
+    }
+  };
   tmem_fence_before_sync();
   int alive = 1;
   uint32_t seg_phase = 0;
@@ -396,44 +460,24 @@ __global__ void __launch_bounds__(32 * Cfg::W, 1)
   bool w_in_flight = false;    // DEC: a copy into this warp's region not yet waited for
   int64_t u = u0;
   while (u < u1) {
-    // the segment group holding entry u (a run of list entries with the same group)
-    const int64_t uu = unit_at(u);
-    const int b = find_spectrum(p, uu);
     const SpecDesc d = spectrum_desc(p, b);
-    const int64_t grp = (uu - d.unit_base) / d.Z;
-    const int64_t z_first = (uu - d.unit_base) % d.Z;
     int64_t grp_end;
     if constexpr (LIST) {
       grp_end = u + 1;
-      while (grp_end < u1 && unit_at(grp_end) / d.Z == grp) ++grp_end;
+      while (grp_end < u1 && unit_at(grp_end) < (grp + 1) * d.Z) ++grp_end;
     } else {
-      grp_end = d.unit_base + (grp + 1) * d.Z;
+      grp_end = u + (d.Z - z_first);
     }
     const int64_t a = u - u0;
     const int64_t bpos = (grp_end < u1 ? grp_end : u1) - u0;
     u = u0 + bpos;
-    // every warp is done with its region (previous exchanges) before segments land in it
-    alive = __syncthreads_and(alive && !*abort_flag);
-    tmem_fence_after_sync();
-    if (!alive) break;
-    if (tid == 0) {
-      // a2: bulk copies of the in-range part of every segment of the group
-      uint32_t bytes = 0;
-      for (int j = 0; j < G; ++j) {
-        const int64_t x0 = (grp * G + j) * (int64_t)p.V - p.h;
-        const int64_t c0 = x0 > 0 ? x0 : 0;
-        const int64_t c1 = x0 + L < d.n_bins ? x0 + L : d.n_bins;
-        if (c1 > c0) bytes += (uint32_t)((c1 - c0) * 8);
-      }
-      mbar_arrive_expect_tx(segbar, bytes);
-      for (int j = 0; j < G; ++j) {
-        const int ws = j / Cfg::F, wj = P == 2 ? (ws & 3) + 8 * (ws >> 2) : ws;   // the segment's first warp
-        float2* dst = reinterpret_cast<float2*>(sReg + (size_t)wj * Cfg::REGION) + (size_t)(j % Cfg::F) * L;
-        const int64_t x0 = (grp * G + j) * (int64_t)p.V - p.h;
-        const int64_t c0 = x0 > 0 ? x0 : 0;
-        const int64_t c1 = x0 + L < d.n_bins ? x0 + L : d.n_bins;
-        if (c1 > c0) bulk_g2s(dst + (c0 - x0), d.spec + c0, (uint32_t)((c1 - c0) * 8), segbar);
-      }
+    if (a > 0) {
+      // every warp is done with its region (previous exchanges) before segments land in it
+      fence_proxy_async_smem();
+      alive = __syncthreads_and(alive && !*abort_flag);
+      tmem_fence_after_sync();
+      if (!alive) break;
+      if (warp == 0) fetch_segments(d);
     }
     if (P == 1 || par == 0) {
       // zeros outside [0, n_b) in this lane group's window
@@ -565,6 +609,7 @@ __global__ void __launch_bounds__(32 * Cfg::W, 1)
         i = inext;
       }
       // after a timeout the abort flag is set: every warp leaves at the group barrier above
+      next_group(u);
       tmem_fence_before_sync();
       continue;
     }
@@ -634,6 +679,7 @@ __global__ void __launch_bounds__(32 * Cfg::W, 1)
         }
       });
     }
+    next_group(u);
     tmem_fence_before_sync();
   }
 
@@ -649,7 +695,7 @@ __global__ void __launch_bounds__(32 * Cfg::W, 1)
   if constexpr (DEC) {
     if (lane == 0 && w_in_flight) (void)mbar_wait(&wbar[warp], w_phase);   // bounded
   }
-  if (warp == 0) tmem_dealloc(*tmem_slot, Cfg::TMEM_COLS);
+  if (warp == 2) tmem_dealloc(*tmem_slot, Cfg::TMEM_COLS);
 }
 
 // Pair-list kernel (one transform per warp, L = 2048).  The listed (segment s, template z) pairs,
@@ -689,18 +735,20 @@ __global__ void __launch_bounds__(256, 1) fdas_convolve_pairs_kernel(const PairP
     *abort_flag = 0;
     fence_barrier_init();
   }
-  if (warp == 0) {
+  if (warp == 2) {
     tmem_alloc(tmem_slot, Cfg::TMEM_COLS);
     tmem_relinquish();
   }
+  // twiddle pairs of lane k1, one warp per quadrant (stored once the tensor memory is there)
+  float4 tw[H2];
+  if (warp >= 4) load_twiddles<H2>(tw, p.twist, N1, k1);
   tmem_fence_before_sync();
   __syncthreads();
   tmem_fence_after_sync();
   const uint32_t tmem_row = *tmem_slot + ((uint32_t)(32 * (warp & 3)) << 16);
   const uint32_t tw_addr = tmem_row + Cfg::COL_TW;
   const uint32_t x_addr = tmem_row + Cfg::COL_X + (uint32_t)(warp >> 2) * (2 * Cfg::N2);
-  // twiddle pairs of lane k1 into this quadrant's TMEM rows (one warp per quadrant)
-  if (warp < 4) twiddles_to_tmem<H2>(p.twist, N1, k1, tw_addr);
+  if (warp >= 4) twiddles_to_tmem<H2>(tw, tw_addr);
   tmem_fence_before_sync();
   __syncthreads();
   tmem_fence_after_sync();
@@ -825,7 +873,7 @@ __global__ void __launch_bounds__(256, 1) fdas_convolve_pairs_kernel(const PairP
   tmem_fence_before_sync();
   __syncthreads();
   tmem_fence_after_sync();
-  if (warp == 0) tmem_dealloc(*tmem_slot, Cfg::TMEM_COLS);
+  if (warp == 2) tmem_dealloc(*tmem_slot, Cfg::TMEM_COLS);
 }
 
 // Forward transforms only (steps a2 + a3), natural-order output, for tests of the FFT.
@@ -927,8 +975,14 @@ static cudaError_t launch_tmem_nv(const ListParams& p, int sm_count, cudaStream_
       return launch(fdas_convolve_tmem_kernel<ListCfg, NV, true, true>, ListCfg::W, ListCfg::SMEM, p);
     if (p.unit_list) return launch(fdas_convolve_tmem_kernel<ListCfg, NV, true>, ListCfg::W, ListCfg::SMEM, p);
   }
-  return launch(fdas_convolve_tmem_kernel<PlaneCfg, NV, false>, PlaneCfg::W, PlaneCfg::SMEM,
-                static_cast<const BatchParams&>(p));
+  BatchParams q = p;
+  // a group's start costs about one position (its forward transforms; two with P = 2, where half of the
+  // warps run them)
+  if (q.descs == nullptr && q.units > grid) q.group_cost = PlaneCfg::P;
+  const int64_t total = q.units + q.group_cost * q.single.ngroups;
+  q.span = total / grid;
+  q.span_extra = (int)(total % grid);
+  return launch(fdas_convolve_tmem_kernel<PlaneCfg, NV, false>, PlaneCfg::W, PlaneCfg::SMEM, q);
 }
 
 // Smallest instantiated NV >= ceil(V / N2): N1*3/4, N1*7/8 or N1.

@@ -54,7 +54,7 @@ struct WideCfg {
   static_assert(N1 * N2 == L && (SPLIT == 1 || SPLIT == 2) && W % 4 == 0 && 4 % WT == 0, "bad decomposition");
   static_assert(2 * N2 * (1 + W / 4) <= (int)TMEM_COLS, "TMEM columns");
   static_assert(SMEM <= 232448, "shared memory budget");
-  static_assert(R * 20 + 40 <= 256, "barrier area");
+  static_assert(R * 20 + 48 <= 256, "barrier area");
 };
 
 template <class Cfg>
@@ -118,6 +118,16 @@ __device__ __forceinline__ void exchange_pass2(const cp2 (&v)[Cfg::H2], cp2 (&u)
   fft_split_pairs<Cfg::M, SIGN>(u);
 }
 
+// First unit of CTA k: the units are cut into equal ranges, every segment group counting group_cost
+// units more than its templates (what fetching and transforming its segments costs).
+__device__ __forceinline__ int64_t first_unit(const ConvParams& p, int Z, unsigned k) {
+  const int64_t v = (int64_t)k * p.span + (k < (unsigned)p.span_extra ? k : (unsigned)p.span_extra);
+  if (p.group_cost == 0) return v;
+  const int per = Z + p.group_cost;
+  const int64_t g = quotient(v, per), r = v - g * per - p.group_cost;
+  return g * Z + (r > 0 ? r : 0);
+}
+
 // NV (eighths of the rows): pass-2 rows n1 >= NV*N1/8 hold no valid output and are dropped at compile
 // time.  FWD: only the forward transforms, natural order, into p.plane (complex64).
 template <class Cfg, int NV, bool FWD>
@@ -131,6 +141,7 @@ __global__ void __launch_bounds__(32 * Cfg::W, 1) fdas_convolve_wide_kernel(cons
   unsigned* cnt = reinterpret_cast<unsigned*>(issued_pos + R);    // [R] consumer arrivals per slot
   volatile int* abort_flag = reinterpret_cast<volatile int*>(cnt + R);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(cnt + R + 1);
+  int* next_z = reinterpret_cast<int*>(cnt + R + 2);              // template of the next part to issue
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int g = warp / Cfg::WT, k1 = 32 * (warp % Cfg::WT) + lane;
@@ -141,50 +152,76 @@ __global__ void __launch_bounds__(32 * Cfg::W, 1) fdas_convolve_wide_kernel(cons
   float2* mySeg = reinterpret_cast<float2*>(region);
   float4* tile = reinterpret_cast<float4*>(region);
 
-  const int64_t U = FWD ? (p.nseg + G - 1) / G : p.units;
   const int Z = FWD ? 1 : p.Z;
-  const int64_t u0 = (int64_t)blockIdx.x * U / gridDim.x;
-  const int64_t u1 = ((int64_t)blockIdx.x + 1) * U / gridDim.x;
+  const int64_t u0 = first_unit(p, Z, blockIdx.x), u1 = first_unit(p, Z, blockIdx.x + 1);
   const int64_t npos = u1 - u0;
   if (npos <= 0) return;
+  int64_t grp = quotient(u0, Z);
+  int z = (int)(u0 - grp * Z);
 
-  if (tid == 0) {
-    for (int r = 0; r < R; ++r) {
-      mbar_init(&full[r], 1);
-      cnt[r] = 0u;
-      issued_pos[r] = -1;
+  // a2: bulk copies of the in-range part of every segment of the group, one lane per segment
+  auto fetch_segments = [&]() {   // a whole warp
+    const int64_t x0 = (grp * G + lane) * (int64_t)p.V - p.h;
+    const int64_t c0 = x0 > 0 ? x0 : 0, c1 = x0 + L < p.n_bins ? x0 + L : p.n_bins;
+    const uint32_t bytes = lane < G && c1 > c0 ? (uint32_t)((c1 - c0) * 8) : 0u;
+    const uint32_t total = __reduce_add_sync(0xffffffffu, bytes);
+    if (lane == 0) mbar_arrive_expect_tx(segbar, total);
+    __syncwarp();
+    if (bytes) {
+      float2* dst = reinterpret_cast<float2*>(smem + Cfg::OFF_REG + (size_t)lane * Cfg::REGION);
+      bulk_g2s(dst + (c0 - x0), p.spectrum + c0, bytes, segbar);
     }
-    mbar_init(segbar, 1);
-    *abort_flag = 0;
-    fence_barrier_init();
-  }
+  };
+  // The first group's segments, the first templates, the twiddles and the tensor memory are asked for at
+  // once by different warps.
   if (warp == 0) {
+    if (lane == 0) {
+      mbar_init(segbar, 1);
+      *abort_flag = 0;
+      fence_barrier_init();
+    }
+    __syncwarp();
+    fetch_segments();
+  } else if (warp == 1) {
+    if (lane < R) {
+      mbar_init(&full[lane], 1);
+      cnt[lane] = 0u;
+      issued_pos[lane] = -1;
+      fence_barrier_init();
+    }
+    __syncwarp();
+  } else if (warp == 2) {
     tmem_alloc(tmem_slot, Cfg::TMEM_COLS);
     tmem_relinquish();
   }
+
+  // ring position e = PARTS * (unit - u0) + part
+  auto issue_part = [&](int64_t e) {
+    const int slot = (int)(e % R);
+    const int zr = *next_z;   // parts are issued in order, one thread at a time
+    if (PARTS == 1 || e % PARTS == PARTS - 1) *next_z = zr + 1 == Z ? 0 : zr + 1;
+    issued_pos[slot] = e;
+    mbar_arrive_expect_tx(&full[slot], (uint32_t)Cfg::PART_BYTES);
+    bulk_g2s(smem + Cfg::OFF_T + slot * Cfg::PART_BYTES,
+             reinterpret_cast<const unsigned char*>(p.templates + (size_t)zr * L) + (e % PARTS) * Cfg::PART_BYTES,
+             (uint32_t)Cfg::PART_BYTES, &full[slot]);
+  };
+  if (!FWD && tid == 32) {
+    *next_z = z;
+    const int64_t first = npos * PARTS < R ? npos * PARTS : R;
+    for (int64_t e = 0; e < first; ++e) issue_part(e);
+  }
+  // warps w, w + 4, ... hold the same lanes of their transforms (WT divides 4): one copy of the twiddles
+  // per quadrant (stored once the tensor memory is there)
+  float4 tw[H2];
+  if (warp >= 4 && warp < 8) load_twiddles<H2>(tw, p.twist, N1, k1);
   tmem_fence_before_sync();
   __syncthreads();
   tmem_fence_after_sync();
   const uint32_t tmem_row = *tmem_slot + ((uint32_t)(32 * (warp & 3)) << 16);
   const uint32_t tw_addr = tmem_row + Cfg::COL_TW;
   const uint32_t x_addr = tmem_row + Cfg::COL_X + (uint32_t)(warp >> 2) * (2 * N2);
-
-  // ring position e = PARTS * (unit - u0) + part
-  auto issue_part = [&](int64_t e) {
-    const int slot = (int)(e % R);
-    const int64_t z = (u0 + e / PARTS) % Z;
-    issued_pos[slot] = e;
-    mbar_arrive_expect_tx(&full[slot], (uint32_t)Cfg::PART_BYTES);
-    bulk_g2s(smem + Cfg::OFF_T + slot * Cfg::PART_BYTES,
-             reinterpret_cast<const unsigned char*>(p.templates + (size_t)z * L) + (e % PARTS) * Cfg::PART_BYTES,
-             (uint32_t)Cfg::PART_BYTES, &full[slot]);
-  };
-  if (!FWD && tid == 0) {
-    const int64_t first = npos * PARTS < R ? npos * PARTS : R;
-    for (int64_t e = 0; e < first; ++e) issue_part(e);
-  }
-  // warps w, w + 4, ... hold the same lanes of their transforms (WT divides 4): one copy per quadrant
-  if (warp < 4) twiddles_to_tmem<H2>(p.twist, N1, k1, tw_addr);
+  if (warp >= 4 && warp < 8) twiddles_to_tmem<H2>(tw, tw_addr);
   tmem_fence_before_sync();
 
   int alive = 1;
@@ -192,31 +229,16 @@ __global__ void __launch_bounds__(32 * Cfg::W, 1) fdas_convolve_wide_kernel(cons
   bool seg_in_flight = false;
   int64_t u = u0;
   while (u < u1) {
-    const int64_t grp = u / Z;
-    int z = (int)(u - grp * Z);
     const int64_t a = u - u0;
-    const int64_t bpos = ((grp + 1) * Z < u1 ? (grp + 1) * Z : u1) - u0;
+    const int64_t bpos = (u + (Z - z) < u1 ? u + (Z - z) : u1) - u0;
     u = u0 + bpos;
-    // every warp is done with its region (previous exchanges) before segments land in it
-    fence_proxy_async_smem();
-    alive = __syncthreads_and(alive && !*abort_flag);
-    tmem_fence_after_sync();
-    if (!alive) break;
-    if (tid == 0) {
-      // a2: bulk copies of the in-range part of every segment of the group
-      uint32_t bytes = 0;
-      for (int j = 0; j < G; ++j) {
-        const int64_t x0 = (grp * G + j) * (int64_t)p.V - p.h;
-        const int64_t c0 = x0 > 0 ? x0 : 0, c1 = x0 + L < p.n_bins ? x0 + L : p.n_bins;
-        if (c1 > c0) bytes += (uint32_t)((c1 - c0) * 8);
-      }
-      mbar_arrive_expect_tx(segbar, bytes);
-      for (int j = 0; j < G; ++j) {
-        const int64_t x0 = (grp * G + j) * (int64_t)p.V - p.h;
-        const int64_t c0 = x0 > 0 ? x0 : 0, c1 = x0 + L < p.n_bins ? x0 + L : p.n_bins;
-        float2* dst = reinterpret_cast<float2*>(smem + Cfg::OFF_REG + (size_t)j * Cfg::REGION);
-        if (c1 > c0) bulk_g2s(dst + (c0 - x0), p.spectrum + c0, (uint32_t)((c1 - c0) * 8), segbar);
-      }
+    if (a > 0) {
+      // every warp is done with its region (previous exchanges) before segments land in it
+      fence_proxy_async_smem();
+      alive = __syncthreads_and(alive && !*abort_flag);
+      tmem_fence_after_sync();
+      if (!alive) break;
+      if (warp == 0) fetch_segments();
     }
     const int64_t s = grp * G + g;
     const int64_t segbase = s * (int64_t)p.V;
@@ -258,6 +280,7 @@ __global__ void __launch_bounds__(32 * Cfg::W, 1) fdas_convolve_wide_kernel(cons
             out[k1 + N1 * j] = make_float2(x[j].re.x, x[j].im.x);
             out[k1 + N1 * (j + M / 2)] = make_float2(x[j].re.y, x[j].im.y);
           });
+        ++grp;
         tmem_fence_before_sync();
         continue;
       }
@@ -341,6 +364,8 @@ __global__ void __launch_bounds__(32 * Cfg::W, 1) fdas_convolve_wide_kernel(cons
         }
       });
     }
+    ++grp;
+    z = 0;
     tmem_fence_before_sync();
   }
 
@@ -353,7 +378,7 @@ __global__ void __launch_bounds__(32 * Cfg::W, 1) fdas_convolve_wide_kernel(cons
       if (issued_pos[r] >= 0) (void)mbar_wait(&full[r], (uint32_t)((issued_pos[r] / R) & 1));
     if (seg_in_flight) (void)mbar_wait(segbar, seg_phase);
   }
-  if (warp == 0) tmem_dealloc(*tmem_slot, Cfg::TMEM_COLS);
+  if (warp == 2) tmem_dealloc(*tmem_slot, Cfg::TMEM_COLS);
 }
 
 using Wide1024 = WideCfg<1024, 1, 32, 16, 1, 4>;
@@ -367,9 +392,13 @@ cudaError_t launch_wide(const ConvParams& p, int sm_count, cudaStream_t st) {
   if (e != cudaSuccess) return e;
   ConvParams q = p;
   const int64_t ngroups = (p.nseg + Cfg::G - 1) / Cfg::G;
-  q.units = ngroups * p.Z;
-  const int64_t work = FWD ? ngroups : q.units;
-  kern<<<(unsigned)(work < sm_count ? work : sm_count), 32 * Cfg::W, Cfg::SMEM, st>>>(q);
+  const int64_t units = FWD ? ngroups : ngroups * p.Z;
+  const int64_t grid = units < sm_count ? units : sm_count;
+  q.group_cost = !FWD && units > grid ? 1 : 0;   // about one position
+  const int64_t total = units + q.group_cost * ngroups;
+  q.span = total / grid;
+  q.span_extra = (int)(total % grid);
+  kern<<<(unsigned)grid, 32 * Cfg::W, Cfg::SMEM, st>>>(q);
   return cudaGetLastError();
 }
 

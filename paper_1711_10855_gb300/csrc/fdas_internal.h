@@ -22,8 +22,12 @@ struct ConvParams {
   int* status;              // device status word (kStatusTimeout | kStatusBadList)
   int64_t n_bins;
   int64_t nseg;             // ceil(n_bins / V)
-  int64_t units;            // (number of segment groups) x Z
   int Z, V, h;
+  // work split (set by the launch): CTA k starts at unit k * span + min(k, span_extra) of a count in which
+  // every segment group has group_cost units more than its templates
+  int64_t span;
+  int span_extra;
+  int group_cost;
 };
 
 // One spectrum of a batch, as the persistent kernel reads it (device table or inline).
@@ -49,6 +53,11 @@ struct BatchParams {
   int64_t units;            // total units over all spectra (or entries of unit_list)
   const int32_t* unit_list; // single spectrum only: ascending units g*Z + z to compute, or nullptr: all
   int V, h;
+  // full planes (set by the launch): CTA k starts at unit k * span + min(k, span_extra) of a count in
+  // which every segment group has group_cost units more than its templates
+  int64_t span;
+  int span_extra;
+  int group_cost = 0;
   // with unit_list: per entry, bit j = segment j of the unit's group is computed (nullptr: all)
   const uint16_t* unit_mask = nullptr;
 };

@@ -113,7 +113,6 @@ extern "C" int fdas_convolve_power_static(int64_t n_bins, int zmax, int zstep, i
   q.status = status;
   q.n_bins = n_bins;
   q.nseg = (n_bins + V - 1) / V;
-  q.units = 0;
   q.Z = Z;
   q.V = V;
   q.h = h;
