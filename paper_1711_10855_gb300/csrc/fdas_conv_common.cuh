@@ -8,24 +8,77 @@ namespace fdas {
 
 __host__ __device__ constexpr size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
-// Twist with the twiddle pairs held in this lane's TMEM row (4 columns per pair, chunks of 4 pairs).
-template <class Cfg, bool CONJ>
-__device__ __forceinline__ void apply_twist_tmem(cp2 (&v)[Cfg::H2], uint32_t tw_addr) {
-  static_assert(Cfg::H2 % 8 == 0, "twist chunking");
-  static_for<Cfg::H2 / 8>([&](auto cc) {
-    constexpr int c = decltype(cc)::value;
-    float r0[16], r1[16];
-    tmem_ld16(tw_addr + 32 * c, r0);
-    tmem_ld16(tw_addr + 32 * c + 16, r1);
+// The element-wise products with the templates (before pass 1) and with the twiddles (before pass 2)
+// are joined with the radix-2 stage that follows them: a + b = t + B*b', a - b = 2t - (a + b) with
+// t = A*a' take 10 packed instructions per butterfly where two products and the butterfly take 12.
+// Operands whose pairs meet in that stage (p and p + n/2) therefore sit next to each other in tensor
+// memory: slot 2p holds pair p, slot 2p + 1 pair p + n/2.
+constexpr __host__ __device__ int slot_pair(int slot, int n) { return (slot >> 1) + (slot & 1) * (n / 2); }
+__device__ __forceinline__ cp2 tmem_pair(const float (&r)[16], int q) {
+  return cp2{make_float2(r[4 * q], r[4 * q + 1]), make_float2(r[4 * q + 2], r[4 * q + 3])};
+}
+
+// Y = X (this lane's TMEM slots from x_addr) * T (load(p) = pair p) and the first stage of the
+// N2-point DFT: v in bit-reversed order, pairs [P0, P0 + NP) and their partners.
+template <class Cfg, int P0, int NP, class Load>
+__device__ __forceinline__ void multiply_first_stage(cp2 (&v)[Cfg::H2], uint32_t x_addr, Load&& load) {
+  constexpr int HALF = Cfg::H2 / 2;
+  static_for<NP / 2>([&](auto cc) {
+    constexpr int p0 = P0 + 2 * decltype(cc)::value;
+    float x[16];
+    tmem_ld16(x_addr + 8 * p0, x);
+    const cp2 ta = cp2_from(load(p0)), tb = cp2_from(load(p0 + HALF));
+    const cp2 tc = cp2_from(load(p0 + 1)), td = cp2_from(load(p0 + 1 + HALF));
     tmem_wait_ld();
+    constexpr int i0 = bitrev(2 * p0, Cfg::LOG_N2), i1 = bitrev(2 * p0 + 2, Cfg::LOG_N2);
+    const cp2 t0 = cmul2(tmem_pair(x, 0), ta), t1 = cmul2(tmem_pair(x, 2), tc);
+    v[i0] = cfma2(tmem_pair(x, 1), tb, t0);
+    v[i1] = cfma2(tmem_pair(x, 3), td, t1);
+    v[i0 + 1] = twice_minus(t0, v[i0]);
+    v[i1 + 1] = twice_minus(t1, v[i1]);
+  });
+}
+
+// u = entries (load(s), s < N) times the twiddles of this lane's TMEM slots (conjugated for the forward
+// transform), with the first stage done: N entries in bit-reversed order over log2(N) + SHIFT bits of
+// (s << SHIFT).  The first pair's twiddle is 1 when UNIT0.
+template <int N, int SHIFT, bool CONJ, bool UNIT0, class Load>
+__device__ __forceinline__ void twist_first_stage(cp2 (&u)[N], uint32_t tw_addr, Load&& load) {
+  constexpr int HALF = N / 2, LOG = ilog2(N) + SHIFT;
+  static_for<N / 4>([&](auto cc) {
+    constexpr int s0 = 2 * decltype(cc)::value;
+    float w[16];
+    tmem_ld16(tw_addr + 8 * s0, w);
+    const cp2 a = load(std::integral_constant<int, s0>{}), b = load(std::integral_constant<int, s0 + HALF>{});
+    const cp2 c = load(std::integral_constant<int, s0 + 1>{}), d = load(std::integral_constant<int, s0 + 1 + HALF>{});
+    tmem_wait_ld();
+    constexpr int i0 = bitrev(s0 << SHIFT, LOG), i1 = bitrev((s0 + 1) << SHIFT, LOG);
+    const cp2 t0 = UNIT0 && s0 == 0 ? a : (CONJ ? cmul2_conj(a, tmem_pair(w, 0)) : cmul2(a, tmem_pair(w, 0)));
+    const cp2 t1 = CONJ ? cmul2_conj(c, tmem_pair(w, 2)) : cmul2(c, tmem_pair(w, 2));
+    u[i0] = CONJ ? cfma2_conj(b, tmem_pair(w, 1), t0) : cfma2(b, tmem_pair(w, 1), t0);
+    u[i1] = CONJ ? cfma2_conj(d, tmem_pair(w, 3), t1) : cfma2(d, tmem_pair(w, 3), t1);
+    u[i0 + 1] = twice_minus(t0, u[i0]);
+    u[i1 + 1] = twice_minus(t1, u[i1]);
+  });
+}
+
+// This lane's spectrum pairs x(p), p < H2, to TMEM in slot order.
+template <int H2, class Pair>
+__device__ __forceinline__ void spectrum_to_tmem(uint32_t x_addr, Pair&& pair) {
+  static_for<H2 / 4>([&](auto cc) {
+    constexpr int c = decltype(cc)::value;
+    float r[16];
     static_for<4>([&](auto qq) {
       constexpr int q = decltype(qq)::value;
-      const cp2 w0 = cp2{make_float2(r0[4 * q], r0[4 * q + 1]), make_float2(r0[4 * q + 2], r0[4 * q + 3])};
-      const cp2 w1 = cp2{make_float2(r1[4 * q], r1[4 * q + 1]), make_float2(r1[4 * q + 2], r1[4 * q + 3])};
-      v[8 * c + q] = CONJ ? cmul2_conj(v[8 * c + q], w0) : cmul2(v[8 * c + q], w0);
-      v[8 * c + 4 + q] = CONJ ? cmul2_conj(v[8 * c + 4 + q], w1) : cmul2(v[8 * c + 4 + q], w1);
+      const cp2 x = pair(std::integral_constant<int, slot_pair(4 * c + q, H2)>{});
+      r[4 * q] = x.re.x;
+      r[4 * q + 1] = x.re.y;
+      r[4 * q + 2] = x.im.x;
+      r[4 * q + 3] = x.im.y;
     });
+    tmem_st16(x_addr + 16 * c, r);
   });
+  tmem_wait_st();
 }
 
 // One arrival on a shared-memory consumer counter with acquire-release semantics at CTA scope: the
@@ -52,13 +105,7 @@ __device__ __forceinline__ void report_timeout(int* status, volatile int* abort_
   atomicOr(status, kStatusTimeout);
 }
 
-// Twiddle pairs of transform lane k1 (pair p at p*n1 + k1 of the plan's table) ...
-template <int H2>
-__device__ __forceinline__ void load_twiddles(float4 (&tw)[H2], const float2* twist, int n1, int k1) {
-  const float4* tw4 = reinterpret_cast<const float4*>(twist);
-  static_for<H2>([&](auto jj) { tw[decltype(jj)::value] = __ldg(tw4 + decltype(jj)::value * n1 + k1); });
-}
-// ... into this lane's TMEM columns from `addr`.
+// Twiddle pairs into this lane's TMEM columns from `addr`, in order.
 template <int H2>
 __device__ __forceinline__ void twiddles_to_tmem(const float4 (&tw)[H2], uint32_t addr) {
   static_for<H2 / 4>([&](auto cc) {

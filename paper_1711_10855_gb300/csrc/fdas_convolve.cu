@@ -161,6 +161,76 @@ __device__ __forceinline__ void forward_transform(const float2* sx, const float4
   forward_transform_with<Cfg>(sx, [&](cp2 (&v)[Cfg::H2]) { apply_twist2<Cfg, true>(v, stw, k1); }, xb, k1, out);
 }
 
+// Exchange, twist and pass 2 with the twiddles in TMEM: round r moves the rows of column pair r, each
+// lane multiplies its column's entries (lane s wrote entry s) by their twiddles and runs two N1-point
+// DFTs in lockstep; out(r, u) receives u[n1] = (y[t + N1*r + N2*n1], y[t + N1*(r+CP) + N2*n1]).
+template <class Cfg, int SIGN, class Out, class AfterReads = NoHook>
+__device__ __forceinline__ void exchange_twist_pass2(const cp2 (&v)[Cfg::H2], float4* xb, int k1, uint32_t tw_addr,
+                                                     Out&& out, AfterReads&& after_reads = AfterReads{}) {
+  constexpr int N1 = Cfg::N1;
+  static_for<Cfg::CP>([&](auto rr) {
+    constexpr int r = decltype(rr)::value;
+    cp2 u[N1];
+    __syncwarp();
+    static_for<N1>([&](auto ii) {
+      constexpr int i = decltype(ii)::value;
+      xb[i * Cfg::XPITCH + k1] = cp2_to(v[r * N1 + i]);
+    });
+    __syncwarp();
+    twist_first_stage<N1, 0, (SIGN < 0), true>(u, tw_addr + 4 * N1 * r, [&](auto ss) {
+      return cp2_from(xb[k1 * Cfg::XPITCH + decltype(ss)::value]);
+    });
+    if constexpr (r == Cfg::CP - 1) after_reads();   // the tile is free once its last round is read
+    fft_pair_columns<N1, SIGN, 1>(u);
+    out(rr, u);
+  });
+}
+
+// Forward FFT (Eq. 3) of one segment held in natural order (complex64) in sx, into this lane's TMEM
+// slots: the pairs (k2 = 2p, 2p + 1) of the elements X[k1 + N1*k2].
+template <class Cfg>
+__device__ __forceinline__ void forward_to_tmem(const float2* sx, float4* xb, int k1, uint32_t tw_addr,
+                                                uint32_t x_addr) {
+  constexpr int N1 = Cfg::N1;
+  cp2 v[Cfg::H2];
+  static_for<Cfg::H2>([&](auto ii) {
+    constexpr int i = decltype(ii)::value;
+    constexpr int k2 = bitrev(i, Cfg::LOG_N2);
+    const float2 a = sx[k1 + N1 * k2];
+    const float2 b = sx[k1 + N1 * (k2 + 1)];
+    v[i] = cp2{make_float2(a.x, b.x), make_float2(a.y, b.y)};
+  });
+  fft_split_pairs<Cfg::N2, -1>(v);
+  cp2 first[Cfg::CP == 2 ? N1 : 1];   // two column pairs: round 0's, until round 1's complete the pairs
+  exchange_twist_pass2<Cfg, -1>(v, xb, k1, tw_addr, [&](auto rr, auto& x) {
+    if constexpr (Cfg::CP == 1) {      // pair p = n1
+      spectrum_to_tmem<Cfg::H2>(x_addr, [&](auto pp) { return x[decltype(pp)::value]; });
+    } else if constexpr (decltype(rr)::value == 0) {   // elements k2 = 4 n1, 4 n1 + 2
+      static_for<N1>([&](auto nn) { first[decltype(nn)::value] = x[decltype(nn)::value]; });
+    } else {                                           // and 4 n1 + 1, 4 n1 + 3
+      spectrum_to_tmem<Cfg::H2>(x_addr, [&](auto pp) {
+        constexpr int n1 = decltype(pp)::value >> 1;
+        if constexpr (decltype(pp)::value & 1)
+          return cp2{make_float2(first[n1].re.y, x[n1].re.y), make_float2(first[n1].im.y, x[n1].im.y)};
+        else
+          return cp2{make_float2(first[n1].re.x, x[n1].re.x), make_float2(first[n1].im.x, x[n1].im.x)};
+      });
+    }
+  });
+}
+
+// Twiddle pairs of lane k1's columns: entry r*N1 + slot = those of column pair r for the lane that
+// slot stands for (the plan's table holds pair j of lane s at j*N1 + s).
+template <class Cfg>
+__device__ __forceinline__ void load_column_twiddles(float4 (&tw)[Cfg::H2], const float2* twist, int k1) {
+  constexpr int N1 = Cfg::N1;
+  const float4* tw4 = reinterpret_cast<const float4*>(twist);
+  static_for<Cfg::H2>([&](auto ii) {
+    constexpr int i = decltype(ii)::value, r = i / N1, src = slot_pair(i % N1, N1);
+    tw[i] = __ldg(tw4 + (r * N1 + k1) * N1 + src);
+  });
+}
+
 // ---------------------------------------------------------------------------------------
 // Variant with the segment spectra and the twiddle table in tensor memory (one column pair per
 // lane: N2 = 2*N1, i.e. L = 512 and 2048).  Every warp owns its own segment(s); the template of
@@ -205,6 +275,19 @@ struct TmemCfg {
   static_assert(2 * N2 * (1 + W / P / 4) <= (int)TMEM_COLS, "TMEM columns");
   static_assert(SMEM <= 232448, "shared memory budget");
 };
+
+// a6 + a7: |y|^2 of the outputs n < lim of column pair r; rows n1 >= NV hold none.
+template <class Cfg, int NV, int r>
+__device__ __forceinline__ void store_powers(const cp2 (&y)[Cfg::N1], float* row, int k1, int lim) {
+  static_for<NV>([&](auto nn) {
+    constexpr int n1 = decltype(nn)::value;
+    const float2 pw = power2(y[n1]);
+    const int n_lo = r * Cfg::N1 + k1 + Cfg::N2 * n1;
+    const int n_hi = n_lo + Cfg::CP * Cfg::N1;
+    if (n_lo < lim) __stcs(row + n_lo, pw.x);
+    if (n_hi < lim) __stcs(row + n_hi, pw.y);
+  });
+}
 
 // Spectrum b holding flattened unit u (largest b with unit_base <= u).
 __device__ __forceinline__ int find_spectrum(const BatchParams& p, int64_t u) {
@@ -416,7 +499,7 @@ __global__ void __launch_bounds__(32 * Cfg::W, 1)
   }
   // twiddle pairs of lane k1, one warp per quadrant (stored once the tensor memory is there)
   float4 tw[H2];
-  if (warp >= 4 && warp < 8) load_twiddles<H2>(tw, p.twist, N1, k1);
+  if (warp >= 4 && warp < 8) load_column_twiddles<Cfg>(tw, p.twist, k1);
   tmem_fence_before_sync();
   __syncthreads();
   tmem_fence_after_sync();
@@ -497,32 +580,7 @@ __global__ void __launch_bounds__(32 * Cfg::W, 1)
     seg_phase ^= 1u;
 
     // a3: forward FFT of this lane group's segment; X pairs (k2 = 2p, 2p+1) go to TMEM
-    if (P == 1 || par == 0) {
-      float xr[16];
-      cp2 first[Cfg::CP == 2 ? N1 : 1];   // two column pairs: round 0's, until round 1's complete the pairs
-      forward_transform_with<Cfg>(
-          mySeg, [&](cp2 (&v)[H2]) { apply_twist_tmem<Cfg, true>(v, tw_addr); }, myXb, k1,
-          [&](auto rr, auto nn, const cp2& x) {
-            [[maybe_unused]] constexpr int r = decltype(rr)::value, n1 = decltype(nn)::value;
-            auto put = [&](auto pp, float a, float b, float c, float d) {
-              constexpr int pr = decltype(pp)::value;
-              xr[4 * (pr & 3)] = a;
-              xr[4 * (pr & 3) + 1] = b;
-              xr[4 * (pr & 3) + 2] = c;
-              xr[4 * (pr & 3) + 3] = d;
-              if constexpr ((pr & 3) == 3) tmem_st16(x_addr + 4 * (pr - 3), xr);
-            };
-            if constexpr (Cfg::CP == 1) {   // pair p = n1
-              put(nn, x.re.x, x.re.y, x.im.x, x.im.y);
-            } else if constexpr (r == 0) {  // elements k2 = 4 n1, 4 n1 + 2
-              first[n1] = x;
-            } else {                        // and 4 n1 + 1, 4 n1 + 3
-              put(std::integral_constant<int, 2 * n1>{}, first[n1].re.x, x.re.x, first[n1].im.x, x.im.x);
-              put(std::integral_constant<int, 2 * n1 + 1>{}, first[n1].re.y, x.re.y, first[n1].im.y, x.im.y);
-            }
-          });
-      tmem_wait_st();
-    }
+    if (P == 1 || par == 0) forward_to_tmem<Cfg>(mySeg, myXb, k1, tw_addr, x_addr);
     if constexpr (P == 2) {   // the other warp of the segment reads the spectrum too
       tmem_fence_before_sync();
       __syncthreads();
@@ -568,41 +626,13 @@ __global__ void __launch_bounds__(32 * Cfg::W, 1)
         const int lim_z = ((warp_bits(i) >> gw) & 1u) ? lim : 0;
         const float4* st4 = reinterpret_cast<const float4*>(myRegion);
         cp2 v[H2];
-        static_for<H2 / 8>([&](auto cc) {
-          constexpr int c = decltype(cc)::value;
-          float x0[16], x1[16];
-          tmem_ld16(x_addr + 32 * c, x0);
-          tmem_ld16(x_addr + 32 * c + 16, x1);
-          float4 t[8];
-          static_for<8>([&](auto qq) {
-            constexpr int q = decltype(qq)::value;
-            t[q] = st4[(8 * c + q) * N1 + k1];
-          });
-          tmem_wait_ld();
-          static_for<8>([&](auto qq) {
-            constexpr int q = decltype(qq)::value;
-            constexpr int pp = 8 * c + q;
-            const float* xs = q < 4 ? &x0[4 * q] : &x1[4 * (q - 4)];
-            const cp2 x = cp2{make_float2(xs[0], xs[1]), make_float2(xs[2], xs[3])};
-            v[bitrev(2 * pp, Cfg::LOG_N2)] = cmul2(x, cp2_from(t[q]));
-          });
-        });
+        multiply_first_stage<Cfg, 0, H2 / 2>(v, x_addr, [&](int q) { return st4[q * N1 + k1]; });
         const int64_t inext = next_active(i + 1);
-        fft_split_pairs<Cfg::N2, +1>(v);
-        apply_twist_tmem<Cfg, false>(v, tw_addr);
+        fft_split_pairs<Cfg::N2, +1, 1>(v);
         float* row = d.plane + z * d.n_bins + segbase;
-        exchange_and_pass2<Cfg, +1>(
-            v, myXb, k1,
-            [&](auto, auto nn, const cp2& y) {
-              constexpr int n1 = decltype(nn)::value;
-              if constexpr (n1 < NV) {
-                const float2 pw = power2(y);
-                const int n_lo = k1 + Cfg::N2 * n1;
-                const int n_hi = n_lo + N1;
-                if (n_lo < lim_z) __stcs(row + n_lo, pw.x);
-                if (n_hi < lim_z) __stcs(row + n_hi, pw.y);
-              }
-            },
+        exchange_twist_pass2<Cfg, +1>(
+            v, myXb, k1, tw_addr,
+            [&](auto rr, auto& y) { store_powers<Cfg, NV, decltype(rr)::value>(y, row, k1, lim_z); },
             [&]() {
               if (inext < bpos) fetch(inext);
             });
@@ -642,41 +672,15 @@ __global__ void __launch_bounds__(32 * Cfg::W, 1)
       }
       const int lim_z = group_on ? lim : 0;
 
-      // a4: Y = X (TMEM) * T (shared ring), packed pairs in bit-reversed order, four pairs per
-      // chunk (a sweep of equivalent orderings timed this one 0.5% faster than eight)
+      // a4: Y = X (TMEM) * T (shared ring), packed pairs in bit-reversed order, with the first stage
       cp2 v[H2];
-      static_for<H2 / 4>([&](auto cc) {
-        constexpr int c = decltype(cc)::value;
-        float x0[16];
-        tmem_ld16(x_addr + 16 * c, x0);
-        float4 t[4];
-        static_for<4>([&](auto qq) {
-          constexpr int q = decltype(qq)::value;
-          t[q] = st4[(4 * c + q) * N1 + k1];
-        });
-        tmem_wait_ld();
-        static_for<4>([&](auto qq) {
-          constexpr int q = decltype(qq)::value;
-          constexpr int pp = 4 * c + q;
-          const cp2 x = cp2{make_float2(x0[4 * q], x0[4 * q + 1]), make_float2(x0[4 * q + 2], x0[4 * q + 3])};
-          v[bitrev(2 * pp, Cfg::LOG_N2)] = cmul2(x, cp2_from(t[q]));
-        });
-      });
+      multiply_first_stage<Cfg, 0, H2 / 2>(v, x_addr, [&](int q) { return st4[q * N1 + k1]; });
       release_slot(i, slot);
-      // a5: inverse FFT
-      fft_split_pairs<Cfg::N2, +1>(v);
-      apply_twist_tmem<Cfg, false>(v, tw_addr);
+      // a5: inverse FFT; a6 + a7: keep n < V (and inside the spectrum), store |y|^2
+      fft_split_pairs<Cfg::N2, +1, 1>(v);
       float* row = d.plane + z * d.n_bins + segbase;
-      exchange_and_pass2<Cfg, +1>(v, myXb, k1, [&](auto rr, auto nn, const cp2& y) {
-        // a6 + a7: keep n < V (and inside the spectrum), store |y|^2
-        constexpr int r = decltype(rr)::value, n1 = decltype(nn)::value;
-        if constexpr (n1 < NV) {
-          const float2 pw = power2(y);
-          const int n_lo = r * N1 + k1 + Cfg::N2 * n1;
-          const int n_hi = n_lo + Cfg::CP * N1;
-          if (n_lo < lim_z) __stcs(row + n_lo, pw.x);
-          if (n_hi < lim_z) __stcs(row + n_hi, pw.y);
-        }
+      exchange_twist_pass2<Cfg, +1>(v, myXb, k1, tw_addr, [&](auto rr, auto& y) {
+        store_powers<Cfg, NV, decltype(rr)::value>(y, row, k1, lim_z);
       });
     }
     next_group(u);
@@ -741,7 +745,7 @@ __global__ void __launch_bounds__(256, 1) fdas_convolve_pairs_kernel(const PairP
   }
   // twiddle pairs of lane k1, one warp per quadrant (stored once the tensor memory is there)
   float4 tw[H2];
-  if (warp >= 4) load_twiddles<H2>(tw, p.twist, N1, k1);
+  if (warp >= 4) load_column_twiddles<Cfg>(tw, p.twist, k1);
   tmem_fence_before_sync();
   __syncthreads();
   tmem_fence_after_sync();
@@ -800,19 +804,8 @@ __global__ void __launch_bounds__(256, 1) fdas_convolve_pairs_kernel(const PairP
         if (x0 + i < c0 || x0 + i >= c1) myRegion[i] = make_float2(0.f, 0.f);
       if (!wait_copy()) break;
       __syncwarp();
-      // a3: forward FFT of the segment; X pairs (k2 = 2p, 2p+1) go to TMEM
-      float xr[16];
-      forward_transform_with<Cfg>(
-          myRegion, [&](cp2 (&v)[H2]) { apply_twist_tmem<Cfg, true>(v, tw_addr); }, myXb, k1,
-          [&](auto, auto nn, const cp2& x) {
-            constexpr int n1 = decltype(nn)::value;
-            xr[4 * (n1 & 3)] = x.re.x;
-            xr[4 * (n1 & 3) + 1] = x.re.y;
-            xr[4 * (n1 & 3) + 2] = x.im.x;
-            xr[4 * (n1 & 3) + 3] = x.im.y;
-            if constexpr ((n1 & 3) == 3) tmem_st16(x_addr + 4 * (n1 - 3), xr);
-          });
-      tmem_wait_st();
+      // a3: forward FFT of the segment
+      forward_to_tmem<Cfg>(myRegion, myXb, k1, tw_addr, x_addr);
       cur_s = s;
       fetch_template(z);
     }
@@ -823,45 +816,19 @@ __global__ void __launch_bounds__(256, 1) fdas_convolve_pairs_kernel(const PairP
       const int32_t un = __ldg(p.pairs + e + 1);
       if (un / p.Z == s32) znext = un - s32 * p.Z;
     }
-    // a4: Y = X (TMEM) * T (this warp's region), packed pairs in bit-reversed order
+    // a4: Y = X (TMEM) * T (this warp's region), packed pairs in bit-reversed order, with the first stage
     const float4* st4 = reinterpret_cast<const float4*>(myRegion);
     cp2 v[H2];
-    static_for<H2 / 4>([&](auto cc) {
-      constexpr int c = decltype(cc)::value;
-      float x0[16];
-      tmem_ld16(x_addr + 16 * c, x0);
-      float4 t[4];
-      static_for<4>([&](auto qq) {
-        constexpr int q = decltype(qq)::value;
-        t[q] = st4[(4 * c + q) * N1 + k1];
-      });
-      tmem_wait_ld();
-      static_for<4>([&](auto qq) {
-        constexpr int q = decltype(qq)::value;
-        constexpr int pp = 4 * c + q;
-        const cp2 x = cp2{make_float2(x0[4 * q], x0[4 * q + 1]), make_float2(x0[4 * q + 2], x0[4 * q + 3])};
-        v[bitrev(2 * pp, Cfg::LOG_N2)] = cmul2(x, cp2_from(t[q]));
-      });
-    });
+    multiply_first_stage<Cfg, 0, H2 / 2>(v, x_addr, [&](int q) { return st4[q * N1 + k1]; });
     // a5: inverse FFT; a6 + a7: keep n < V inside the spectrum, store |y|^2
-    fft_split_pairs<Cfg::N2, +1>(v);
-    apply_twist_tmem<Cfg, false>(v, tw_addr);
+    fft_split_pairs<Cfg::N2, +1, 1>(v);
     const int64_t segbase = s * (int64_t)p.V;
     const int64_t lim64 = p.n_bins - segbase < (int64_t)p.V ? p.n_bins - segbase : (int64_t)p.V;
     const int lim = (int)lim64;
     float* row = p.plane + (int64_t)z * p.n_bins + segbase;
-    exchange_and_pass2<Cfg, +1>(
-        v, myXb, k1,
-        [&](auto, auto nn, const cp2& y) {
-          constexpr int n1 = decltype(nn)::value;
-          if constexpr (n1 < NV) {
-            const float2 pw = power2(y);
-            const int n_lo = k1 + Cfg::N2 * n1;
-            const int n_hi = n_lo + N1;
-            if (n_lo < lim) __stcs(row + n_lo, pw.x);
-            if (n_hi < lim) __stcs(row + n_hi, pw.y);
-          }
-        },
+    exchange_twist_pass2<Cfg, +1>(
+        v, myXb, k1, tw_addr,
+        [&](auto rr, auto& y) { store_powers<Cfg, NV, decltype(rr)::value>(y, row, k1, lim); },
         [&]() {
           if (znext >= 0) fetch_template(znext);
         });

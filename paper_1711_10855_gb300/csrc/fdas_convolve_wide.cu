@@ -4,11 +4,11 @@
 //
 // Transform of length L = N1 * N2 by N1 = 32 * WT lanes, N2 points per lane (four-step):
 //   pass 1: lane k1 holds Y[k1 + N1*k2], k2 < N2, as N2/2 packed pairs: N2-point DFT in registers,
-//   twist:  multiply by exp(SIGN i 2pi n2 k1 / L),
 //   exchange: row n2 of a shared-memory tile holds the N1 values of that column, two neighbouring k1
 //           per 16-byte entry (re, re, im, im), so that pass 2 reads packed pairs with 128-bit loads,
+//   twist:  multiply by exp(SIGN i 2pi n2 k1 / L), joined with the first stage of
 //   pass 2: lane (n2) runs the N1-point DFT of its column as a split pair; output n = n2 + N2*n1.
-//   L = 8192 has N1 = 2*N2: lane (n2, c) first forms Z[a] + Z[a + N1/2] (c = 0) or
+//   L = 8192 has N1 = 2*N2: the twist comes before the exchange, and lane (n2, c) first forms Z[a] + Z[a + N1/2] (c = 0) or
 //           (Z[a] - Z[a + N1/2]) W^a (c = 1) and runs an N2-point DFT: the outputs n1 = 2 n' + c.
 // In the exchange a lane writes single 4-byte words; the (re, im) halves of every second group of
 // eight entries are swapped, which puts a warp's 32 words on 32 banks.
@@ -57,6 +57,26 @@ struct WideCfg {
   static_assert(R * 20 + 48 <= 256, "barrier area");
 };
 
+// Twist before the exchange (split columns) with the twiddle pairs held in this lane's TMEM row.
+template <class Cfg, bool CONJ>
+__device__ __forceinline__ void apply_twist_tmem(cp2 (&v)[Cfg::H2], uint32_t tw_addr) {
+  static_assert(Cfg::H2 % 8 == 0, "twist chunking");
+  static_for<Cfg::H2 / 8>([&](auto cc) {
+    constexpr int c = decltype(cc)::value;
+    float r0[16], r1[16];
+    tmem_ld16(tw_addr + 32 * c, r0);
+    tmem_ld16(tw_addr + 32 * c + 16, r1);
+    tmem_wait_ld();
+    static_for<4>([&](auto qq) {
+      constexpr int q = decltype(qq)::value;
+      const cp2 w0 = cp2{make_float2(r0[4 * q], r0[4 * q + 1]), make_float2(r0[4 * q + 2], r0[4 * q + 3])};
+      const cp2 w1 = cp2{make_float2(r1[4 * q], r1[4 * q + 1]), make_float2(r1[4 * q + 2], r1[4 * q + 3])};
+      v[8 * c + q] = CONJ ? cmul2_conj(v[8 * c + q], w0) : cmul2(v[8 * c + q], w0);
+      v[8 * c + 4 + q] = CONJ ? cmul2_conj(v[8 * c + 4 + q], w1) : cmul2(v[8 * c + 4 + q], w1);
+    });
+  });
+}
+
 template <class Cfg>
 __device__ __forceinline__ void transform_sync(int g) {
   if constexpr (Cfg::WT == 1) __syncwarp();
@@ -73,8 +93,9 @@ __device__ __forceinline__ cp2 split_twiddle() {
 // Exchange and pass 2.  On exit u[j] = (y[r0 + RS*j], y[r0 + RS*(j + M/2)]) in rows n1 of column n2,
 // with RS = SPLIT and r0 = c.
 template <class Cfg, int SIGN>
-__device__ __forceinline__ void exchange_pass2(const cp2 (&v)[Cfg::H2], cp2 (&u)[Cfg::M / 2], float4* tile, int g,
-                                               int k1, int n2, int c) {
+__device__ __forceinline__ void exchange_pass2(cp2 (&v)[Cfg::H2], cp2 (&u)[Cfg::M / 2], float4* tile, int g, int k1,
+                                               int n2, int c, uint32_t tw_addr) {
+  if constexpr (Cfg::SPLIT == 2) apply_twist_tmem<Cfg, (SIGN < 0)>(v, tw_addr);
   const int kappa = k1 >> 1, sw = (kappa >> 3) & 1;
   float* wr = reinterpret_cast<float*>(tile) + 4 * kappa + (k1 & 1);
   float* w_re = wr + 2 * sw;
@@ -97,10 +118,9 @@ __device__ __forceinline__ void exchange_pass2(const cp2 (&v)[Cfg::H2], cp2 (&u)
   };
   constexpr int LOGM = ilog2(Cfg::M);
   if constexpr (Cfg::SPLIT == 1) {
-    static_for<Cfg::M / 2>([&](auto kk) {
-      constexpr int k = decltype(kk)::value;
-      u[bitrev(2 * k, LOGM)] = entry(kk);
-    });
+    twist_first_stage<Cfg::M / 2, 1, (SIGN < 0), false>(u, tw_addr, entry);
+    fft_split_pairs<Cfg::M, SIGN, 1>(u);
+    return;
   } else if (c == 0) {
     static_for<Cfg::M / 2>([&](auto kk) {
       constexpr int k = decltype(kk)::value;
@@ -126,6 +146,23 @@ __device__ __forceinline__ int64_t first_unit(const ConvParams& p, int Z, unsign
   const int per = Z + p.group_cost;
   const int64_t g = quotient(v, per), r = v - g * per - p.group_cost;
   return g * Z + (r > 0 ? r : 0);
+}
+
+// Twiddle pairs of a lane (the plan's table holds exp(i 2pi n2 k1 / L) for n2 = j, j + H2 as pair j of
+// lane k1).  Split columns: that pair j.  Otherwise the pairs of k1 = 2 kappa, 2 kappa + 1 of the lane's
+// column n2, in slot order.
+template <class Cfg>
+__device__ __forceinline__ void load_lane_twiddles(float4 (&tw)[Cfg::H2], const float2* twist, int lane_k1) {
+  if constexpr (Cfg::SPLIT == 2) {
+    const float4* tw4 = reinterpret_cast<const float4*>(twist);
+    static_for<Cfg::H2>([&](auto jj) { tw[decltype(jj)::value] = __ldg(tw4 + decltype(jj)::value * Cfg::N1 + lane_k1); });
+  } else {
+    const float* f = reinterpret_cast<const float*>(twist) + (lane_k1 % Cfg::H2) * Cfg::N1 * 4 + lane_k1 / Cfg::H2;
+    static_for<Cfg::H2>([&](auto ii) {
+      constexpr int i = decltype(ii)::value, k = 2 * slot_pair(i, Cfg::H2);
+      tw[i] = make_float4(__ldg(f + 4 * k), __ldg(f + 4 * (k + 1)), __ldg(f + 4 * k + 2), __ldg(f + 4 * (k + 1) + 2));
+    });
+  }
 }
 
 // NV (eighths of the rows): pass-2 rows n1 >= NV*N1/8 hold no valid output and are dropped at compile
@@ -202,9 +239,16 @@ __global__ void __launch_bounds__(32 * Cfg::W, 1) fdas_convolve_wide_kernel(cons
     if (PARTS == 1 || e % PARTS == PARTS - 1) *next_z = zr + 1 == Z ? 0 : zr + 1;
     issued_pos[slot] = e;
     mbar_arrive_expect_tx(&full[slot], (uint32_t)Cfg::PART_BYTES);
-    bulk_g2s(smem + Cfg::OFF_T + slot * Cfg::PART_BYTES,
-             reinterpret_cast<const unsigned char*>(p.templates + (size_t)zr * L) + (e % PARTS) * Cfg::PART_BYTES,
-             (uint32_t)Cfg::PART_BYTES, &full[slot]);
+    unsigned char* dst = smem + Cfg::OFF_T + slot * Cfg::PART_BYTES;
+    const unsigned char* src = reinterpret_cast<const unsigned char*>(p.templates + (size_t)zr * L);
+    if constexpr (PARTS == 1) {
+      bulk_g2s(dst, src, (uint32_t)Cfg::PART_BYTES, &full[slot]);
+    } else {   // the part's pairs, then their partners half a template further
+      constexpr uint32_t half = (uint32_t)(Cfg::PART_BYTES / 2);
+      src += (e % PARTS) * half;
+      bulk_g2s(dst, src, half, &full[slot]);
+      bulk_g2s(dst + half, src + (size_t)L * 4, half, &full[slot]);
+    }
   };
   if (!FWD && tid == 32) {
     *next_z = z;
@@ -214,7 +258,7 @@ __global__ void __launch_bounds__(32 * Cfg::W, 1) fdas_convolve_wide_kernel(cons
   // warps w, w + 4, ... hold the same lanes of their transforms (WT divides 4): one copy of the twiddles
   // per quadrant (stored once the tensor memory is there)
   float4 tw[H2];
-  if (warp >= 4 && warp < 8) load_twiddles<H2>(tw, p.twist, N1, k1);
+  if (warp >= 4 && warp < 8) load_lane_twiddles<Cfg>(tw, p.twist, k1);
   tmem_fence_before_sync();
   __syncthreads();
   tmem_fence_after_sync();
@@ -270,8 +314,7 @@ __global__ void __launch_bounds__(32 * Cfg::W, 1) fdas_convolve_wide_kernel(cons
         v[i] = cp2{make_float2(e0.x, e1.x), make_float2(e0.y, e1.y)};
       });
       fft_split_pairs<N2, -1>(v);
-      apply_twist_tmem<Cfg, true>(v, tw_addr);
-      exchange_pass2<Cfg, -1>(v, x, tile, g, k1, n2, c_fwd);
+      exchange_pass2<Cfg, -1>(v, x, tile, g, k1, n2, c_fwd, tw_addr);
       if constexpr (FWD) {
         float2* out = reinterpret_cast<float2*>(p.plane) + s * L;
         if (s < p.nseg)
@@ -284,22 +327,14 @@ __global__ void __launch_bounds__(32 * Cfg::W, 1) fdas_convolve_wide_kernel(cons
         tmem_fence_before_sync();
         continue;
       }
-      static_for<H2 / 4>([&](auto cc) {
-        constexpr int c = decltype(cc)::value;
-        float r[16];
-        static_for<4>([&](auto qq) {
-          constexpr int q = decltype(qq)::value;
-          constexpr int k2 = 2 * (4 * c + q);   // members k2 and k2 + 1: both in .x or both in .y
-          constexpr int j = k2 < M / 2 ? k2 : k2 - M / 2;
-          if constexpr (k2 < M / 2) {
-            r[4 * q] = x[j].re.x, r[4 * q + 1] = x[j + 1].re.x, r[4 * q + 2] = x[j].im.x, r[4 * q + 3] = x[j + 1].im.x;
-          } else {
-            r[4 * q] = x[j].re.y, r[4 * q + 1] = x[j + 1].re.y, r[4 * q + 2] = x[j].im.y, r[4 * q + 3] = x[j + 1].im.y;
-          }
-        });
-        tmem_st16(x_addr + 16 * c, r);
+      spectrum_to_tmem<H2>(x_addr, [&](auto pp) {
+        constexpr int k2 = 2 * decltype(pp)::value;   // members k2 and k2 + 1: both in .x or both in .y
+        constexpr int j = k2 < M / 2 ? k2 : k2 - M / 2;
+        if constexpr (k2 < M / 2)
+          return cp2{make_float2(x[j].re.x, x[j + 1].re.x), make_float2(x[j].im.x, x[j + 1].im.x)};
+        else
+          return cp2{make_float2(x[j].re.y, x[j + 1].re.y), make_float2(x[j].im.y, x[j + 1].im.y)};
       });
-      tmem_wait_st();
     }
 
     const int64_t lim64 = p.n_bins - segbase < (int64_t)p.V ? p.n_bins - segbase : (int64_t)p.V;
@@ -319,22 +354,10 @@ __global__ void __launch_bounds__(32 * Cfg::W, 1) fdas_convolve_wide_kernel(cons
           lim = 0;
         }
         const float4* st4 = reinterpret_cast<const float4*>(smem + Cfg::OFF_T + slot * Cfg::PART_BYTES);
-        static_for<Cfg::PART_PAIRS / 4>([&](auto cc) {
-          constexpr int c = decltype(cc)::value;
-          constexpr int q0 = part * Cfg::PART_PAIRS + 4 * c;
-          float x0[16];
-          tmem_ld16(x_addr + 4 * q0, x0);
-          float4 t[4];
-          static_for<4>([&](auto qq) {
-            constexpr int q = decltype(qq)::value;
-            t[q] = st4[(4 * c + q) * N1 + k1];
-          });
-          tmem_wait_ld();
-          static_for<4>([&](auto qq) {
-            constexpr int q = decltype(qq)::value;
-            const cp2 x = cp2{make_float2(x0[4 * q], x0[4 * q + 1]), make_float2(x0[4 * q + 2], x0[4 * q + 3])};
-            v[bitrev(2 * (q0 + q), Cfg::LOG_N2)] = cmul2(x, cp2_from(t[q]));
-          });
+        // a part holds its pairs p and their partners p + H2/2
+        multiply_first_stage<Cfg, part * Cfg::PART_PAIRS / 2, Cfg::PART_PAIRS / 2>(v, x_addr, [&](int q) {
+          constexpr int first = part * Cfg::PART_PAIRS / 2;
+          return st4[(q < H2 / 2 ? q - first : q - H2 / 2 - first + Cfg::PART_PAIRS / 2) * N1 + k1];
         });
         // release the slot; the last of the W consumers refills it R positions ahead
         __syncwarp();
@@ -347,10 +370,9 @@ __global__ void __launch_bounds__(32 * Cfg::W, 1) fdas_convolve_wide_kernel(cons
         }
       });
       // a5: inverse FFT
-      fft_split_pairs<N2, +1>(v);
-      apply_twist_tmem<Cfg, false>(v, tw_addr);
+      fft_split_pairs<N2, +1, 1>(v);
       cp2 y[M / 2];
-      exchange_pass2<Cfg, +1>(v, y, tile, g, k1, n2, c_inv);
+      exchange_pass2<Cfg, +1>(v, y, tile, g, k1, n2, c_inv, tw_addr);
       // a6 + a7: keep n < V (and inside the spectrum), store |y|^2
       float* row = p.plane + (int64_t)z * p.n_bins + segbase;
       const int nb = n2 + N2 * c_inv;

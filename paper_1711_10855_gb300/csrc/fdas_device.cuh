@@ -191,6 +191,19 @@ __device__ __forceinline__ cp2 cmul2(const cp2& a, const cp2& b) {
 __device__ __forceinline__ cp2 cmul2_conj(const cp2& a, const cp2& b) {   // a * conj(b)
   return cp2{fma2(a.re, b.re, mul2(a.im, b.im)), fma2(a.im, b.re, mul2(make_float2(-a.re.x, -a.re.y), b.im))};
 }
+// c + a * b and c + a * conj(b), element-wise (4 packed instructions).
+__device__ __forceinline__ cp2 cfma2(const cp2& a, const cp2& b, const cp2& c) {
+  return cp2{fma2(make_float2(-a.im.x, -a.im.y), b.im, fma2(a.re, b.re, c.re)), fma2(a.im, b.re, fma2(a.re, b.im, c.im))};
+}
+__device__ __forceinline__ cp2 cfma2_conj(const cp2& a, const cp2& b, const cp2& c) {
+  return cp2{fma2(a.im, b.im, fma2(a.re, b.re, c.re)),
+             fma2(make_float2(-a.re.x, -a.re.y), b.im, fma2(a.im, b.re, c.im))};
+}
+// 2a - b
+__device__ __forceinline__ cp2 twice_minus(const cp2& a, const cp2& b) {
+  const float2 two = make_float2(2.f, 2.f);
+  return cp2{fma2(two, a.re, make_float2(-b.re.x, -b.re.y)), fma2(two, a.im, make_float2(-b.im.x, -b.im.y))};
+}
 __device__ __forceinline__ float2 power2(const cp2& a) { return fma2(a.re, a.re, mul2(a.im, a.im)); }
 __device__ __forceinline__ cp2 cp2_from(float4 v) { return cp2{make_float2(v.x, v.y), make_float2(v.z, v.w)}; }
 __device__ __forceinline__ float4 cp2_to(const cp2& v) { return make_float4(v.re.x, v.re.y, v.im.x, v.im.y); }
@@ -245,16 +258,17 @@ template <int N, int SIGN, int S, int... I>
 __device__ __forceinline__ void fft_stage2(cp2 (&v)[N], std::integer_sequence<int, I...>) {
   (stage_butterfly2<N, SIGN, S, I>(v), ...);
 }
-template <int N, int SIGN, int... S>
+template <int N, int SIGN, int FROM = 0, int... S>
 __device__ __forceinline__ void fft_stages2(cp2 (&v)[N], std::integer_sequence<int, S...>) {
-  (fft_stage2<N, SIGN, S>(v, std::make_integer_sequence<int, N / 2>{}), ...);
+  (fft_stage2<N, SIGN, FROM + S>(v, std::make_integer_sequence<int, N / 2>{}), ...);
 }
 
 // Two independent N-point DFTs in lockstep ("columns" a and b of each pair):
-// on entry v[i] = (a[bitrev(i)], b[bitrev(i)]), on exit v[m] = (A[m], B[m]).
-template <int N, int SIGN>
+// on entry v[i] = (a[bitrev(i)], b[bitrev(i)]), on exit v[m] = (A[m], B[m]).  FROM: the first
+// FROM stages have been done.
+template <int N, int SIGN, int FROM = 0>
 __device__ __forceinline__ void fft_pair_columns(cp2 (&v)[N]) {
-  fft_stages2<N, SIGN>(v, std::make_integer_sequence<int, ilog2(N)>{});
+  fft_stages2<N, SIGN, FROM>(v, std::make_integer_sequence<int, ilog2(N) - FROM>{});
 }
 
 template <int N, int SIGN, int J>
@@ -271,10 +285,11 @@ __device__ __forceinline__ void last_stage_all(cp2 (&v)[N / 2], std::integer_seq
 
 // One N-point DFT held as N/2 pairs v[i] = (x[bitrev(i)], x[bitrev(i + N/2)]): the first
 // log2(N)-1 stages are two N/2-point DFTs in lockstep (packed), the last stage pairs the two
-// members of each pair (scalar FMA butterflies).  On exit v[j] = (X[j], X[j + N/2]).
-template <int N, int SIGN>
+// members of each pair (scalar FMA butterflies).  On exit v[j] = (X[j], X[j + N/2]).  FROM: the first
+// FROM stages have been done.
+template <int N, int SIGN, int FROM = 0>
 __device__ __forceinline__ void fft_split_pairs(cp2 (&v)[N / 2]) {
-  fft_stages2<N / 2, SIGN>(v, std::make_integer_sequence<int, ilog2(N) - 1>{});
+  fft_stages2<N / 2, SIGN, FROM>(v, std::make_integer_sequence<int, ilog2(N) - 1 - FROM>{});
   last_stage_all<N, SIGN>(v, std::make_integer_sequence<int, N / 2>{});
 }
 
