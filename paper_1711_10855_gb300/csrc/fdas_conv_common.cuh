@@ -18,22 +18,36 @@ __device__ __forceinline__ cp2 tmem_pair(const float (&r)[16], int q) {
   return cp2{make_float2(r[4 * q], r[4 * q + 1]), make_float2(r[4 * q + 2], r[4 * q + 3])};
 }
 
+// Both products go in chunks of two butterflies.  PIPE: a chunk's operands are fetched before the
+// previous chunk is computed; the kernels with one column pair per lane and a ring shared by eight
+// warps are faster without (2048: 1313 against 1366 us per survey plane), the others with it (4096: 1847
+// against 1877 us, 8192: 1680 against 1713 us for their timed planes).
+
 // Y = X (this lane's TMEM slots from x_addr) * T (load(p) = pair p) and the first stage of the
 // N2-point DFT: v in bit-reversed order, pairs [P0, P0 + NP) and their partners.
 template <class Cfg, int P0, int NP, class Load>
 __device__ __forceinline__ void multiply_first_stage(cp2 (&v)[Cfg::H2], uint32_t x_addr, Load&& load) {
-  constexpr int HALF = Cfg::H2 / 2;
-  static_for<NP / 2>([&](auto cc) {
-    constexpr int p0 = P0 + 2 * decltype(cc)::value;
-    float x[16];
-    tmem_ld16(x_addr + 8 * p0, x);
-    const cp2 ta = cp2_from(load(p0)), tb = cp2_from(load(p0 + HALF));
-    const cp2 tc = cp2_from(load(p0 + 1)), td = cp2_from(load(p0 + 1 + HALF));
+  constexpr int HALF = Cfg::H2 / 2, NC = NP / 2;
+  float x[2][16];
+  float4 t[2][4];
+  auto fetch = [&](auto cc) {
+    constexpr int b = decltype(cc)::value & 1, p0 = P0 + 2 * decltype(cc)::value;
+    tmem_ld16(x_addr + 8 * p0, x[b]);
+    t[b][0] = load(p0);
+    t[b][1] = load(p0 + HALF);
+    t[b][2] = load(p0 + 1);
+    t[b][3] = load(p0 + 1 + HALF);
+  };
+  if constexpr (Cfg::PIPE) fetch(std::integral_constant<int, 0>{});
+  static_for<NC>([&](auto cc) {
+    constexpr int c = decltype(cc)::value, b = c & 1, p0 = P0 + 2 * c;
+    if constexpr (!Cfg::PIPE) fetch(cc);
     tmem_wait_ld();
+    if constexpr (Cfg::PIPE && c + 1 < NC) fetch(std::integral_constant<int, c + 1>{});
     constexpr int i0 = bitrev(2 * p0, Cfg::LOG_N2), i1 = bitrev(2 * p0 + 2, Cfg::LOG_N2);
-    const cp2 t0 = cmul2(tmem_pair(x, 0), ta), t1 = cmul2(tmem_pair(x, 2), tc);
-    v[i0] = cfma2(tmem_pair(x, 1), tb, t0);
-    v[i1] = cfma2(tmem_pair(x, 3), td, t1);
+    const cp2 t0 = cmul2(tmem_pair(x[b], 0), cp2_from(t[b][0])), t1 = cmul2(tmem_pair(x[b], 2), cp2_from(t[b][2]));
+    v[i0] = cfma2(tmem_pair(x[b], 1), cp2_from(t[b][1]), t0);
+    v[i1] = cfma2(tmem_pair(x[b], 3), cp2_from(t[b][3]), t1);
     v[i0 + 1] = twice_minus(t0, v[i0]);
     v[i1 + 1] = twice_minus(t1, v[i1]);
   });
@@ -42,21 +56,32 @@ __device__ __forceinline__ void multiply_first_stage(cp2 (&v)[Cfg::H2], uint32_t
 // u = entries (load(s), s < N) times the twiddles of this lane's TMEM slots (conjugated for the forward
 // transform), with the first stage done: N entries in bit-reversed order over log2(N) + SHIFT bits of
 // (s << SHIFT).  The first pair's twiddle is 1 when UNIT0.
-template <int N, int SHIFT, bool CONJ, bool UNIT0, class Load>
+template <int N, int SHIFT, bool CONJ, bool UNIT0, bool PIPE, class Load>
 __device__ __forceinline__ void twist_first_stage(cp2 (&u)[N], uint32_t tw_addr, Load&& load) {
-  constexpr int HALF = N / 2, LOG = ilog2(N) + SHIFT;
-  static_for<N / 4>([&](auto cc) {
-    constexpr int s0 = 2 * decltype(cc)::value;
-    float w[16];
-    tmem_ld16(tw_addr + 8 * s0, w);
-    const cp2 a = load(std::integral_constant<int, s0>{}), b = load(std::integral_constant<int, s0 + HALF>{});
-    const cp2 c = load(std::integral_constant<int, s0 + 1>{}), d = load(std::integral_constant<int, s0 + 1 + HALF>{});
+  constexpr int HALF = N / 2, LOG = ilog2(N) + SHIFT, NC = N / 4;
+  float w[2][16];
+  cp2 e[2][4];
+  auto fetch = [&](auto cc) {
+    constexpr int b = decltype(cc)::value & 1, s0 = 2 * decltype(cc)::value;
+    tmem_ld16(tw_addr + 8 * s0, w[b]);
+    e[b][0] = load(std::integral_constant<int, s0>{});
+    e[b][1] = load(std::integral_constant<int, s0 + HALF>{});
+    e[b][2] = load(std::integral_constant<int, s0 + 1>{});
+    e[b][3] = load(std::integral_constant<int, s0 + 1 + HALF>{});
+  };
+  auto times = [](const cp2& a, const cp2& t) { return CONJ ? cmul2_conj(a, t) : cmul2(a, t); };
+  auto times_add = [](const cp2& a, const cp2& t, const cp2& c) { return CONJ ? cfma2_conj(a, t, c) : cfma2(a, t, c); };
+  if constexpr (PIPE) fetch(std::integral_constant<int, 0>{});
+  static_for<NC>([&](auto cc) {
+    constexpr int c = decltype(cc)::value, b = c & 1, s0 = 2 * c;
+    if constexpr (!PIPE) fetch(cc);
     tmem_wait_ld();
+    if constexpr (PIPE && c + 1 < NC) fetch(std::integral_constant<int, c + 1>{});
     constexpr int i0 = bitrev(s0 << SHIFT, LOG), i1 = bitrev((s0 + 1) << SHIFT, LOG);
-    const cp2 t0 = UNIT0 && s0 == 0 ? a : (CONJ ? cmul2_conj(a, tmem_pair(w, 0)) : cmul2(a, tmem_pair(w, 0)));
-    const cp2 t1 = CONJ ? cmul2_conj(c, tmem_pair(w, 2)) : cmul2(c, tmem_pair(w, 2));
-    u[i0] = CONJ ? cfma2_conj(b, tmem_pair(w, 1), t0) : cfma2(b, tmem_pair(w, 1), t0);
-    u[i1] = CONJ ? cfma2_conj(d, tmem_pair(w, 3), t1) : cfma2(d, tmem_pair(w, 3), t1);
+    const cp2 t0 = UNIT0 && s0 == 0 ? e[b][0] : times(e[b][0], tmem_pair(w[b], 0));
+    const cp2 t1 = times(e[b][2], tmem_pair(w[b], 2));
+    u[i0] = times_add(e[b][1], tmem_pair(w[b], 1), t0);
+    u[i1] = times_add(e[b][3], tmem_pair(w[b], 3), t1);
     u[i0 + 1] = twice_minus(t0, u[i0]);
     u[i1 + 1] = twice_minus(t1, u[i1]);
   });

@@ -177,7 +177,7 @@ __device__ __forceinline__ void exchange_twist_pass2(const cp2 (&v)[Cfg::H2], fl
       xb[i * Cfg::XPITCH + k1] = cp2_to(v[r * N1 + i]);
     });
     __syncwarp();
-    twist_first_stage<N1, 0, (SIGN < 0), true>(u, tw_addr + 4 * N1 * r, [&](auto ss) {
+    twist_first_stage<N1, 0, (SIGN < 0), true, Cfg::PIPE>(u, tw_addr + 4 * N1 * r, [&](auto ss) {
       return cp2_from(xb[k1 * Cfg::XPITCH + decltype(ss)::value]);
     });
     if constexpr (r == Cfg::CP - 1) after_reads();   // the tile is free once its last round is read
@@ -250,6 +250,7 @@ struct TmemCfg {
   static constexpr int P = P_;             // warps sharing a segment, taking alternate templates
   static constexpr int G = F * W / P;      // segments resident per CTA: one group of lanes each
   static constexpr int R = 4;
+  static constexpr bool PIPE = false;      // see multiply_first_stage
   static constexpr int C = N2 / N1;        // pass-2 columns per lane
   static constexpr int CP = C / 2;         // and column pairs (exchange rounds)
   static constexpr int XR = 1;

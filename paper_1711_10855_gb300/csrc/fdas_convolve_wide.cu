@@ -35,6 +35,7 @@ struct WideCfg {
   static constexpr int G = W / WT;           // segments resident per CTA
   static constexpr int PARTS = PARTS_;       // ring slots per template
   static constexpr int R = R_;               // ring slots
+  static constexpr bool PIPE = true;         // see multiply_first_stage
   static constexpr int SPLIT = N1 / N2;      // lanes per column of pass 2
   static constexpr int M = N1 / SPLIT;       // points of a lane's pass-2 DFT (= N2)
   static constexpr int LOG_N2 = ilog2(N2);
@@ -118,7 +119,7 @@ __device__ __forceinline__ void exchange_pass2(cp2 (&v)[Cfg::H2], cp2 (&u)[Cfg::
   };
   constexpr int LOGM = ilog2(Cfg::M);
   if constexpr (Cfg::SPLIT == 1) {
-    twist_first_stage<Cfg::M / 2, 1, (SIGN < 0), false>(u, tw_addr, entry);
+    twist_first_stage<Cfg::M / 2, 1, (SIGN < 0), false, Cfg::PIPE>(u, tw_addr, entry);
     fft_split_pairs<Cfg::M, SIGN, 1>(u);
     return;
   } else if (c == 0) {
