@@ -343,48 +343,54 @@ __global__ void __launch_bounds__(256) write_units_kernel(const uint16_t* masks,
 // positions [w*hop, (w+1)*hop) and recomputes the +-84-position halo its three layers need
 // (dilations 1, 4, 16):
 //   x   at P0-84 + j, j < 128*T1 + 8     (prefetched into registers one block ahead)
-//   h1  at P0-80 + r, r < 128*T2 + 32    (layer 1 as an im2col GEMM: K = 9 taps padded to 16)
-//   h2  at P0-64 + r, r < hop + 128      (layer 2: T2 = T3 + 1 M-tiles of 128 positions)
-//   h3  at P0 + r,    r < hop            (layer 3: T3 = hop/128 M-tiles), max-pooled per channel
-// Activations sit in shared memory "chunk-planar": channel chunk j (8 channels, 16 B) of
-// position row r at plane j, offset 16*r.  A K-major no-swizzle operand whose rows are
-// positions is then one descriptor per (tap k, K-half c): start row + k d, LBO = plane size,
-// SBO = 128 B -- the im2col of a dilated k = 9 convolution costs no copies.
+//   h1  at P0-80 + r, r < hop + 160      (layer 1 as an im2col GEMM: K = 9 taps padded to 16, M = positions)
+//   h2  at P0-64 + r, r < hop + 128      (layer 2)
+//   h3  at P0 + r,    r < hop            (layer 3, max-pooled per channel)
+// Layers 2 and 3 (dilation d) put the weights on the M side: row 32 i + c of the accumulator is channel c
+// at the positions t = 4 d a + d i + b (phase i < 4, 0 <= b < d), column P = d a + b.  Tap k of phase i
+// reads input position t + d k, which is phase (i + k) mod 4 of the same split, d ((i + k) div 4) columns
+// further: for each of the 12 offsets o = i + k one MMA multiplies [W_o; W_{o-1}; W_{o-2}; W_{o-3}]
+// (zero where o - i is no tap) by the input rows of phase o mod 4 from column d (o div 4) on.  The
+// weight rows are kept once, as the stack [0 0 0 W_8 ... W_0 0 0 0]: offset o starts at its block 11 - o.
+// N is (hop + 128)/4 and hop/4 columns instead of 32 channels, where an MMA's time no longer has
+// its floor of about 50 cycles: 24 MMAs of 80 and 64 cycles per layer for 512 positions, against 90
+// and 72 of 64 cycles with one tap, 128 positions and N = 32 each (kernel 330 to 225 us at 2^22
+// bins).  The zero blocks are a quarter of the multiply-adds.
+// Activations sit in shared memory K-major "chunk-planar": channel chunk j (8 channels, 16 B) of row q at
+// plane j, offset 16*q, rows ordered (phase, column) for the layer that reads them.  h2 overwrites
+// h1, and h1 the layer-1 im2col, each after the MMAs that read them.
 // ---------------------------------------------------------------------------------------
 constexpr int kMaxHop = 512;
-constexpr int kT3max = kMaxHop / 128;
-constexpr int kT2max = kT3max + 1;
-constexpr int kT1max = kT2max + 1;
-constexpr int kNP1 = 128 * kT2max + 8 * kDil2;  // h1 rows (plane height)
-constexpr int kNP2 = 128 * kT2max;              // h2 rows (plane height)
+constexpr int kT1max = kMaxHop / 128 + 2;       // layer-1 M-tiles
+constexpr int kNP1 = (kMaxHop + 160) / 4 + 4;   // h1 rows per phase (+4: a quarter-warp's rows on all banks)
+constexpr int kNP2 = (kMaxHop + 128) / 4;       // h2 rows per phase
 constexpr int kNA1 = 128 * kT1max;              // im2col rows of layer 1
 constexpr int kNX = kNA1 + 8;                   // staged x values
 constexpr int kGroupThreads = 128;
 constexpr int kXPer = (kNX + kGroupThreads - 1) / kGroupThreads;   // prefetched x per thread
 constexpr int kZStage = 256;                    // head weights staged in shared memory up to this Z
-constexpr uint32_t kPlaneH1 = kNP1 * 16, kPlaneH2 = kNP2 * 16, kPlaneA1 = kNA1 * 16;
+constexpr uint32_t kPlaneH1 = 4 * kNP1 * 16, kPlaneA1 = kNA1 * 16;
+constexpr uint32_t kPlaneH2 = 4 * kNP2 * 16 + 16;   // + 16: the four planes of a row on different banks
+constexpr int kStackRows = 15 * kC;             // weight rows of layers 2 and 3
+constexpr uint32_t kPlaneW = kStackRows * 16;
 constexpr int kOffW1 = 0;                       // layer-1 weights: 2 K-chunks x 512 B
-constexpr int kOffW2 = kOffW1 + 1024;           // 9 taps x 4 K-chunks x 512 B
-constexpr int kOffW3 = kOffW2 + 9 * 2048;
-constexpr int kOffWl = kOffW3 + 9 * 2048;       // head weights [Z][32] FP16
+constexpr int kOffW2 = kOffW1 + 1024;           // 4 K-chunks x 480 rows
+constexpr int kOffW3 = kOffW2 + 4 * kPlaneW;
+constexpr int kOffWl = kOffW3 + 4 * kPlaneW;    // head weights [Z][32] FP16
 constexpr int kOffBl = kOffWl + kZStage * kC * 2;
 constexpr int kOffBias = kOffBl + kZStage * 4;  // b1, b2, b3 (FP32 values of the FP16 copy)
-constexpr int kOffSlot = kOffBias + 3 * kC * 4; // two activation slots
-constexpr int kSlotH1 = 0;                      // also holds the staged x (dead before h1 is written)
-constexpr int kSlotH2 = 4 * kPlaneH1;           // also holds the layer-1 im2col (dead before h2)
-constexpr int kSlotBytes = kSlotH2 + 4 * kPlaneH2;
+constexpr int kOffSlot = (kOffBias + 3 * kC * 4 + 127) / 128 * 128;   // two activation slots
+constexpr int kSlotX = 4 * kPlaneH1;            // staged x behind the planes
+constexpr int kSlotBytes = (kSlotX + kNX * 4 + 127) / 128 * 128;
 constexpr int kOffGroup = kOffSlot + 2 * kSlotBytes;   // per group: channel maxima, mbarrier
 constexpr int kGroupMisc = 256;
 constexpr int kOffTslot = kOffGroup + 2 * kGroupMisc;
 constexpr int kProposeSmem = kOffTslot + 16;
-constexpr uint32_t kIdesc = fdas::umma_idesc_f16(128, kC);
+constexpr uint32_t kIdesc1 = fdas::umma_idesc_f16(128, kC);
 constexpr uint32_t kTmemCols = 512;             // 256 columns per group (<= 6 x 32 used)
 static_assert(kDil1 == 1, "layer 1 is an im2col of adjacent x values");
-static_assert(8 * kDil3 <= 128 && 8 * kDil2 <= 128, "each layer's halo fits in one extra 128-row tile");
-static_assert(2 * kPlaneA1 <= 4 * kPlaneH2, "im2col must fit in the h2 planes");
-static_assert(kNX * 4 <= (int)(4 * kPlaneH1), "staged x must fit in the h1 planes");
-static_assert(32 * kT1max <= (int)kTmemCols / 2, "accumulators must fit a group's TMEM half");
-static_assert(kOffSlot % 128 == 0 && kSlotBytes % 128 == 0, "slot alignment");
+static_assert(kPlaneH2 <= kPlaneH1 && 2 * kPlaneA1 <= 4 * kPlaneH1, "h2 and the im2col fit in the h1 planes");
+static_assert(32 * kT1max <= (int)kTmemCols / 2 && kNP2 <= (int)kTmemCols / 2, "a group's TMEM half");
 static_assert(kProposeSmem <= 227 * 1024, "shared memory");
 
 struct ProposeParams {
@@ -399,7 +405,7 @@ struct ProposeParams {
   int* status;              // bit 0: a bounded wait gave up
 };
 
-// B operand (weights) of one tap in the K-major no-swizzle layout: rows o (N = 32), K = in-ch.
+// B operand (layer-1 weights) in the K-major no-swizzle layout: rows o (N = 32), K = tap.
 __device__ __forceinline__ int wb_off(int o, int i) { return (i >> 3) * 512 + (o >> 3) * 128 + (o & 7) * 16 + (i & 7) * 2; }
 
 // Named barrier of one 128-thread group (ids 1, 2; id 0 is __syncthreads).
@@ -421,8 +427,6 @@ __global__ void __launch_bounds__(256, 1) propose_kernel(const ProposeParams p) 
   using namespace fdas;
   extern __shared__ __align__(1024) unsigned char sm[];
   __half* sW1 = reinterpret_cast<__half*>(sm + kOffW1);
-  __half* sW2 = reinterpret_cast<__half*>(sm + kOffW2);
-  __half* sW3 = reinterpret_cast<__half*>(sm + kOffW3);
   __half* sWl = reinterpret_cast<__half*>(sm + kOffWl);
   float* sBl = reinterpret_cast<float*>(sm + kOffBl);
   float* sBias = reinterpret_cast<float*>(sm + kOffBias);
@@ -431,10 +435,7 @@ __global__ void __launch_bounds__(256, 1) propose_kernel(const ProposeParams p) 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int g = warp >> 2, q = warp & 3, gt = tid & (kGroupThreads - 1);
   unsigned char* slot = sm + kOffSlot + g * kSlotBytes;
-  float* sX = reinterpret_cast<float*>(slot + kSlotH1);
-  unsigned char* sH1 = slot + kSlotH1;
-  unsigned char* sH2 = slot + kSlotH2;
-  unsigned char* sA1 = slot + kSlotH2;
+  float* sX = reinterpret_cast<float*>(slot + kSlotX);
   unsigned* sMax = reinterpret_cast<unsigned*>(sm + kOffGroup + g * kGroupMisc);
   uint64_t* bar = reinterpret_cast<uint64_t*>(sm + kOffGroup + g * kGroupMisc + 128);
   const bool wl_staged = p.Z <= kZStage;
@@ -444,10 +445,14 @@ __global__ void __launch_bounds__(256, 1) propose_kernel(const ProposeParams p) 
     const int o = idx >> 4, k = idx & 15;
     sW1[wb_off(o, k) / 2] = k < kK ? p.w[p.oW1 + o * kK + k] : __float2half_rn(0.f);
   }
-  for (int idx = tid; idx < kK * kC * kC; idx += 256) {
-    const int k = idx / (kC * kC), o = (idx / kC) % kC, i = idx % kC;
-    sW2[k * 1024 + wb_off(o, i) / 2] = p.w[p.oW2 + (o * kC + i) * kK + k];
-    sW3[k * 1024 + wb_off(o, i) / 2] = p.w[p.oW3 + (o * kC + i) * kK + k];
+  for (int idx = tid; idx < 2 * 4 * kStackRows; idx += 256) {   // 8 input channels of a stack row at a time
+    const int layer = idx / (4 * kStackRows), j = idx / kStackRows % 4, row = idx % kStackRows;
+    const int k = 11 - row / kC, o = row % kC;
+    __half h[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e)
+      h[e] = k >= 0 && k < kK ? p.w[(layer ? p.oW3 : p.oW2) + (o * kC + 8 * j + e) * kK + k] : __float2half_rn(0.f);
+    *reinterpret_cast<uint4*>(sm + (layer ? kOffW3 : kOffW2) + j * kPlaneW + row * 16) = *reinterpret_cast<uint4*>(h);
   }
   if (wl_staged) {
     for (int idx = tid; idx < p.Z * kC; idx += 256) sWl[idx] = p.w[p.oWl + idx];
@@ -472,10 +477,10 @@ __global__ void __launch_bounds__(256, 1) propose_kernel(const ProposeParams p) 
   tmem_fence_after_sync();
   const uint32_t tm = *tslot + 256u * g;
   const uint32_t tm_lane = tm + ((uint32_t)(32 * q) << 16);
-  const uint32_t aW1 = smem_u32(sW1), aW2 = smem_u32(sW2), aW3 = smem_u32(sW3);
-  const uint32_t aH1 = smem_u32(sH1), aH2 = smem_u32(sH2), aA1 = smem_u32(sA1);
+  const uint32_t aW1 = smem_u32(sW1), aW2 = smem_u32(sm + kOffW2), aW3 = smem_u32(sm + kOffW3);
+  const uint32_t aSlot = smem_u32(slot);
   const float sc = *p.scale;
-  constexpr int T3 = HOP / 128, T2 = T3 + 1, T1 = T2 + 1;
+  constexpr int T1 = HOP / 128 + 2, N2 = (HOP + 128) / 4, N3 = HOP / 4;
   constexpr int nx = 128 * T1 + 8;
   uint32_t phase = 0;
   bool ok = true;
@@ -504,23 +509,24 @@ __global__ void __launch_bounds__(256, 1) propose_kernel(const ProposeParams p) 
     group_sync(g);
     tmem_fence_after_sync();
   };
-  // accumulator tile t (lanes = rows 128t + 32q + lane) + bias -> relu -> FP16 planes, rows < limit.
-  // The next tile's TMEM load is issued before this tile is converted (tcgen05.wait::ld waits for
-  // every earlier load, so the wait comes first and the two buffers alternate).
-  auto store_layer = [&](auto ntiles, int limit, const float* bias, unsigned char* dst, uint32_t plane) {
-    constexpr int NT = decltype(ntiles)::value;
+  // layer 1's accumulator tiles (lanes = positions r = 128t + 32q + lane, columns = channels) + bias -> relu
+  // -> FP16 rows of layer 2's input, r < HOP + 160.  The next tile's TMEM load is issued before this
+  // tile is converted (tcgen05.wait::ld waits for every earlier load, so the wait comes first and the two
+  // buffers alternate).
+  auto store_h1 = [&]() {
     float a[2][16], b[2][16];
     tmem_ld16(tm_lane, a[0]);
     tmem_ld16(tm_lane + 16, b[0]);
-    static_for<NT>([&](auto tt) {
+    unsigned char* dst = slot + (((lane >> 2) & 3) * kNP1 + 8 * q + 4 * (lane >> 4) + (lane & 3)) * 16;
+    static_for<T1>([&](auto tt) {
       constexpr int t = decltype(tt)::value, cur = t & 1;
       tmem_wait_ld();
-      if constexpr (t + 1 < NT) {
+      if constexpr (t + 1 < T1) {
         tmem_ld16(tm_lane + 32 * (t + 1), a[cur ^ 1]);
         tmem_ld16(tm_lane + 32 * (t + 1) + 16, b[cur ^ 1]);
       }
       const int r = 128 * t + 32 * q + lane;
-      if (r < limit) {
+      if (r < HOP + 160) {
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
           __half2 h[4];
@@ -528,30 +534,43 @@ __global__ void __launch_bounds__(256, 1) propose_kernel(const ProposeParams p) 
           for (int e = 0; e < 4; ++e) {
             const int c = 8 * j + 2 * e;
             const float v0 = c < 16 ? a[cur][c] : b[cur][c - 16], v1 = c + 1 < 16 ? a[cur][c + 1] : b[cur][c - 15];
-            h[e] = __floats2half2_rn(fmaxf(v0 + bias[c], 0.f), fmaxf(v1 + bias[c + 1], 0.f));
+            h[e] = __floats2half2_rn(fmaxf(v0 + sBias[c], 0.f), fmaxf(v1 + sBias[c + 1], 0.f));
           }
-          *reinterpret_cast<uint4*>(dst + j * plane + r * 16) = *reinterpret_cast<uint4*>(h);
+          *reinterpret_cast<uint4*>(dst + j * kPlaneH1 + t * (32 * 16)) = *reinterpret_cast<uint4*>(h);
         }
       }
     });
   };
-  // one k = 9 convolution layer with dilation D: NT M-tiles, A rows start at 128t + kD in the
-  // source planes; tiles innermost, so consecutive MMAs feed independent accumulators.  A
+  // layer 2's accumulator (lanes = channel `lane` of phase q, columns P = 4a + b: position 16a + 4q + b)
+  // + bias -> relu -> FP16 rows of layer 3's input
+  auto store_h2 = [&]() {
+    float v[2][16];
+    tmem_ld16(tm_lane, v[0]);
+    const float bias = sBias[kC + lane];
+    unsigned char* dst = slot + (lane >> 3) * kPlaneH2 + (lane & 7) * 2 + 4 * q * 16;
+    static_for<N2 / 16>([&](auto cc) {
+      constexpr int c = decltype(cc)::value, cur = c & 1;
+      tmem_wait_ld();
+      if constexpr (c + 1 < N2 / 16) tmem_ld16(tm_lane + 16 * (c + 1), v[cur ^ 1]);
+#pragma unroll
+      for (int e = 0; e < 16; ++e)   // a = 4c + e/4: phase e/4, column 16c + 4q + e%4 of dilation 16
+        *reinterpret_cast<__half*>(dst + ((e >> 2) * kNP2 + 16 * c + (e & 3)) * 16) =
+            __float2half_rn(fmaxf(v[cur][e] + bias, 0.f));
+    });
+  };
+  // one k = 9 convolution layer with dilation D: 12 offsets x 2 halves of the input channels.  A
   // descriptor's start address is its low field, so every operand is a base descriptor plus a
   // constant.
-  auto issue_conv = [&](auto ntiles, auto dil, uint32_t src, uint32_t plane, uint32_t wts) {
-    constexpr int NT = decltype(ntiles)::value, D = decltype(dil)::value;
-    const uint64_t a0 = umma_desc(src, plane, 128), b0 = umma_desc(wts, 512, 128);
-    static_for<kK>([&](auto kk) {
-      constexpr int k = decltype(kk)::value;
+  auto issue_conv = [&](auto dil, auto cols, uint32_t wts, uint32_t plane, uint32_t rows_per_phase) {
+    constexpr int D = decltype(dil)::value, N = decltype(cols)::value;
+    const uint64_t a0 = umma_desc(wts, kPlaneW, 128), b0 = umma_desc(aSlot, plane, 128);
+    static_for<12>([&](auto oo) {
+      constexpr int o = decltype(oo)::value;
       static_for<2>([&](auto cc) {
         constexpr int c = decltype(cc)::value;
-        const uint64_t bd = b0 + (uint64_t)((k * 2048 + c * 1024) >> 4);
-        const uint64_t ac = a0 + (uint64_t)(((uint32_t)(k * D) * 16 + 2u * c * plane) >> 4);
-        static_for<NT>([&](auto tt) {
-          constexpr int t = decltype(tt)::value;
-          umma_f16(tm + 32 * t, ac + (uint64_t)(128 * t), bd, kIdesc, (k | c) != 0);
-        });
+        const uint64_t ad = a0 + (uint64_t)((2u * c * kPlaneW + (11 - o) * kC * 16) >> 4);
+        const uint64_t bd = b0 + (uint64_t)((2u * c * plane + ((o & 3) * rows_per_phase + D * (o >> 2)) * 16) >> 4);
+        umma_f16(tm, ad, bd, umma_idesc_f16(128, N), (o | c) != 0);
       });
     });
     umma_commit(bar);
@@ -576,51 +595,43 @@ __global__ void __launch_bounds__(256, 1) propose_kernel(const ProposeParams p) 
       for (int e = 0; e < 4; ++e) h[e] = __floats2half2_rn(sX[r + 2 * e], sX[r + 2 * e + 1]);
       h[4] = __floats2half2_rn(sX[r + 8], 0.f);
       h[5] = h[6] = h[7] = __floats2half2_rn(0.f, 0.f);
-      *reinterpret_cast<uint4*>(sA1 + r * 16) = *reinterpret_cast<uint4*>(&h[0]);
-      *reinterpret_cast<uint4*>(sA1 + kPlaneA1 + r * 16) = *reinterpret_cast<uint4*>(&h[4]);
+      *reinterpret_cast<uint4*>(slot + r * 16) = *reinterpret_cast<uint4*>(&h[0]);
+      *reinterpret_cast<uint4*>(slot + kPlaneA1 + r * 16) = *reinterpret_cast<uint4*>(&h[4]);
     }
     sync_for_mma();
     if (gt == 0) {
-      const uint64_t bd = umma_desc(aW1, 512, 128), a0 = umma_desc(aA1, kPlaneA1, 128);
+      const uint64_t bd = umma_desc(aW1, 512, 128), a0 = umma_desc(aSlot, kPlaneA1, 128);
       static_for<T1>([&](auto tt) {
         constexpr int t = decltype(tt)::value;
-        umma_f16(tm + 32 * t, a0 + (uint64_t)(128 * t), bd, kIdesc, 0u);   // 128 rows x 16 B = 2048 B
+        umma_f16(tm + 32 * t, a0 + (uint64_t)(128 * t), bd, kIdesc1, 0u);   // 128 rows x 16 B = 2048 B
       });
       umma_commit(bar);
     }
     if (!(ok = wait_mma())) break;
-    store_layer(std::integral_constant<int, T1>{}, 128 * T2 + 8 * kDil2, sBias, sH1, kPlaneH1);
+    store_h1();
     sync_for_mma();
-    if (gt == 0) issue_conv(std::integral_constant<int, T2>{}, std::integral_constant<int, kDil2>{}, aH1, kPlaneH1, aW2);
+    if (gt == 0)
+      issue_conv(std::integral_constant<int, kDil2>{}, std::integral_constant<int, N2>{}, aW2, kPlaneH1, kNP1);
     if (!(ok = wait_mma())) break;
-    store_layer(std::integral_constant<int, T2>{}, HOP + 8 * kDil3, sBias + kC, sH2, kPlaneH2);
+    store_h2();
     sync_for_mma();
-    if (gt == 0) issue_conv(std::integral_constant<int, T3>{}, std::integral_constant<int, kDil3>{}, aH2, kPlaneH2, aW3);
+    if (gt == 0)
+      issue_conv(std::integral_constant<int, kDil3>{}, std::integral_constant<int, N3>{}, aW3, kPlaneH2, kNP2);
     if (!(ok = wait_mma())) break;
-    // layer 3: relu(acc + b3), channel maxima over the block: each thread keeps the maximum of
-    // its rows, then one warp reduction per channel (non-negative floats order as unsigned)
+    // layer 3: relu(acc + b3), channel maxima over the block: this lane's channel at its warp's phase,
+    // then the four phases (adding the bias after the maximum changes nothing; non-negative floats
+    // order as unsigned)
     {
-      float mx[kC];
-#pragma unroll
-      for (int c = 0; c < kC; ++c) mx[c] = 0.f;
-      float a[2][16], b[2][16];
-      tmem_ld16(tm_lane, a[0]);
-      tmem_ld16(tm_lane + 16, b[0]);
-      static_for<T3>([&](auto tt) {
-        constexpr int t = decltype(tt)::value, cur = t & 1;
+      float mx = -INFINITY, v[2][16];
+      tmem_ld16(tm_lane, v[0]);
+      static_for<N3 / 16>([&](auto cc) {
+        constexpr int c = decltype(cc)::value, cur = c & 1;
         tmem_wait_ld();
-        if constexpr (t + 1 < T3) {
-          tmem_ld16(tm_lane + 32 * (t + 1), a[cur ^ 1]);
-          tmem_ld16(tm_lane + 32 * (t + 1) + 16, b[cur ^ 1]);
-        }
+        if constexpr (c + 1 < N3 / 16) tmem_ld16(tm_lane + 16 * (c + 1), v[cur ^ 1]);
 #pragma unroll
-        for (int c = 0; c < kC; ++c) mx[c] = fmaxf(mx[c], (c < 16 ? a[cur][c] : b[cur][c - 16]) + sBias[2 * kC + c]);
+        for (int e = 0; e < 16; ++e) mx = fmaxf(mx, v[cur][e]);
       });
-#pragma unroll
-      for (int c = 0; c < kC; ++c) {
-        const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(fmaxf(mx[c], 0.f)));
-        if (lane == c) atomicMax(&sMax[c], m);
-      }
+      atomicMax(&sMax[lane], __float_as_uint(fmaxf(mx + sBias[2 * kC + lane], 0.f)));
     }
     tmem_fence_before_sync();
     group_sync(g);
