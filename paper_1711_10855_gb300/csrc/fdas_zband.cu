@@ -41,58 +41,91 @@ constexpr int kDil1 = 1, kDil2 = 4, kDil3 = 16;    // layer dilations
 constexpr int kRF = kPad * (kDil1 + kDil2 + kDil3);   // receptive field of a layer-3 position
 
 constexpr float kXCap = 64.f;   // input cap: x_r = min(|A_r|^2 ln 2 / median |A|^2, 64)
-constexpr int kSelBlocks = 2048; // grid cap of the median's first pass
-constexpr int kSelBlocks12 = 304; // and of its second and third (2 blocks per SM of a GB300)
+constexpr int kSelBlocks0 = 456;   // grid caps of the median's passes: 3 blocks of the first fit an SM of a GB300,
+constexpr int kSelBlocks = 608;    // and the later ones flush up to 4096 bins per block
 
 // Exact lower median of |A_r|^2 (rank (n-1)/2) by radix selection on the FP32 bit patterns
-// (non-negative floats order as unsigned integers): three passes over the spectrum histogram the
-// top 8 bits (sign and exponent: most values share a few bins, so each warp counts into its own
-// copy), then the next 12 bits of the values matching the digit found so far, then the last 12;
-// after each pass one block finds the digit holding the rank (a block scan of the histogram).
-// scale = ln 2 / median.
-constexpr int kSelBins0 = 256, kSelBins = 4096;
+// (non-negative floats order as unsigned integers; the sign bit is 0): three passes over the spectrum
+// histogram 8 bits (the exponent: most values share a few bins, so each thread counts into bytes of
+// its own), then 12 bits of the values that match the digit found so far, then the last 11.  The block of a pass that finishes last
+// finds the digit holding the rank; the last pass leaves scale = ln 2 / median.  The state is cleared
+// before the first pass.
+constexpr int kSelBins0 = 256, kSelBins1 = 4096, kSelBins2 = 2048;
 constexpr int kSelPer = 8;   // complex values per thread and pass iteration (four 16-byte loads)
 struct SelectState {
   long long k;                 // rank of the median among the values matching `prefix`
-  unsigned prefix, mask;       // bits fixed so far and their mask
-  unsigned hist0[kSelBins0];   // bits 31..24
-  unsigned hist1[kSelBins];    // bits 23..12 of the values matching digit 0
-  unsigned hist2[kSelBins];    // bits 11..0 of the values matching digits 0 and 1
+  unsigned prefix, done;       // bits fixed so far; blocks of the current pass that have finished
+  unsigned hist0[kSelBins0];   // bits 30..23
+  unsigned hist1[kSelBins1];   // bits 22..11 of the values matching digit 0
+  unsigned hist2[kSelBins2];   // bits 10..0 of the values matching digits 0 and 1
 };
 
 __device__ __forceinline__ float power_of(const float2 a) { return fmaf(a.x, a.x, a.y * a.y); }
 
-// PASS 0: top 8 bits of every value (one histogram per warp, summed at the end); PASS 1, 2: the
-// next 12 bits of the values whose higher bits equal st->prefix.  Values are read in 16-byte pairs from the first 16-byte boundary (an
-// 8-byte aligned spectrum's first value is counted on its own); the tail element by element.
+// PASS 0: bits 30..23 of every value, one byte per thread and bin (the four warps w, w + 1, ... of a
+// 128-byte row of lanes use one byte of each word: no conflicts, no atomics), summed per block before a
+// byte can overflow; PASS 1, 2: the next bits of the values whose higher bits equal st->prefix, by
+// shared atomics.  Values are read in 16-byte pairs from the first 16-byte boundary (an 8-byte aligned
+// spectrum's first value is counted on its own); the tail element by element.
 template <int PASS>
-__global__ void __launch_bounds__(256) select_pass_kernel(const float2* spec, int64_t n, SelectState* st) {
-  constexpr int NB = PASS == 0 ? kSelBins0 : kSelBins;
-  constexpr int SHIFT = PASS == 0 ? 24 : (PASS == 1 ? 12 : 0);
-  constexpr int COPIES = PASS == 0 ? 8 : 1;   // per-warp histograms in pass 0
-  __shared__ unsigned h[COPIES * NB];
-  for (int i = threadIdx.x; i < COPIES * NB; i += 256) h[i] = 0u;
-  const unsigned prefix = PASS == 0 ? 0u : st->prefix, mask = PASS == 0 ? 0u : st->mask;
+__host__ __device__ constexpr size_t select_smem() {
+  return PASS == 0 ? 256 * kSelBins0 : sizeof(unsigned) * (PASS == 1 ? kSelBins1 : kSelBins2);
+}
+
+template <int PASS>
+__global__ void __launch_bounds__(256) select_pass_kernel(const float2* spec, int64_t n, SelectState* st,
+                                                          float* scale) {
+  constexpr int NB = PASS == 0 ? kSelBins0 : (PASS == 1 ? kSelBins1 : kSelBins2);
+  constexpr int SHIFT = PASS == 0 ? 23 : (PASS == 1 ? 11 : 0);
+  constexpr unsigned MASK = PASS == 0 ? 0u : (PASS == 1 ? 0xFF800000u : 0xFFFFF800u);
+  extern __shared__ __align__(16) unsigned char sel_smem[];
+  unsigned* h = reinterpret_cast<unsigned*>(sel_smem);
+  __shared__ bool last;
+  const int64_t total = n;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  unsigned char* mine = sel_smem + (warp >> 2) * 128 + lane * 4 + (warp & 3);   // + 256 * bin
+  for (int i = threadIdx.x; i < (int)(select_smem<PASS>() / 16); i += 256)
+    reinterpret_cast<uint4*>(sel_smem)[i] = make_uint4(0u, 0u, 0u, 0u);
+  const unsigned prefix = PASS == 0 ? 0u : st->prefix;
+  unsigned* hist = PASS == 0 ? st->hist0 : (PASS == 1 ? st->hist1 : st->hist2);
   __syncthreads();
-  const int lane = threadIdx.x & 31;
-  unsigned* hw = h + (COPIES > 1 ? (threadIdx.x >> 5) * NB : 0);
   auto count = [&](float2 a, bool valid) {
-    unsigned bucket = 0xFFFFFFFFu;
-    if (valid) {
-      const unsigned bits = __float_as_uint(power_of(a));
-      if ((bits & mask) == prefix) bucket = (bits >> SHIFT) & (unsigned)(NB - 1);
+    const unsigned bits = __float_as_uint(power_of(a)) & 0x7FFFFFFFu;
+    const unsigned bucket = (bits >> SHIFT) & (unsigned)(NB - 1);
+    if constexpr (PASS == 0) {
+      if (valid) mine[256 * bucket] = (unsigned char)(mine[256 * bucket] + 1);
+    } else {
+      if (valid && (bits & MASK) == prefix) atomicAdd(&h[bucket], 1u);
     }
-    // one shared atomic per distinct bucket of the warp
-    const unsigned peers = __match_any_sync(0xffffffffu, bucket);
-    if (bucket != 0xFFFFFFFFu && lane == __ffs(peers) - 1) atomicAdd(&hw[bucket], (unsigned)__popc(peers));
+  };
+  // PASS 0: the block's bytes of bin threadIdx.x added to the histogram and cleared (between barriers);
+  // threads start at different words of their rows
+  auto flush_bytes = [&]() {
+    __syncthreads();
+    unsigned c = 0u;
+    unsigned* row = h + 64 * threadIdx.x;
+    for (int i = 0; i < 64; ++i) {
+      const unsigned w = row[(i + lane) & 63];
+      row[(i + lane) & 63] = 0u;
+      c += (w & 0xFFu) + ((w >> 8) & 0xFFu) + ((w >> 16) & 0xFFu) + (w >> 24);
+    }
+    if (c) atomicAdd(&hist[threadIdx.x], c);
+    __syncthreads();
   };
   const int off = (reinterpret_cast<uintptr_t>(spec) & 15u) ? 1 : 0;
-  if (off && blockIdx.x == 0 && threadIdx.x < 32)
-    count(threadIdx.x == 0 ? __ldg(spec) : make_float2(0.f, 0.f), threadIdx.x == 0 && n > 0);
+  if (off && blockIdx.x == 0 && threadIdx.x == 0 && n > 0) count(__ldg(spec), true);
   spec += off;
   n -= off;
   const int64_t step = (int64_t)gridDim.x * 256 * kSelPer;
+  int held = 0;   // PASS 0: values counted since the last flush, per thread
   for (int64_t base = (int64_t)blockIdx.x * 256 * kSelPer; base < n; base += step) {
+    if constexpr (PASS == 0) {
+      if (held + kSelPer + 1 > 255) {   // uniform over the block
+        flush_bytes();
+        held = 0;
+      }
+      held += kSelPer;
+    }
     // thread t reads the pairs (base + 2(t + 256 j), +1), j < kSelPer / 2: coalesced 16-byte loads
     float4 v[kSelPer / 2];
 #pragma unroll
@@ -108,45 +141,43 @@ __global__ void __launch_bounds__(256) select_pass_kernel(const float2* spec, in
       count(make_float2(v[j].z, v[j].w), r + 1 < n);
     }
   }
-  __syncthreads();
-  unsigned* out = PASS == 0 ? st->hist0 : (PASS == 1 ? st->hist1 : st->hist2);
-  for (int i = threadIdx.x; i < NB; i += 256) {
-    unsigned c = 0u;
-#pragma unroll
-    for (int w = 0; w < COPIES; ++w) c += h[w * NB + i];
-    if (c) atomicAdd(&out[i], c);
+  if constexpr (PASS == 0) {
+    flush_bytes();
+  } else {
+    __syncthreads();
+    for (int i = threadIdx.x; i < NB; i += 256)
+      if (h[i]) atomicAdd(&hist[i], h[i]);
   }
-}
-
-// One block of 256 threads: the digit of histogram PASS holding rank st->k (thread t owns the
-// bins [t*NB/256, (t+1)*NB/256); a block scan of their sums leaves exactly one thread whose range
-// holds the rank), appended to st->prefix; after the last digit, scale = ln 2 / median.
-template <int PASS>
-__global__ void __launch_bounds__(256) select_digit_kernel(SelectState* st, float* scale) {
-  constexpr int NB = PASS == 0 ? kSelBins0 : kSelBins;
-  constexpr int SHIFT = PASS == 0 ? 24 : (PASS == 1 ? 12 : 0);
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(&st->done, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  // The last block: the digit of the histogram that holds rank st->k (thread t owns NB/256 bins; a block
+  // scan of their sums leaves exactly one thread whose range holds the rank), appended to st->prefix.
+  __threadfence();
   constexpr int per = NB / 256;
   __shared__ long long wsum[8];
-  const unsigned* hist = PASS == 0 ? st->hist0 : (PASS == 1 ? st->hist1 : st->hist2);
-  const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+  const int t = threadIdx.x, wid = t >> 5;
   unsigned c[per];
   long long own = 0;
 #pragma unroll
   for (int i = 0; i < per; ++i) {
-    c[i] = hist[t * per + i];
+    c[i] = __ldcg(&hist[t * per + i]);
     own += c[i];
   }
   long long inc = own;
 #pragma unroll
-  for (int off = 1; off < 32; off <<= 1) {
-    const long long y = __shfl_up_sync(0xffffffffu, inc, off);
-    if (lane >= off) inc += y;
+  for (int o = 1; o < 32; o <<= 1) {
+    const long long y = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += y;
   }
   if (lane == 31) wsum[wid] = inc;
   __syncthreads();
   long long excl = inc - own;
   for (int i = 0; i < wid; ++i) excl += wsum[i];
-  const long long k = st->k;
+  const long long k = PASS == 0 ? (total - 1) / 2 : st->k;
+  __syncthreads();   // st->k is read by every thread before one of them replaces it
   if (k >= excl && k < excl + own) {
     long long r = k - excl;
     int d = t * per;
@@ -156,28 +187,15 @@ __global__ void __launch_bounds__(256) select_digit_kernel(SelectState* st, floa
         r -= c[i];
         ++d;
       }
-    const unsigned prefix = (PASS == 0 ? 0u : st->prefix) | ((unsigned)d << SHIFT);
+    const unsigned found = prefix | ((unsigned)d << SHIFT);
     st->k = r;
-    st->prefix = prefix;
-    st->mask = PASS == 0 ? 0xFF000000u : (PASS == 1 ? 0xFFFFF000u : 0xFFFFFFFFu);
+    st->prefix = found;
     if (PASS == 2) {
-      const float med = __uint_as_float(prefix);
+      const float med = __uint_as_float(found);
       *scale = med > 0.f ? 0.69314718055994531f / med : 0.f;
     }
   }
-}
-
-__global__ void __launch_bounds__(256) select_init_kernel(SelectState* st, int64_t n) {
-  if (threadIdx.x == 0) {
-    st->k = (n - 1) / 2;
-    st->prefix = 0u;
-    st->mask = 0u;
-  }
-  for (int i = threadIdx.x; i < kSelBins0; i += 256) st->hist0[i] = 0u;
-  for (int i = threadIdx.x; i < kSelBins; i += 256) {
-    st->hist1[i] = 0u;
-    st->hist2[i] = 0u;
-  }
+  if (t == 0) st->done = 0u;
 }
 
 __device__ __forceinline__ float power_x(const float2* spec, int64_t n, int64_t r, float scale) {
@@ -337,7 +355,7 @@ __global__ void __launch_bounds__(256) write_units_kernel(const uint16_t* masks,
 // ---------------------------------------------------------------------------------------
 // Fused inference over a whole spectrum on the tensor cores (tcgen05.mma kind::f16: FP16
 // weights and activations, FP32 accumulation in TMEM).  A CTA holds the weights once and runs
-// two independent groups of 4 warps, each with its own activation slot, half of the TMEM
+// two independent groups of 8 warps, each with its own activation slot, half of the TMEM
 // allocation, mbarrier and named barriers, so one group's MMAs overlap the other's epilogues.
 // Group g of CTA b walks blocks w = 2b + g, 2b + g + 2*gridDim.x, ...; block w owns output
 // positions [w*hop, (w+1)*hop) and recomputes the +-84-position halo its three layers need
@@ -354,11 +372,13 @@ __global__ void __launch_bounds__(256) write_units_kernel(const uint16_t* masks,
 // weight rows are kept once, as the stack [0 0 0 W_8 ... W_0 0 0 0]: offset o starts at its block 11 - o.
 // N is (hop + 128)/4 and hop/4 columns instead of 32 channels, where an MMA's time no longer has
 // its floor of about 50 cycles: 24 MMAs of 80 and 64 cycles per layer for 512 positions, against 90
-// and 72 of 64 cycles with one tap, 128 positions and N = 32 each (kernel 330 to 225 us at 2^22
+// and 72 of 64 cycles with one tap, 128 positions and N = 32 each (kernel 330 to 200 us at 2^22
 // bins).  The zero blocks are a quarter of the multiply-adds.
 // Activations sit in shared memory K-major "chunk-planar": channel chunk j (8 channels, 16 B) of row q at
 // plane j, offset 16*q, rows ordered (phase, column) for the layer that reads them.  h2 overwrites
-// h1, and h1 the layer-1 im2col, each after the MMAs that read them.
+// h1 after the MMAs that read it.  While a group's layer-2 MMAs run it does the previous block's head, and
+// during layer 3 the next block's staging and im2col; what is left between MMAs is the conversion of the
+// two activation layers.
 // ---------------------------------------------------------------------------------------
 constexpr int kMaxHop = 512;
 constexpr int kT1max = kMaxHop / 128 + 2;       // layer-1 M-tiles
@@ -366,7 +386,8 @@ constexpr int kNP1 = (kMaxHop + 160) / 4 + 4;   // h1 rows per phase (+4: a quar
 constexpr int kNP2 = (kMaxHop + 128) / 4;       // h2 rows per phase
 constexpr int kNA1 = 128 * kT1max;              // im2col rows of layer 1
 constexpr int kNX = kNA1 + 8;                   // staged x values
-constexpr int kGroupThreads = 128;
+constexpr int kGroupThreads = 256;             // two warps per TMEM quadrant share its columns
+constexpr int kProposeThreads = 2 * kGroupThreads;
 constexpr int kXPer = (kNX + kGroupThreads - 1) / kGroupThreads;   // prefetched x per thread
 constexpr int kZStage = 256;                    // head weights staged in shared memory up to this Z
 constexpr uint32_t kPlaneH1 = 4 * kNP1 * 16, kPlaneA1 = kNA1 * 16;
@@ -380,16 +401,17 @@ constexpr int kOffWl = kOffW3 + 4 * kPlaneW;    // head weights [Z][32] FP16
 constexpr int kOffBl = kOffWl + kZStage * kC * 2;
 constexpr int kOffBias = kOffBl + kZStage * 4;  // b1, b2, b3 (FP32 values of the FP16 copy)
 constexpr int kOffSlot = (kOffBias + 3 * kC * 4 + 127) / 128 * 128;   // two activation slots
-constexpr int kSlotX = 4 * kPlaneH1;            // staged x behind the planes
+constexpr int kSlotA1 = 4 * kPlaneH1;           // layer-1 im2col of the next block
+constexpr int kSlotX = kSlotA1 + 2 * kPlaneA1;  // staged x
 constexpr int kSlotBytes = (kSlotX + kNX * 4 + 127) / 128 * 128;
 constexpr int kOffGroup = kOffSlot + 2 * kSlotBytes;   // per group: channel maxima, mbarrier
-constexpr int kGroupMisc = 256;
+constexpr int kGroupMisc = 384;
 constexpr int kOffTslot = kOffGroup + 2 * kGroupMisc;
 constexpr int kProposeSmem = kOffTslot + 16;
 constexpr uint32_t kIdesc1 = fdas::umma_idesc_f16(128, kC);
 constexpr uint32_t kTmemCols = 512;             // 256 columns per group (<= 6 x 32 used)
 static_assert(kDil1 == 1, "layer 1 is an im2col of adjacent x values");
-static_assert(kPlaneH2 <= kPlaneH1 && 2 * kPlaneA1 <= 4 * kPlaneH1, "h2 and the im2col fit in the h1 planes");
+static_assert(kPlaneH2 <= kPlaneH1, "h2 fits in the h1 planes");
 static_assert(32 * kT1max <= (int)kTmemCols / 2 && kNP2 <= (int)kTmemCols / 2, "a group's TMEM half");
 static_assert(kProposeSmem <= 227 * 1024, "shared memory");
 
@@ -408,21 +430,23 @@ struct ProposeParams {
 // B operand (layer-1 weights) in the K-major no-swizzle layout: rows o (N = 32), K = tap.
 __device__ __forceinline__ int wb_off(int o, int i) { return (i >> 3) * 512 + (o >> 3) * 128 + (o & 7) * 16 + (i & 7) * 2; }
 
-// Named barrier of one 128-thread group (ids 1, 2; id 0 is __syncthreads).
-__device__ __forceinline__ void group_sync(int g) { asm volatile("bar.sync %0, 128;" ::"r"(g + 1) : "memory"); }
+// Named barrier of one group (ids 1, 2; id 0 is __syncthreads).
+__device__ __forceinline__ void group_sync(int g) {
+  asm volatile("bar.sync %0, %1;" ::"r"(g + 1), "n"(kGroupThreads) : "memory");
+}
 __device__ __forceinline__ int group_all(int g, int v) {
   int r;
   asm volatile(
-      "{\n\t.reg .pred p, q;\n\tsetp.ne.s32 p, %1, 0;\n\tbar.red.and.pred q, %2, 128, p;\n\t"
+      "{\n\t.reg .pred p, q;\n\tsetp.ne.s32 p, %1, 0;\n\tbar.red.and.pred q, %2, %3, p;\n\t"
       "selp.s32 %0, 1, 0, q;\n\t}"
       : "=r"(r)
-      : "r"(v), "r"(g + 1)
+      : "r"(v), "r"(g + 1), "n"(kGroupThreads)
       : "memory");
   return r;
 }
 
 template <int HOP>
-__global__ void __launch_bounds__(256, 1) propose_kernel(const ProposeParams p) {
+__global__ void __launch_bounds__(kProposeThreads, 1) propose_kernel(const ProposeParams p) {
   static_assert(HOP % 128 == 0 && HOP <= kMaxHop, "hop");
   using namespace fdas;
   extern __shared__ __align__(1024) unsigned char sm[];
@@ -433,19 +457,19 @@ __global__ void __launch_bounds__(256, 1) propose_kernel(const ProposeParams p) 
   uint32_t* tslot = reinterpret_cast<uint32_t*>(sm + kOffTslot);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int g = warp >> 2, q = warp & 3, gt = tid & (kGroupThreads - 1);
+  const int g = warp >> 3, q = warp & 3, half = (warp >> 2) & 1, gt = tid & (kGroupThreads - 1);
   unsigned char* slot = sm + kOffSlot + g * kSlotBytes;
   float* sX = reinterpret_cast<float*>(slot + kSlotX);
-  unsigned* sMax = reinterpret_cast<unsigned*>(sm + kOffGroup + g * kGroupMisc);
-  uint64_t* bar = reinterpret_cast<uint64_t*>(sm + kOffGroup + g * kGroupMisc + 128);
+  unsigned* sMax = reinterpret_cast<unsigned*>(sm + kOffGroup + g * kGroupMisc);   // two blocks' channel maxima
+  uint64_t* bar = reinterpret_cast<uint64_t*>(sm + kOffGroup + g * kGroupMisc + 256);
   const bool wl_staged = p.Z <= kZStage;
 
   // weights into the B layouts (FP16) and the head; biases as FP32 values of the FP16 copy
-  for (int idx = tid; idx < kC * 16; idx += 256) {
+  for (int idx = tid; idx < kC * 16; idx += kProposeThreads) {
     const int o = idx >> 4, k = idx & 15;
     sW1[wb_off(o, k) / 2] = k < kK ? p.w[p.oW1 + o * kK + k] : __float2half_rn(0.f);
   }
-  for (int idx = tid; idx < 2 * 4 * kStackRows; idx += 256) {   // 8 input channels of a stack row at a time
+  for (int idx = tid; idx < 2 * 4 * kStackRows; idx += kProposeThreads) {   // 8 input channels of a stack row at a time
     const int layer = idx / (4 * kStackRows), j = idx / kStackRows % 4, row = idx % kStackRows;
     const int k = 11 - row / kC, o = row % kC;
     __half h[8];
@@ -455,8 +479,8 @@ __global__ void __launch_bounds__(256, 1) propose_kernel(const ProposeParams p) 
     *reinterpret_cast<uint4*>(sm + (layer ? kOffW3 : kOffW2) + j * kPlaneW + row * 16) = *reinterpret_cast<uint4*>(h);
   }
   if (wl_staged) {
-    for (int idx = tid; idx < p.Z * kC; idx += 256) sWl[idx] = p.w[p.oWl + idx];
-    for (int j = tid; j < p.Z; j += 256) sBl[j] = __half2float(p.w[p.obl + j]);
+    for (int idx = tid; idx < p.Z * kC; idx += kProposeThreads) sWl[idx] = p.w[p.oWl + idx];
+    for (int j = tid; j < p.Z; j += kProposeThreads) sBl[j] = __half2float(p.w[p.obl + j]);
   }
   if (tid < kC) {
     sBias[tid] = __half2float(p.w[p.ob1 + tid]);
@@ -509,34 +533,38 @@ __global__ void __launch_bounds__(256, 1) propose_kernel(const ProposeParams p) 
     group_sync(g);
     tmem_fence_after_sync();
   };
+  const __half2 zero2 = __floats2half2_rn(0.f, 0.f);
   // layer 1's accumulator tiles (lanes = positions r = 128t + 32q + lane, columns = channels) + bias -> relu
   // -> FP16 rows of layer 2's input, r < HOP + 160.  The next tile's TMEM load is issued before this
   // tile is converted (tcgen05.wait::ld waits for every earlier load, so the wait comes first and the two
   // buffers alternate).
   auto store_h1 = [&]() {
     float a[2][16], b[2][16];
-    tmem_ld16(tm_lane, a[0]);
-    tmem_ld16(tm_lane + 16, b[0]);
-    unsigned char* dst = slot + (((lane >> 2) & 3) * kNP1 + 8 * q + 4 * (lane >> 4) + (lane & 3)) * 16;
-    static_for<T1>([&](auto tt) {
+    const uint32_t src = tm_lane + 32 * half;   // this warp's tiles: half, half + 2, ...
+    tmem_ld16(src, a[0]);
+    tmem_ld16(src + 16, b[0]);
+    unsigned char* dst =
+        slot + (32 * half + ((lane >> 2) & 3) * kNP1 + 8 * q + 4 * (lane >> 4) + (lane & 3)) * 16;
+    constexpr int NT = (T1 + 1) / 2;
+    static_for<NT>([&](auto tt) {
       constexpr int t = decltype(tt)::value, cur = t & 1;
       tmem_wait_ld();
-      if constexpr (t + 1 < T1) {
-        tmem_ld16(tm_lane + 32 * (t + 1), a[cur ^ 1]);
-        tmem_ld16(tm_lane + 32 * (t + 1) + 16, b[cur ^ 1]);
+      if constexpr (t + 1 < NT) {
+        tmem_ld16(src + 64 * (t + 1), a[cur ^ 1]);
+        tmem_ld16(src + 64 * (t + 1) + 16, b[cur ^ 1]);
       }
-      const int r = 128 * t + 32 * q + lane;
+      const int r = 128 * (2 * t + half) + 32 * q + lane;
       if (r < HOP + 160) {
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
           __half2 h[4];
 #pragma unroll
-          for (int e = 0; e < 4; ++e) {
+          for (int e = 0; e < 4; ++e) {   // rounding is monotonic: relu after it is the same
             const int c = 8 * j + 2 * e;
-            const float v0 = c < 16 ? a[cur][c] : b[cur][c - 16], v1 = c + 1 < 16 ? a[cur][c + 1] : b[cur][c - 15];
-            h[e] = __floats2half2_rn(fmaxf(v0 + sBias[c], 0.f), fmaxf(v1 + sBias[c + 1], 0.f));
+            const float2 v = c < 16 ? make_float2(a[cur][c], a[cur][c + 1]) : make_float2(b[cur][c - 16], b[cur][c - 15]);
+            h[e] = __hmax2(__float22half2_rn(add2(v, *reinterpret_cast<const float2*>(sBias + c))), zero2);
           }
-          *reinterpret_cast<uint4*>(dst + j * kPlaneH1 + t * (32 * 16)) = *reinterpret_cast<uint4*>(h);
+          *reinterpret_cast<uint4*>(dst + j * kPlaneH1 + t * (64 * 16)) = *reinterpret_cast<uint4*>(h);
         }
       }
     });
@@ -545,17 +573,22 @@ __global__ void __launch_bounds__(256, 1) propose_kernel(const ProposeParams p) 
   // + bias -> relu -> FP16 rows of layer 3's input
   auto store_h2 = [&]() {
     float v[2][16];
-    tmem_ld16(tm_lane, v[0]);
-    const float bias = sBias[kC + lane];
-    unsigned char* dst = slot + (lane >> 3) * kPlaneH2 + (lane & 7) * 2 + 4 * q * 16;
-    static_for<N2 / 16>([&](auto cc) {
+    const uint32_t src = tm_lane + 16 * half;   // this warp's column chunks c' = 2c + half
+    tmem_ld16(src, v[0]);
+    const float2 bias = bc(sBias[kC + lane]);
+    unsigned char* dst = slot + (lane >> 3) * kPlaneH2 + (lane & 7) * 2 + (16 * half + 4 * q) * 16;
+    static_assert(N2 % 32 == 0, "two warps share the columns");
+    static_for<N2 / 32>([&](auto cc) {
       constexpr int c = decltype(cc)::value, cur = c & 1;
       tmem_wait_ld();
-      if constexpr (c + 1 < N2 / 16) tmem_ld16(tm_lane + 16 * (c + 1), v[cur ^ 1]);
+      if constexpr (c + 1 < N2 / 32) tmem_ld16(src + 32 * (c + 1), v[cur ^ 1]);
 #pragma unroll
-      for (int e = 0; e < 16; ++e)   // a = 4c + e/4: phase e/4, column 16c + 4q + e%4 of dilation 16
-        *reinterpret_cast<__half*>(dst + ((e >> 2) * kNP2 + 16 * c + (e & 3)) * 16) =
-            __float2half_rn(fmaxf(v[cur][e] + bias, 0.f));
+      for (int e = 0; e < 16; e += 2) {   // a = 4c' + e/4: phase e/4, column 16c' + 4q + e%4 of dilation 16
+        const __half2 h = __hmax2(__float22half2_rn(add2(make_float2(v[cur][e], v[cur][e + 1]), bias)), zero2);
+        unsigned char* at = dst + ((e >> 2) * kNP2 + 32 * c + (e & 3)) * 16;
+        *reinterpret_cast<__half*>(at) = __low2half(h);
+        *reinterpret_cast<__half*>(at + 16) = __high2half(h);
+      }
     });
   };
   // one k = 9 convolution layer with dilation D: 12 offsets x 2 halves of the input channels.  A
@@ -576,69 +609,31 @@ __global__ void __launch_bounds__(256, 1) propose_kernel(const ProposeParams p) 
     umma_commit(bar);
   };
 
-  const int64_t wstep = 2 * (int64_t)gridDim.x;
-  int64_t w = 2 * (int64_t)blockIdx.x + g;
-  if (w < p.n_blocks) load_x(w * HOP);
-  for (; w < p.n_blocks; w += wstep) {
+  // x of the block in registers -> layer-1 im2col: row r (position P0-80+r) = x[r .. r+8], zero for K in [9, 16)
+  unsigned char* sA1 = slot + kSlotA1;
+  auto stage_x = [&]() {
 #pragma unroll
     for (int e = 0; e < kXPer; ++e) {
       const int j = gt + kGroupThreads * e;
       if (j < nx) sX[j] = fminf(power_of(xa[e]) * sc, kXCap);
     }
-    if (gt < kC) sMax[gt] = 0u;
-    group_sync(g);
-    if (w + wstep < p.n_blocks) load_x((w + wstep) * HOP);   // next block, used next iteration
-    // layer-1 im2col: row r (position P0-80+r) = x[r .. r+8], zero for K in [9, 16)
+  };
+  auto im2col = [&]() {
     for (int r = gt; r < 128 * T1; r += kGroupThreads) {
       __half2 h[8];
 #pragma unroll
       for (int e = 0; e < 4; ++e) h[e] = __floats2half2_rn(sX[r + 2 * e], sX[r + 2 * e + 1]);
       h[4] = __floats2half2_rn(sX[r + 8], 0.f);
-      h[5] = h[6] = h[7] = __floats2half2_rn(0.f, 0.f);
-      *reinterpret_cast<uint4*>(slot + r * 16) = *reinterpret_cast<uint4*>(&h[0]);
-      *reinterpret_cast<uint4*>(slot + kPlaneA1 + r * 16) = *reinterpret_cast<uint4*>(&h[4]);
+      h[5] = h[6] = h[7] = zero2;
+      *reinterpret_cast<uint4*>(sA1 + r * 16) = *reinterpret_cast<uint4*>(&h[0]);
+      *reinterpret_cast<uint4*>(sA1 + kPlaneA1 + r * 16) = *reinterpret_cast<uint4*>(&h[4]);
     }
-    sync_for_mma();
-    if (gt == 0) {
-      const uint64_t bd = umma_desc(aW1, 512, 128), a0 = umma_desc(aSlot, kPlaneA1, 128);
-      static_for<T1>([&](auto tt) {
-        constexpr int t = decltype(tt)::value;
-        umma_f16(tm + 32 * t, a0 + (uint64_t)(128 * t), bd, kIdesc1, 0u);   // 128 rows x 16 B = 2048 B
-      });
-      umma_commit(bar);
-    }
-    if (!(ok = wait_mma())) break;
-    store_h1();
-    sync_for_mma();
-    if (gt == 0)
-      issue_conv(std::integral_constant<int, kDil2>{}, std::integral_constant<int, N2>{}, aW2, kPlaneH1, kNP1);
-    if (!(ok = wait_mma())) break;
-    store_h2();
-    sync_for_mma();
-    if (gt == 0)
-      issue_conv(std::integral_constant<int, kDil3>{}, std::integral_constant<int, N3>{}, aW3, kPlaneH2, kNP2);
-    if (!(ok = wait_mma())) break;
-    // layer 3: relu(acc + b3), channel maxima over the block: this lane's channel at its warp's phase,
-    // then the four phases (adding the bias after the maximum changes nothing; non-negative floats
-    // order as unsigned)
-    {
-      float mx = -INFINITY, v[2][16];
-      tmem_ld16(tm_lane, v[0]);
-      static_for<N3 / 16>([&](auto cc) {
-        constexpr int c = decltype(cc)::value, cur = c & 1;
-        tmem_wait_ld();
-        if constexpr (c + 1 < N3 / 16) tmem_ld16(tm_lane + 16 * (c + 1), v[cur ^ 1]);
-#pragma unroll
-        for (int e = 0; e < 16; ++e) mx = fmaxf(mx, v[cur][e]);
-      });
-      atomicMax(&sMax[lane], __float_as_uint(fmaxf(mx + sBias[2 * kC + lane], 0.f)));
-    }
-    tmem_fence_before_sync();
-    group_sync(g);
-    // head: logits[w][j] = bl[j] + sum_c Wl[j][c] m[c]  (FP16 weights, FP32 sums)
+  };
+  // logits[w][j] = bl[j] + sum_c Wl[j][c] m[c]  (FP16 weights, FP32 sums)
+  auto head = [&](int64_t w, const unsigned* smax) {
     float mc[kC];
 #pragma unroll
-    for (int c = 0; c < kC; ++c) mc[c] = __uint_as_float(sMax[c]);
+    for (int c = 0; c < kC; ++c) mc[c] = __uint_as_float(smax[c]);
     for (int j = gt; j < p.Z; j += kGroupThreads) {
       const __half* wl = wl_staged ? sWl + j * kC : p.w + p.oWl + (size_t)j * kC;
       float s = wl_staged ? sBl[j] : __half2float(p.w[p.obl + j]);
@@ -655,7 +650,75 @@ __global__ void __launch_bounds__(256, 1) propose_kernel(const ProposeParams p) 
       }
       p.logits[w * p.Z + j] = s;
     }
-    group_sync(g);   // sMax and the staging area are reused by the next block
+  };
+
+  const int64_t wstep = 2 * (int64_t)gridDim.x;
+  int64_t w = 2 * (int64_t)blockIdx.x + g, w_prev = -1;
+  unsigned* max_cur = sMax;           // this block's maxima (zero when its layer 3 is read)
+  unsigned* max_prev = sMax + kC;     // the previous block's
+  if (w < p.n_blocks) {
+    load_x(w * HOP);
+    stage_x();
+    if (gt < kC) max_cur[gt] = 0u;
+    group_sync(g);
+    if (w + wstep < p.n_blocks) load_x((w + wstep) * HOP);
+    im2col();
+  }
+  for (; w < p.n_blocks; w += wstep) {
+    sync_for_mma();
+    if (gt == 0) {
+      const uint64_t bd = umma_desc(aW1, 512, 128), a0 = umma_desc(aSlot + kSlotA1, kPlaneA1, 128);
+      static_for<T1>([&](auto tt) {
+        constexpr int t = decltype(tt)::value;
+        umma_f16(tm + 32 * t, a0 + (uint64_t)(128 * t), bd, kIdesc1, 0u);   // 128 rows x 16 B = 2048 B
+      });
+      umma_commit(bar);
+    }
+    if (!(ok = wait_mma())) break;
+    store_h1();
+    sync_for_mma();
+    if (gt == 0)
+      issue_conv(std::integral_constant<int, kDil2>{}, std::integral_constant<int, N2>{}, aW2, kPlaneH1, kNP1);
+    if (w_prev >= 0) head(w_prev, max_prev);
+    if (!(ok = wait_mma())) break;
+    store_h2();
+    sync_for_mma();
+    if (gt == 0)
+      issue_conv(std::integral_constant<int, kDil3>{}, std::integral_constant<int, N3>{}, aW3, kPlaneH2, kNP2);
+    // the next block's input (every thread has left the head that read max_prev)
+    if (gt < kC) max_prev[gt] = 0u;
+    if (w + wstep < p.n_blocks) {
+      stage_x();
+      group_sync(g);
+      if (w + 2 * wstep < p.n_blocks) load_x((w + 2 * wstep) * HOP);
+      im2col();
+    }
+    if (!(ok = wait_mma())) break;
+    // layer 3: relu(acc + b3), channel maxima over the block: this lane's channel at its warp's phase,
+    // then the four phases (adding the bias after the maximum changes nothing; non-negative floats
+    // order as unsigned)
+    {
+      float mx = -INFINITY, v[2][16];
+      const uint32_t src = tm_lane + 16 * half;
+      static_assert(N3 % 32 == 0, "two warps share the columns");
+      tmem_ld16(src, v[0]);
+      static_for<N3 / 32>([&](auto cc) {
+        constexpr int c = decltype(cc)::value, cur = c & 1;
+        tmem_wait_ld();
+        if constexpr (c + 1 < N3 / 32) tmem_ld16(src + 32 * (c + 1), v[cur ^ 1]);
+#pragma unroll
+        for (int e = 0; e < 16; ++e) mx = fmaxf(mx, v[cur][e]);
+      });
+      atomicMax(&max_cur[lane], __float_as_uint(fmaxf(mx + sBias[2 * kC + lane], 0.f)));
+    }
+    unsigned* const t = max_cur;
+    max_cur = max_prev;
+    max_prev = t;
+    w_prev = w;
+  }
+  if (ok && w_prev >= 0) {
+    group_sync(g);
+    head(w_prev, max_prev);
   }
   if (!ok && gt == 0) {
     atomicOr(p.status, 1);
@@ -693,7 +756,7 @@ namespace {
 void free_zband(fdas_zband* z) {
   const fdas::NetState& s = z->net;
   void* ptrs[] = {s.p,      s.ph,   s.pr,   s.packs,  s.g,    s.m,         s.v,        s.h1,    s.h2,    s.d2,    s.pool,
-                  s.pool_arg, s.pooled, s.seed, s.arg, s.logits, s.dlog, s.loss, s.loss_part, s.db2_part, s.part1, s.part2,
+                  s.pool_arg, s.pooled, s.seed, s.arg, s.logits, s.dlog, s.loss, s.loss_part, s.db2_part, s.part1, s.sum1, s.part2,
                   s.part3,  s.gl,   z->sel, z->scale, z->status};
   for (void* q : ptrs) cudaFree(q);
   if (z->graph_exec) cudaGraphExecDestroy(z->graph_exec);
@@ -723,19 +786,17 @@ int host_copy(fdas_zband* z, void* dst, const void* src, size_t bytes, cudaMemcp
   return FDAS_OK;
 }
 
-// scale = ln 2 / median |A|^2 into `scale`: seven launches.
+// scale = ln 2 / median |A|^2 into `scale`: a clear and three launches.
 void launch_power_scale(const float2* spec, int64_t n, SelectState* sel, float* scale, cudaStream_t st) {
-  select_init_kernel<<<1, 256, 0, st>>>(sel, n);
   const int64_t blocks = (n + 256 * kSelPer - 1) / (256 * kSelPer);
-  const unsigned grid = (unsigned)(blocks < kSelBlocks ? blocks : kSelBlocks);
-  // passes 1 and 2 flush up to 4096 bins per block: fewer, longer blocks
-  const unsigned grid12 = (unsigned)(blocks < kSelBlocks12 ? blocks : kSelBlocks12);
-  select_pass_kernel<0><<<grid, 256, 0, st>>>(spec, n, sel);
-  select_digit_kernel<0><<<1, 256, 0, st>>>(sel, scale);
-  select_pass_kernel<1><<<grid12, 256, 0, st>>>(spec, n, sel);
-  select_digit_kernel<1><<<1, 256, 0, st>>>(sel, scale);
-  select_pass_kernel<2><<<grid12, 256, 0, st>>>(spec, n, sel);
-  select_digit_kernel<2><<<1, 256, 0, st>>>(sel, scale);
+  auto grid = [&](int64_t cap) { return (unsigned)(blocks < cap ? blocks : cap); };
+  cudaMemsetAsync(sel, 0, sizeof(SelectState), st);
+  select_pass_kernel<0><<<grid(kSelBlocks0), 256, select_smem<0>(), st>>>(spec, n, sel, scale);
+  select_pass_kernel<1><<<grid(kSelBlocks), 256, select_smem<1>(), st>>>(spec, n, sel, scale);
+  select_pass_kernel<2><<<grid(kSelBlocks), 256, select_smem<2>(), st>>>(spec, n, sel, scale);
+}
+cudaError_t prepare_power_scale() {
+  return cudaFuncSetAttribute(select_pass_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)select_smem<0>());
 }
 }  // namespace
 
@@ -754,7 +815,7 @@ fdas_zband* fdas_zband_create(int window, int n_out, int max_batch) {
     cudaGetLastError();
     return nullptr;
   }
-  if (fdas::net_prepare() != cudaSuccess ||
+  if (fdas::net_prepare() != cudaSuccess || prepare_power_scale() != cudaSuccess ||
       cudaFuncSetAttribute(propose_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, kProposeSmem) !=
           cudaSuccess ||
       cudaFuncSetAttribute(propose_kernel<384>, cudaFuncAttributeMaxDynamicSharedMemorySize, kProposeSmem) !=
@@ -787,7 +848,7 @@ fdas_zband* fdas_zband_create(int window, int n_out, int max_batch) {
             cudaMalloc(&s.logits, B * (size_t)n_out * 4) == cudaSuccess &&
             cudaMalloc(&s.dlog, B * (size_t)n_out * 4) == cudaSuccess && cudaMalloc(&s.loss, 4) == cudaSuccess &&
             cudaMalloc(&s.loss_part, B * 4) == cudaSuccess && cudaMalloc(&s.db2_part, B * kC * 4) == cudaSuccess &&
-            cudaMalloc(&s.part1, n.part1 * 4) == cudaSuccess && cudaMalloc(&s.part2, n.part2 * 4) == cudaSuccess &&
+            cudaMalloc(&s.part1, n.part1 * 4) == cudaSuccess && cudaMalloc(&s.sum1, n.sum1 * 4) == cudaSuccess && cudaMalloc(&s.part2, n.part2 * 4) == cudaSuccess &&
             cudaMalloc(&s.part3, n.part3 * 4) == cudaSuccess && cudaMalloc(&s.gl, n.gl * 4) == cudaSuccess &&
             cudaMalloc(&z->sel, sizeof(SelectState)) == cudaSuccess &&
             cudaMalloc(&z->scale, 4) == cudaSuccess && cudaMalloc(&z->status, 4) == cudaSuccess &&
@@ -906,9 +967,9 @@ static cudaError_t launch_propose(fdas_zband* z, const float* d_spectrum, int64_
   const int64_t pairs = (nb + 1) / 2;
   const unsigned grid = (unsigned)(pairs < z->sm_count ? pairs : z->sm_count);
   switch (hop) {
-    case 256: propose_kernel<256><<<grid, 256, kProposeSmem, st>>>(q); break;
-    case 384: propose_kernel<384><<<grid, 256, kProposeSmem, st>>>(q); break;
-    default: propose_kernel<512><<<grid, 256, kProposeSmem, st>>>(q); break;
+    case 256: propose_kernel<256><<<grid, kProposeThreads, kProposeSmem, st>>>(q); break;
+    case 384: propose_kernel<384><<<grid, kProposeThreads, kProposeSmem, st>>>(q); break;
+    default: propose_kernel<512><<<grid, kProposeThreads, kProposeSmem, st>>>(q); break;
   }
   return cudaGetLastError();
 }
@@ -921,7 +982,7 @@ int fdas_zband_propose(fdas_zband* z, const float* d_spectrum, int64_t n_bins, f
   if ((reinterpret_cast<uintptr_t>(d_spectrum) & 7u) || (reinterpret_cast<uintptr_t>(d_logits) & 3u))
     return FDAS_ERR_ALIGN;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  // eight launches replayed as one graph: captured again when the spectrum, its length or the
+  // a clear and four launches replayed as one graph: captured again when the spectrum, its length or the
   // logits buffer change (the weights are read through fixed pointers, so training needs none)
   if (!(z->graph_exec && z->cap_spec == d_spectrum && z->cap_n == n_bins && z->cap_logits == d_logits)) {
     if (z->graph_exec) cudaGraphExecDestroy(z->graph_exec);
@@ -980,6 +1041,7 @@ int fdas_zband_spectrum_windows(const float* d_spectrum, int64_t n_bins, int win
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   SelectState* sel = nullptr;
   float* scale = nullptr;
+  if (prepare_power_scale() != cudaSuccess) return FDAS_ERR_CUDA;
   if (cudaMallocAsync(&sel, sizeof(SelectState), st) != cudaSuccess) return FDAS_ERR_ALLOC;
   if (cudaMallocAsync(&scale, 4, st) != cudaSuccess) {
     cudaFreeAsync(sel, st);
