@@ -209,7 +209,8 @@ struct NetState {
   float* loss = nullptr;       // device scalar
   float* loss_part = nullptr;  // [B]
   float* db2_part = nullptr;   // [B][32]
-  float* part1 = nullptr;      // weight-gradient partials of the three layers
+  float* part1 = nullptr;      // weight-gradient partials of the three layers (sum1: layer 1's, summed once)
+  float* sum1 = nullptr;
   float* part2 = nullptr;
   float* part3 = nullptr;
   float* gl = nullptr;         // head gradients
@@ -217,7 +218,7 @@ struct NetState {
 
 // Element counts of the buffers whose size is not plain from their shape.
 struct NetSizes {
-  size_t act, pool, part1, part2, part3, gl, packs;
+  size_t act, pool, part1, sum1, part2, part3, gl, packs;
 };
 NetSizes net_sizes(int W, int Z, int max_batch, int sm_count);
 cudaError_t net_prepare();   // function attributes, once per created net

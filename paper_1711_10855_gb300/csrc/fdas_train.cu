@@ -32,8 +32,10 @@ constexpr int kWgThreads = 256;          // layer-2 weight gradient: lane = inpu
 constexpr int kWgUnit = 32;              // positions per unit of its work split
 constexpr int kWgHalo = 32;              // 8 taps x dilation 4
 constexpr int kWgPitch = kTile + kWgHalo + 4;   // floats; an odd number of 16-byte chunks
-constexpr int kScatter = 320;            // positions of the layer-2 gradient built at a time
-constexpr int kL3Chunks = 8;             // window ranges of the layer-3 weight gradient
+constexpr int kScatter = 640;            // positions of the layer-2 gradient built at a time
+constexpr int kL3Chunks = 32;            // window ranges of the layer-3 weight gradient
+constexpr int kHeadChunks = 4;           // window ranges of the head's gradient
+constexpr int kW1Chunks = 32;            // tile ranges layer 1's partials are summed over first
 constexpr int kL3Part = kC * kC * kK + kC;
 constexpr int kW1Part = kC * kK + kC;
 
@@ -42,7 +44,9 @@ __device__ __forceinline__ int padded(int pos) { return pos + (pos >> 4) * 4; }
 // Adds 9 taps of one input channel to acc[chunk][element][channel]: x0 = the thread's first chunk,
 // STEP floats between successive chunks (padding included where it is regular), w = 9 x 32 weights.
 template <int D>
-__device__ __forceinline__ void conv_channel(float (&acc)[4][4][4], const float* __restrict__ x0,
+// Channels are paired (packed FP32x2): an FMA instruction then reads three register pairs in two cycles, where
+// scalar FMAs with three different registers issue at about 60%.
+__device__ __forceinline__ void conv_channel(float2 (&acc)[4][4][2], const float* __restrict__ x0,
                                              const float* __restrict__ w, int og) {
   float4 wk[kK];
 #pragma unroll
@@ -52,16 +56,17 @@ __device__ __forceinline__ void conv_channel(float (&acc)[4][4][4], const float*
     // chunk j is j*D positions further: 4j + 4(j/4) floats for D = 4 (the thread starts on a multiple
     // of 16), 20j for D = 16
     const float4 x = *reinterpret_cast<const float4*>(x0 + (D == 4 ? 4 * j + 4 * (j / 4) : 20 * j));
-    const float xe[4] = {x.x, x.y, x.z, x.w};
+    const float2 xe[4] = {bc(x.x), bc(x.y), bc(x.z), bc(x.w)};
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
       const int k = j - c;
       if (k < 0 || k >= kK) continue;
-      const float we[4] = {wk[k].x, wk[k].y, wk[k].z, wk[k].w};
+      const float2 w01 = make_float2(wk[k].x, wk[k].y), w23 = make_float2(wk[k].z, wk[k].w);
 #pragma unroll
-      for (int e = 0; e < 4; ++e)
-#pragma unroll
-        for (int o = 0; o < 4; ++o) acc[c][e][o] = fmaf(we[o], xe[e], acc[c][e][o]);
+      for (int e = 0; e < 4; ++e) {
+        acc[c][e][0] = fma2(w01, xe[e], acc[c][e][0]);
+        acc[c][e][1] = fma2(w23, xe[e], acc[c][e][1]);
+      }
     }
   }
 }
@@ -117,15 +122,16 @@ __global__ void __launch_bounds__(kConvThreads) net_conv_kernel(const ConvArgs a
     for (int i = tid; i < kC; i += kConvThreads) sW1[kC * kK + i] = a.b1[i];
   }
 
-  float acc[4][4][4];
+  float2 acc[4][4][2];   // [chunk][element][channel pair]
 #pragma unroll
-  for (int o = 0; o < 4; ++o) {
-    const float v = MODE == kConvBwd2 ? 0.f : a.bias[4 * og + o];
+  for (int o = 0; o < 2; ++o) {
+    const float2 v = MODE == kConvBwd2 ? bc(0.f) : make_float2(a.bias[4 * og + 2 * o], a.bias[4 * og + 2 * o + 1]);
 #pragma unroll
     for (int c = 0; c < 4; ++c)
 #pragma unroll
       for (int e = 0; e < 4; ++e) acc[c][e][o] = v;
   }
+  auto at = [&](int c, int e, int o) { return o & 1 ? acc[c][e][o >> 1].y : acc[c][e][o >> 1].x; };
 
   for (int c0 = 0; c0 < kC; c0 += kStage) {
     __syncthreads();
@@ -173,38 +179,38 @@ __global__ void __launch_bounds__(kConvThreads) net_conv_kernel(const ConvArgs a
         const int p = p0 + pos0 + D * c;
         if (p < n2)
           *reinterpret_cast<float4*>(a.h2 + rows + (size_t)(4 * og + o) * W + p) =
-              make_float4(fmaxf(acc[c][0][o], 0.f), fmaxf(acc[c][1][o], 0.f), fmaxf(acc[c][2][o], 0.f),
-                          fmaxf(acc[c][3][o], 0.f));
+              make_float4(fmaxf(at(c, 0, o), 0.f), fmaxf(at(c, 1, o), 0.f), fmaxf(at(c, 2, o), 0.f),
+                          fmaxf(at(c, 3, o), 0.f));
       }
   } else if constexpr (MODE == kConvL3) {
 #pragma unroll
     for (int o = 0; o < 4; ++o) {
       float best = -1.f;
-      int at = 0;
+      int where = 0;
 #pragma unroll
       for (int c = 0; c < 4; ++c)
 #pragma unroll
         for (int e = 0; e < 4; ++e) {   // increasing positions
           const int p = p0 + pos0 + D * c + e;
-          const float v = fmaxf(acc[c][e][o], 0.f);
+          const float v = fmaxf(at(c, e, o), 0.f);
           if (p < n3 && v > best) {
             best = v;
-            at = p;
+            where = p;
           }
         }
 #pragma unroll
       for (int off = 4; off > 0; off >>= 1) {
         const float ov = __shfl_down_sync(0xffffffffu, best, off, 8);
-        const int oa = __shfl_down_sync(0xffffffffu, at, off, 8);
-        if (ov > best || (ov == best && oa < at)) {
+        const int oa = __shfl_down_sync(0xffffffffu, where, off, 8);
+        if (ov > best || (ov == best && oa < where)) {
           best = ov;
-          at = oa;
+          where = oa;
         }
       }
       if (pt == 0) {
         const size_t at_out = ((size_t)b * gridDim.x + blockIdx.x) * kC + 4 * og + o;
         a.pool[at_out] = best;
-        a.arg[at_out] = at;
+        a.arg[at_out] = where;
       }
     }
   } else {
@@ -229,7 +235,7 @@ __global__ void __launch_bounds__(kConvThreads) net_conv_kernel(const ConvArgs a
         const float he[4] = {h.x, h.y, h.z, h.w};
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-          const float d = he[e] > 0.f ? acc[c][e][o] : 0.f;
+          const float d = he[e] > 0.f ? at(c, e, o) : 0.f;
 #pragma unroll
           for (int k = 0; k < kK; ++k) g[k] = fmaf(d, xv[4 * c + e + k], g[k]);
           g[kK] += d;
@@ -268,12 +274,14 @@ struct HeadArgs {
 };
 
 // One CTA per window: pooled maxima, head; in training also the loss, the pooled gradient, layer 3's
-// data gradient scattered to layer 2's positions, and layer 2's bias gradient.
+// data gradient scattered to layer 2's positions, and layer 2's bias gradient.  It waits on memory, not
+// on arithmetic: the head's weights are staged 256 rows at a time (coalesced, used twice), the scatter
+// covers all positions of a 1024-bin window at once and loads a channel's nine taps together.
 template <bool TRAIN>
 __global__ void __launch_bounds__(256) net_head_kernel(const HeadArgs a) {
-  __shared__ float sM[kC], sS[kC], sRed[8][kC], sLoss[256];
+  __shared__ float sM[kC], sS[kC], sRed[8][kC], sLoss[256], sDl[256];
   __shared__ int sA[kC];
-  extern __shared__ float sD[];   // TRAIN: [32][kScatter + 1]
+  extern __shared__ __align__(16) float dyn[];   // head weights [256][33]; TRAIN, later: gradient [32][kScatter + 1]
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, b = blockIdx.x, Z = a.Z;
   if (tid < kC) {
     float best = -1.f;
@@ -288,84 +296,98 @@ __global__ void __launch_bounds__(256) net_head_kernel(const HeadArgs a) {
     sM[tid] = best;
     sA[tid] = at;
   }
-  __syncthreads();
-  float loss = 0.f;
-  for (int j = tid; j < Z; j += 256) {
-    float s = a.bl[j];
-#pragma unroll
-    for (int c = 0; c < kC; ++c) s = fmaf(a.Wl[(size_t)j * kC + c], sM[c], s);
-    const size_t at = (size_t)b * Z + j;
-    a.logits[at] = s;
-    if constexpr (TRAIN) {
-      const float t = a.target[at];
-      a.dlog[at] = (1.f / (1.f + expf(-s)) - t) / a.count;
-      loss += fmaxf(s, 0.f) - s * t + log1pf(expf(-fabsf(s)));
-    }
-  }
-  if constexpr (!TRAIN) return;
-  sLoss[tid] = loss;
-  __syncthreads();   // dlog of this window is visible to the CTA
-  for (int s = 128; s > 0; s >>= 1) {
-    if (tid < s) sLoss[tid] += sLoss[tid + s];
+  float loss = 0.f, dm = 0.f;   // dm: warp w's share (j = w, w + 8, ...) of channel `lane`
+  for (int j0 = 0; j0 < Z; j0 += 256) {
+    const int nj = Z - j0 < 256 ? Z - j0 : 256;
     __syncthreads();
-  }
-  // dm[c] = sum_j dlog[j] Wl[j][c]: warp w takes j = w, w + 8, ...
-  {
-    float s = 0.f;
-    for (int j = warp; j < Z; j += 8) s = fmaf(a.dlog[(size_t)b * Z + j], a.Wl[(size_t)j * kC + lane], s);
-    sRed[warp][lane] = s;
-  }
-  __syncthreads();
-  if (tid < kC) {
-    float s = 0.f;
-#pragma unroll
-    for (int w = 0; w < 8; ++w) s += sRed[w][tid];
-    s = sM[tid] > 0.f ? s : 0.f;
-    sS[tid] = s;
-    a.pooled[(size_t)b * kC + tid] = sM[tid];
-    a.seed[(size_t)b * kC + tid] = s;
-    a.arg[(size_t)b * kC + tid] = sA[tid];
-  }
-  if (tid == 0) a.loss_part[b] = sLoss[0] / a.count;
-  // layer 3's data gradient at compact layer-2 position t = arg + 16k: sum over (o, k) of W3[o][i][k]
-  // seed[o].  Warp w adds the channels o whose arg is 2w or 2w + 1 mod 16, so no two warps meet.
-  const int n2 = a.W / 2 + 128;
-  float db[4] = {0.f, 0.f, 0.f, 0.f};
-  for (int t0 = 0; t0 < n2; t0 += kScatter) {
-    const int nt = n2 - t0 < kScatter ? n2 - t0 : kScatter;
-    for (int i = tid; i < kC * (kScatter + 1); i += 256) sD[i] = 0.f;
+    for (int i = tid; i < nj * kC; i += 256) dyn[(i >> 5) * (kC + 1) + (i & 31)] = a.Wl[(size_t)j0 * kC + i];
     __syncthreads();
-    for (int o = 0; o < kC; ++o) {
-      const int p = sA[o];
-      const float s = sS[o];
-      if (((p & 15) >> 1) != warp || s == 0.f) continue;
-      float w[kK];
+    if (tid < nj) {
+      const float* w = dyn + tid * (kC + 1);
+      float s = a.bl[j0 + tid];
 #pragma unroll
-      for (int k = 0; k < kK; ++k) w[k] = a.w3b[(o * kK + k) * kC + lane];
-#pragma unroll
-      for (int k = 0; k < kK; ++k) {
-        const int t = p + 16 * k - t0;
-        if (t >= 0 && t < nt) sD[lane * (kScatter + 1) + t] = fmaf(w[k], s, sD[lane * (kScatter + 1) + t]);
+      for (int c = 0; c < kC; ++c) s = fmaf(w[c], sM[c], s);
+      const size_t at = (size_t)b * Z + j0 + tid;
+      a.logits[at] = s;
+      if constexpr (TRAIN) {
+        const float t = a.target[at];
+        const float d = (1.f / (1.f + expf(-s)) - t) / a.count;
+        a.dlog[at] = d;
+        sDl[tid] = d;
+        loss += fmaxf(s, 0.f) - s * t + log1pf(expf(-fabsf(s)));
       }
     }
+    if constexpr (TRAIN) {
+      __syncthreads();
+      for (int j = warp; j < nj; j += 8) dm = fmaf(sDl[j], dyn[j * (kC + 1) + lane], dm);
+    }
+  }
+  if constexpr (TRAIN) {
+    sRed[warp][lane] = dm;
+    sLoss[tid] = loss;
     __syncthreads();
+    for (int s = 128; s > 0; s >>= 1) {
+      if (tid < s) sLoss[tid] += sLoss[tid + s];
+      __syncthreads();
+    }
+    if (tid < kC) {
+      float s = 0.f;
+#pragma unroll
+      for (int w = 0; w < 8; ++w) s += sRed[w][tid];
+      s = sM[tid] > 0.f ? s : 0.f;
+      sS[tid] = s;
+      a.pooled[(size_t)b * kC + tid] = sM[tid];
+      a.seed[(size_t)b * kC + tid] = s;
+      a.arg[(size_t)b * kC + tid] = sA[tid];
+    }
+    if (tid == 0) a.loss_part[b] = sLoss[0] / a.count;
+    // layer 3's data gradient at compact layer-2 position t = arg + 16k: sum over (o, k) of W3[o][i][k]
+    // seed[o].  Warp w adds the channels o whose arg is 2w or 2w + 1 mod 16, so no two warps meet.
+    const int n2 = a.W / 2 + 128;
+    float* col = dyn + lane * (kScatter + 1);
+    float db[4] = {0.f, 0.f, 0.f, 0.f};
+    for (int t0 = 0; t0 < n2; t0 += kScatter) {
+      const int nt = n2 - t0 < kScatter ? n2 - t0 : kScatter;
+      __syncthreads();
+      for (int i = tid; i < kC * (kScatter + 1) / 4; i += 256) reinterpret_cast<float4*>(dyn)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+      __syncthreads();
+      for (int o = 0; o < kC; ++o) {
+        const int p = sA[o];
+        const float s = sS[o];
+        if (((p & 15) >> 1) != warp || s == 0.f) continue;
+        float w[kK], v[kK];
+#pragma unroll
+        for (int k = 0; k < kK; ++k) w[k] = a.w3b[(o * kK + k) * kC + lane];
+#pragma unroll
+        for (int k = 0; k < kK; ++k) {   // nine different positions
+          const int t = p + 16 * k - t0;
+          v[k] = t >= 0 && t < nt ? col[t] : 0.f;
+        }
+#pragma unroll
+        for (int k = 0; k < kK; ++k) {
+          const int t = p + 16 * k - t0;
+          if (t >= 0 && t < nt) col[t] = fmaf(w[k], s, v[k]);
+        }
+      }
+      __syncthreads();
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const int ch = warp + 8 * r;
+        const size_t row = ((size_t)b * kC + ch) * a.W + t0;
+#pragma unroll 5
+        for (int t = lane; t < nt; t += 32) {
+          const float v = a.h2[row + t] > 0.f ? dyn[ch * (kScatter + 1) + t] : 0.f;
+          a.d2[row + t] = v;
+          db[r] += v;
+        }
+      }
+    }
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
-      const int ch = warp + 8 * r;
-      const size_t row = ((size_t)b * kC + ch) * a.W + t0;
-      for (int t = lane; t < nt; t += 32) {
-        const float v = a.h2[row + t] > 0.f ? sD[ch * (kScatter + 1) + t] : 0.f;
-        a.d2[row + t] = v;
-        db[r] += v;
-      }
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) db[r] += __shfl_down_sync(0xffffffffu, db[r], off);
+      if (lane == 0) a.db2_part[(size_t)b * kC + warp + 8 * r] = db[r];
     }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int r = 0; r < 4; ++r) {
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) db[r] += __shfl_down_sync(0xffffffffu, db[r], off);
-    if (lane == 0) a.db2_part[(size_t)b * kC + warp + 8 * r] = db[r];
   }
 }
 
@@ -387,11 +409,11 @@ __global__ void __launch_bounds__(kWgThreads, 2) net_wgrad2_kernel(const WgArgs 
   const int64_t U = (int64_t)a.B * per;
   int64_t u = (int64_t)blockIdx.x * U / gridDim.x;
   const int64_t u1 = ((int64_t)blockIdx.x + 1) * U / gridDim.x;
-  float acc[4][kK];
+  float2 acc[4][kK];   // sums over even and odd positions (packed FP32x2)
 #pragma unroll
   for (int o = 0; o < 4; ++o)
 #pragma unroll
-    for (int k = 0; k < kK; ++k) acc[o][k] = 0.f;
+    for (int k = 0; k < kK; ++k) acc[o][k] = bc(0.f);
   while (u < u1) {
     const int64_t b = u / per;
     const int q = (int)(u - b * per);
@@ -415,25 +437,24 @@ __global__ void __launch_bounds__(kWgThreads, 2) net_wgrad2_kernel(const WgArgs 
     }
     __syncthreads();
 #pragma unroll 1
-    for (int t = 0; t < nt; t += 16) {
-      float4 d[4][4];
+    for (int t = 0; t < nt; t += 8) {
+      float4 d[4][2];
 #pragma unroll
       for (int o = 0; o < 4; ++o)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) d[o][c] = *reinterpret_cast<const float4*>(sD + (4 * warp + o) * kTile + t + 4 * c);
+        for (int c = 0; c < 2; ++c) d[o][c] = *reinterpret_cast<const float4*>(sD + (4 * warp + o) * kTile + t + 4 * c);
 #pragma unroll
-      for (int j = 0; j < 12; ++j) {
+      for (int j = 0; j < 10; ++j) {
         const float4 h = *reinterpret_cast<const float4*>(sH + lane * kWgPitch + t + 4 * j);
+        const float2 h01 = make_float2(h.x, h.y), h23 = make_float2(h.z, h.w);
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
+        for (int c = 0; c < 2; ++c) {
           const int k = j - c;
           if (k < 0 || k >= kK) continue;
 #pragma unroll
           for (int o = 0; o < 4; ++o) {
-            acc[o][k] = fmaf(d[o][c].x, h.x, acc[o][k]);
-            acc[o][k] = fmaf(d[o][c].y, h.y, acc[o][k]);
-            acc[o][k] = fmaf(d[o][c].z, h.z, acc[o][k]);
-            acc[o][k] = fmaf(d[o][c].w, h.w, acc[o][k]);
+            acc[o][k] = fma2(make_float2(d[o][c].x, d[o][c].y), h01, acc[o][k]);
+            acc[o][k] = fma2(make_float2(d[o][c].z, d[o][c].w), h23, acc[o][k]);
           }
         }
       }
@@ -443,7 +464,7 @@ __global__ void __launch_bounds__(kWgThreads, 2) net_wgrad2_kernel(const WgArgs 
 #pragma unroll
   for (int o = 0; o < 4; ++o)
 #pragma unroll
-    for (int k = 0; k < kK; ++k) out[((4 * warp + o) * kK + k) * kC + lane] = acc[o][k];
+    for (int k = 0; k < kK; ++k) out[((4 * warp + o) * kK + k) * kC + lane] = acc[o][k].x + acc[o][k].y;
 }
 
 struct SparseArgs {
@@ -452,20 +473,24 @@ struct SparseArgs {
   const int* arg;
   const float* pooled;
   const float* dlog;
+  const float* part1;    // [tiles1][kW1Part]
+  float* sum1;           // [kW1Chunks][kW1Part]
   float* part3;          // [kL3Chunks][32][9][32] then [32]
-  float* gl;             // dWl [Z][32], dbl [Z]
-  int B, W, Z;
+  float* gl;             // [kHeadChunks] of dWl [Z][32], dbl [Z]
+  int B, W, Z, tiles1;
 };
 
-// Layer 3's weight gradient from the pooled values (blocks o + 32 * chunk of windows), and the head's
-// (the remaining blocks, 8 outputs each): 288 threads.
+// The small gradients, 288 threads a block: layer 3's weights from the pooled values (blocks o + 32 *
+// chunk of windows), a first sum of layer 1's partials (kW1Chunks blocks), and the head's (8 outputs
+// and a range of windows each).  All are chains of loads, so the ranges are short.
 __global__ void __launch_bounds__(288) net_sparse_grad_kernel(const SparseArgs a) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (blockIdx.x < kC * kL3Chunks) {
-    const int o = blockIdx.x % kC, chunk = blockIdx.x / kC;
+  int blk = blockIdx.x;
+  if (blk < kC * kL3Chunks) {
+    const int o = blk % kC, chunk = blk / kC;
     const int b0 = (int)((int64_t)chunk * a.B / kL3Chunks), b1 = (int)((int64_t)(chunk + 1) * a.B / kL3Chunks);
     float s = 0.f, sb = 0.f;   // warp = tap, lane = input channel
-#pragma unroll 4
+#pragma unroll 8
     for (int b = b0; b < b1; ++b) {
       const float g = a.seed[(size_t)b * kC + o];
       const int p = a.arg[(size_t)b * kC + o];
@@ -477,16 +502,29 @@ __global__ void __launch_bounds__(288) net_sparse_grad_kernel(const SparseArgs a
     if (tid == 0) out[kC * kC * kK + o] = sb;
     return;
   }
+  blk -= kC * kL3Chunks;
+  if (blk < kW1Chunks) {
+    const int t0 = (int)((int64_t)blk * a.tiles1 / kW1Chunks), t1 = (int)((int64_t)(blk + 1) * a.tiles1 / kW1Chunks);
+    for (int e = tid; e < kW1Part; e += 288) {
+      float s = 0.f;
+#pragma unroll 16
+      for (int t = t0; t < t1; ++t) s += a.part1[(size_t)t * kW1Part + e];
+      a.sum1[(size_t)blk * kW1Part + e] = s;
+    }
+    return;
+  }
+  blk -= kW1Chunks;
   // dWl[j][c] = sum_b dlog[b][j] m[b][c], dbl[j] = sum_b dlog[b][j]
-  const int j = (blockIdx.x - kC * kL3Chunks) * 8 + tid / (kC + 1), c = tid % (kC + 1);
+  const int chunk = blk % kHeadChunks, j = blk / kHeadChunks * 8 + tid / (kC + 1), c = tid % (kC + 1);
   if (tid >= 8 * (kC + 1) || j >= a.Z) return;
+  const int b0 = (int)((int64_t)chunk * a.B / kHeadChunks), b1 = (int)((int64_t)(chunk + 1) * a.B / kHeadChunks);
   float s = 0.f;
-#pragma unroll 8
-  for (int b = 0; b < a.B; ++b) {
+#pragma unroll 16
+  for (int b = b0; b < b1; ++b) {
     const float m = c < kC ? a.pooled[(size_t)b * kC + c] : 1.f;
     s = fmaf(a.dlog[(size_t)b * a.Z + j], m, s);
   }
-  a.gl[c < kC ? (size_t)j * kC + c : (size_t)a.Z * kC + j] = s;
+  a.gl[(size_t)chunk * a.Z * (kC + 1) + (c < kC ? (size_t)j * kC + c : (size_t)a.Z * kC + j)] = s;
 }
 
 // Where a parameter's copies go (net layout: NetLayout in fdas_internal.h).
@@ -586,7 +624,9 @@ int wg_ctas(const NetState& s, int B) {
 }
 Copies copies_of(const NetState& s) { return Copies{s.ph, s.pr, s.packs, s.lay.W2, s.lay.W3}; }
 
-constexpr size_t kHeadSmem = sizeof(float) * kC * (kScatter + 1);
+constexpr size_t kHeadTrainSmem = sizeof(float) * kC * (kScatter + 1);
+constexpr size_t kHeadSmem = sizeof(float) * 256 * (kC + 1);
+static_assert(kHeadSmem <= kHeadTrainSmem, "the head's weights share the gradient's space");
 
 void launch_forward(const NetState& s, const float* windows, int B, const float* params, int pack2, int pack3,
                     cudaStream_t st) {
@@ -632,13 +672,14 @@ NetSizes net_sizes(int W, int Z, int max_batch, int sm_count) {
   z.part1 = B * tiles_of(W / 2 + 160) * kW1Part;
   z.part2 = (size_t)2 * sm_count * kC * kC * kK;
   z.part3 = (size_t)kL3Chunks * kL3Part;
-  z.gl = (size_t)Z * (kC + 1);
+  z.sum1 = (size_t)kW1Chunks * kW1Part;
+  z.gl = (size_t)kHeadChunks * Z * (kC + 1);
   z.packs = (size_t)kNetPacks * kC * kC * kK;
   return z;
 }
 
 cudaError_t net_prepare() {
-  return cudaFuncSetAttribute(net_head_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kHeadSmem);
+  return cudaFuncSetAttribute(net_head_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kHeadTrainSmem);
 }
 
 void net_publish(const NetState& s, cudaStream_t st) {
@@ -649,7 +690,7 @@ cudaError_t net_predict(const NetState& s, const float* windows, int B, bool hal
                         cudaStream_t st) {
   const float* params = half_weights ? s.pr : s.p;
   launch_forward(s, windows, B, params, half_weights ? kPackW2Half : kPackW2, half_weights ? kPackW3Half : kPackW3, st);
-  net_head_kernel<false><<<B, 256, 0, st>>>(head_args(s, params, logits));
+  net_head_kernel<false><<<B, 256, kHeadSmem, st>>>(head_args(s, params, logits));
   return cudaGetLastError();
 }
 
@@ -670,7 +711,7 @@ cudaError_t net_train_step(const NetState& s, const float* windows, const float*
   h.d2 = s.d2;
   h.db2_part = s.db2_part;
   h.count = (float)((int64_t)B * Z);
-  net_head_kernel<true><<<B, 256, kHeadSmem, st>>>(h);
+  net_head_kernel<true><<<B, 256, kHeadTrainSmem, st>>>(h);
 
   ConvArgs c{};
   c.x = windows;
@@ -683,8 +724,8 @@ cudaError_t net_train_step(const NetState& s, const float* windows, const float*
   net_conv_kernel<kConvBwd2><<<dim3(tiles1, B), kConvThreads, 0, st>>>(c);
   const int wg = wg_ctas(s, B);
   net_wgrad2_kernel<<<wg, kWgThreads, 0, st>>>(WgArgs{s.h1, s.d2, s.part2, B, W});
-  net_sparse_grad_kernel<<<kC * kL3Chunks + (Z + 7) / 8, 288, 0, st>>>(
-      SparseArgs{s.h2, s.seed, s.arg, s.pooled, s.dlog, s.part3, s.gl, B, W, Z});
+  net_sparse_grad_kernel<<<kC * kL3Chunks + kW1Chunks + kHeadChunks * ((Z + 7) / 8), 288, 0, st>>>(
+      SparseArgs{s.h2, s.seed, s.arg, s.pooled, s.dlog, s.part1, s.sum1, s.part3, s.gl, B, W, Z, B * tiles1});
 
   AdamArgs a{};
   int blk = 0, k = 0;
@@ -692,14 +733,14 @@ cudaError_t net_train_step(const NetState& s, const float* windows, const float*
     a.seg[k++] = {part, stride, parts, count, at, blk, oki};
     blk += (count + 31) / 32;
   };
-  seg(s.part1, kW1Part, B * tiles1, kC * kK, s.lay.W1, false);
-  seg(s.part1 + kC * kK, kW1Part, B * tiles1, kC, s.lay.b1, false);
+  seg(s.sum1, kW1Part, kW1Chunks, kC * kK, s.lay.W1, false);
+  seg(s.sum1 + kC * kK, kW1Part, kW1Chunks, kC, s.lay.b1, false);
   seg(s.part2, n, wg, n, s.lay.W2, true);
   seg(s.db2_part, kC, B, kC, s.lay.b2, false);
   seg(s.part3, kL3Part, kL3Chunks, n, s.lay.W3, true);
   seg(s.part3 + n, kL3Part, kL3Chunks, kC, s.lay.b3, false);
-  seg(s.gl, Z * (kC + 1), 1, Z * kC, s.lay.Wl, false);
-  seg(s.gl + Z * kC, Z * (kC + 1), 1, Z, s.lay.bl, false);
+  seg(s.gl, Z * (kC + 1), kHeadChunks, Z * kC, s.lay.Wl, false);
+  seg(s.gl + Z * kC, Z * (kC + 1), kHeadChunks, Z, s.lay.bl, false);
   a.p = s.p;
   a.g = s.g;
   a.m = s.m;
