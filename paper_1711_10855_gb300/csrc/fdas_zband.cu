@@ -372,13 +372,15 @@ __global__ void __launch_bounds__(256) write_units_kernel(const uint16_t* masks,
 // weight rows are kept once, as the stack [0 0 0 W_8 ... W_0 0 0 0]: offset o starts at its block 11 - o.
 // N is (hop + 128)/4 and hop/4 columns instead of 32 channels, where an MMA's time no longer has
 // its floor of about 50 cycles: 24 MMAs of 80 and 64 cycles per layer for 512 positions, against 90
-// and 72 of 64 cycles with one tap, 128 positions and N = 32 each (kernel 330 to 200 us at 2^22
+// and 72 of 64 cycles with one tap, 128 positions and N = 32 each (kernel 330 to 176 us at 2^22
 // bins).  The zero blocks are a quarter of the multiply-adds.
 // Activations sit in shared memory K-major "chunk-planar": channel chunk j (8 channels, 16 B) of row q at
 // plane j, offset 16*q, rows ordered (phase, column) for the layer that reads them.  h2 overwrites
-// h1 after the MMAs that read it.  While a group's layer-2 MMAs run it does the previous block's head, and
-// during layer 3 the next block's staging and im2col; what is left between MMAs is the conversion of the
-// two activation layers.
+// h1 after the MMAs that read it.  While a group's layer-2 MMAs are issued (the issuing thread is held to
+// their pace) its other seven warps do the previous block's head, and during layer 3 the next block's
+// staging and im2col; what is left between MMAs is the conversion of the two activation layers.  The
+// groups issue layers 2 and 3 one at a time (a token): left alone they fall into step, both in their MMAs
+// at half speed and then both outside (14.0k cycles per block and group; 12.5k with the token).
 // ---------------------------------------------------------------------------------------
 constexpr int kMaxHop = 512;
 constexpr int kT1max = kMaxHop / 128 + 2;       // layer-1 M-tiles
@@ -388,7 +390,8 @@ constexpr int kNA1 = 128 * kT1max;              // im2col rows of layer 1
 constexpr int kNX = kNA1 + 8;                   // staged x values
 constexpr int kGroupThreads = 256;             // two warps per TMEM quadrant share its columns
 constexpr int kProposeThreads = 2 * kGroupThreads;
-constexpr int kXPer = (kNX + kGroupThreads - 1) / kGroupThreads;   // prefetched x per thread
+constexpr int kSideThreads = kGroupThreads - 32;   // a group without its issuing warp
+constexpr int kXPer = (kNX + kSideThreads - 1) / kSideThreads;   // prefetched x per thread
 constexpr int kZStage = 256;                    // head weights staged in shared memory up to this Z
 constexpr uint32_t kPlaneH1 = 4 * kNP1 * 16, kPlaneA1 = kNA1 * 16;
 constexpr uint32_t kPlaneH2 = 4 * kNP2 * 16 + 16;   // + 16: the four planes of a row on different banks
@@ -407,7 +410,7 @@ constexpr int kSlotBytes = (kSlotX + kNX * 4 + 127) / 128 * 128;
 constexpr int kOffGroup = kOffSlot + 2 * kSlotBytes;   // per group: channel maxima, mbarrier
 constexpr int kGroupMisc = 384;
 constexpr int kOffTslot = kOffGroup + 2 * kGroupMisc;
-constexpr int kProposeSmem = kOffTslot + 16;
+constexpr int kProposeSmem = kOffTslot + 16;   // TMEM base, MMA token
 constexpr uint32_t kIdesc1 = fdas::umma_idesc_f16(128, kC);
 constexpr uint32_t kTmemCols = 512;             // 256 columns per group (<= 6 x 32 used)
 static_assert(kDil1 == 1, "layer 1 is an im2col of adjacent x values");
@@ -434,6 +437,18 @@ __device__ __forceinline__ int wb_off(int o, int i) { return (i >> 3) * 512 + (o
 __device__ __forceinline__ void group_sync(int g) {
   asm volatile("bar.sync %0, %1;" ::"r"(g + 1), "n"(kGroupThreads) : "memory");
 }
+// The group without its first warp (ids 3, 4).
+__device__ __forceinline__ void side_sync(int g) {
+  asm volatile("bar.sync %0, %1;" ::"r"(g + 3), "n"(kSideThreads) : "memory");
+}
+// Bounded acquisition of the CTA's MMA token (0: free) by one thread; false if it gave up.
+__device__ __forceinline__ bool take_token(int* token) {
+  if (atomicCAS(token, 0, 1) == 0) return true;
+  const unsigned long long t0 = fdas::globaltimer_ns();
+  while (atomicCAS(token, 0, 1) != 0)
+    if (fdas::globaltimer_ns() - t0 > fdas::kWaitLimitNs) return false;
+  return true;
+}
 __device__ __forceinline__ int group_all(int g, int v) {
   int r;
   asm volatile(
@@ -455,6 +470,7 @@ __global__ void __launch_bounds__(kProposeThreads, 1) propose_kernel(const Propo
   float* sBl = reinterpret_cast<float*>(sm + kOffBl);
   float* sBias = reinterpret_cast<float*>(sm + kOffBias);
   uint32_t* tslot = reinterpret_cast<uint32_t*>(sm + kOffTslot);
+  int* token = reinterpret_cast<int*>(sm + kOffTslot + 4);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int g = warp >> 3, q = warp & 3, half = (warp >> 2) & 1, gt = tid & (kGroupThreads - 1);
@@ -490,6 +506,7 @@ __global__ void __launch_bounds__(kProposeThreads, 1) propose_kernel(const Propo
   if (gt == 0) {
     mbar_init(bar, 1);
     fence_barrier_init();
+    *token = 0;
   }
   if (warp == 0) {
     tmem_alloc(tslot, kTmemCols);
@@ -507,22 +524,23 @@ __global__ void __launch_bounds__(kProposeThreads, 1) propose_kernel(const Propo
   constexpr int T1 = HOP / 128 + 2, N2 = (HOP + 128) / 4, N3 = HOP / 4;
   constexpr int nx = 128 * T1 + 8;
   uint32_t phase = 0;
-  bool ok = true;
+  bool ok = true, issued = true;   // issued: the issuing thread got the token
 
+  const int st = gt - 32;   // the input and the head are the work of the warps that issue no MMAs
   // x values of block w's staging window into registers (all loads issued before any use)
   float2 xa[kXPer];
   auto load_x = [&](int64_t P0) {
 #pragma unroll
     for (int e = 0; e < kXPer; ++e) {
-      const int j = gt + kGroupThreads * e;
+      const int j = st + kSideThreads * e;
       const int64_t r = P0 - kRF + j;
-      xa[e] = (j < nx && r >= 0 && r < p.n) ? __ldg(p.spec + r) : make_float2(0.f, 0.f);
+      xa[e] = (st >= 0 && j < nx && r >= 0 && r < p.n) ? __ldg(p.spec + r) : make_float2(0.f, 0.f);
     }
   };
   // wait for this group's committed MMAs: one thread polls (bounded), the others sleep in the
   // group's hardware barrier
   auto wait_mma = [&]() -> bool {
-    const int good = group_all(g, gt == 0 ? (mbar_wait(bar, phase) ? 1 : 0) : 1);
+    const int good = group_all(g, gt == 0 ? (issued && mbar_wait(bar, phase) ? 1 : 0) : 1);
     phase ^= 1u;
     tmem_fence_after_sync();
     return good != 0;
@@ -597,6 +615,8 @@ __global__ void __launch_bounds__(kProposeThreads, 1) propose_kernel(const Propo
   auto issue_conv = [&](auto dil, auto cols, uint32_t wts, uint32_t plane, uint32_t rows_per_phase) {
     constexpr int D = decltype(dil)::value, N = decltype(cols)::value;
     const uint64_t a0 = umma_desc(wts, kPlaneW, 128), b0 = umma_desc(aSlot, plane, 128);
+    issued = take_token(token);
+    if (!issued) return;
     static_for<12>([&](auto oo) {
       constexpr int o = decltype(oo)::value;
       static_for<2>([&](auto cc) {
@@ -607,6 +627,7 @@ __global__ void __launch_bounds__(kProposeThreads, 1) propose_kernel(const Propo
       });
     });
     umma_commit(bar);
+    atomicExch(token, 0);
   };
 
   // x of the block in registers -> layer-1 im2col: row r (position P0-80+r) = x[r .. r+8], zero for K in [9, 16)
@@ -614,12 +635,12 @@ __global__ void __launch_bounds__(kProposeThreads, 1) propose_kernel(const Propo
   auto stage_x = [&]() {
 #pragma unroll
     for (int e = 0; e < kXPer; ++e) {
-      const int j = gt + kGroupThreads * e;
-      if (j < nx) sX[j] = fminf(power_of(xa[e]) * sc, kXCap);
+      const int j = st + kSideThreads * e;
+      if (st >= 0 && j < nx) sX[j] = fminf(power_of(xa[e]) * sc, kXCap);
     }
   };
   auto im2col = [&]() {
-    for (int r = gt; r < 128 * T1; r += kGroupThreads) {
+    for (int r = st; r < 128 * T1; r += kSideThreads) {
       __half2 h[8];
 #pragma unroll
       for (int e = 0; e < 4; ++e) h[e] = __floats2half2_rn(sX[r + 2 * e], sX[r + 2 * e + 1]);
@@ -634,7 +655,7 @@ __global__ void __launch_bounds__(kProposeThreads, 1) propose_kernel(const Propo
     float mc[kC];
 #pragma unroll
     for (int c = 0; c < kC; ++c) mc[c] = __uint_as_float(smax[c]);
-    for (int j = gt; j < p.Z; j += kGroupThreads) {
+    for (int j = st; j < p.Z; j += kSideThreads) {
       const __half* wl = wl_staged ? sWl + j * kC : p.w + p.oWl + (size_t)j * kC;
       float s = wl_staged ? sBl[j] : __half2float(p.w[p.obl + j]);
 #pragma unroll
@@ -657,12 +678,15 @@ __global__ void __launch_bounds__(kProposeThreads, 1) propose_kernel(const Propo
   unsigned* max_cur = sMax;           // this block's maxima (zero when its layer 3 is read)
   unsigned* max_prev = sMax + kC;     // the previous block's
   if (w < p.n_blocks) {
-    load_x(w * HOP);
-    stage_x();
-    if (gt < kC) max_cur[gt] = 0u;
-    group_sync(g);
-    if (w + wstep < p.n_blocks) load_x((w + wstep) * HOP);
-    im2col();
+    if (st >= 0) {
+      load_x(w * HOP);
+      stage_x();
+      side_sync(g);
+      if (w + wstep < p.n_blocks) load_x((w + wstep) * HOP);
+      im2col();
+    } else {
+      max_cur[lane] = 0u;
+    }
   }
   for (; w < p.n_blocks; w += wstep) {
     sync_for_mma();
@@ -679,17 +703,18 @@ __global__ void __launch_bounds__(kProposeThreads, 1) propose_kernel(const Propo
     sync_for_mma();
     if (gt == 0)
       issue_conv(std::integral_constant<int, kDil2>{}, std::integral_constant<int, N2>{}, aW2, kPlaneH1, kNP1);
-    if (w_prev >= 0) head(w_prev, max_prev);
+    if (st >= 0 && w_prev >= 0) head(w_prev, max_prev);
     if (!(ok = wait_mma())) break;
     store_h2();
     sync_for_mma();
     if (gt == 0)
       issue_conv(std::integral_constant<int, kDil3>{}, std::integral_constant<int, N3>{}, aW3, kPlaneH2, kNP2);
     // the next block's input (every thread has left the head that read max_prev)
-    if (gt < kC) max_prev[gt] = 0u;
-    if (w + wstep < p.n_blocks) {
+    if (st < 0) {
+      max_prev[lane] = 0u;
+    } else if (w + wstep < p.n_blocks) {
       stage_x();
-      group_sync(g);
+      side_sync(g);
       if (w + 2 * wstep < p.n_blocks) load_x((w + 2 * wstep) * HOP);
       im2col();
     }
@@ -718,7 +743,7 @@ __global__ void __launch_bounds__(kProposeThreads, 1) propose_kernel(const Propo
   }
   if (ok && w_prev >= 0) {
     group_sync(g);
-    head(w_prev, max_prev);
+    if (st >= 0) head(w_prev, max_prev);
   }
   if (!ok && gt == 0) {
     atomicOr(p.status, 1);
