@@ -286,11 +286,14 @@ __global__ void __launch_bounds__(256) net_head_kernel(const HeadArgs a) {
   if (tid < kC) {
     float best = -1.f;
     int at = 0;
+#pragma unroll 4
     for (int t = 0; t < a.tiles; ++t) {   // increasing positions: the first maximum
       const size_t i = ((size_t)b * a.tiles + t) * kC + tid;
-      if (a.pool[i] > best) {
-        best = a.pool[i];
-        at = a.pool_arg[i];
+      const float v = a.pool[i];
+      const int where = a.pool_arg[i];
+      if (v > best) {
+        best = v;
+        at = where;
       }
     }
     sM[tid] = best;
@@ -300,7 +303,12 @@ __global__ void __launch_bounds__(256) net_head_kernel(const HeadArgs a) {
   for (int j0 = 0; j0 < Z; j0 += 256) {
     const int nj = Z - j0 < 256 ? Z - j0 : 256;
     __syncthreads();
-    for (int i = tid; i < nj * kC; i += 256) dyn[(i >> 5) * (kC + 1) + (i & 31)] = a.Wl[(size_t)j0 * kC + i];
+#pragma unroll 8
+    for (int i = tid; i < nj * kC / 4; i += 256) {
+      const float4 v = reinterpret_cast<const float4*>(a.Wl + (size_t)j0 * kC)[i];   // 16-byte aligned (NetLayout)
+      float* d = dyn + (i >> 3) * (kC + 1) + 4 * (i & 7);
+      d[0] = v.x, d[1] = v.y, d[2] = v.z, d[3] = v.w;
+    }
     __syncthreads();
     if (tid < nj) {
       const float* w = dyn + tid * (kC + 1);
@@ -351,13 +359,22 @@ __global__ void __launch_bounds__(256) net_head_kernel(const HeadArgs a) {
       __syncthreads();
       for (int i = tid; i < kC * (kScatter + 1) / 4; i += 256) reinterpret_cast<float4*>(dyn)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
       __syncthreads();
-      for (int o = 0; o < kC; ++o) {
-        const int p = sA[o];
-        const float s = sS[o];
-        if (((p & 15) >> 1) != warp || s == 0.f) continue;
-        float w[kK], v[kK];
+      // this warp's channels, the next one's weights loaded before the current one's are used
+      unsigned mine = __ballot_sync(0xffffffffu, ((sA[lane] & 15) >> 1) == warp && sS[lane] != 0.f);
+      float w[kK];
+      auto load = [&](int o) {
 #pragma unroll
         for (int k = 0; k < kK; ++k) w[k] = a.w3b[(o * kK + k) * kC + lane];
+      };
+      if (mine) load(__ffs(mine) - 1);
+      while (mine) {
+        const int o = __ffs(mine) - 1, p = sA[o];
+        const float s = sS[o];
+        mine &= mine - 1;
+        float v[kK], wc[kK];
+#pragma unroll
+        for (int k = 0; k < kK; ++k) wc[k] = w[k];
+        if (mine) load(__ffs(mine) - 1);
 #pragma unroll
         for (int k = 0; k < kK; ++k) {   // nine different positions
           const int t = p + 16 * k - t0;
@@ -366,7 +383,7 @@ __global__ void __launch_bounds__(256) net_head_kernel(const HeadArgs a) {
 #pragma unroll
         for (int k = 0; k < kK; ++k) {
           const int t = p + 16 * k - t0;
-          if (t >= 0 && t < nt) col[t] = fmaf(w[k], s, v[k]);
+          if (t >= 0 && t < nt) col[t] = fmaf(wc[k], s, v[k]);
         }
       }
       __syncthreads();
@@ -374,11 +391,16 @@ __global__ void __launch_bounds__(256) net_head_kernel(const HeadArgs a) {
       for (int r = 0; r < 4; ++r) {
         const int ch = warp + 8 * r;
         const size_t row = ((size_t)b * kC + ch) * a.W + t0;
-#pragma unroll 5
-        for (int t = lane; t < nt; t += 32) {
-          const float v = a.h2[row + t] > 0.f ? dyn[ch * (kScatter + 1) + t] : 0.f;
-          a.d2[row + t] = v;
-          db[r] += v;
+        const float* src = dyn + ch * (kScatter + 1);
+#pragma unroll
+        for (int i = 0; i < kScatter / 128; ++i) {
+          const int t = 128 * i + 4 * lane;   // nt is a multiple of 4
+          if (t >= nt) continue;
+          const float4 h = *reinterpret_cast<const float4*>(a.h2 + row + t);
+          const float4 v = make_float4(h.x > 0.f ? src[t] : 0.f, h.y > 0.f ? src[t + 1] : 0.f,
+                                       h.z > 0.f ? src[t + 2] : 0.f, h.w > 0.f ? src[t + 3] : 0.f);
+          *reinterpret_cast<float4*>(a.d2 + row + t) = v;
+          db[r] += (v.x + v.y) + (v.z + v.w);
         }
       }
     }

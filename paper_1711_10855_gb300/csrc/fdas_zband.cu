@@ -42,22 +42,23 @@ constexpr int kRF = kPad * (kDil1 + kDil2 + kDil3);   // receptive field of a la
 
 constexpr float kXCap = 64.f;   // input cap: x_r = min(|A_r|^2 ln 2 / median |A|^2, 64)
 constexpr int kSelBlocks0 = 456;   // grid caps of the median's passes: 3 blocks of the first fit an SM of a GB300,
-constexpr int kSelBlocks = 608;    // and the later ones flush up to 4096 bins per block
+constexpr int kSelBlocks = 304;    // and the later ones flush their bins once per block
 
 // Exact lower median of |A_r|^2 (rank (n-1)/2) by radix selection on the FP32 bit patterns
 // (non-negative floats order as unsigned integers; the sign bit is 0): three passes over the spectrum
 // histogram 8 bits (the exponent: most values share a few bins, so each thread counts into bytes of
-// its own), then 12 bits of the values that match the digit found so far, then the last 11.  The block of a pass that finishes last
+// its own), then 10 bits of the values that match the digit found so far (a third of them, spread
+// over every bin: few bins keep the blocks' flush short), then the last 13.  The block of a pass that finishes last
 // finds the digit holding the rank; the last pass leaves scale = ln 2 / median.  The state is cleared
 // before the first pass.
-constexpr int kSelBins0 = 256, kSelBins1 = 4096, kSelBins2 = 2048;
+constexpr int kSelBins0 = 256, kSelBins1 = 1024, kSelBins2 = 8192;
 constexpr int kSelPer = 8;   // complex values per thread and pass iteration (four 16-byte loads)
 struct SelectState {
   long long k;                 // rank of the median among the values matching `prefix`
   unsigned prefix, done;       // bits fixed so far; blocks of the current pass that have finished
   unsigned hist0[kSelBins0];   // bits 30..23
-  unsigned hist1[kSelBins1];   // bits 22..11 of the values matching digit 0
-  unsigned hist2[kSelBins2];   // bits 10..0 of the values matching digits 0 and 1
+  unsigned hist1[kSelBins1];   // bits 22..13 of the values matching digit 0
+  unsigned hist2[kSelBins2];   // bits 12..0 of the values matching digits 0 and 1
 };
 
 __device__ __forceinline__ float power_of(const float2 a) { return fmaf(a.x, a.x, a.y * a.y); }
@@ -76,8 +77,8 @@ template <int PASS>
 __global__ void __launch_bounds__(256) select_pass_kernel(const float2* spec, int64_t n, SelectState* st,
                                                           float* scale) {
   constexpr int NB = PASS == 0 ? kSelBins0 : (PASS == 1 ? kSelBins1 : kSelBins2);
-  constexpr int SHIFT = PASS == 0 ? 23 : (PASS == 1 ? 11 : 0);
-  constexpr unsigned MASK = PASS == 0 ? 0u : (PASS == 1 ? 0xFF800000u : 0xFFFFF800u);
+  constexpr int SHIFT = PASS == 0 ? 23 : (PASS == 1 ? 13 : 0);
+  constexpr unsigned MASK = PASS == 0 ? 0u : (PASS == 1 ? 0xFF800000u : 0xFFFFE000u);
   extern __shared__ __align__(16) unsigned char sel_smem[];
   unsigned* h = reinterpret_cast<unsigned*>(sel_smem);
   __shared__ bool last;
