@@ -20,6 +20,7 @@ struct fdas_plan {
   int zmax = 0, zstep = 1, L = 0, m = 0, h = 0, V = 0, Z = 0;
   int64_t nseg = 0;
   int n1 = 0;                        // lanes per transform group for this L
+  void* memory = nullptr;            // one allocation holding the four buffers below
   float2* d_templates = nullptr;     // Z x L complex64, IFFT first-pass layout
   double2* d_taps = nullptr;         // Z x (m+1) complex128 normalised taps
   float2* d_twist = nullptr;         // L complex64 inter-pass twiddles, same layout
@@ -144,14 +145,8 @@ void free_plan_memory(fdas_plan* p) {
   free_tc_memory(p);
   if (p->done) cudaEventDestroy(p->done);
   p->done = nullptr;
-  cudaFree(p->d_templates);
-  cudaFree(p->d_taps);
-  cudaFree(p->d_twist);
-  cudaFree(p->d_status);
-  p->d_templates = nullptr;
-  p->d_taps = nullptr;
-  p->d_twist = nullptr;
-  p->d_status = nullptr;
+  cudaFree(p->memory);
+  p->memory = nullptr;
 }
 
 }  // namespace
@@ -218,10 +213,11 @@ fdas_plan* fdas_plan_create(int64_t n_bins, int zmax, int zstep, int seg_len, in
   p->nseg = (n_bins + p->V - 1) / p->V;
   p->n1 = fdas::conv_group_threads(seg_len);
   const size_t ntap = (size_t)tmpl_len + 1;
-  if (cudaMalloc(&p->d_templates, sizeof(float2) * (size_t)p->Z * p->L) != cudaSuccess ||
-      cudaMalloc(&p->d_taps, sizeof(double2) * (size_t)p->Z * ntap) != cudaSuccess ||
-      cudaMalloc(&p->d_twist, sizeof(float2) * (size_t)p->L) != cudaSuccess ||
-      cudaMalloc(&p->d_status, sizeof(int)) != cudaSuccess ||
+  auto round256 = [](size_t x) { return (x + 255) / 256 * 256; };
+  const size_t off_taps = round256(sizeof(float2) * (size_t)p->Z * p->L);
+  const size_t off_twist = off_taps + round256(sizeof(double2) * (size_t)p->Z * ntap);
+  const size_t off_status = off_twist + round256(sizeof(float2) * (size_t)p->L);
+  if (cudaMalloc(&p->memory, off_status + sizeof(int)) != cudaSuccess ||
       cudaEventCreateWithFlags(&p->done, cudaEventDisableTiming) != cudaSuccess) {
     cudaGetLastError();
     free_plan_memory(p);
@@ -229,6 +225,11 @@ fdas_plan* fdas_plan_create(int64_t n_bins, int zmax, int zstep, int seg_len, in
     g_last_error = FDAS_ERR_ALLOC;
     return nullptr;
   }
+  unsigned char* base = static_cast<unsigned char*>(p->memory);
+  p->d_templates = reinterpret_cast<float2*>(base);
+  p->d_taps = reinterpret_cast<double2*>(base + off_taps);
+  p->d_twist = reinterpret_cast<float2*>(base + off_twist);
+  p->d_status = reinterpret_cast<int*>(base + off_status);
   // cleared before any stream can use the plan (a non-blocking stream is not ordered after
   // default-stream work)
   if (cudaMemsetAsync(p->d_status, 0, sizeof(int), 0) != cudaSuccess || cudaStreamSynchronize(0) != cudaSuccess) {

@@ -53,6 +53,8 @@ class FdasError(RuntimeError):
 def lib() -> ctypes.CDLL:
     """Load the in-tree libfdas.so (built by paper_1711_10855_gb300.build / __graft_entry__.build)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is None:
             if not os.path.exists(LIB_PATH):
@@ -157,7 +159,7 @@ def lib() -> ctypes.CDLL:
             L.fdas_zband_work_pairs.restype = i32
             L.fdas_static_selftest_wait_timeout.argtypes = [i64, vp]
             L.fdas_static_selftest_wait_timeout.restype = i32
-            _lib = L
+            _lib = L   # published complete: readers take it without the lock
     return _lib
 
 
@@ -184,10 +186,19 @@ def _ptr(x) -> int:
     raise TypeError(f"cannot take a device pointer of {type(x)!r}")
 
 
+_raw_stream = None   # torch's (device) -> current stream handle, and its current-device query
+
+
 def _stream(stream) -> int:
+    """Handle of a CUDA stream; None: the current stream of the current device (the raw handle: building a
+    torch stream object for it costs more than the launch's own bookkeeping)."""
     if stream is None:
-        import torch
-        return int(torch.cuda.current_stream().cuda_stream)
+        global _raw_stream
+        if _raw_stream is None:
+            import torch
+            torch.cuda.init()
+            _raw_stream = (torch._C._cuda_getCurrentRawStream, torch.cuda.current_device)
+        return _raw_stream[0](_raw_stream[1]())
     if isinstance(stream, int):
         return stream
     return int(stream.cuda_stream)
