@@ -3,8 +3,8 @@
 // One launch computes the whole f-fdot power plane (Adamek et al. 2017, Section 1 Eq. 2, by
 // the overlap-and-save method of Section 2):
 //
-//   a2  TMA (cp.async.bulk.tensor, zero fill outside [0, n_bins)) brings each segment's L bins
-//       A[s*V - h .. s*V - h + L) into shared memory,
+//   a2  bulk copies (cp.async.bulk) bring the part inside [0, n_bins) of each segment's L bins
+//       A[s*V - h .. s*V - h + L) into shared memory, the rest is zero-filled,
 //   a3  forward FFT of the segment, kept in shared memory for all Z templates,
 //   a4  for every template z: multiply by the template spectrum T_z (streamed from L2 into a
 //       ring of shared-memory slots by bulk copies),
@@ -17,18 +17,21 @@
 //   pass 1: lane k1 holds Y[k1 + N1*k2], k2 < N2, as N2/2 packed pairs and does its N2-point DFT
 //           in registers (two N2/2-point DFTs in lockstep with packed f32x2 butterflies, then one
 //           scalar stage joining them),
-//   twist:  multiply by exp(SIGN i 2pi n2 k1 / L) (packed),
 //   exchange: one shared-memory transposition of 16-byte pair entries through a padded tile,
+//   twist:  multiply by exp(SIGN i 2pi n2 k1 / L), joined with the first stage of
 //   pass 2: lane t holds two columns n2 (a packed pair) and runs two N1-point DFTs in lockstep;
 //           output index n = n2 + N2*n1, so lane t ends with outputs n = t (mod N1).
 // The paper's design (Section 2: shuffle stage for N <= 32, shared memory above, 4 elements per
 // thread) is replaced by two register passes with compile-time FMA butterflies on packed pairs
 // and a single shared-memory exchange per transform.
 //
-// Work decomposition: a CTA of 8 warps owns G consecutive segments at a time ("group"); the
-// flattened (group, z) list is split into contiguous equal ranges, one per CTA (grid = #SMs),
-// so every CTA does the same number of inverse transforms.  P warps share a segment and take
-// alternate templates.
+// Work decomposition: a CTA owns G consecutive segments at a time ("group"); the flattened (group,
+// z) list is split into contiguous equal ranges, one per CTA (grid = #SMs).  The FP32 pipe bounds the kernel:
+// 71.8k lane operations per 2048-point transform, 0.98 ms per 2^22 x 201 plane of which 1.31 ms is
+// measured (1.36 with separate products; DRAM writes at 38% of their rate).  L = 2048 holds 64 points a
+// lane (8 warps of 217 registers); L = 256 and 512 hold 32 (16 warps of 128, P = 2 warps per segment
+// on alternate templates: 3e6 x 51 at L = 512 takes 228 us against 240 with 8 warps, 1e6 x 17 at 256 35
+// against 45 with everything in shared memory).
 #include <cstdio>
 #include <type_traits>
 
@@ -232,9 +235,9 @@ __device__ __forceinline__ void load_column_twiddles(float4 (&tw)[Cfg::H2], cons
 }
 
 // ---------------------------------------------------------------------------------------
-// Variant with the segment spectra and the twiddle table in tensor memory (one column pair per
-// lane: N2 = 2*N1, i.e. L = 512 and 2048).  Every warp owns its own segment(s); the template of
-// each position is read from the shared-memory ring by all 8 warps.  Per inverse transform the
+// The kernel: segment spectra and twiddle table in tensor memory (one column pair per lane at L = 512
+// and 2048, two at 256).  Every warp holds its segment(s); the template of
+// each position is read from the shared-memory ring by 8 warps.  Per inverse transform the
 // shared-memory traffic is the template (L*8 bytes) and the exchange (2*L*8 bytes); the
 // spectrum and the twiddles come from TMEM, a separate store, which relieves the shared-memory
 // bandwidth that otherwise co-limits the kernel with the FP32 pipe.
