@@ -824,7 +824,7 @@ def kernel_rev() -> str:
     """Content hash of the kernel sources; ncu traffic figures are valid only for this hash."""
     import hashlib
     h = hashlib.sha256()
-    for name in ("fdas_convolve.cu", "fdas_device.cuh"):
+    for name in ("fdas_convolve.cu", "fdas_conv_common.cuh", "fdas_device.cuh"):
         with open(os.path.join(ROOT, "paper_1711_10855_gb300", "csrc", name), "rb") as f:
             h.update(f.read())
     return h.hexdigest()[:16]

@@ -6,7 +6,6 @@
 #include <cstring>
 #include <new>
 
-#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include "fdas.h"
@@ -26,8 +25,6 @@ struct fdas_plan {
   float2* d_twist = nullptr;         // L complex64 inter-pass twiddles, same layout
   int* d_status = nullptr;
   bool built = false;
-  const void* map_ptr = nullptr;     // spectrum pointer the cached tensor map describes
-  CUtensorMap map;
   // tensor-core variant (fdas_convolve_power_tc), allocated on its first call
   float2* tc_bank = nullptr;         // Z x L natural-order template spectra
   float2* tc_seg = nullptr;          // nseg x L forward segment spectra of the current call
@@ -72,28 +69,6 @@ int validate(int64_t n_bins, int zmax, int zstep, int seg_len, int tmpl_len) {
   return FDAS_OK;
 }
 
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-EncodeTiledFn lookup_encode_fn() {
-  void* ptr = nullptr;
-  cudaDriverEntryPointQueryResult q;
-  if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &ptr, 12000, cudaEnableDefault, &q) !=
-          cudaSuccess ||
-      q != cudaDriverEntryPointSuccess)
-    return nullptr;
-  return reinterpret_cast<EncodeTiledFn>(ptr);
-}
-EncodeTiledFn get_encode_fn() {
-  static const EncodeTiledFn fn = lookup_encode_fn();   // looked up once, thread-safe
-  return fn;
-}
-
-// fdas_segment_spectra of the short lengths reads the spectrum through a tensor map; every other kernel
-// fetches its in-range part by bulk copies.
-bool needs_spectrum_map(int L) { return L <= 512 || L == 2048; }
-
 // Record the plan's completion event after work enqueued on `st` (skipped while the stream is
 // being captured into a CUDA graph: a captured record is not an event the host can wait on).
 int note_work(fdas_plan* p, cudaStream_t st) {
@@ -105,28 +80,6 @@ int note_work(fdas_plan* p, cudaStream_t st) {
 int enqueued(fdas_plan* p, cudaStream_t st, cudaError_t launch) {
   if (launch != cudaSuccess) return FDAS_ERR_CUDA;
   return note_work(p, st);
-}
-
-// 1-D tensor map over the spectrum: n_bins elements of 8 bytes, box of min(L, 256) elements,
-// zero fill outside [0, n_bins).
-int make_spectrum_map(fdas_plan* p, const void* d_spectrum) {
-  if (!needs_spectrum_map(p->L)) return FDAS_OK;
-  if (p->map_ptr == d_spectrum) return FDAS_OK;
-  EncodeTiledFn enc = get_encode_fn();
-  if (!enc) return FDAS_ERR_CUDA;
-  cuuint64_t gdim[1] = {(cuuint64_t)p->n_bins};
-  cuuint64_t gstride[1] = {0};
-  cuuint32_t box[1] = {(cuuint32_t)(p->L < 256 ? p->L : 256)};
-  cuuint32_t estride[1] = {1};
-  CUresult r = enc(&p->map, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 1, const_cast<void*>(d_spectrum), gdim, gstride, box,
-                   estride, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                   CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  if (r != CUDA_SUCCESS) {
-    p->map_ptr = nullptr;
-    return FDAS_ERR_CUDA;
-  }
-  p->map_ptr = d_spectrum;
-  return FDAS_OK;
 }
 
 void free_tc_memory(fdas_plan* p) {
@@ -377,8 +330,6 @@ int fdas_segment_spectra(fdas_plan* p, const float* d_spectrum, float* d_out, fd
   if (!p->built) return FDAS_ERR_NOT_BUILT;
   if ((reinterpret_cast<uintptr_t>(d_spectrum) & 15u) || (reinterpret_cast<uintptr_t>(d_out) & 15u))
     return FDAS_ERR_ALIGN;
-  int rc = make_spectrum_map(p, d_spectrum);
-  if (rc != FDAS_OK) return rc;
   fdas::SegParams q;
   q.twist = p->d_twist;
   q.spectrum_in = reinterpret_cast<const float2*>(d_spectrum);
@@ -389,7 +340,7 @@ int fdas_segment_spectra(fdas_plan* p, const float* d_spectrum, float* d_out, fd
   q.V = p->V;
   q.h = p->h;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  return enqueued(p, st, fdas::launch_segment_spectra(p->L, &p->map, q, p->sm_count, st));
+  return enqueued(p, st, fdas::launch_segment_spectra(p->L, q, p->sm_count, st));
 }
 
 namespace {
@@ -543,8 +494,8 @@ int fdas_template_spectrum(fdas_plan* p, int z_idx, float* host_out) {
 }  // extern "C"
 
 // ---------------------------------------------------------------------------------------
-// Helpers for the allocation-free entry point (fdas_static.cu): the same validation and
-// tensor-map encoding as the plan-based calls above, on caller-given memory.
+// Helpers for the allocation-free entry point (fdas_static.cu): the plan-based calls' validation and
+// wait self test.
 // ---------------------------------------------------------------------------------------
 namespace fdas {
 

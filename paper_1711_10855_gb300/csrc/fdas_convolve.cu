@@ -43,39 +43,6 @@
 
 namespace fdas {
 
-template <int L_, int N1_, int P_, int XR_, int R_ = 4>
-struct ConvCfg {
-  static constexpr int L = L_;
-  static constexpr int N1 = N1_;           // lanes per transform
-  static constexpr int N2 = L / N1;        // points per lane in pass 1
-  static constexpr int H2 = N2 / 2;        // pass-1 pairs per lane
-  static constexpr int F = 32 / N1;        // transform groups per warp
-  static constexpr int W = 8;              // compute warps per CTA
-  static constexpr int P = P_;             // warps sharing one segment
-  static constexpr int G = F * W / P;      // segments resident per CTA
-  static constexpr int R = R_;             // template ring slots
-  static constexpr int C = N2 / N1;        // pass-2 columns per lane
-  static constexpr int CP = C / 2;         // pass-2 column pairs per lane (= exchange row rounds)
-  static constexpr int XR = XR_;           // exchange sub-rounds (lane halves writing in turn)
-  static constexpr int XCOLS = N1 / XR;    // exchange tile columns per sub-round
-  static constexpr int XPITCH = XCOLS + 1; // 16-byte entries per tile row (odd: conflict-free)
-  static constexpr int XGROUP = N1 * XPITCH;
-  static constexpr int XWARP = F * XGROUP;
-  static constexpr int LOG_N1 = ilog2(N1);
-  static constexpr int LOG_N2 = ilog2(N2);
-  static constexpr int BOX = L < 256 ? L : 256;   // TMA box (elements of 8 bytes)
-  static constexpr size_t OFF_X = 0;
-  static constexpr size_t OFF_T = OFF_X + (size_t)G * L * 8;
-  static constexpr size_t OFF_TW = OFF_T + (size_t)R * L * 8;
-  static constexpr size_t OFF_XB = OFF_TW + (size_t)L * 8;
-  static constexpr size_t OFF_BAR = align_up(OFF_XB + (size_t)W * XWARP * 16, 128);
-  static constexpr size_t SMEM = OFF_BAR + 256;
-  static_assert(N1 * N2 == L && C >= 2 && C % 2 == 0 && 32 % N1 == 0, "bad decomposition");
-  static_assert(N1 % XR == 0 && XCOLS % 2 == 0, "bad exchange split");
-  static_assert(L % BOX == 0, "segment must be whole boxes");
-  static_assert(SMEM <= 232448, "shared memory budget");
-};
-
 // ---------------------------------------------------------------------------------------
 // Shared per-lane pieces of the transform
 //
@@ -87,82 +54,9 @@ struct ConvCfg {
 // for n2 = p and p + H2.  One 128-bit load gives a packed pair ready for f32x2 arithmetic.
 // ---------------------------------------------------------------------------------------
 
-// Pass 1 of the inverse transform on entry: v[i] = (Y[k1 + N1*bitrev(i)], Y[k1 + N1*(bitrev(i)+1)]),
-// i < H2 (bitrev over log2 N2 bits of an even index is < H2).  After fft_split_pairs:
-// v[j] = (Z[j], Z[j + H2]) for the lane's N2-point DFT; the twist then multiplies by the
-// twiddle pair of row j.
-template <class Cfg, bool CONJ>
-__device__ __forceinline__ void apply_twist2(cp2 (&v)[Cfg::H2], const float4* __restrict__ stw, int k1) {
-  static_for<Cfg::H2>([&](auto jj) {
-    constexpr int j = decltype(jj)::value;
-    const cp2 w = cp2_from(stw[j * Cfg::N1 + k1]);
-    v[j] = CONJ ? cmul2_conj(v[j], w) : cmul2(v[j], w);
-  });
-}
-
-// Exchange + pass 2.  Lane k1's pair j = r*N1 + t holds columns n2 = t + N1*r and
-// t + N1*(r + CP) of row k1; lane t gathers, for its column pair r, the entries of all N1 lanes
-// and runs two N1-point DFTs in lockstep.  Round r moves rows j in [r*N1, (r+1)*N1) through a
-// tile of N1 rows x XCOLS lanes (XR sub-rounds, lanes [h*XCOLS, (h+1)*XCOLS) writing in turn).
-// out(r, n1, pair) receives (y[t + N1*r + N2*n1], y[t + N1*(r+CP) + N2*n1]).
 struct NoHook {
   __device__ __forceinline__ void operator()() const {}
 };
-
-template <class Cfg, int SIGN, class Out, class AfterReads = NoHook>
-__device__ __forceinline__ void exchange_and_pass2(cp2 (&v)[Cfg::H2], float4* xb, int k1, Out&& out,
-                                                   AfterReads&& after_reads = AfterReads{}) {
-  static_for<Cfg::CP>([&](auto rr) {
-    constexpr int r = decltype(rr)::value;
-    cp2 u[Cfg::N1];
-    static_for<Cfg::XR>([&](auto hh) {
-      constexpr int h = decltype(hh)::value;
-      __syncwarp();
-      if (k1 / Cfg::XCOLS == h) {
-        const int c = k1 - h * Cfg::XCOLS;
-        static_for<Cfg::N1>([&](auto ii) {
-          constexpr int i = decltype(ii)::value;
-          xb[i * Cfg::XPITCH + c] = cp2_to(v[r * Cfg::N1 + i]);
-        });
-      }
-      __syncwarp();
-      static_for<Cfg::XCOLS>([&](auto cc) {
-        constexpr int c = decltype(cc)::value;
-        constexpr int src = h * Cfg::XCOLS + c;   // the writing lane k1'
-        u[bitrev(src, Cfg::LOG_N1)] = cp2_from(xb[k1 * Cfg::XPITCH + c]);
-      });
-    });
-    if constexpr (r == Cfg::CP - 1) after_reads();   // the tile is free once its last round is read
-    fft_pair_columns<Cfg::N1, SIGN>(u);
-    static_for<Cfg::N1>([&](auto nn) {
-      constexpr int n1 = decltype(nn)::value;
-      out(std::integral_constant<int, r>{}, std::integral_constant<int, n1>{}, u[n1]);
-    });
-  });
-}
-
-// Forward FFT (Eq. 3) of one segment held in natural order (complex64) in sx;
-// out(r, n1, pair) receives (X[t + N1*r + N2*n1], X[t + N1*(r+CP) + N2*n1]).
-template <class Cfg, class Twist, class Out>
-__device__ __forceinline__ void forward_transform_with(const float2* sx, Twist&& twist_conj, float4* xb, int k1,
-                                                       Out&& out) {
-  cp2 v[Cfg::H2];
-  static_for<Cfg::H2>([&](auto ii) {
-    constexpr int i = decltype(ii)::value;
-    constexpr int k2 = bitrev(i, Cfg::LOG_N2);
-    const float2 a = sx[k1 + Cfg::N1 * k2];
-    const float2 b = sx[k1 + Cfg::N1 * (k2 + 1)];
-    v[i] = cp2{make_float2(a.x, b.x), make_float2(a.y, b.y)};
-  });
-  fft_split_pairs<Cfg::N2, -1>(v);
-  twist_conj(v);
-  exchange_and_pass2<Cfg, -1>(v, xb, k1, out);
-}
-template <class Cfg, class Out>
-__device__ __forceinline__ void forward_transform(const float2* sx, const float4* __restrict__ stw, float4* xb,
-                                                  int k1, Out&& out) {
-  forward_transform_with<Cfg>(sx, [&](cp2 (&v)[Cfg::H2]) { apply_twist2<Cfg, true>(v, stw, k1); }, xb, k1, out);
-}
 
 // Exchange, twist and pass 2 with the twiddles in TMEM: round r moves the rows of column pair r, each
 // lane multiplies its column's entries (lane s wrote entry s) by their twiddles and runs two N1-point
@@ -189,23 +83,28 @@ __device__ __forceinline__ void exchange_twist_pass2(const cp2 (&v)[Cfg::H2], fl
   });
 }
 
-// Forward FFT (Eq. 3) of one segment held in natural order (complex64) in sx, into this lane's TMEM
-// slots: the pairs (k2 = 2p, 2p + 1) of the elements X[k1 + N1*k2].
-template <class Cfg>
-__device__ __forceinline__ void forward_to_tmem(const float2* sx, float4* xb, int k1, uint32_t tw_addr,
-                                                uint32_t x_addr) {
-  constexpr int N1 = Cfg::N1;
+// Forward FFT (Eq. 3) of one segment held in natural order (complex64) in sx; out as in
+// exchange_twist_pass2: u[n1] = (X[t + N1*r + N2*n1], X[t + N1*(r+CP) + N2*n1]).
+template <class Cfg, class Out>
+__device__ __forceinline__ void forward_transform(const float2* sx, float4* xb, int k1, uint32_t tw_addr, Out&& out) {
   cp2 v[Cfg::H2];
   static_for<Cfg::H2>([&](auto ii) {
     constexpr int i = decltype(ii)::value;
     constexpr int k2 = bitrev(i, Cfg::LOG_N2);
-    const float2 a = sx[k1 + N1 * k2];
-    const float2 b = sx[k1 + N1 * (k2 + 1)];
+    const float2 a = sx[k1 + Cfg::N1 * k2];
+    const float2 b = sx[k1 + Cfg::N1 * (k2 + 1)];
     v[i] = cp2{make_float2(a.x, b.x), make_float2(a.y, b.y)};
   });
   fft_split_pairs<Cfg::N2, -1>(v);
+  exchange_twist_pass2<Cfg, -1>(v, xb, k1, tw_addr, out);
+}
+// The same into this lane's TMEM slots: the pairs (k2 = 2p, 2p + 1) of the elements X[k1 + N1*k2].
+template <class Cfg>
+__device__ __forceinline__ void forward_to_tmem(const float2* sx, float4* xb, int k1, uint32_t tw_addr,
+                                                uint32_t x_addr) {
+  constexpr int N1 = Cfg::N1;
   cp2 first[Cfg::CP == 2 ? N1 : 1];   // two column pairs: round 0's, until round 1's complete the pairs
-  exchange_twist_pass2<Cfg, -1>(v, xb, k1, tw_addr, [&](auto rr, auto& x) {
+  forward_transform<Cfg>(sx, xb, k1, tw_addr, [&](auto rr, auto& x) {
     if constexpr (Cfg::CP == 1) {      // pair p = n1
       spectrum_to_tmem<Cfg::H2>(x_addr, [&](auto pp) { return x[decltype(pp)::value]; });
     } else if constexpr (decltype(rr)::value == 0) {   // elements k2 = 4 n1, 4 n1 + 2
@@ -256,8 +155,6 @@ struct TmemCfg {
   static constexpr bool PIPE = false;      // see multiply_first_stage
   static constexpr int C = N2 / N1;        // pass-2 columns per lane
   static constexpr int CP = C / 2;         // and column pairs (exchange rounds)
-  static constexpr int XR = 1;
-  static constexpr int XCOLS = N1;
   static constexpr int XPITCH = N1 + 1;
   static constexpr int XGROUP = N1 * XPITCH;
   static constexpr int XWARP = F * XGROUP;
@@ -847,54 +744,83 @@ __global__ void __launch_bounds__(256, 1) fdas_convolve_pairs_kernel(const PairP
   if (warp == 2) tmem_dealloc(*tmem_slot, Cfg::TMEM_COLS);
 }
 
-// Forward transforms only (steps a2 + a3), natural-order output, for tests of the FFT.
+// Forward transforms only (steps a2 + a3), natural-order output, for tests of the FFT: the forward code of
+// the kernels above, one CTA per segment group.
 template <class Cfg>
-__global__ void __launch_bounds__(256, 1)
-    fdas_segment_spectra_kernel(const __grid_constant__ CUtensorMap spec_map, const SegParams p) {
-  constexpr int L = Cfg::L, N1 = Cfg::N1;
-  constexpr int GS = 8 * Cfg::F;   // segments per CTA (one per transform group)
+constexpr size_t seg_smem() {
+  return (size_t)Cfg::W * Cfg::REGION + 64;
+}
+template <class Cfg>
+__global__ void __launch_bounds__(32 * Cfg::W, 1) fdas_segment_spectra_kernel(const SegParams p) {
+  constexpr int L = Cfg::L, N1 = Cfg::N1, N2 = Cfg::N2, H2 = Cfg::H2, G = Cfg::G;
+  static_assert(Cfg::P == 1 && Cfg::W == 8 && G <= 32, "one warp per segment set, one lane per segment");
   extern __shared__ __align__(1024) unsigned char smem[];
-  float2* sX = reinterpret_cast<float2*>(smem);
-  float2* sTw = sX + (size_t)GS * L;
-  float4* sXb = reinterpret_cast<float4*>(sTw + L);
-  uint64_t* bar = reinterpret_cast<uint64_t*>(smem + align_up(((size_t)GS * L + L) * 8 + (size_t)8 * Cfg::XWARP * 16, 128));
+  uint64_t* bar = reinterpret_cast<uint64_t*>(smem + (size_t)Cfg::W * Cfg::REGION);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar + 1);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int gw = lane / N1, k1 = lane % N1;
-  const int slot = warp * Cfg::F + gw;
-  const int64_t s0 = (int64_t)blockIdx.x * GS;
-  if (tid == 0) {
-    mbar_init(bar, 1);
-    fence_barrier_init();
+  float2* region = reinterpret_cast<float2*>(smem + (size_t)warp * Cfg::REGION);
+  float2* mySeg = region + (size_t)gw * L;
+  float4* myXb = reinterpret_cast<float4*>(region) + gw * Cfg::XGROUP;
+  const int64_t s0 = (int64_t)blockIdx.x * G;
+  if (warp == 0) {
+    if (lane == 0) {
+      mbar_init(bar, 1);
+      fence_barrier_init();
+    }
+    __syncwarp();
+    const int64_t x0 = (s0 + lane) * (int64_t)p.V - p.h;
+    const int64_t c0 = x0 > 0 ? x0 : 0, c1 = x0 + L < p.n_bins ? x0 + L : p.n_bins;
+    const uint32_t bytes = lane < G && c1 > c0 ? (uint32_t)((c1 - c0) * 8) : 0u;
+    const uint32_t total = __reduce_add_sync(0xffffffffu, bytes);
+    if (lane == 0) mbar_arrive_expect_tx(bar, total);
+    __syncwarp();
+    if (bytes) {
+      float2* dst = reinterpret_cast<float2*>(smem + (size_t)(lane / Cfg::F) * Cfg::REGION) + (lane % Cfg::F) * L;
+      bulk_g2s(dst + (c0 - x0), p.spectrum_in + c0, bytes, bar);
+    }
+  } else if (warp == 2) {
+    tmem_alloc(tmem_slot, Cfg::TMEM_COLS);
+    tmem_relinquish();
   }
+  const int64_t s = s0 + warp * Cfg::F + gw;
+  {
+    // zeros outside [0, n) in this lane group's window
+    const int64_t x0 = s * (int64_t)p.V - p.h;
+    for (int e = k1; e < L; e += N1)
+      if (x0 + e < 0 || x0 + e >= p.n_bins) mySeg[e] = make_float2(0.f, 0.f);
+  }
+  float4 tw[H2];
+  if (warp >= 4) load_column_twiddles<Cfg>(tw, p.twist, k1);
+  tmem_fence_before_sync();
   __syncthreads();
-  if (tid == 0) {
-    mbar_arrive_expect_tx(bar, (GS + 1) * L * 8);
-    bulk_g2s(sTw, p.twist, L * 8, bar);
-    for (int j = 0; j < GS; ++j) {
-      const int64_t x0 = (s0 + j) * (int64_t)p.V - p.h;
-      for (int bx = 0; bx < L / Cfg::BOX; ++bx)
-        tma_load_1d(sX + (size_t)j * L + bx * Cfg::BOX, &spec_map, (int32_t)(x0 + bx * Cfg::BOX), bar);
-    }
-  }
+  tmem_fence_after_sync();
+  const uint32_t tw_addr = *tmem_slot + ((uint32_t)(32 * (warp & 3)) << 16) + Cfg::COL_TW;
+  if (warp >= 4) twiddles_to_tmem<H2>(tw, tw_addr);
+  tmem_fence_before_sync();
   const int ok = __syncthreads_and(mbar_wait(bar, 0) ? 1 : 0);
-  if (!ok) {
-    if (tid == 0) {
-      atomicOr(p.status, kStatusTimeout);
-      (void)mbar_wait(bar, 0);   // bounded wait for copies still in flight
-    }
-    return;
+  tmem_fence_after_sync();
+  if (ok) {
+    float2* dst = p.out + s * L;
+    const bool valid = s < p.nseg;
+    forward_transform<Cfg>(mySeg, myXb, k1, tw_addr, [&](auto rr, auto& x) {
+      static_for<N1>([&](auto nn) {
+        constexpr int n1 = decltype(nn)::value;
+        const int n = decltype(rr)::value * N1 + k1 + N2 * n1;
+        if (valid) {
+          dst[n] = make_float2(x[n1].re.x, x[n1].im.x);
+          dst[n + Cfg::CP * N1] = make_float2(x[n1].re.y, x[n1].im.y);
+        }
+      });
+    });
+  } else if (tid == 0) {
+    atomicOr(p.status, kStatusTimeout);
+    (void)mbar_wait(bar, 0);   // bounded wait for copies still in flight
   }
-  const int64_t s = s0 + slot;
-  float2* dst = p.out + s * L;
-  const bool valid = s < p.nseg;
-  forward_transform<Cfg>(sX + (size_t)slot * L, reinterpret_cast<const float4*>(sTw),
-                         sXb + warp * Cfg::XWARP + gw * Cfg::XGROUP, k1, [&](auto rr, auto nn, const cp2& x) {
-                           const int n = decltype(rr)::value * N1 + k1 + Cfg::N2 * decltype(nn)::value;
-                           if (valid) {
-                             dst[n] = make_float2(x.re.x, x.im.x);
-                             dst[n + Cfg::CP * N1] = make_float2(x.re.y, x.im.y);
-                           }
-                         });
+  tmem_fence_before_sync();
+  __syncthreads();
+  tmem_fence_after_sync();
+  if (warp == 2) tmem_dealloc(*tmem_slot, Cfg::TMEM_COLS);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -912,20 +838,15 @@ int conv_group_threads(int L) {
 }
 
 template <class Cfg>
-static cudaError_t launch_seg_cfg(const CUtensorMap* map, const SegParams& p, cudaStream_t st) {
-  constexpr int GS = 8 * Cfg::F;
-  constexpr size_t smem = align_up(((size_t)GS * Cfg::L + Cfg::L) * 8 + (size_t)8 * Cfg::XWARP * 16, 128) + 64;
-  static_assert(smem <= 232448, "shared memory budget of the segment-spectra kernel");
+static cudaError_t launch_seg_cfg(const SegParams& p, cudaStream_t st) {
+  static_assert(seg_smem<Cfg>() <= 232448, "shared memory budget of the segment-spectra kernel");
   auto kern = fdas_segment_spectra_kernel<Cfg>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)seg_smem<Cfg>());
   if (e != cudaSuccess) return e;
-  const int64_t grid = (p.nseg + GS - 1) / GS;
-  kern<<<(unsigned)grid, 256, smem, st>>>(*map, p);
+  const int64_t grid = (p.nseg + Cfg::G - 1) / Cfg::G;
+  kern<<<(unsigned)grid, 32 * Cfg::W, seg_smem<Cfg>(), st>>>(p);
   return cudaGetLastError();
 }
-
-using Cfg256 = ConvCfg<256, 8, 1, 1>;
-using Cfg512 = ConvCfg<512, 16, 1, 1>;
 
 // Full planes: PlaneCfg.  Work lists: ListCfg (the same segments per CTA; void: none), separate
 // instantiations with their own parameter type, so that the full-plane code stays free of them.
@@ -1109,11 +1030,11 @@ cudaError_t launch_convolve(int L, const ConvParams& p, int sm_count, cudaStream
   }
 }
 
-cudaError_t launch_segment_spectra(int L, const CUtensorMap* map, const SegParams& p, int sm_count, cudaStream_t st) {
+cudaError_t launch_segment_spectra(int L, const SegParams& p, int sm_count, cudaStream_t st) {
   switch (L) {
-    case 256: return launch_seg_cfg<Cfg256>(map, p, st);
-    case 512: return launch_seg_cfg<Cfg512>(map, p, st);
-    case 2048: return launch_seg_cfg<ConvCfg<2048, 32, 2, 2>>(map, p, st);   // two-round exchange fits
+    case 256: return launch_seg_cfg<TmemCfg<256, 8>>(p, st);
+    case 512: return launch_seg_cfg<Tmem512List>(p, st);
+    case 2048: return launch_seg_cfg<Tmem2048>(p, st);
     default: return launch_segment_spectra_wide(L, p, sm_count, st);
   }
 }

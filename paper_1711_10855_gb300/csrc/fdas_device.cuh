@@ -92,17 +92,6 @@ __device__ __forceinline__ void static_for(F&& f) {
 }
 
 // ---------------------------------------------------------------------------------------
-// Complex helpers
-// ---------------------------------------------------------------------------------------
-__device__ __forceinline__ float2 cmul(float2 a, float2 b) {
-  return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
-}
-__device__ __forceinline__ float2 cmul_conj_b(float2 a, float2 b) {   // a * conj(b)
-  return make_float2(fmaf(a.x, b.x, a.y * b.y), fmaf(a.y, b.x, -a.x * b.y));
-}
-__device__ __forceinline__ float power(float2 a) { return fmaf(a.x, a.x, a.y * a.y); }
-
-// ---------------------------------------------------------------------------------------
 // Radix-2 DIT butterfly a' = a + w b, b' = a - w b with w = exp(SIGN * i * 2*pi*J/M)
 // ---------------------------------------------------------------------------------------
 template <int J, int M, int SIGN>
@@ -143,29 +132,6 @@ __device__ __forceinline__ void butterfly(float2& a, float2& b) {
     a = make_float2(fmaf(sn, ur, s.x), fmaf(sn, ui, s.y));
     b = make_float2(fmaf(-sn, ur, s.x), fmaf(-sn, ui, s.y));
   }
-}
-
-template <int N, int SIGN, int S, int I>
-__device__ __forceinline__ void stage_butterfly(float2 (&v)[N]) {
-  constexpr int span = 1 << S;
-  constexpr int blk = (I / span) * (2 * span);
-  constexpr int j = I % span;
-  butterfly<j, 2 * span, SIGN>(v[blk + j], v[blk + j + span]);
-}
-template <int N, int SIGN, int S, int... I>
-__device__ __forceinline__ void fft_stage(float2 (&v)[N], std::integer_sequence<int, I...>) {
-  (stage_butterfly<N, SIGN, S, I>(v), ...);
-}
-template <int N, int SIGN, int... S>
-__device__ __forceinline__ void fft_stages(float2 (&v)[N], std::integer_sequence<int, S...>) {
-  (fft_stage<N, SIGN, S>(v, std::make_integer_sequence<int, N / 2>{}), ...);
-}
-
-// In-register DFT of N points: on entry v[i] = x[bitrev(i)], on exit v[m] = X[m] =
-// sum_n x[n] exp(SIGN * i * 2*pi*n*m/N)  (Eq. 3 for SIGN = -1).
-template <int N, int SIGN>
-__device__ __forceinline__ void fft_dit(float2 (&v)[N]) {
-  fft_stages<N, SIGN>(v, std::make_integer_sequence<int, ilog2(N)>{});
 }
 
 // ---------------------------------------------------------------------------------------
@@ -349,18 +315,6 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
       "l"(src), "r"(bytes), "r"(smem_u32(bar))
       : "memory");
 }
-// 1-D tiled tensor copy global -> shared of one box starting at element x (may be negative or
-// beyond the extent: those elements are zero-filled).  x * element size must be a multiple of
-// 16 bytes.
-__device__ __forceinline__ void tma_load_1d(void* dst, const void* tmap, int32_t x, uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.1d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2}], "
-      "[%3];" ::"r"(smem_u32(dst)),
-      "l"(tmap), "r"(x), "r"(smem_u32(bar))
-      : "memory");
-}
-
-
 // ---------------------------------------------------------------------------------------
 // Tensor memory (TMEM, sm_100+): 128 lanes x 512 columns of 32-bit cells per SM, a store
 // separate from shared memory.  Warp w of a CTA may access lanes [32*(w%4), 32*(w%4)+32);

@@ -3,7 +3,6 @@
 
 #include <cstdint>
 
-#include <cuda.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
@@ -88,7 +87,7 @@ struct PairParams {
 // Parameters of the forward-transform-only kernel (steps a2 + a3, for tests).
 struct SegParams {
   const float2* twist;
-  const float2* spectrum_in; // n_bins complex64 (bulk copies of the L = 1024, 4096, 8192 kernel)
+  const float2* spectrum_in; // n_bins complex64 (read by bulk copies)
   float2* out;              // nseg x L, natural order
   int* status;
   int64_t n_bins;
@@ -117,8 +116,7 @@ cudaError_t launch_pairs(int L, const PairParams& p, int sm_count, cudaStream_t 
 
 // Launch helpers (defined in fdas_convolve.cu).  Return a cudaError_t from the launch.
 cudaError_t launch_convolve(int L, const ConvParams& p, int sm_count, cudaStream_t stream);
-cudaError_t launch_segment_spectra(int L, const CUtensorMap* spec_map, const SegParams& p,
-                                   int sm_count, cudaStream_t stream);
+cudaError_t launch_segment_spectra(int L, const SegParams& p, int sm_count, cudaStream_t stream);
 // Tensor-core variant for L = 2048 (fdas_tc.cu): inverse transforms as DFT-matrix contractions.
 struct TcParams {
   const float2* seg;        // nseg x 2048 forward segment spectra, natural order (inverse pass)
@@ -143,7 +141,7 @@ cudaError_t launch_tc_prepare(const float2* bank, int Z, float2* nat, unsigned* 
 // forward = true: the segment transforms (spectrum -> seg_out); false: the correlation (seg -> plane).
 cudaError_t launch_tc(const TcParams& p, int precision, bool forward, int sm_count, cudaStream_t stream);
 
-// Segment lengths 1024, 4096 and 8192 (fdas_convolve_wide.cu); no tensor map.
+// Segment lengths 1024, 4096 and 8192 (fdas_convolve_wide.cu).
 cudaError_t launch_convolve_wide(int L, const ConvParams& p, int sm_count, cudaStream_t stream);
 cudaError_t launch_segment_spectra_wide(int L, const SegParams& p, int sm_count, cudaStream_t stream);
 

@@ -5,7 +5,6 @@
 #include <cstdint>
 #include <mutex>
 
-#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include "fdas.h"

@@ -323,7 +323,9 @@ cudaError_t build_templates_into(double2* taps, float2* templates, float2* twist
   }
   b.gc = 1;
   while (b.M && b.gc < kHalf && 2 * b.gc * (b.M + extra) <= b.nbuf) b.gc *= 2;
-  cudaError_t e = cudaFuncSetAttribute(template_bank_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // the same limit whatever the shape: threads that build different banks at once do not undo each other's
+  cudaError_t e =
+      cudaFuncSetAttribute(template_bank_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
   if (e != cudaSuccess) return e;
   if (!b.M) taps_kernel<<<2 * (zmax / zstep) + 1, kThreads, 0, st>>>(taps, zmax, zstep, b.h);
   const int grid = zmax / zstep + 1 + (L + kTwistPer - 1) / kTwistPer;
