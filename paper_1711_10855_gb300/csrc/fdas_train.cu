@@ -12,10 +12,12 @@
 // four chunks of 4 spaced by the dilation D, so tap k of chunk c is chunk c + k and each 16-byte
 // input load feeds up to 64 FMAs (one load per FMA without the tile: 8 times slower, bound by
 // shared memory).  Rows are padded by one 16-byte chunk in five, which spreads a quarter-warp's
-// loads over all banks for D = 4 and D = 16.
+// loads over all banks for D = 4 and D = 16.  The next stage's operands are copied asynchronously while one
+// is computed: with one buffer a fifth to a quarter of the warps' time went to waiting for them.
 //
 // Every reduction has a fixed shape, so one seed gives one network.
 #include <cuda_fp16.h>
+#include <cuda_pipeline.h>
 #include <cuda_runtime.h>
 
 #include "fdas_device.cuh"
@@ -27,11 +29,12 @@ namespace {
 constexpr int kC = kNetC, kK = kNetK;
 constexpr int kTile = 128;               // positions per conv CTA
 constexpr int kConvThreads = 64;         // 8 position threads x 8 channel groups of 4
-constexpr int kStage = 16;               // input channels staged at a time
+constexpr int kStage = 8;                // input channels staged at a time (two stages in shared memory)
 constexpr int kWgThreads = 256;          // layer-2 weight gradient: lane = input channel, warp = 4 output channels
 constexpr int kWgUnit = 32;              // positions per unit of its work split
 constexpr int kWgHalo = 32;              // 8 taps x dilation 4
 constexpr int kWgPitch = kTile + kWgHalo + 4;   // floats; an odd number of 16-byte chunks
+constexpr int kWgBuffer = kC * (kWgPitch + kTile);
 constexpr int kScatter = 640;            // positions of the layer-2 gradient built at a time
 constexpr int kL3Chunks = 32;            // window ranges of the layer-3 weight gradient
 constexpr int kHeadChunks = 4;           // window ranges of the head's gradient
@@ -98,8 +101,8 @@ __global__ void __launch_bounds__(kConvThreads) net_conv_kernel(const ConvArgs a
   constexpr int S = kTile + 8 * D;         // staged positions
   constexpr int SP = S / 4 * 5;            // padded row
   constexpr int XS = MODE == kConvL2 ? S + 8 : (MODE == kConvBwd2 ? kTile + 8 : 4);   // staged x
-  __shared__ __align__(16) float sIn[kStage * SP];
-  __shared__ __align__(16) float sW[kStage * kK * kC];
+  __shared__ __align__(16) float sIn[2][kStage * SP];
+  __shared__ __align__(16) float sW[2][kStage * kK * kC];
   __shared__ __align__(16) float sX[XS];
   __shared__ float sW1[kC * (kK + 1)];
 
@@ -133,14 +136,33 @@ __global__ void __launch_bounds__(kConvThreads) net_conv_kernel(const ConvArgs a
   }
   auto at = [&](int c, int e, int o) { return o & 1 ? acc[c][e][o >> 1].y : acc[c][e][o >> 1].x; };
 
-  for (int c0 = 0; c0 < kC; c0 += kStage) {
-    __syncthreads();
-    const float4* w4 = reinterpret_cast<const float4*>(a.w + c0 * kK * kC);
-    for (int i = tid; i < kStage * kK * kC / 4; i += kConvThreads) reinterpret_cast<float4*>(sW)[i] = w4[i];
-    for (int i = tid; i < kStage * (S / 4); i += kConvThreads) {
-      const int ch = i / (S / 4), u = 4 * (i - ch * (S / 4));
-      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-      if constexpr (MODE == kConvL2) {
+  // stage st's weights and (layers 3, 2 backward) input channels into buffer st & 1
+  auto fetch = [&](int st) {
+    const int c0 = st * kStage;
+    const float* w = a.w + c0 * kK * kC;
+    for (int i = tid; i < kStage * kK * kC / 4; i += kConvThreads)
+      __pipeline_memcpy_async(sW[st & 1] + 4 * i, w + 4 * i, 16);
+    if constexpr (MODE != kConvL2) {
+      for (int i = tid; i < kStage * (S / 4); i += kConvThreads) {
+        const int ch = i / (S / 4), u = 4 * (i - ch * (S / 4));
+        const int t = MODE == kConvL3 ? p0 + u : p0 - 32 + u;   // a compact layer-2 position
+        const bool in = t >= 0 && t < n2;
+        const float* row = a.in + rows + (size_t)(c0 + ch) * W;
+        __pipeline_memcpy_async(sIn[st & 1] + ch * SP + padded(u), row + (in ? t : 0), 16, in ? 0 : 16);
+      }
+    }
+    __pipeline_commit();
+  };
+  constexpr int kStages = kC / kStage;
+  fetch(0);
+  __syncthreads();   // x and the layer-1 weights
+#pragma unroll 1
+  for (int st = 0; st < kStages; ++st) {
+    const int c0 = st * kStage;
+    if (st + 1 < kStages) fetch(st + 1);
+    if constexpr (MODE == kConvL2) {
+      for (int i = tid; i < kStage * (S / 4); i += kConvThreads) {
+        const int ch = i / (S / 4), u = 4 * (i - ch * (S / 4));
         const float* w1 = sW1 + (c0 + ch) * kK;
         float xv[12], r[4];
 #pragma unroll
@@ -156,19 +178,19 @@ __global__ void __launch_bounds__(kConvThreads) net_conv_kernel(const ConvArgs a
 #pragma unroll
           for (int e = 0; e < 4; ++e) r[e] = fmaf(w, xv[e + k], r[e]);
         }
-        v = make_float4(fmaxf(r[0], 0.f), fmaxf(r[1], 0.f), fmaxf(r[2], 0.f), fmaxf(r[3], 0.f));
+        const float4 v = make_float4(fmaxf(r[0], 0.f), fmaxf(r[1], 0.f), fmaxf(r[2], 0.f), fmaxf(r[3], 0.f));
         // the tile keeps its own positions; the last one also the halo beyond layer 2's
         if ((u < kTile || p0 + kTile >= n2) && p0 + u < n1)
           *reinterpret_cast<float4*>(a.h1 + rows + (size_t)(c0 + ch) * W + p0 + u) = v;
-      } else {
-        const int t = MODE == kConvL3 ? p0 + u : p0 - 32 + u;   // a compact layer-2 position
-        if (t >= 0 && t < n2) v = *reinterpret_cast<const float4*>(a.in + rows + (size_t)(c0 + ch) * W + t);
+        *reinterpret_cast<float4*>(sIn[st & 1] + ch * SP + padded(u)) = v;
       }
-      *reinterpret_cast<float4*>(sIn + ch * SP + padded(u)) = v;
     }
+    if (st + 1 < kStages) __pipeline_wait_prior(1);
+    else __pipeline_wait_prior(0);
     __syncthreads();
 #pragma unroll 1
-    for (int i = 0; i < kStage; ++i) conv_channel<D>(acc, sIn + i * SP + x0, sW + i * kK * kC, og);
+    for (int i = 0; i < kStage; ++i) conv_channel<D>(acc, sIn[st & 1] + i * SP + x0, sW[st & 1] + i * kK * kC, og);
+    __syncthreads();   // the buffer is free for stage st + 2
   }
 
   if constexpr (MODE == kConvL2) {
@@ -424,8 +446,7 @@ struct WgArgs {
 // (compact positions).  The positions are cut into equal contiguous ranges of 32-position units, one
 // per CTA; lane = i, warp = 4 output channels, 36 sums per thread in registers over the CTA's whole range.
 __global__ void __launch_bounds__(kWgThreads, 2) net_wgrad2_kernel(const WgArgs a) {
-  __shared__ __align__(16) float sH[kC * kWgPitch];
-  __shared__ __align__(16) float sD[kC * kTile];
+  extern __shared__ __align__(16) float wg_smem[];   // two buffers of h1 rows, then gradient rows
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, W = a.W;
   const int n2 = W / 2 + 128, per = n2 / kWgUnit;
   const int64_t U = (int64_t)a.B * per;
@@ -436,28 +457,46 @@ __global__ void __launch_bounds__(kWgThreads, 2) net_wgrad2_kernel(const WgArgs 
   for (int o = 0; o < 4; ++o)
 #pragma unroll
     for (int k = 0; k < kK; ++k) acc[o][k] = bc(0.f);
-  while (u < u1) {
+  // the next run of units within one window: its first element and length (0: none left)
+  auto take = [&](size_t& rows) -> int {
+    if (u >= u1) return 0;
     const int64_t b = u / per;
     const int q = (int)(u - b * per);
     int len = per - q;                                   // units to the end of the window
     if (len > kTile / kWgUnit) len = kTile / kWgUnit;
     if (len > u1 - u) len = (int)(u1 - u);
     u += len;
-    const int t0 = q * kWgUnit, nt = len * kWgUnit;
-    const size_t rows = (size_t)b * kC * W + t0;
-    __syncthreads();
+    rows = (size_t)b * kC * W + q * kWgUnit;
+    return len * kWgUnit;
+  };
+  auto fetch = [&](int buf, size_t rows, int nt) {
+    float* h = wg_smem + buf * kWgBuffer;
+    float* d = h + kC * kWgPitch;
     const int hc = (nt + kWgHalo) / 4, dc = nt / 4;
     for (int i = tid; i < kC * hc; i += kWgThreads) {
       const int ch = i / hc, m = i - ch * hc;
-      *reinterpret_cast<float4*>(sH + ch * kWgPitch + 4 * m) =
-          *reinterpret_cast<const float4*>(a.h1 + rows + (size_t)ch * W + 4 * m);
+      __pipeline_memcpy_async(h + ch * kWgPitch + 4 * m, a.h1 + rows + (size_t)ch * W + 4 * m, 16);
     }
     for (int i = tid; i < kC * dc; i += kWgThreads) {
       const int ch = i / dc, m = i - ch * dc;
-      *reinterpret_cast<float4*>(sD + ch * kTile + 4 * m) =
-          *reinterpret_cast<const float4*>(a.d2 + rows + (size_t)ch * W + 4 * m);
+      __pipeline_memcpy_async(d + ch * kTile + 4 * m, a.d2 + rows + (size_t)ch * W + 4 * m, 16);
+    }
+    __pipeline_commit();
+  };
+  size_t rows = 0;
+  int nt = take(rows), buf = 0;
+  if (nt) fetch(0, rows, nt);
+  while (nt) {
+    const int nt_next = take(rows);
+    if (nt_next) {
+      fetch(buf ^ 1, rows, nt_next);
+      __pipeline_wait_prior(1);
+    } else {
+      __pipeline_wait_prior(0);
     }
     __syncthreads();
+    const float* sH = wg_smem + buf * kWgBuffer;
+    const float* sD = sH + kC * kWgPitch;
 #pragma unroll 1
     for (int t = 0; t < nt; t += 8) {
       float4 d[4][2];
@@ -481,6 +520,9 @@ __global__ void __launch_bounds__(kWgThreads, 2) net_wgrad2_kernel(const WgArgs 
         }
       }
     }
+    __syncthreads();   // the buffer is free
+    nt = nt_next;
+    buf ^= 1;
   }
   float* out = a.part2 + (size_t)blockIdx.x * (kC * kC * kK);
 #pragma unroll
@@ -648,6 +690,7 @@ Copies copies_of(const NetState& s) { return Copies{s.ph, s.pr, s.packs, s.lay.W
 
 constexpr size_t kHeadTrainSmem = sizeof(float) * kC * (kScatter + 1);
 constexpr size_t kHeadSmem = sizeof(float) * 256 * (kC + 1);
+constexpr size_t kWgSmem = sizeof(float) * 2 * kWgBuffer;
 static_assert(kHeadSmem <= kHeadTrainSmem, "the head's weights share the gradient's space");
 
 void launch_forward(const NetState& s, const float* windows, int B, const float* params, int pack2, int pack3,
@@ -701,6 +744,9 @@ NetSizes net_sizes(int W, int Z, int max_batch, int sm_count) {
 }
 
 cudaError_t net_prepare() {
+  const cudaError_t e =
+      cudaFuncSetAttribute(net_wgrad2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWgSmem);
+  if (e != cudaSuccess) return e;
   return cudaFuncSetAttribute(net_head_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kHeadTrainSmem);
 }
 
@@ -745,7 +791,7 @@ cudaError_t net_train_step(const NetState& s, const float* windows, const float*
   const int tiles1 = tiles_of(W / 2 + 160);
   net_conv_kernel<kConvBwd2><<<dim3(tiles1, B), kConvThreads, 0, st>>>(c);
   const int wg = wg_ctas(s, B);
-  net_wgrad2_kernel<<<wg, kWgThreads, 0, st>>>(WgArgs{s.h1, s.d2, s.part2, B, W});
+  net_wgrad2_kernel<<<wg, kWgThreads, kWgSmem, st>>>(WgArgs{s.h1, s.d2, s.part2, B, W});
   net_sparse_grad_kernel<<<kC * kL3Chunks + kW1Chunks + kHeadChunks * ((Z + 7) / 8), 288, 0, st>>>(
       SparseArgs{s.h2, s.seed, s.arg, s.pooled, s.dlog, s.part1, s.sum1, s.part3, s.gl, B, W, Z, B * tiles1});
 
