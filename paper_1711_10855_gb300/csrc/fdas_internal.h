@@ -114,7 +114,11 @@ bool pairs_supported(int L);
 // Single spectrum restricted to a list of pairs s*Z + z (checked on the device first).
 cudaError_t launch_pairs(int L, const PairParams& p, int sm_count, cudaStream_t stream);
 
-// Launch helpers (defined in fdas_convolve.cu).  Return a cudaError_t from the launch.
+// Launch helpers (defined in fdas_convolve.cu).  Return a cudaError_t from the launch.  The segment length
+// alone picks the kernel: 2048 and the short ones give every lane a pair of columns of the second pass
+// (16-byte exchange entries); 1024, 4096 and 8192 have as many lanes as columns or more
+// (fdas_convolve_wide.cu; 1024 with pairs of columns, 16 lanes and everything in shared memory took 611
+// us where it now takes 482).
 cudaError_t launch_convolve(int L, const ConvParams& p, int sm_count, cudaStream_t stream);
 cudaError_t launch_segment_spectra(int L, const SegParams& p, int sm_count, cudaStream_t stream);
 // Tensor-core variant for L = 2048 (fdas_tc.cu): inverse transforms as DFT-matrix contractions.

@@ -15,6 +15,10 @@
 // loads over all banks for D = 4 and D = 16.  The next stage's operands are copied asynchronously while one
 // is computed: with one buffer a fifth to a quarter of the warps' time went to waiting for them.
 //
+// A step on 256 windows of 1024 (Z = 201) takes 316 us, of which the four convolutions are about 260 at
+// 60-65% of the FP32 pipe; with every position in every layer, dense gradients and untiled loops it
+// took 3.46 ms.
+//
 // Every reduction has a fixed shape, so one seed gives one network.
 #include <cuda_fp16.h>
 #include <cuda_pipeline.h>
