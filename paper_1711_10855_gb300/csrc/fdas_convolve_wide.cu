@@ -304,6 +304,7 @@ __global__ void __launch_bounds__(32 * Cfg::W, 1) fdas_convolve_wide_kernel(cons
     }
     seg_in_flight = true;
     alive = __syncthreads_and(mbar_wait(segbar, seg_phase) ? 1 : 0);
+    tmem_fence_after_sync();   // the twiddles were stored by other warps
     if (!alive) {
       if (tid == 0) report_timeout(p.status, abort_flag);
       break;
