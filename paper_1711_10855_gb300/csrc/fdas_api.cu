@@ -22,7 +22,7 @@ struct fdas_plan {
   void* memory = nullptr;            // one allocation holding the four buffers below
   float2* d_templates = nullptr;     // Z x L complex64, IFFT first-pass layout
   double2* d_taps = nullptr;         // Z x (m+1) complex128 normalised taps
-  float2* d_twist = nullptr;         // L complex64 inter-pass twiddles, same layout
+  float2* d_twist = nullptr;         // L complex64 inter-pass twiddles (twist_re)
   int* d_status = nullptr;
   bool built = false;
   // tensor-core variant (fdas_convolve_power_tc), allocated on its first call

@@ -46,12 +46,11 @@ namespace fdas {
 // ---------------------------------------------------------------------------------------
 // Shared per-lane pieces of the transform
 //
-// Buffer layout of a segment spectrum, a template spectrum and the twiddle table (L complex
-// values each), "pair-major structure of arrays": lane k1 of the first pass owns the pairs
+// Buffer layout of a segment spectrum and a template spectrum (L complex values each), "pair-major structure of arrays": lane k1 of the first pass owns the pairs
 // p = 0..H2-1; pair p of lane k1 is the float4 at index p*N1 + k1 holding
 // (re(e0), re(e1), im(e0), im(e1)).  For spectra and templates e0, e1 are the elements
-// k = k1 + N1*(2p) and k1 + N1*(2p+1); for the twiddle table they are exp(+i 2pi n2 k1 / L)
-// for n2 = p and p + H2.  One 128-bit load gives a packed pair ready for f32x2 arithmetic.
+// k = k1 + N1*(2p) and k1 + N1*(2p+1); the twiddle table's order is twist_re's.  One 128-bit load gives
+// a packed pair ready for f32x2 arithmetic.
 // ---------------------------------------------------------------------------------------
 
 struct NoHook {
@@ -122,14 +121,14 @@ __device__ __forceinline__ void forward_to_tmem(const float2* sx, float4* xb, in
 }
 
 // Twiddle pairs of lane k1's columns: entry r*N1 + slot = those of column pair r for the lane that
-// slot stands for (the plan's table holds pair j of lane s at j*N1 + s).
+// slot stands for (contiguous over the lanes: twist_re).
 template <class Cfg>
 __device__ __forceinline__ void load_column_twiddles(float4 (&tw)[Cfg::H2], const float2* twist, int k1) {
   constexpr int N1 = Cfg::N1;
   const float4* tw4 = reinterpret_cast<const float4*>(twist);
   static_for<Cfg::H2>([&](auto ii) {
     constexpr int i = decltype(ii)::value, r = i / N1, src = slot_pair(i % N1, N1);
-    tw[i] = __ldg(tw4 + (r * N1 + k1) * N1 + src);
+    tw[i] = __ldg(tw4 + (r * N1 + src) * N1 + k1);
   });
 }
 

@@ -156,20 +156,25 @@ __device__ __forceinline__ int64_t first_unit(const ConvParams& p, int Z, unsign
 }
 
 // Twiddle pairs of a lane (the plan's table holds exp(i 2pi n2 k1 / L) for n2 = j, j + H2 as pair j of
-// lane k1).  Split columns: that pair j.  Otherwise the pairs of k1 = 2 kappa, 2 kappa + 1 of the lane's
-// column n2, in slot order.
+// lane k1, contiguous over the lanes).  Split columns: that pair j.  Otherwise the pairs of k1 = 2 kappa,
+// 2 kappa + 1 of the lane's column n2, in slot order; N1 = N2 makes the table symmetric, so they are the
+// lane's own pairs with n2 and k1 exchanged.
 template <class Cfg>
 __device__ __forceinline__ void load_lane_twiddles(float4 (&tw)[Cfg::H2], const float2* twist, int lane_k1) {
-  if constexpr (Cfg::SPLIT == 2) {
-    const float4* tw4 = reinterpret_cast<const float4*>(twist);
-    static_for<Cfg::H2>([&](auto jj) { tw[decltype(jj)::value] = __ldg(tw4 + decltype(jj)::value * Cfg::N1 + lane_k1); });
-  } else {
-    const float* f = reinterpret_cast<const float*>(twist) + (lane_k1 % Cfg::H2) * Cfg::N1 * 4 + lane_k1 / Cfg::H2;
-    static_for<Cfg::H2>([&](auto ii) {
-      constexpr int i = decltype(ii)::value, k = 2 * slot_pair(i, Cfg::H2);
-      tw[i] = make_float4(__ldg(f + 4 * k), __ldg(f + 4 * (k + 1)), __ldg(f + 4 * k + 2), __ldg(f + 4 * (k + 1) + 2));
-    });
-  }
+  float4 own[Cfg::H2];
+  const float4* tw4 = reinterpret_cast<const float4*>(twist);
+  static_for<Cfg::H2>([&](auto jj) { own[decltype(jj)::value] = __ldg(tw4 + decltype(jj)::value * Cfg::N1 + lane_k1); });
+  static_for<Cfg::H2>([&](auto ii) {
+    constexpr int i = decltype(ii)::value, k = 2 * slot_pair(i, Cfg::H2);
+    if constexpr (Cfg::SPLIT == 2) {
+      tw[i] = own[i];
+    } else if constexpr (k < Cfg::H2) {
+      tw[i] = make_float4(own[k].x, own[k + 1].x, own[k].z, own[k + 1].z);
+    } else {
+      const float4 a = own[k - Cfg::H2], b = own[k + 1 - Cfg::H2];
+      tw[i] = make_float4(a.y, b.y, a.w, b.w);
+    }
+  });
 }
 
 // NV (eighths of the rows): pass-2 rows n1 >= NV*N1/8 hold no valid output and are dropped at compile

@@ -16,7 +16,7 @@ constexpr int kStatusBadList = 2;   // a work list failed its check and was not 
 struct ConvParams {
   const float2* spectrum;   // n_bins complex64 (read by bulk copies in the descriptor-driven kernel)
   const float2* templates;  // Z x L template spectra, per-template layout of the IFFT's first pass
-  const float2* twist;      // L inter-pass twiddles exp(+i 2pi n2 k1 / L), same layout
+  const float2* twist;      // L inter-pass twiddles exp(+i 2pi n2 k1 / L) (twist_re)
   float* plane;             // Z x n_bins output, row pitch n_bins
   int* status;              // device status word (kStatusTimeout | kStatusBadList)
   int64_t n_bins;
@@ -44,7 +44,7 @@ struct SpecDesc {
 // Parameters of the descriptor-driven fused kernel (TMEM variant): one or many spectra.
 struct BatchParams {
   const float2* templates;  // Z_bank x L template spectra (pair-major layout)
-  const float2* twist;      // L inter-pass twiddles (pair-major layout)
+  const float2* twist;      // L inter-pass twiddles (twist_re)
   int* status;              // device status word (kStatusTimeout | kStatusBadList)
   const SpecDesc* descs;    // device table of `count` spectra, or nullptr: use `single`
   SpecDesc single;
@@ -74,7 +74,7 @@ struct PairParams {
   const float2* spec;       // n_bins complex64, 16-byte aligned
   float* plane;             // Z x n_bins float32, row pitch n_bins
   const float2* templates;  // Z x L template spectra (pair-major layout)
-  const float2* twist;      // L inter-pass twiddles (pair-major layout)
+  const float2* twist;      // L inter-pass twiddles (twist_re)
   int* status;              // device status word (kStatusTimeout | kStatusBadList)
   const int32_t* pairs;     // ascending entries s*Z + z
   const int64_t* pair_count;  // list length in device memory (checked), or nullptr: n_pairs
@@ -99,6 +99,19 @@ struct SegParams {
 // twiddle table are stored in the layout of that decomposition (element k = k1 + N1*k2 at
 // ((k2/2)*N1 + k1)*2 + k2%2).
 int conv_group_threads(int L);
+
+// Float offset of the real part of the twiddle exp(+i 2pi n2 k1 / L), n2 < N2 = 2*h2, k1 < n1, in the plan's
+// table (the imaginary part is 2 floats further): a float4 (re, re, im, im) holds n2 = j and j + h2.  The
+// kernels whose lanes own column pairs of the second pass (n1 <= h2: 256, 512 and 2048) read the pair of
+// column j = r*n1 + t for one k1 at a time, lane t: entry (r*n1 + k1)*n1 + t.  The others read one k1 or
+// one column per lane (the table is symmetric where n1 = N2): entry j*n1 + k1.  Either way a warp's load is
+// one contiguous row; with the second order in all of them a warp touched 32 lines per load, which cost a
+// CTA's start 3,400 cycles at 2048 and 11,500 at 4096 (4096 bins, one template: 14.4 us where it takes 12.3,
+// and 20.5 us where it takes 12.4).
+__host__ __device__ inline int twist_re(int n2, int k1, int n1, int h2) {
+  const int j = n2 % h2, e = n1 <= h2 ? (j / n1 * n1 + k1) * n1 + j % n1 : j * n1 + k1;
+  return 4 * e + n2 / h2;
+}
 
 // Segments resident per CTA of the descriptor-driven kernel for segment length L, or 0 if L has
 // no descriptor-driven kernel (then only the single-spectrum plan path serves it).
@@ -127,7 +140,7 @@ struct TcParams {
   float2* seg_out;          // the same, written by the forward pass
   const float2* spectrum;   // n_bins complex64 (forward pass)
   const float2* bank;       // Z x 2048 template spectra, natural order
-  const float2* twist;      // the plan's twist table (pair-major layout, N1 = 32)
+  const float2* twist;      // the plan's twist table
   const unsigned char* mats;  // DFT matrices of the precision and direction, operand layout (hi, lo)
   const unsigned* tmax;     // bits of max |Re|, |Im| over the bank
   float* plane;

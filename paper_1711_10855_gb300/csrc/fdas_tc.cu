@@ -200,13 +200,12 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_convolve_kernel(const TcPara
     const uint4* src = reinterpret_cast<const uint4*>(p.mats);
     uint4* dst = reinterpret_cast<uint4*>(sm + kOffW1h);
     for (int i = tid; i < kMatBytes / 16; i += kTcThreads) dst[i] = __ldg(src + i);
-    // the plan's table holds w2048^(k1 n2) at float ((n2 % 32) * 32 + k1) * 4 + n2 / 32, Im + 2
     const float* tw = reinterpret_cast<const float*>(p.twist);
     float4* tdst = reinterpret_cast<float4*>(sm + kOffTw);
     const float s2 = PREC == 1 ? 0.015625f : 1.f, s2i = FWD ? -s2 : s2;
     for (int i = tid; i < kTL / 2; i += kTcThreads) {
       const int j = i >> 6, n2 = i & 63;
-      const int off0 = ((n2 & 31) * 32 + 2 * j) * 4 + (n2 >> 5), off1 = off0 + 4;   // k1 = 2j, 2j + 1
+      const int off0 = twist_re(n2, 2 * j, 32, 32), off1 = twist_re(n2, 2 * j + 1, 32, 32);
       tdst[i] = make_float4(__ldg(tw + off0) * s2, __ldg(tw + off1) * s2, __ldg(tw + off0 + 2) * s2i,
                             __ldg(tw + off1 + 2) * s2i);
     }

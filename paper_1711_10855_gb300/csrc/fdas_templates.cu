@@ -117,14 +117,12 @@ struct BankShape {
   int gc;     // nodes per chunk
 };
 
-// Inter-pass twiddles exp(+i 2pi n2 k1 / L), n2 < N2 = L/n1, k1 < n1: lane k1's pair j holds
-// n2 = j and n2 = j + N2/2 (float4 at j*n1 + k1: re, re, im, im).
+// Inter-pass twiddles exp(+i 2pi n2 k1 / L), n2 < N2 = L/n1, k1 < n1, where twist_re puts them.
 __device__ void write_twist(float2* tw, int idx, int L, int n1) {
   const int k1 = idx % n1, n2 = idx / n1;
-  const int h2 = L / n1 / 2;
   const double2 w = cispi(2.0 * (double)(((long long)n2 * k1) % L) / (double)L);
   float* dst = reinterpret_cast<float*>(tw);
-  const int off = ((n2 % h2) * n1 + k1) * 4 + n2 / h2;
+  const int off = fdas::twist_re(n2, k1, n1, L / n1 / 2);
   dst[off] = (float)w.x;
   dst[off + 2] = (float)w.y;
 }

@@ -1,0 +1,62 @@
+"""Layouts that the host side and several kernels share, checked by a small program compiled from the
+library's own header: what one warp loads at a time is one contiguous row."""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+NVCC = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+
+TWIST = r"""
+#include <cstdio>
+#include <vector>
+#include "fdas_internal.h"
+// 0: every twiddle has a place of its own and every warp load is contiguous (float4 by float4)
+int check(int L, int n1, bool columns) {
+  const int N2 = L / n1, h2 = N2 / 2;
+  std::vector<int> seen(2 * L, 0);
+  for (int n2 = 0; n2 < N2; ++n2)
+    for (int k1 = 0; k1 < n1; ++k1) {
+      const int at = fdas::twist_re(n2, k1, n1, h2);
+      if (at < 0 || at + 2 >= 2 * L || seen[at]++ || seen[at + 2]++) return 1;
+      // the pair (j, j + h2) is one float4: re, re, im, im
+      if (n2 < h2 && (at % 4 != 0 || fdas::twist_re(n2 + h2, k1, n1, h2) != at + 1)) return 2;
+    }
+  if (columns) {   // lane t loads column pair r*n1 + t for one k1 at a time
+    for (int r = 0; r < h2 / n1; ++r)
+      for (int k1 = 0; k1 < n1; ++k1)
+        for (int t = 0; t < n1; ++t)
+          if (fdas::twist_re(r * n1 + t, k1, n1, h2) != fdas::twist_re(r * n1, k1, n1, h2) + 4 * t) return 3;
+  } else {         // lane k1 loads pair j
+    for (int j = 0; j < h2; ++j)
+      for (int k1 = 0; k1 < n1; ++k1)
+        if (fdas::twist_re(j, k1, n1, h2) != fdas::twist_re(j, 0, n1, h2) + 4 * k1) return 4;
+  }
+  return 0;
+}
+int main() {
+  const int len[6] = {256, 512, 1024, 2048, 4096, 8192}, lanes[6] = {8, 16, 32, 32, 64, 128};
+  const bool columns[6] = {true, true, false, true, false, false};
+  for (int i = 0; i < 6; ++i)
+    if (int rc = check(len[i], lanes[i], columns[i])) return std::printf("L = %d: %d\n", len[i], rc), 1;
+  return 0;
+}
+"""
+
+
+def run(tmp_path, source):
+    if not os.path.exists(NVCC):
+        pytest.skip("no nvcc")
+    src, exe = tmp_path / "t.cu", tmp_path / "t"
+    src.write_text(source)
+    inc = ["-I" + os.path.join(ROOT, "include"), "-I" + os.path.join(ROOT, "paper_1711_10855_gb300", "csrc")]
+    subprocess.run([NVCC, "-std=c++17", "-gencode", "arch=compute_103a,code=sm_103a", *inc, str(src), "-o", str(exe)],
+                   check=True)
+    r = subprocess.run([str(exe)], capture_output=True, text=True)
+    assert r.returncode == 0, r.stdout
+
+
+def test_twiddle_table_is_contiguous_over_the_lanes_of_a_load(tmp_path):
+    run(tmp_path, TWIST)
