@@ -201,12 +201,22 @@ struct NetLayout {
 // Packed copies of the 32 x 32 x 9 weights, each [32 inputs of the pass][9 taps][32 outputs].
 enum { kPackW2, kPackW3, kPackW2Back, kPackW3Back, kPackW2Half, kPackW3Half, kNetPacks };
 
+// The inference kernel's FP16 image of the weights of layers 2 and 3: [layer][4 planes of 8 input
+// channels][480 rows][8], row 32 b + o = output channel o of tap 11 - b, zero where that is no tap (the
+// stack [0 0 0 W_8 ... W_0 0 0 0] of fdas_zband.cu).
+constexpr int kStackRows = 15 * kNetC;
+constexpr int kStackHalves = 2 * 4 * kStackRows * 8;
+__host__ __device__ inline int stack_at(int layer, int o, int i, int k) {
+  return ((layer * 4 + (i >> 3)) * kStackRows + (11 - k) * kNetC + o) * 8 + (i & 7);
+}
+
 struct NetState {
   NetLayout lay{0};
   int W = 0, sm_count = 0;
   float* p = nullptr;          // FP32 master parameters
   __half* ph = nullptr;        // FP16 copy for inference
   float* pr = nullptr;         // the FP16 copy's values as FP32
+  __half* stack = nullptr;     // kStackHalves: layers 2 and 3 for the inference kernel (of ph)
   float* packs = nullptr;      // kNetPacks packed weight matrices (of p, and of pr: *Half)
   float* g = nullptr;          // gradients
   float* m = nullptr;          // Adam moments
@@ -237,7 +247,7 @@ struct NetSizes {
 };
 NetSizes net_sizes(int W, int Z, int max_batch, int sm_count);
 cudaError_t net_prepare();   // function attributes, once per created net
-// The copies (ph, pr, packs) of the parameters p.
+// The copies (ph, pr, stack, packs) of the parameters p.
 void net_publish(const NetState& s, cudaStream_t st);
 cudaError_t net_predict(const NetState& s, const float* windows, int B, bool half_weights, float* logits,
                         cudaStream_t st);

@@ -599,6 +599,7 @@ __global__ void __launch_bounds__(288) net_sparse_grad_kernel(const SparseArgs a
 struct Copies {
   __half* ph;            // FP16 copy
   float* pr;             // its values as FP32
+  __half* stack;         // layers 2 and 3 in the inference kernel's order
   float* packs;          // kNetPacks packed weight matrices
   int W2, W3;            // offsets of the two layers' weights in the parameter vector
 };
@@ -613,6 +614,7 @@ __device__ __forceinline__ void publish(const Copies& c, int idx, float v) {
   if (!l2 && !l3) return;
   const int e = idx - (l2 ? c.W2 : c.W3), o = e / (kC * kK), i = e / kK % kC, k = e % kK;
   const int fwd = (i * kK + k) * kC + o;
+  c.stack[stack_at(l3 ? 1 : 0, o, i, k)] = hv;
   c.packs[(l2 ? kPackW2 : kPackW3) * n + fwd] = v;
   c.packs[(l2 ? kPackW2Half : kPackW3Half) * n + fwd] = r;
   // layer 2's data gradient is a convolution with the taps reversed; layer 3's is scattered tap by tap
@@ -690,7 +692,7 @@ int wg_ctas(const NetState& s, int B) {
   const int64_t units = (int64_t)B * ((s.W / 2 + 128) / kWgUnit);
   return (int)(units < 2 * s.sm_count ? units : 2 * s.sm_count);
 }
-Copies copies_of(const NetState& s) { return Copies{s.ph, s.pr, s.packs, s.lay.W2, s.lay.W3}; }
+Copies copies_of(const NetState& s) { return Copies{s.ph, s.pr, s.stack, s.packs, s.lay.W2, s.lay.W3}; }
 
 constexpr size_t kHeadTrainSmem = sizeof(float) * kC * (kScatter + 1);
 constexpr size_t kHeadSmem = sizeof(float) * 256 * (kC + 1);

@@ -45,6 +45,30 @@ int main() {
 }
 """
 
+STACK = r"""
+#include <cstdio>
+#include <vector>
+#include "fdas_internal.h"
+int main() {
+  std::vector<int> seen(fdas::kStackHalves, 0);
+  for (int layer = 0; layer < 2; ++layer)
+    for (int o = 0; o < 32; ++o)
+      for (int i = 0; i < 32; ++i)
+        for (int k = 0; k < 9; ++k) {
+          const int at = fdas::stack_at(layer, o, i, k);
+          if (at < 0 || at >= fdas::kStackHalves || seen[at]++) return std::puts("place"), 1;
+        }
+  // plane j, row 32 b + o: tap 11 - b of input channels 8j .. 8j + 7, and nothing where that is no tap
+  for (int at = 0; at < fdas::kStackHalves; ++at) {
+    const int e = at % 8, row = at / 8 % 480, j = at / (8 * 480) % 4, layer = at / (8 * 480 * 4), k = 11 - row / 32;
+    const bool tap = k >= 0 && k < 9;
+    if (seen[at] != (tap ? 1 : 0)) return std::puts("zero blocks"), 1;
+    if (tap && fdas::stack_at(layer, row % 32, 8 * j + e, k) != at) return std::puts("row"), 1;
+  }
+  return 0;
+}
+"""
+
 
 def run(tmp_path, source):
     if not os.path.exists(NVCC):
@@ -60,3 +84,7 @@ def run(tmp_path, source):
 
 def test_twiddle_table_is_contiguous_over_the_lanes_of_a_load(tmp_path):
     run(tmp_path, TWIST)
+
+
+def test_inference_weight_image_is_a_straight_copy(tmp_path):
+    run(tmp_path, STACK)
