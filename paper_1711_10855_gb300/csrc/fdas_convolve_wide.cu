@@ -181,7 +181,7 @@ __device__ __forceinline__ void load_lane_twiddles(float4 (&tw)[Cfg::H2], const 
 // time.  FWD: only the forward transforms, natural order, into p.plane (complex64).
 template <class Cfg, int NV, bool FWD>
 __global__ void __launch_bounds__(32 * Cfg::W, 1) fdas_convolve_wide_kernel(const ConvParams p) {
-  constexpr int L = Cfg::L, N1 = Cfg::N1, N2 = Cfg::N2, H2 = Cfg::H2, R = Cfg::R, G = Cfg::G, W = Cfg::W;
+  constexpr int L = Cfg::L, N1 = Cfg::N1, N2 = Cfg::N2, H2 = Cfg::H2, R = Cfg::R, W = Cfg::W;
   constexpr int M = Cfg::M, PARTS = Cfg::PARTS, RS = Cfg::SPLIT;
   extern __shared__ __align__(1024) unsigned char smem[];
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + Cfg::OFF_BAR);
@@ -210,9 +210,9 @@ __global__ void __launch_bounds__(32 * Cfg::W, 1) fdas_convolve_wide_kernel(cons
 
   // a2: bulk copies of the in-range part of every segment of the group, one lane per segment
   auto fetch_segments = [&]() {   // a whole warp
-    const int64_t x0 = (grp * G + lane) * (int64_t)p.V - p.h;
+    const int64_t x0 = (grp * p.segs + lane) * (int64_t)p.V - p.h;
     const int64_t c0 = x0 > 0 ? x0 : 0, c1 = x0 + L < p.n_bins ? x0 + L : p.n_bins;
-    const uint32_t bytes = lane < G && c1 > c0 ? (uint32_t)((c1 - c0) * 8) : 0u;
+    const uint32_t bytes = lane < p.segs && c1 > c0 ? (uint32_t)((c1 - c0) * 8) : 0u;
     const uint32_t total = __reduce_add_sync(0xffffffffu, bytes);
     if (lane == 0) mbar_arrive_expect_tx(segbar, total);
     __syncwarp();
@@ -296,17 +296,11 @@ __global__ void __launch_bounds__(32 * Cfg::W, 1) fdas_convolve_wide_kernel(cons
       if (!alive) break;
       if (warp == 0) fetch_segments();
     }
-    const int64_t s = grp * G + g;
+    const int64_t s = grp * p.segs + g;
     const int64_t segbase = s * (int64_t)p.V;
-    {
-      // zeros outside [0, n) in this transform's window
-      const int64_t x0 = segbase - p.h;
-      const int64_t lo = x0 < 0 ? (-x0 < L ? -x0 : L) : 0;
-      const int64_t hi = p.n_bins - x0 < L ? (p.n_bins - x0 > 0 ? p.n_bins - x0 : 0) : L;
-      if (lo > 0 || hi < L)
-        for (int e = k1; e < L; e += N1)
-          if (e < lo || e >= hi) mySeg[e] = make_float2(0.f, 0.f);
-    }
+    // the warps of a transform without a segment only keep the barriers and the ring going
+    const bool on = g < p.segs && s < p.nseg;
+    if (on) zero_outside<L>(mySeg, segbase - p.h, p.n_bins, k1, N1);
     seg_in_flight = true;
     alive = __syncthreads_and(mbar_wait(segbar, seg_phase) ? 1 : 0);
     tmem_fence_after_sync();   // the twiddles were stored by other warps
@@ -318,7 +312,7 @@ __global__ void __launch_bounds__(32 * Cfg::W, 1) fdas_convolve_wide_kernel(cons
     seg_phase ^= 1u;
 
     // a3: forward FFT; lane k1's elements X[k1 + N1*k2] end in the lane itself: pairs (2q, 2q + 1) to TMEM
-    {
+    if (on) {
       cp2 v[H2], x[M / 2];
       static_for<H2>([&](auto ii) {
         constexpr int i = decltype(ii)::value;
@@ -330,17 +324,12 @@ __global__ void __launch_bounds__(32 * Cfg::W, 1) fdas_convolve_wide_kernel(cons
       exchange_pass2<Cfg, -1>(v, x, tile, g, k1, n2, c_fwd, tw_addr);
       if constexpr (FWD) {
         float2* out = reinterpret_cast<float2*>(p.plane) + s * L;
-        if (s < p.nseg)
-          static_for<M / 2>([&](auto jj) {
-            constexpr int j = decltype(jj)::value;
-            out[k1 + N1 * j] = make_float2(x[j].re.x, x[j].im.x);
-            out[k1 + N1 * (j + M / 2)] = make_float2(x[j].re.y, x[j].im.y);
-          });
-        ++grp;
-        tmem_fence_before_sync();
-        continue;
-      }
-      spectrum_to_tmem<H2>(x_addr, [&](auto pp) {
+        static_for<M / 2>([&](auto jj) {
+          constexpr int j = decltype(jj)::value;
+          out[k1 + N1 * j] = make_float2(x[j].re.x, x[j].im.x);
+          out[k1 + N1 * (j + M / 2)] = make_float2(x[j].re.y, x[j].im.y);
+        });
+      } else spectrum_to_tmem<H2>(x_addr, [&](auto pp) {
         constexpr int k2 = 2 * decltype(pp)::value;   // members k2 and k2 + 1: both in .x or both in .y
         constexpr int j = k2 < M / 2 ? k2 : k2 - M / 2;
         if constexpr (k2 < M / 2)
@@ -350,9 +339,33 @@ __global__ void __launch_bounds__(32 * Cfg::W, 1) fdas_convolve_wide_kernel(cons
       });
     }
 
+    if constexpr (FWD) {
+      ++grp;
+      tmem_fence_before_sync();
+      continue;
+    }
+
     const int64_t lim64 = p.n_bins - segbase < (int64_t)p.V ? p.n_bins - segbase : (int64_t)p.V;
     int lim = lim64 > 0 ? (int)lim64 : 0;   // outputs n < lim of this segment are stored
-    for (int64_t i = a; i < bpos; ++i, ++z) {
+    // release the slot of ring position e; the last of the W consumers refills it R positions ahead
+    auto release_part = [&](int64_t e, int slot, int ok) {
+      __syncwarp();
+      if (lane == 0) {
+        const unsigned old = arrive_count(&cnt[slot]);
+        if ((old + 1u) % (unsigned)W == 0u && e + R < npos * PARTS && ok) {
+          fence_proxy_async_smem();
+          issue_part(e + R);
+        }
+      }
+    };
+    if (!on) {
+      for (int64_t e = a * PARTS; e < bpos * PARTS; ++e) {
+        const int slot = (int)(e % R);
+        const int ok = __all_sync(0xffffffffu, wait_slot(&full[slot], (uint32_t)((e / R) & 1), abort_flag));
+        if (!ok && lane == 0) report_timeout(p.status, abort_flag);
+        release_part(e, slot, ok);
+      }
+    } else for (int64_t i = a; i < bpos; ++i, ++z) {
       // a4: Y = X (TMEM) * T (shared ring), packed pairs in bit-reversed order.  A wait that gives up ends
       // the stores, not the loop: the warps of a transform keep meeting at their barriers until the
       // group ends.
@@ -372,15 +385,7 @@ __global__ void __launch_bounds__(32 * Cfg::W, 1) fdas_convolve_wide_kernel(cons
           constexpr int first = part * Cfg::PART_PAIRS / 2;
           return st4[(q < H2 / 2 ? q - first : q - H2 / 2 - first + Cfg::PART_PAIRS / 2) * N1 + k1];
         });
-        // release the slot; the last of the W consumers refills it R positions ahead
-        __syncwarp();
-        if (lane == 0) {
-          const unsigned old = arrive_count(&cnt[slot]);
-          if ((old + 1u) % (unsigned)W == 0u && e + R < npos * PARTS && ok) {
-            fence_proxy_async_smem();
-            issue_part(e + R);
-          }
-        }
+        release_part(e, slot, ok);
       });
       // a5: inverse FFT
       fft_split_pairs<N2, +1, 1>(v);
@@ -426,7 +431,10 @@ cudaError_t launch_wide(const ConvParams& p, int sm_count, cudaStream_t st) {
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::SMEM);
   if (e != cudaSuccess) return e;
   ConvParams q = p;
-  const int64_t ngroups = (p.nseg + Cfg::G - 1) / Cfg::G;
+  // With G segments per CTA always, and transforms of segments that do not exist, 4096 bins took: one template
+  // at 4096 12.4 us (now 9.3) and at 8192 16.4 us (10.3), 201 templates at 1024 14.4 us (10.3).
+  q.segs = FWD ? Cfg::G : wide_segments(p.nseg, p.Z, Cfg::G, sm_count);
+  const int64_t ngroups = (p.nseg + q.segs - 1) / q.segs;
   const int64_t units = FWD ? ngroups : ngroups * p.Z;
   const int64_t grid = units < sm_count ? units : sm_count;
   q.group_cost = !FWD && units > grid ? 1 : 0;   // about one position

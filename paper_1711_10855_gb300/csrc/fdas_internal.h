@@ -27,6 +27,7 @@ struct ConvParams {
   int64_t span;
   int span_extra;
   int group_cost;
+  int segs;                 // segments per group (set by the launch; fdas_convolve_wide.cu)
 };
 
 // One spectrum of a batch, as the persistent kernel reads it (device table or inline).
@@ -99,6 +100,14 @@ struct SegParams {
 // twiddle table are stored in the layout of that decomposition (element k = k1 + N1*k2 at
 // ((k2/2)*N1 + k1)*2 + k2%2).
 int conv_group_threads(int L);
+
+// Segments per group of a full plane at 1024, 4096 and 8192, at most `most` (those a CTA has room for): while
+// every unit has an SM of its own, halved, since a CTA's warps then share its four schedulers with fewer others.
+inline int wide_segments(int64_t nseg, int Z, int most, int sm_count) {
+  int segs = most;
+  while (segs > 1 && (nseg + segs / 2 - 1) / (segs / 2) * Z <= sm_count) segs /= 2;
+  return segs;
+}
 
 // Float offset of the real part of the twiddle exp(+i 2pi n2 k1 / L), n2 < N2 = 2*h2, k1 < n1, in the plan's
 // table (the imaginary part is 2 floats further): a float4 (re, re, im, im) holds n2 = j and j + h2.  The

@@ -69,6 +69,24 @@ int main() {
 }
 """
 
+SEGMENTS = r"""
+#include <cstdio>
+#include "fdas_internal.h"
+int main() {
+  for (int sms : {148, 152})
+    for (int most : {2, 4, 16})
+      for (int64_t nseg = 1; nseg < 3000; nseg += 1 + nseg / 40)
+        for (int Z = 1; Z <= 401; Z += 2) {
+          const int s = fdas::wide_segments(nseg, Z, most, sms);
+          const auto units = [&](int k) { return (nseg + k - 1) / k * Z; };
+          const bool full = s == most, fits = units(s) <= sms, half_fits = s > 1 && units(s / 2) <= sms;
+          if (s < 1 || s > most || most % s || !(full || fits) || half_fits)
+            return std::printf("%ld segments x %d, %d: %d\n", (long)nseg, Z, most, s), 1;
+        }
+  return 0;
+}
+"""
+
 
 def run(tmp_path, source):
     if not os.path.exists(NVCC):
@@ -88,3 +106,7 @@ def test_twiddle_table_is_contiguous_over_the_lanes_of_a_load(tmp_path):
 
 def test_inference_weight_image_is_a_straight_copy(tmp_path):
     run(tmp_path, STACK)
+
+
+def test_fewest_segments_per_cta_while_every_unit_has_an_sm(tmp_path):
+    run(tmp_path, SEGMENTS)
