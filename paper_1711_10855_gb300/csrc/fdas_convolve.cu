@@ -210,15 +210,9 @@ __device__ __forceinline__ int64_t unit_total(const BatchParams& p) { return p.u
 __device__ __forceinline__ int64_t unit_total(const ListParams& p) { return p.unit_count ? *p.unit_count : p.units; }
 
 // First unit of CTA k.  The units are cut into equal ranges; one spectrum's groups count group_cost
-// more units each (what fetching and transforming a group's segments costs), so that a CTA whose
-// range enters a second group gets fewer templates.
+// units more each.  A batch's do not: its spectra have their own template counts, and its CTAs many positions.
 __device__ __forceinline__ int64_t first_unit(const BatchParams& p, unsigned k) {
-  const int64_t v = (int64_t)k * p.span + (k < (unsigned)p.span_extra ? k : (unsigned)p.span_extra);
-  if (p.group_cost == 0) return v;
-  const int per = p.single.Z + p.group_cost;
-  const int64_t g = quotient(v, per);
-  const int64_t r = v - g * per - p.group_cost;
-  return g * p.single.Z + (r > 0 ? r : 0);
+  return first_unit_of(k, p.span, p.span_extra, p.group_cost, p.single.Z);
 }
 
 // NV: pass-2 output rows n1 < NV can hold valid outputs (NV >= ceil(V / N2)); rows n1 >= NV are
@@ -868,9 +862,9 @@ static cudaError_t launch_tmem_nv(const ListParams& p, int sm_count, cudaStream_
     if (p.unit_list) return launch(fdas_convolve_tmem_kernel<ListCfg, NV, true>, ListCfg::W, ListCfg::SMEM, p);
   }
   BatchParams q = p;
-  // a group's start costs about one position (its forward transforms; two with P = 2, where half of the
-  // warps run them)
-  if (q.descs == nullptr && q.units > grid) q.group_cost = PlaneCfg::P;
+  // (P = 2: two positions, half of the warps run the forward transforms)
+  if (q.descs == nullptr && q.units > grid)
+    q.group_cost = PlaneCfg::P == 2 ? 2 : group_cost_of(q.units, q.single.ngroups, grid);
   const int64_t total = q.units + q.group_cost * q.single.ngroups;
   q.span = total / grid;
   q.span_extra = (int)(total % grid);

@@ -148,11 +148,7 @@ __device__ __forceinline__ void exchange_pass2(cp2 (&v)[Cfg::H2], cp2 (&u)[Cfg::
 // First unit of CTA k: the units are cut into equal ranges, every segment group counting group_cost
 // units more than its templates (what fetching and transforming its segments costs).
 __device__ __forceinline__ int64_t first_unit(const ConvParams& p, int Z, unsigned k) {
-  const int64_t v = (int64_t)k * p.span + (k < (unsigned)p.span_extra ? k : (unsigned)p.span_extra);
-  if (p.group_cost == 0) return v;
-  const int per = Z + p.group_cost;
-  const int64_t g = quotient(v, per), r = v - g * per - p.group_cost;
-  return g * Z + (r > 0 ? r : 0);
+  return first_unit_of(k, p.span, p.span_extra, p.group_cost, Z);
 }
 
 // Twiddle pairs of a lane (the plan's table holds exp(i 2pi n2 k1 / L) for n2 = j, j + H2 as pair j of
@@ -437,7 +433,7 @@ cudaError_t launch_wide(const ConvParams& p, int sm_count, cudaStream_t st) {
   const int64_t ngroups = (p.nseg + q.segs - 1) / q.segs;
   const int64_t units = FWD ? ngroups : ngroups * p.Z;
   const int64_t grid = units < sm_count ? units : sm_count;
-  q.group_cost = !FWD && units > grid ? 1 : 0;   // about one position
+  q.group_cost = !FWD && units > grid ? 1 : 0;   // about one position (2: 4096 and 8192 0.5% slower)
   const int64_t total = units + q.group_cost * ngroups;
   q.span = total / grid;
   q.span_extra = (int)(total % grid);

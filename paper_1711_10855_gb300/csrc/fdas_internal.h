@@ -109,6 +109,27 @@ inline int wide_segments(int64_t nseg, int Z, int most, int sm_count) {
   return segs;
 }
 
+// group_cost of a full plane at 2048 whose units outnumber its CTAs: what a group's start,
+// its segments' copy and forward transforms, counts in units (10,000 cycles against 7,600 per position at
+// 2048), so that a CTA whose range enters a second group gets fewer templates.  2, unless that makes the
+// longest range longer than 1 does; 0 where equal ranges end with the groups.  With 1 throughout, a CTA of
+// two groups was the last one on planes of a few positions per CTA: 49,152 x 201 at 2048 30.2 us, now 28.7.
+inline int group_cost_of(int64_t units, int64_t ngroups, int64_t grid) {
+  if (units % grid == 0 && grid % ngroups == 0) return 0;
+  const auto longest = [&](int cost) { return (units + cost * ngroups + grid - 1) / grid; };
+  return longest(2) == longest(1) ? 2 : 1;
+}
+// First unit of CTA k in that count (span, span_extra: ConvParams), Z units per group.
+__host__ __device__ inline int64_t first_unit_of(int64_t k, int64_t span, int span_extra, int group_cost, int Z) {
+  const int64_t v = k * span + (k < span_extra ? k : span_extra);
+  if (group_cost == 0) return v;
+  const int per = Z + group_cost;
+  // 32-bit division where v fits
+  const int64_t g = (uint64_t)v <= 0xffffffffull ? (int64_t)((uint32_t)v / (uint32_t)per) : v / per;
+  const int64_t r = v - g * per - group_cost;
+  return g * Z + (r > 0 ? r : 0);
+}
+
 // Float offset of the real part of the twiddle exp(+i 2pi n2 k1 / L), n2 < N2 = 2*h2, k1 < n1, in the plan's
 // table (the imaginary part is 2 floats further): a float4 (re, re, im, im) holds n2 = j and j + h2.  The
 // kernels whose lanes own column pairs of the second pass (n1 <= h2: 256, 512 and 2048) read the pair of

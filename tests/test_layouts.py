@@ -87,6 +87,41 @@ int main() {
 }
 """
 
+SPLIT = r"""
+#include <cstdio>
+#include "fdas_internal.h"
+// Longest CTA in positions when every group's start but the CTA's first counts 1.3 of them.
+template <class First>
+double longest(int64_t grid, int Z, const First& first) {
+  double worst = 0;
+  for (int64_t k = 0; k < grid; ++k) {
+    const int64_t u0 = first(k), u1 = first(k + 1);
+    if (u1 <= u0) continue;
+    const double t = (double)(u1 - u0) + 1.3 * (double)((u1 - 1) / Z - u0 / Z);
+    if (t > worst) worst = t;
+  }
+  return worst;
+}
+int main() {
+  for (int64_t grid : {148, 152})
+    for (int64_t ng = 1; ng < 40; ++ng)
+      for (int Z = 1; Z <= 401; Z += 2) {
+        const int64_t units = ng * Z;
+        if (units <= grid) continue;
+        const int cost = fdas::group_cost_of(units, ng, grid);
+        const int64_t total = units + cost * ng, span = total / grid;
+        const int extra = (int)(total % grid);
+        auto first = [&](int64_t k) { return fdas::first_unit_of(k, span, extra, cost, Z); };
+        if (first(0) != 0 || first(grid) != units) return std::printf("ends: %ld x %d\n", (long)ng, Z), 1;
+        for (int64_t k = 0; k < grid; ++k)
+          if (first(k + 1) < first(k)) return std::printf("order: %ld x %d\n", (long)ng, Z), 1;
+        const double plain = longest(grid, Z, [&](int64_t k) { return k * units / grid; });
+        if (longest(grid, Z, first) > plain + 1e-9) return std::printf("longer: %ld x %d\n", (long)ng, Z), 1;
+      }
+  return 0;
+}
+"""
+
 
 def run(tmp_path, source):
     if not os.path.exists(NVCC):
@@ -110,3 +145,7 @@ def test_inference_weight_image_is_a_straight_copy(tmp_path):
 
 def test_fewest_segments_per_cta_while_every_unit_has_an_sm(tmp_path):
     run(tmp_path, SEGMENTS)
+
+
+def test_unit_split_is_never_longer_than_equal_ranges(tmp_path):
+    run(tmp_path, SPLIT)
