@@ -375,7 +375,8 @@ __global__ void __launch_bounds__(256) write_units_kernel(const uint16_t* masks,
 // N is (hop + 128)/4 and hop/4 columns instead of 32 channels, where an MMA's time no longer has
 // its floor of about 50 cycles: 24 MMAs of 80 and 64 cycles per layer for 512 positions, against 90
 // and 72 of 64 cycles with one tap, 128 positions and N = 32 each (kernel 330 to 176 us at 2^22
-// bins).  The zero blocks are a quarter of the multiply-adds.
+// bins).  The zero blocks are a quarter of the multiply-adds; their rows' lanes are switched off, since an
+// activation that overflowed FP16 times zero would be NaN where no tap reaches.
 // Activations sit in shared memory K-major "chunk-planar": channel chunk j (8 channels, 16 B) of row q at
 // plane j, offset 16*q, rows ordered (phase, column) for the layer that reads them.  h2 overwrites
 // h1 after the MMAs that read it.  While a group's layer-2 MMAs are issued (the issuing thread is held to
@@ -619,13 +620,19 @@ __global__ void __launch_bounds__(kProposeThreads, 1) propose_kernel(const Propo
     const uint64_t a0 = umma_desc(wts, kPlaneW, 128), b0 = umma_desc(aSlot, plane, 128);
     issued = take_token(token);
     if (!issued) return;
+    // D = 0: from row 384 of the stack on, its last three blocks and the next plane's first three are zero
+    const uint64_t zero = umma_desc(aW2 + 12 * kC * 16, kPlaneW, 128);
+    static_assert(N <= 6 * kC, "rows of zeros");
+    umma_f16(tm, zero, zero, umma_idesc_f16(128, N), 0u);
     static_for<12>([&](auto oo) {
       constexpr int o = decltype(oo)::value;
       static_for<2>([&](auto cc) {
         constexpr int c = decltype(cc)::value;
         const uint64_t ad = a0 + (uint64_t)((2u * c * kPlaneW + (11 - o) * kC * 16) >> 4);
         const uint64_t bd = b0 + (uint64_t)((2u * c * plane + ((o & 3) * rows_per_phase + D * (o >> 2)) * 16) >> 4);
-        umma_f16(tm, ad, bd, umma_idesc_f16(128, N), (o | c) != 0);
+        // the phases i for which o - i is no tap
+        constexpr uint32_t off = o < 3 ? (0xEu << o) & 0xFu : (o > 8 ? (1u << (o - 8)) - 1u : 0u);
+        umma_f16_lanes<off>(tm, ad, bd, umma_idesc_f16(128, N));
       });
     });
     umma_commit(bar);
