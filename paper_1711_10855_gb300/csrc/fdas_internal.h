@@ -242,7 +242,7 @@ __host__ __device__ inline int stack_at(int layer, int o, int i, int k) {
 
 struct NetState {
   NetLayout lay{0};
-  int W = 0, sm_count = 0;
+  int W = 0;
   float* p = nullptr;          // FP32 master parameters
   __half* ph = nullptr;        // FP16 copy for inference
   float* pr = nullptr;         // the FP16 copy's values as FP32
@@ -275,7 +275,7 @@ struct NetState {
 struct NetSizes {
   size_t act, pool, part1, sum1, part2, part3, gl, packs;
 };
-NetSizes net_sizes(int W, int Z, int max_batch, int sm_count);
+NetSizes net_sizes(int W, int Z, int max_batch);
 cudaError_t net_prepare();   // function attributes, once per created net
 // The copies (ph, pr, stack, packs) of the parameters p.
 void net_publish(const NetState& s, cudaStream_t st);

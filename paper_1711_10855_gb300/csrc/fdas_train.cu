@@ -19,7 +19,7 @@
 // 60-65% of the FP32 pipe; with every position in every layer, dense gradients and untiled loops it
 // took 3.46 ms.
 //
-// Every reduction has a fixed shape, so one seed gives one network.
+// Every reduction has a fixed shape, which no device property enters, so one seed gives one network.
 #include <cuda_fp16.h>
 #include <cuda_pipeline.h>
 #include <cuda_runtime.h>
@@ -39,6 +39,9 @@ constexpr int kWgUnit = 32;              // positions per unit of its work split
 constexpr int kWgHalo = 32;              // 8 taps x dilation 4
 constexpr int kWgPitch = kTile + kWgHalo + 4;   // floats; an odd number of 16-byte chunks
 constexpr int kWgBuffer = kC * (kWgPitch + kTile);
+// CTAs (and partial sums) of that gradient, at most: two for each of a GB300's 152 SMs, and as many on a device with
+// another count, so that the sums' order and with it a training run's bits do not depend on the device.
+constexpr int kWgCtas = 304;
 constexpr int kScatter = 640;            // positions of the layer-2 gradient built at a time
 constexpr int kL3Chunks = 32;            // window ranges of the layer-3 weight gradient
 constexpr int kHeadChunks = 4;           // window ranges of the head's gradient
@@ -50,9 +53,9 @@ __device__ __forceinline__ int padded(int pos) { return pos + (pos >> 4) * 4; }
 
 // Adds 9 taps of one input channel to acc[chunk][element][channel]: x0 = the thread's first chunk,
 // STEP floats between successive chunks (padding included where it is regular), w = 9 x 32 weights.
-template <int D>
 // Channels are paired (packed FP32x2): an FMA instruction then reads three register pairs in two cycles, where
 // scalar FMAs with three different registers issue at about 60%.
+template <int D>
 __device__ __forceinline__ void conv_channel(float2 (&acc)[4][4][2], const float* __restrict__ x0,
                                              const float* __restrict__ w, int og) {
   float4 wk[kK];
@@ -690,7 +693,7 @@ __global__ void __launch_bounds__(256) net_adam_kernel(const AdamArgs a) {
 int tiles_of(int n) { return (n + kTile - 1) / kTile; }
 int wg_ctas(const NetState& s, int B) {
   const int64_t units = (int64_t)B * ((s.W / 2 + 128) / kWgUnit);
-  return (int)(units < 2 * s.sm_count ? units : 2 * s.sm_count);
+  return (int)(units < kWgCtas ? units : kWgCtas);
 }
 Copies copies_of(const NetState& s) { return Copies{s.ph, s.pr, s.stack, s.packs, s.lay.W2, s.lay.W3}; }
 
@@ -735,13 +738,13 @@ HeadArgs head_args(const NetState& s, const float* params, float* logits) {
 
 }  // namespace
 
-NetSizes net_sizes(int W, int Z, int max_batch, int sm_count) {
+NetSizes net_sizes(int W, int Z, int max_batch) {
   NetSizes z;
   const size_t B = (size_t)max_batch;
   z.act = B * kC * (size_t)W;
   z.pool = B * tiles_of(W / 2) * kC;
   z.part1 = B * tiles_of(W / 2 + 160) * kW1Part;
-  z.part2 = (size_t)2 * sm_count * kC * kC * kK;
+  z.part2 = (size_t)kWgCtas * kC * kC * kK;
   z.part3 = (size_t)kL3Chunks * kL3Part;
   z.sum1 = (size_t)kW1Chunks * kW1Part;
   z.gl = (size_t)kHeadChunks * Z * (kC + 1);

@@ -868,9 +868,8 @@ fdas_zband* fdas_zband_create(int window, int n_out, int max_batch) {
   fdas::NetState& s = z->net;
   s.lay = Layout(n_out);
   s.W = window;
-  s.sm_count = sms;
   const size_t P = (size_t)s.lay.total, B = (size_t)max_batch;
-  const fdas::NetSizes n = fdas::net_sizes(window, n_out, max_batch, sms);
+  const fdas::NetSizes n = fdas::net_sizes(window, n_out, max_batch);
   bool ok = cudaMalloc(&s.p, P * 4) == cudaSuccess && cudaMalloc(&s.ph, P * 2) == cudaSuccess &&
             cudaMalloc(&s.pr, P * 4) == cudaSuccess && cudaMalloc(&s.packs, n.packs * 4) == cudaSuccess &&
             cudaMalloc(&s.stack, fdas::kStackHalves * 2) == cudaSuccess &&
