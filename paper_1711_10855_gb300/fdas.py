@@ -186,19 +186,28 @@ def _ptr(x) -> int:
     raise TypeError(f"cannot take a device pointer of {type(x)!r}")
 
 
-_raw_stream = None   # torch's (device) -> current stream handle, and its current-device query
+_raw_stream = None   # () -> handle of torch's current stream on its current device
+
+
+def _raw_stream_query():
+    """The raw handle where this torch has it (building a torch stream object for it costs more than the
+    launch's own bookkeeping), otherwise the public call's."""
+    import torch
+    torch.cuda.init()
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if raw is None:
+        return lambda: int(torch.cuda.current_stream().cuda_stream)
+    device = torch.cuda.current_device
+    return lambda: raw(device())
 
 
 def _stream(stream) -> int:
-    """Handle of a CUDA stream; None: the current stream of the current device (the raw handle: building a
-    torch stream object for it costs more than the launch's own bookkeeping)."""
+    """Handle of a CUDA stream; None: the current stream of the current device."""
     if stream is None:
         global _raw_stream
         if _raw_stream is None:
-            import torch
-            torch.cuda.init()
-            _raw_stream = (torch._C._cuda_getCurrentRawStream, torch.cuda.current_device)
-        return _raw_stream[0](_raw_stream[1]())
+            _raw_stream = _raw_stream_query()
+        return _raw_stream()
     if isinstance(stream, int):
         return stream
     return int(stream.cuda_stream)
