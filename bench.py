@@ -461,7 +461,7 @@ def run_zband(args):
     macs = ps.n_blocks * hop * (9 * 32 + 2 * 9 * 32 * 32) + ps.n_blocks * plan.n_z * 32
     tflops = 2.0 * macs / (propose_ms * 1e-3) / 1e12
     sms = torch.cuda.get_device_properties(dev).multi_processor_count
-    shape_tflops = 2.0 * 128 * 32 * 16 / 64 * sms * 2.07e9 / 1e12   # at the maximum SM clock
+    shape_cycles, shape_tflops = propose_mma_ceiling(hop, sms)
     dense_at = at(dense_points)
     line = {
         "metric": "effective f-fdot cells/s of the learned z-band proposal path (full-plane cells / path time)",
@@ -491,13 +491,11 @@ def run_zband(args):
                      "frac": tflops / float(peaks["bf16_tflops"]),
                      "peak_source": f"bf16_tflops burst ({peak_src}); FP16 dense rate equals BF16",
                      "flops_per_launch": 2.0 * macs, "traffic": zband_traffic(),
-                     # the layers' MMAs are M = 128, N = 32, K = 16: one occupies the tensor pipe ~64
-                     # cycles (a per-instruction floor below N = 128), a quarter of the dense rate
-                     "shape_peak": {"cycles_per_mma": 64, "tflops": shape_tflops,
+                     # what the kernel's own MMAs allow (zero blocks, halo and layer 1's padding count as no work)
+                     "shape_peak": {"cycles_per_block": shape_cycles, "tflops": shape_tflops,
                                     "frac": tflops / shape_tflops}},
-        # per step: median (init, three histogram passes, three digit kernels) and the fused
-        # inference (8), the pair list (3), the list check and the pair correlation (2)
-        "clocks": clk.summary(), "gpu_launches": args.steps * 9,   # median 3, inference, list 3, list check, correlation
+        # per step: median 3, inference, list 3, list check, correlation
+        "clocks": clk.summary(), "gpu_launches": args.steps * 9,
     }
     print(json.dumps(line), flush=True)
     net.close()
@@ -799,6 +797,18 @@ def tc_kernel_rev() -> str:
         with open(os.path.join(ROOT, "paper_1711_10855_gb300", "csrc", name), "rb") as f:
             h.update(f.read())
     return h.hexdigest()[:16]
+
+
+def propose_mma_ceiling(hop: int, sms: int, hz: float = 2.07e9) -> tuple[int, float]:
+    """(tensor-pipe cycles per block of `hop` positions, algorithmic TFLOP/s of a GPU whose tensor pipes did
+    nothing but the inference kernel's MMAs, at the maximum SM clock).  M = 128, K = 16 throughout; an MMA takes
+    N / 2 cycles, at least about 50.  Layer 1: one MMA of N = 32 per 128 of hop + 256
+    positions.  Layers 2 and 3: a clear and 12 tap offsets x 2 halves of the channels, N = (hop + 128) / 4
+    and hop / 4."""
+    mma = lambda n: max(50, n // 2)
+    cycles = (hop // 128 + 2) * mma(32) + 25 * (mma((hop + 128) // 4) + mma(hop // 4))
+    macs = hop * (9 * 32 + 2 * 9 * 32 * 32)
+    return cycles, 2.0 * macs / cycles * sms * hz / 1e12
 
 
 def zband_kernel_rev() -> str:
