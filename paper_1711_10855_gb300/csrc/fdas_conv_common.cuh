@@ -158,9 +158,4 @@ __device__ __forceinline__ void zero_outside(float2* seg, int64_t x0, int64_t n,
   for (int e = (hi > lo ? hi : lo) + lane; e < L; e += lanes) seg[e] = make_float2(0.f, 0.f);
 }
 
-// a / b for a >= 0, in 32 bits where a fits.
-__device__ __forceinline__ int64_t quotient(int64_t a, int b) {
-  return (uint64_t)a <= 0xffffffffull ? (int64_t)((uint32_t)a / (uint32_t)b) : a / b;
-}
-
 }  // namespace fdas

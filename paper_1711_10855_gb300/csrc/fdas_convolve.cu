@@ -212,7 +212,7 @@ __device__ __forceinline__ int64_t unit_total(const ListParams& p) { return p.un
 // First unit of CTA k.  The units are cut into equal ranges; one spectrum's groups count group_cost
 // units more each.  A batch's do not: its spectra have their own template counts, and its CTAs many positions.
 __device__ __forceinline__ int64_t first_unit(const BatchParams& p, unsigned k) {
-  return first_unit_of(k, p.span, p.span_extra, p.group_cost, p.single.Z);
+  return first_unit_of(p, p.single.Z, k);
 }
 
 // NV: pass-2 output rows n1 < NV can hold valid outputs (NV >= ceil(V / N2)); rows n1 >= NV are

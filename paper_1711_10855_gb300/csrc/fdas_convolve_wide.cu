@@ -145,12 +145,6 @@ __device__ __forceinline__ void exchange_pass2(cp2 (&v)[Cfg::H2], cp2 (&u)[Cfg::
   fft_split_pairs<Cfg::M, SIGN>(u);
 }
 
-// First unit of CTA k: the units are cut into equal ranges, every segment group counting group_cost
-// units more than its templates (what fetching and transforming its segments costs).
-__device__ __forceinline__ int64_t first_unit(const ConvParams& p, int Z, unsigned k) {
-  return first_unit_of(k, p.span, p.span_extra, p.group_cost, Z);
-}
-
 // Twiddle pairs of a lane (the plan's table holds exp(i 2pi n2 k1 / L) for n2 = j, j + H2 as pair j of
 // lane k1, contiguous over the lanes).  Split columns: that pair j.  Otherwise the pairs of k1 = 2 kappa,
 // 2 kappa + 1 of the lane's column n2, in slot order; N1 = N2 makes the table symmetric, so they are the
@@ -198,7 +192,7 @@ __global__ void __launch_bounds__(32 * Cfg::W, 1) fdas_convolve_wide_kernel(cons
   float4* tile = reinterpret_cast<float4*>(region);
 
   const int Z = FWD ? 1 : p.Z;
-  const int64_t u0 = first_unit(p, Z, blockIdx.x), u1 = first_unit(p, Z, blockIdx.x + 1);
+  const int64_t u0 = first_unit_of(p, Z, blockIdx.x), u1 = first_unit_of(p, Z, blockIdx.x + 1);
   const int64_t npos = u1 - u0;
   if (npos <= 0) return;
   int64_t grp = quotient(u0, Z);

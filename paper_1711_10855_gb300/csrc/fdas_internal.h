@@ -119,14 +119,19 @@ inline int group_cost_of(int64_t units, int64_t ngroups, int64_t grid) {
   const auto longest = [&](int cost) { return (units + cost * ngroups + grid - 1) / grid; };
   return longest(2) == longest(1) ? 2 : 1;
 }
-// First unit of CTA k in that count (span, span_extra: ConvParams), Z units per group.
-__host__ __device__ inline int64_t first_unit_of(int64_t k, int64_t span, int span_extra, int group_cost, int Z) {
-  const int64_t v = k * span + (k < span_extra ? k : span_extra);
-  if (group_cost == 0) return v;
-  const int per = Z + group_cost;
-  // 32-bit division where v fits
-  const int64_t g = (uint64_t)v <= 0xffffffffull ? (int64_t)((uint32_t)v / (uint32_t)per) : v / per;
-  const int64_t r = v - g * per - group_cost;
+// a / b for a >= 0, in 32 bits where a fits.
+__host__ __device__ __forceinline__ int64_t quotient(int64_t a, int b) {
+  return (uint64_t)a <= 0xffffffffull ? (int64_t)((uint32_t)a / (uint32_t)b) : a / b;
+}
+// First unit of CTA k in that count, Z units per group; p: a struct with span, span_extra and group_cost
+// (ConvParams, BatchParams).
+template <class P>
+__host__ __device__ __forceinline__ int64_t first_unit_of(const P& p, int Z, unsigned k) {
+  const int64_t v = (int64_t)k * p.span + (k < (unsigned)p.span_extra ? k : (unsigned)p.span_extra);
+  if (p.group_cost == 0) return v;
+  const int per = Z + p.group_cost;
+  const int64_t g = quotient(v, per);
+  const int64_t r = v - g * per - p.group_cost;
   return g * Z + (r > 0 ? r : 0);
 }
 

@@ -110,8 +110,8 @@ int main() {
         if (units <= grid) continue;
         const int cost = fdas::group_cost_of(units, ng, grid);
         const int64_t total = units + cost * ng, span = total / grid;
-        const int extra = (int)(total % grid);
-        auto first = [&](int64_t k) { return fdas::first_unit_of(k, span, extra, cost, Z); };
+        struct { int64_t span; int span_extra, group_cost; } split{span, (int)(total % grid), cost};
+        auto first = [&](int64_t k) { return fdas::first_unit_of(split, Z, (unsigned)k); };
         if (first(0) != 0 || first(grid) != units) return std::printf("ends: %ld x %d\n", (long)ng, Z), 1;
         for (int64_t k = 0; k < grid; ++k)
           if (first(k + 1) < first(k)) return std::printf("order: %ld x %d\n", (long)ng, Z), 1;
