@@ -324,7 +324,8 @@ typedef struct fdas_zband fdas_zband;
 /* window W: a multiple of 128 in [384, 65536] (the receptive field, +-84, must fit in a quarter
  * window); n_out = Z in [1, 65535]; max_batch windows per call in [1, 65535].  Requires a compute capability 10.3 device (current device).  NULL on
  * invalid arguments, another device, or allocation failure.  Parameters start at zero: set
- * them before use.  Device memory ~ 5 * max_batch * 32 * W floats. */
+ * them before use.  Device memory ~ max_batch * (3 * 32 * W + 320 * ceil((W/2 + 160) / 128)) floats and
+ * 12 MB of partial sums. */
 fdas_zband* fdas_zband_create(int window, int n_out, int max_batch);
 int fdas_zband_param_count(const fdas_zband* net);
 /* Host copies of the FP32 parameters (param_count floats).  Setting refreshes the FP16 copy and

@@ -102,7 +102,7 @@ cudaError_t launch_per_spectrum(const fdas_batch* b, const float* const* d_spect
     q.status = b->d_status;
     q.n_bins = d.n_bins;
     q.nseg = d.nseg;
-      q.Z = d.Z;
+    q.Z = d.Z;
     q.V = b->V;
     q.h = b->h;
     const cudaError_t e = fdas::launch_convolve(b->L, q, b->sm_count, st);

@@ -5,7 +5,7 @@
 //
 //   a2  bulk copies (cp.async.bulk) bring the part inside [0, n_bins) of each segment's L bins
 //       A[s*V - h .. s*V - h + L) into shared memory, the rest is zero-filled,
-//   a3  forward FFT of the segment, kept in shared memory for all Z templates,
+//   a3  forward FFT of the segment, kept in tensor memory for all Z templates,
 //   a4  for every template z: multiply by the template spectrum T_z (streamed from L2 into a
 //       ring of shared-memory slots by bulk copies),
 //   a5  inverse FFT,
@@ -30,8 +30,8 @@
 // 71.8k lane operations per 2048-point transform, 0.98 ms per 2^22 x 201 plane of which 1.31 ms is
 // measured (1.36 with separate products; DRAM writes at 38% of their rate).  L = 2048 holds 64 points a
 // lane (8 warps of 217 registers); L = 256 and 512 hold 32 (16 warps of 128, P = 2 warps per segment
-// on alternate templates: 3e6 x 51 at L = 512 takes 228 us against 240 with 8 warps, 1e6 x 17 at 256 35
-// against 45 with everything in shared memory).
+// on alternate templates: 3e6 x 51 at L = 512 takes 198 us against 244 with 8 warps and separate products,
+// 1e6 x 17 at 256 35 against 45 with everything in shared memory).
 #include <cstdio>
 #include <type_traits>
 

@@ -20,8 +20,13 @@
 // The FP32 pipe bounds the kernel: 32 points a lane let 1024 run 16 warps of 128 registers, 64 points
 // a lane 4096 and 8192 only 8, which wait at barriers and on the exchange together.  Measured, before
 // (1024: everything in shared memory; 4096, 8192: Stockham passes through it with a CTA barrier each)
-// and now: 3,000,004 x 101 at L = 1024, m = 256: 611, 482 us (pipe 68% busy); 2^21 x 401 at 4096, m = 1024:
-// 2822, 1844 us (58%); 1,500,012 x 401 at 8192, m = 2048: 3151, 1683 us (53%).
+// and now: 3,000,004 x 101 at L = 1024, m = 256: 611, 481 us; 2^21 x 401 at 4096, m = 1024: 2822, 1843 us (236
+// registers); 1,500,012 x 401 at 8192, m = 2048: 3151, 1626 us (255 registers, 20 bytes spilled).
+//
+// A CTA has room for 16 (1024), 4 or 2 segments.  On planes of few units it takes fewer (wide_segments), and
+// warps without a segment only keep the barriers and the ring going.  What remains of a single position is
+// straight-line code run once, from cold instruction caches: one template at 4096 takes 8 us of device time,
+// where a kernel of short loops with 256 threads per transform took 5 at twice the error.
 #include <cuda_runtime.h>
 
 #include "fdas_conv_common.cuh"

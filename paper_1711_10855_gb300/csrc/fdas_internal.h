@@ -96,9 +96,8 @@ struct SegParams {
   int V, h;
 };
 
-// Threads per transform group (N1) used for segment length L; the template bank and the
-// twiddle table are stored in the layout of that decomposition (element k = k1 + N1*k2 at
-// ((k2/2)*N1 + k1)*2 + k2%2).
+// Threads per transform group (N1) used for segment length L; the template bank is stored in the layout
+// of that decomposition (element k = k1 + N1*k2 at ((k2/2)*N1 + k1)*2 + k2%2).
 int conv_group_threads(int L);
 
 // Segments per group of a full plane at 1024, 4096 and 8192, at most `most` (those a CTA has room for): while

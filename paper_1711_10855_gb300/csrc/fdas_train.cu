@@ -42,6 +42,8 @@ constexpr int kWgBuffer = kC * (kWgPitch + kTile);
 // CTAs (and partial sums) of that gradient, at most: two for each of a GB300's 152 SMs, and as many on a device with
 // another count, so that the sums' order and with it a training run's bits do not depend on the device.
 constexpr int kWgCtas = 304;
+// The splits below were chosen on 256 windows of 1024 and hold for any size: longer batches lengthen their chains
+// of loads in proportion, as they do the convolutions, which stay most of a step (1024 windows: 1.09 ms, 256: 0.317).
 constexpr int kScatter = 640;            // positions of the layer-2 gradient built at a time
 constexpr int kL3Chunks = 32;            // window ranges of the layer-3 weight gradient
 constexpr int kHeadChunks = 4;           // window ranges of the head's gradient
