@@ -210,7 +210,8 @@ __device__ __forceinline__ int64_t unit_total(const BatchParams& p) { return p.u
 __device__ __forceinline__ int64_t unit_total(const ListParams& p) { return p.unit_count ? *p.unit_count : p.units; }
 
 // First unit of CTA k.  The units are cut into equal ranges; one spectrum's groups count group_cost
-// units more each.  A batch's do not: its spectra have their own template counts, and its CTAs many positions.
+// units more each.  A batch's do not: with a template count per spectrum the counted units would need a base of
+// their own in every descriptor.
 __device__ __forceinline__ int64_t first_unit(const BatchParams& p, unsigned k) {
   return first_unit_of(p, p.single.Z, k);
 }
@@ -886,6 +887,8 @@ using Tmem512 = TmemCfg<512, 16, 16, 2>;
 using Tmem512List = TmemCfg<512, 16>;
 using Tmem2048 = TmemCfg<2048, 32>;
 
+// Lengths with work lists and with batches in one launch.  256 runs the same kernel but has no work-list form,
+// which a non-zero count also promises: a batch there is one launch per spectrum, as at 1024, 4096 and 8192.
 int batch_segments_per_cta(int L) {
   switch (L) {
     case 512: return Tmem512::G;

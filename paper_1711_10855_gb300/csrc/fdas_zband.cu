@@ -160,8 +160,8 @@ __global__ void __launch_bounds__(256) select_pass_kernel(const float2* spec, in
   constexpr int per = NB / 256;
   __shared__ long long wsum[8];
   const int t = threadIdx.x, wid = t >> 5;
-  // through shared memory: a thread's own bins straight from L2 are a line per lane and load (8192 bins
-  // that way: a proposal over 160,000 bins took 47.1 us, now 43.1; over 113,356, 41.8 and 39.6); threads start at different words of their bins
+  // through shared memory: a thread's own bins straight from L2 are a line per lane and load (8192 bins that
+  // way cost a proposal over 160,000 bins 4 us); threads start at different words of their bins
 #pragma unroll
   for (int i = 0; i < per; ++i) h[t + 256 * i] = __ldcg(&hist[t + 256 * i]);
   __syncthreads();
@@ -373,7 +373,7 @@ __global__ void __launch_bounds__(256) write_units_kernel(const uint16_t* masks,
 // (zero where o - i is no tap) by the input rows of phase o mod 4 from column d (o div 4) on.  The
 // weight rows are kept once, as the stack [0 0 0 W_8 ... W_0 0 0 0]: offset o starts at its block 11 - o.
 // N is (hop + 128)/4 and hop/4 columns instead of 32 channels, where an MMA's time no longer has
-// its floor of about 50 cycles: 24 MMAs of 80 and 64 cycles per layer for 512 positions, against 90
+// its floor of about 50 cycles: 24 MMAs and a clear, of 80 and 64 cycles, per layer for 512 positions, against 90
 // and 72 of 64 cycles with one tap, 128 positions and N = 32 each (kernel 330 to 176 us at 2^22
 // bins).  The zero blocks are a quarter of the multiply-adds; their rows' lanes are switched off, since an
 // activation that overflowed FP16 times zero would be NaN where no tap reaches.
@@ -383,7 +383,7 @@ __global__ void __launch_bounds__(256) write_units_kernel(const uint16_t* masks,
 // their pace) its other seven warps do the previous block's head, and during layer 3 the next block's
 // staging and im2col; what is left between MMAs is the conversion of the two activation layers.  The
 // groups issue layers 2 and 3 one at a time (a token): left alone they fall into step, both in their MMAs
-// at half speed and then both outside (14.0k cycles per block and group; 12.5k with the token).
+// at half speed and then both outside (14.0k cycles per block and group; 12.5k with the token, before the clears).
 // ---------------------------------------------------------------------------------------
 constexpr int kMaxHop = 512;
 constexpr int kT1max = kMaxHop / 128 + 2;       // layer-1 M-tiles
